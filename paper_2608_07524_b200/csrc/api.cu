@@ -130,16 +130,32 @@ int device_info(DeviceInfo* out) {
 // zero-filled.  Consecutive tokens are row_stride elements apart (n_heads * head_dim when the tensor is
 // contiguous; more when it is a group of heads inside a wider tensor).
 int make_map(CUtensorMap* map, const void* base, int32_t total_tokens, int32_t n_heads, int32_t head_dim,
-             int64_t row_stride) {
+             int64_t row_stride, int box_rows = kTile) {
     EncodeTiledFn enc = encode_tiled_fn();
     if (!enc) return fail(DCP_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the CUDA driver");
     const cuuint64_t dims[3] = {(cuuint64_t)head_dim, (cuuint64_t)n_heads, (cuuint64_t)total_tokens};
     const cuuint64_t strides[2] = {(cuuint64_t)head_dim * 2, (cuuint64_t)row_stride * 2};
-    const cuuint32_t box[3] = {64, 1, (cuuint32_t)kTile};
+    const cuuint32_t box[3] = {64, 1, (cuuint32_t)box_rows};
     const cuuint32_t elem_strides[3] = {1, 1, 1};
     const CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box,
                            elem_strides, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) return fail(DCP_ERR_CUDA, "cuTensorMapEncodeTiled failed with CUresult %d", (int)r);
+    return DCP_OK;
+}
+
+// The per-query tiles of the backward, [tile * head][term][128 rows x 8] bf16, as (256, 2, 2 row halves, 2 terms per
+// tile and head): a box holds both terms of 64 rows, 1 KB each.
+int make_stats_map(CUtensorMap* map, const void* base, size_t n_tiles) {
+    EncodeTiledFn enc = encode_tiled_fn();
+    if (!enc) return fail(DCP_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the CUDA driver");
+    const cuuint64_t dims[4] = {256, 2, 2, (cuuint64_t)(2 * n_tiles)};
+    const cuuint64_t strides[3] = {512, 1024, 2048};
+    const cuuint32_t box[4] = {256, 2, 1, 2};
+    const cuuint32_t elem_strides[4] = {1, 1, 1, 1};
+    const CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, elem_strides,
+                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return fail(DCP_ERR_CUDA, "cuTensorMapEncodeTiled failed with CUresult %d", (int)r);
     return DCP_OK;
 }
@@ -270,7 +286,7 @@ static int attn_fwd_impl(const char* fn, bool merge, const void* q, const void* 
     {
         ScopedTimer t(DCP_KERNEL_PREP, stream);
         e = launch_prep(cu_seqlens, n_seqs, total_tokens, max_seqlen, kFwdRowsPerItem, n_heads, sched, bounds, UINT32_MAX,
-                        input_order, stream);
+                        input_order, INT32_MAX, stream);
     }
     if (e != cudaSuccess) return fail(DCP_ERR_CUDA, "%s: work-list kernel: %s", fn, cudaGetErrorString(e));
     g_launches.fetch_add(prep_launches(n_seqs, merge, input_order));
@@ -377,10 +393,12 @@ static int attn_bwd_impl(const char* fn, const void* q, const void* k, const voi
         return DCP_OK;
     }
     const bool input_order = g_input_order.load() != 0;
+    const bool pair = pair_path(head_dim, max_seqlen);
+    const int32_t direct_len = pair ? kPairDirectLen : kTile;      // longest sequence that is a single key block
     {
         ScopedTimer t(DCP_KERNEL_PREP, stream);
-        e = launch_prep(cu_seqlens, n_seqs, total_tokens, max_seqlen, kTile, n_heads, sched, bounds,
-                        (uint32_t)max_tiles(total_tokens, n_seqs), input_order, stream);
+        e = launch_prep(cu_seqlens, n_seqs, total_tokens, max_seqlen, pair ? 2 * kTile : kTile, n_heads, sched, bounds,
+                        (uint32_t)max_tiles(total_tokens, n_seqs), input_order, pair ? kTile + 1 : INT32_MAX, stream);
     }
     if (e != cudaSuccess) return fail(DCP_ERR_CUDA, "%s: work-list kernel: %s", fn, cudaGetErrorString(e));
     g_launches.fetch_add(prep_launches(n_seqs, true, input_order));
@@ -401,7 +419,7 @@ static int attn_bwd_impl(const char* fn, const void* q, const void* k, const voi
         e = launch_bwd_pre(static_cast<const __nv_bfloat16*>(o), static_cast<const __nv_bfloat16*>(d_o), lse, vcu,
                            sched, stats, dq_acc, max_tiles(total_tokens, n_seqs) * kTile * n_heads * padded_dim(head_dim),
                            total_tokens, n_heads, head_dim, token_stride,
-                           softmax_scale > 0.f ? softmax_scale : 1.0f / std::sqrt((float)head_dim), dev.sm_count, stream);
+                           softmax_scale > 0.f ? softmax_scale : 1.0f / std::sqrt((float)head_dim), direct_len, dev.sm_count, stream);
     }
     if (e != cudaSuccess) return fail(DCP_ERR_CUDA, "%s: pre kernel: %s", fn, cudaGetErrorString(e));
     g_launches.fetch_add(1);
@@ -421,8 +439,23 @@ static int attn_bwd_impl(const char* fn, const void* q, const void* k, const voi
     p.row_stride = token_stride;
     p.scale = softmax_scale > 0.f ? softmax_scale : 1.0f / std::sqrt((float)head_dim);
     p.scale_log2 = p.scale * 1.4426950408889634f;
+    PairMaps maps;
+    if (pair) {
+        maps.q = tq;
+        maps.k = tk;
+        maps.v = tv;
+        maps.d_o = tg;
+        if (int rc = make_map(&maps.q_rows, q, total_tokens, n_heads, head_dim, token_stride, 64)) return rc;
+        if (int rc = make_map(&maps.do_rows, d_o, total_tokens, n_heads, head_dim, token_stride, 64)) return rc;
+        if (int rc = make_stats_map(&maps.stats, stats, max_tiles(total_tokens, n_seqs) * n_heads)) return rc;
+    }
     {
         ScopedTimer t(DCP_KERNEL_BWD_MAIN, stream);
+        if (pair) {
+            e = launch_attn_bwd_pair(maps, p, head_dim, causal != 0, dev.sm_count, stream);
+            if (e != cudaSuccess) return fail(DCP_ERR_CUDA, "%s: pair kernel: %s", fn, cudaGetErrorString(e));
+            g_launches.fetch_add(1);
+        }
         e = launch_attn_bwd(tq, tk, tv, tg, tdk, tdv, p, head_dim, causal != 0, dev.sm_count, stream);
     }
     if (e != cudaSuccess) return fail(DCP_ERR_CUDA, "%s: main kernel: %s", fn, cudaGetErrorString(e));
@@ -431,7 +464,7 @@ static int attn_bwd_impl(const char* fn, const void* q, const void* k, const voi
     {
         ScopedTimer t(DCP_KERNEL_BWD_POST, stream);
         e = launch_bwd_post(dq_acc, static_cast<__nv_bfloat16*>(dq), vcu, sched, n_heads, head_dim, token_stride, p.scale,
-                            dev.sm_count, stream);
+                            direct_len, dev.sm_count, stream);
     }
     if (e != cudaSuccess) return fail(DCP_ERR_CUDA, "%s: post kernel: %s", fn, cudaGetErrorString(e));
     g_launches.fetch_add(1);

@@ -310,7 +310,8 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     tc_fence_after();
     const uint32_t tmem = sh.tmem_base;
     // when this CTA started and (at the end) when it ran out of work: the spread over CTAs measures the balance
-    if (tid == 0 && blockIdx.x < kMaxCtas) {
+    const bool record = p.sched.hdr->n_pair_items == 0;      // after the pair kernel the spans are that kernel's
+    if (record && tid == 0 && blockIdx.x < kMaxCtas) {
         p.sched.spans[1 * kMaxCtas + blockIdx.x].begin_ns = global_timer_ns();
         if (blockIdx.x == 0) p.sched.hdr->n_ctas[1] = gridDim.x < kMaxCtas ? gridDim.x : kMaxCtas;
     }
@@ -331,14 +332,14 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             tma_prefetch_desc(&tmap_v);
             tma_prefetch_desc(&tmap_do);
         }
-        const uint32_t n_items = p.sched.hdr->n_items;
+        const uint32_t n_items = p.sched.hdr->n_items, item0 = p.sched.hdr->n_pair_items;     // items before item0: the pair kernel
         uint32_t n_work = 0, g = 0;
         while (true) {
             const uint32_t slot = n_work & 1u;
             WorkItem w;
             if (lane == 0) {
                 if (n_work >= 2) mbar_wait(&sh.work_empty[slot], ((n_work >> 1) - 1) & 1u, guard);
-                const uint32_t item = atomicAdd(&p.sched.hdr->work_counter, 1u);
+                const uint32_t item = item0 + atomicAdd(&p.sched.hdr->work_counter, 1u);
                 if (item < n_items && !sh.abort_flag) {
                     w = decode_item(p.sched, p.cu_seqlens, item, kTile, p.n_heads, false);
                 } else {
@@ -707,7 +708,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
 
     tc_fence_before();
     __syncthreads();
-    if (tid == 0 && blockIdx.x < kMaxCtas) p.sched.spans[1 * kMaxCtas + blockIdx.x].end_ns = global_timer_ns();
+    if (record && tid == 0 && blockIdx.x < kMaxCtas) p.sched.spans[1 * kMaxCtas + blockIdx.x].end_ns = global_timer_ns();
     if (warp == 0) tmem_dealloc(tmem, 512);
 }
 

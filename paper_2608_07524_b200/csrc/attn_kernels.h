@@ -42,6 +42,17 @@ struct BwdParams {
     float scale_log2;
 };
 
+// Tensor maps of the pair kernel: boxes of 64 columns x 128 rows, of 64 rows for the `_rows` maps; `stats` views the
+// per-query tiles as (256, 2, 2, 2 * tiles * heads), so that one box holds both terms of 64 queries.
+struct PairMaps {
+    CUtensorMap q, q_rows, k, v, d_o, do_rows, stats;
+};
+
+// Sequences longer than one tile of a backward call whose head dimension is above 64 go to the pair kernel; a
+// sequence of at most kPairDirectLen tokens is a single work item there, which writes dQ itself.
+constexpr int kPairDirectLen = 2 * kTile;
+inline bool pair_path(int32_t head_dim, int32_t max_seqlen) { return head_dim > 64 && max_seqlen > kTile; }
+
 // Builds the work list (longest sequence first) and resets the work counter and status word.
 // With `bounds` non-null, short sequences are first merged into virtual sequences: sched.vcu and
 // `bounds` are written and the list is built over sched.vcu, which the later kernels must then be
@@ -50,10 +61,11 @@ int prep_launches(int32_t n_seqs, bool merge, bool input_order);   // kernels la
 // tile_capacity = number of 128-row tiles the per-tile storage of the workspace holds (UINT32_MAX if the
 // call uses none).  Inconsistent boundaries or more tiles than that leave an empty work list and
 // kStatusBadLengths in the status word.  input_order = true lists the sequences as they come instead of
-// longest first (a measurement aid: it shows what the ordering is worth).
+// longest first (a measurement aid: it shows what the ordering is worth).  Sequences of at least pair_min_len
+// tokens come first in either order, and their items are counted in the header (n_pair_items).
 cudaError_t launch_prep(const int32_t* cu_seqlens, int32_t n_seqs, int32_t total_tokens, int32_t max_seqlen,
                         int32_t rows_per_block, int32_t n_heads, const SchedView& sched, uint16_t* bounds,
-                        uint32_t tile_capacity, bool input_order, cudaStream_t stream);
+                        uint32_t tile_capacity, bool input_order, int32_t pair_min_len, cudaStream_t stream);
 
 // One CTA that waits, with the kernels' own bounded wait and the given poll limit, on a barrier nobody
 // arrives at, and leaves through the same abort path (status word raised, no trap).
@@ -70,11 +82,14 @@ cudaError_t launch_copy_segments(const void* src, void* dst, const int32_t* seg,
 cudaError_t launch_attn_fwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& to,
                             const FwdParams& p, int head_dim, bool causal, bool short_items, int n_ctas, cudaStream_t stream);
 
-// Tile-aligned row statistics for the backward kernel (see BwdParams::stats) and dq_acc = 0.
+// Tile-aligned row statistics for the backward kernel (see BwdParams::stats) and dq_acc = 0.  Sequences of at most
+// direct_len tokens get their dQ written by the main kernel: here and in the post kernel they have no accumulator.
 cudaError_t launch_bwd_pre(const __nv_bfloat16* o, const __nv_bfloat16* d_o, const float* lse, const int32_t* cu_seqlens,
                            const SchedView& sched, __nv_bfloat16* stats, float* dq_acc, size_t dq_acc_elems,
                            int32_t total_tokens, int32_t n_heads, int32_t head_dim, int64_t row_stride, float scale,
-                           int n_sms, cudaStream_t stream);
+                           int32_t direct_len, int n_sms, cudaStream_t stream);
+
+cudaError_t launch_attn_bwd_pair(const PairMaps& maps, const BwdParams& p, int head_dim, bool causal, int n_ctas, cudaStream_t stream);
 
 // tdk, tdv = maps over dk and dv: whole key blocks leave through shared memory and TMA stores.
 cudaError_t launch_attn_bwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tdo,
@@ -83,7 +98,7 @@ cudaError_t launch_attn_bwd(const CUtensorMap& tq, const CUtensorMap& tk, const 
 
 // dq[T, H, d] = bf16(scale * dq_acc), undoing the tile-blocked layout
 cudaError_t launch_bwd_post(const float* dq_acc, __nv_bfloat16* dq, const int32_t* cu_seqlens, const SchedView& sched,
-                            int32_t n_heads, int32_t head_dim, int64_t row_stride, float scale, int n_sms,
+                            int32_t n_heads, int32_t head_dim, int64_t row_stride, float scale, int32_t direct_len, int n_sms,
                             cudaStream_t stream);
 
 // Batches in which no sequence exceeds kSmallSeqMaxLen tokens (the declared max_seqlen says so) skip the work list

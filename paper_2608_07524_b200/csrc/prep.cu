@@ -208,7 +208,7 @@ __global__ void __launch_bounds__(kPrepThreads) prep_kernel(const int32_t* __res
                                                             int32_t rows_per_block, int32_t n_heads,
                                                             WorkspaceHeader* hdr, int32_t* order, uint32_t* prefix,
                                                             uint32_t* tile_prefix, int ranked, int32_t total_tokens,
-                                                            uint32_t tile_capacity) {
+                                                            uint32_t tile_capacity, int32_t pair_min_len) {
     __shared__ uint32_t scratch[33];
     __shared__ int32_t len_sh[kPrepThreads];
     const int tid = threadIdx.x;
@@ -222,12 +222,20 @@ __global__ void __launch_bounds__(kPrepThreads) prep_kernel(const int32_t* __res
         if (bad) {
             for (int i = tid; i <= n_seqs; i += kPrepThreads) { prefix[i] = 0; tile_prefix[i] = 0; }
             for (int i = tid; i < n_seqs; i += kPrepThreads) order[i] = i;
-            if (tid == 0) { hdr->n_items = 0; hdr->work_counter = 0; }
+            if (tid == 0) hdr->n_items = hdr->n_pair_items = hdr->work_counter = hdr->pair_counter = 0;
             return;
         }
     }
     if (ranked == 2) {
-        for (int i = tid; i < n_seqs; i += kPrepThreads) order[i] = i;
+        // input order, those of the pair kernel first
+        const int chunk = (n_live + kPrepThreads - 1) / kPrepThreads;
+        const int from = min(tid * chunk, n_live), to = min(from + chunk, n_live);
+        uint32_t n_long = 0, all_long = 0;
+        for (int i = from; i < to; ++i) n_long += cu[i + 1] - cu[i] >= pair_min_len ? 1u : 0u;
+        uint32_t at_long = block_exclusive_scan(n_long, scratch, &all_long);
+        uint32_t at_short = all_long + (uint32_t)from - at_long;
+        for (int i = from; i < to; ++i) order[cu[i + 1] - cu[i] >= pair_min_len ? at_long++ : at_short++] = i;
+        for (int i = n_live + tid; i < n_seqs; i += kPrepThreads) order[i] = i;
     } else if (!ranked) {                             // n_seqs <= kRankInKernelMax: one sequence per thread
         len_sh[tid] = tid < n_seqs ? cu[tid + 1] - cu[tid] : -1;
         __syncthreads();
@@ -253,15 +261,19 @@ __global__ void __launch_bounds__(kPrepThreads) prep_kernel(const int32_t* __res
     uint32_t local = 0, total = 0;
     for (int i = begin; i < end; ++i) local += items_of(i);
     uint32_t run = block_exclusive_scan(local, scratch, &total);
+    if (tid == 0) {
+        hdr->n_items = total;
+        hdr->work_counter = hdr->pair_counter = 0;
+        hdr->n_pair_items = 0;
+    }
+    __syncthreads();
+    auto in_pair = [&](int pos) { return pos < n_live && cu[order[pos] + 1] - cu[order[pos]] >= pair_min_len; };
     for (int i = begin; i < end; ++i) {
         prefix[i] = run;
         run += items_of(i);
+        if (in_pair(i) && !in_pair(i + 1)) hdr->n_pair_items = run;      // they come first in the order
     }
     for (int i = n_live + tid; i <= n_seqs; i += kPrepThreads) prefix[i] = total;
-    if (tid == 0) {
-        hdr->n_items = total;
-        hdr->work_counter = 0;
-    }
     // tile_prefix[b] = number of 128-row tiles of sequences 0..b-1 (input order): same two-level scan
     auto tiles_of = [&](int b) -> uint32_t { return (uint32_t)((cu[b + 1] - cu[b] + kTile - 1) / kTile); };
     local = 0;
@@ -272,7 +284,7 @@ __global__ void __launch_bounds__(kPrepThreads) prep_kernel(const int32_t* __res
         // relies on it).  Nothing may index the per-tile storage: no items, no tiles.
         for (int i = tid; i <= n_seqs; i += kPrepThreads) tile_prefix[i] = 0;
         if (tid == 0) {
-            hdr->n_items = 0;
+            hdr->n_items = hdr->n_pair_items = 0;
             atomicMax(&hdr->status, (uint32_t)kStatusBadLengths);
         }
         return;
@@ -290,7 +302,7 @@ int prep_launches(int32_t n_seqs, bool merge, bool input_order) {
 
 cudaError_t launch_prep(const int32_t* cu_seqlens, int32_t n_seqs, int32_t total_tokens, int32_t max_seqlen,
                         int32_t rows_per_block, int32_t n_heads, const SchedView& sched, uint16_t* bounds,
-                        uint32_t tile_capacity, bool input_order, cudaStream_t stream) {
+                        uint32_t tile_capacity, bool input_order, int32_t pair_min_len, cudaStream_t stream) {
     const int32_t* cu = cu_seqlens;
     const uint32_t* n_live = nullptr;
     if (bounds) {                                       // merge short sequences; everything below sees vcu
@@ -312,7 +324,8 @@ cudaError_t launch_prep(const int32_t* cu_seqlens, int32_t n_seqs, int32_t total
     }
     prep_kernel<<<1, kPrepThreads, 0, stream>>>(cu, n_seqs, n_live, rows_per_block, n_heads, sched.hdr,
                                                 const_cast<int32_t*>(sched.order), const_cast<uint32_t*>(sched.prefix),
-                                                const_cast<uint32_t*>(sched.tile_prefix), ranked, total_tokens, tile_capacity);
+                                                const_cast<uint32_t*>(sched.tile_prefix), ranked, total_tokens, tile_capacity,
+                                                pair_min_len);
     return cudaGetLastError();
 }
 
@@ -360,7 +373,7 @@ __global__ void __launch_bounds__(256) bwd_pre_kernel(const __nv_bfloat16* __res
                                                       int32_t n_seqs, __nv_bfloat16* __restrict__ stats,
                                                       float* __restrict__ dq_acc, size_t dq_acc_vec4,
                                                       int32_t total_tokens, int32_t n_heads, int32_t head_dim,
-                                                      int64_t row_stride, float inv_scale) {
+                                                      int64_t row_stride, float inv_scale, int32_t direct_len) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t n_blocks = tile_prefix[n_seqs] * (uint32_t)n_heads;
     for (uint32_t blk = blockIdx.x; blk < n_blocks; blk += gridDim.x) {
@@ -369,9 +382,9 @@ __global__ void __launch_bounds__(256) bwd_pre_kernel(const __nv_bfloat16* __res
         // this kernel slower: 0.39 -> 0.44 ms on 131072 tokens x 16 heads)
         const TileRef ref = find_tile(cu, tile_prefix, n_seqs, t);
         const int row0 = ref.row0, len = ref.len, tok0 = ref.tok0;
-        if (len > kTile) {
-            // this (tile, head) block of the dQ accumulator; a sequence of a single tile needs none (its
-            // one tile pair yields the whole dQ, which the main kernel writes directly)
+        if (len > direct_len) {
+            // this (tile, head) block of the dQ accumulator; a sequence of a single key block needs none (the main
+            // kernel holds its whole dQ and writes it directly)
             float4* acc_blk = reinterpret_cast<float4*>(dq_acc) + (size_t)blk * (kTile * D / 4);
             if ((size_t)(blk + 1) * (kTile * D / 4) <= dq_acc_vec4)
                 for (int e = threadIdx.x; e < kTile * D / 4; e += blockDim.x) acc_blk[e] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -448,16 +461,16 @@ __global__ void __launch_bounds__(256) bwd_pre_kernel(const __nv_bfloat16* __res
 cudaError_t launch_bwd_pre(const __nv_bfloat16* o, const __nv_bfloat16* d_o, const float* lse, const int32_t* cu_seqlens,
                            const SchedView& sched, __nv_bfloat16* stats, float* dq_acc, size_t dq_acc_elems,
                            int32_t total_tokens, int32_t n_heads, int32_t head_dim, int64_t row_stride, float scale,
-                           int n_sms, cudaStream_t stream) {
+                           int32_t direct_len, int n_sms, cudaStream_t stream) {
     const int blocks = n_sms * 8;
     if (head_dim > 64)
         bwd_pre_kernel<128><<<blocks, 256, 0, stream>>>(o, d_o, lse, cu_seqlens, sched.tile_prefix, sched.n_seqs, stats,
                                                         dq_acc, dq_acc_elems / 4, total_tokens, n_heads, head_dim,
-                                                        row_stride, 1.0f / scale);
+                                                        row_stride, 1.0f / scale, direct_len);
     else
         bwd_pre_kernel<64><<<blocks, 256, 0, stream>>>(o, d_o, lse, cu_seqlens, sched.tile_prefix, sched.n_seqs, stats,
                                                        dq_acc, dq_acc_elems / 4, total_tokens, n_heads, head_dim,
-                                                       row_stride, 1.0f / scale);
+                                                       row_stride, 1.0f / scale, direct_len);
     return cudaGetLastError();
 }
 
@@ -469,7 +482,7 @@ template <int D>
 __global__ void __launch_bounds__(256) bwd_post_kernel(const float* __restrict__ dq_acc, __nv_bfloat16* __restrict__ dq,
                                                        const int32_t* __restrict__ cu, const uint32_t* __restrict__ tile_prefix,
                                                        int32_t n_seqs, int32_t n_heads, int32_t head_dim, int64_t row_stride,
-                                                       float scale) {
+                                                       float scale, int32_t direct_len) {
     constexpr int kRowBytes = D * 2 + 16;                    // padded row of bf16
     __shared__ __align__(16) uint8_t tile[kTile * kRowBytes];
     const uint32_t n_blocks = tile_prefix[n_seqs] * (uint32_t)n_heads;
@@ -481,7 +494,7 @@ __global__ void __launch_bounds__(256) bwd_post_kernel(const float* __restrict__
         const uint32_t t_next = (blk + gridDim.x) / n_heads;
         const int row0 = ref.row0, len = ref.len;
         const int rows = min(kTile, len - row0);
-        if (len <= kTile) {               // a single tile pair: the main kernel has written dq itself
+        if (len <= direct_len) {          // a single key block: the main kernel has written dq itself
             if (more) ref_next = find_tile(cu, tile_prefix, n_seqs, t_next);
             continue;
         }
@@ -517,15 +530,15 @@ __global__ void __launch_bounds__(256) bwd_post_kernel(const float* __restrict__
 }
 
 cudaError_t launch_bwd_post(const float* dq_acc, __nv_bfloat16* dq, const int32_t* cu_seqlens, const SchedView& sched,
-                            int32_t n_heads, int32_t head_dim, int64_t row_stride, float scale, int n_sms,
+                            int32_t n_heads, int32_t head_dim, int64_t row_stride, float scale, int32_t direct_len, int n_sms,
                             cudaStream_t stream) {
     const int blocks = n_sms * 6;
     if (head_dim > 64)
         bwd_post_kernel<128><<<blocks, 256, 0, stream>>>(dq_acc, dq, cu_seqlens, sched.tile_prefix, sched.n_seqs, n_heads,
-                                                         head_dim, row_stride, scale);
+                                                         head_dim, row_stride, scale, direct_len);
     else
         bwd_post_kernel<64><<<blocks, 256, 0, stream>>>(dq_acc, dq, cu_seqlens, sched.tile_prefix, sched.n_seqs, n_heads,
-                                                        head_dim, row_stride, scale);
+                                                        head_dim, row_stride, scale, direct_len);
     return cudaGetLastError();
 }
 

@@ -44,7 +44,9 @@ struct WorkspaceHeader {
     uint32_t call_bad;      // this call's boundaries were inconsistent (reset by every call)
     uint32_t magic[2];      // kHeaderMagic0/1 once the header has been initialised
     uint32_t n_ctas[2];     // CTAs of the last forward / backward main launch that recorded a span
-    uint32_t pad[54];
+    uint32_t n_pair_items;  // the first items of the list, which the pair kernel takes (0 where it does not run)
+    uint32_t pair_counter;  // next unclaimed one of those
+    uint32_t pad[52];
 };
 static_assert(sizeof(WorkspaceHeader) == 256, "header is 256 bytes");
 

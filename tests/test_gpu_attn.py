@@ -385,6 +385,17 @@ def test_head_dims_between_the_native_ones(causal, d):
 
 
 
+@pytest.mark.parametrize("causal", [False, True])
+@pytest.mark.parametrize("d", [72, 112, 128])
+@pytest.mark.parametrize("lengths", [[129], [256], [257], [384, 385, 383], [200, 1, 255, 64, 64, 130, 0, 128, 511, 513, 640]],
+                         ids=lambda x: "-".join(map(str, x)))
+def test_backward_on_cta_pairs(causal, d, lengths):
+    """Head dimensions above 64 and sequences of more than 128 tokens: blocks of 256 keys over two CTAs.  Edges of the
+    block (its second half empty, one row, full), one block (dQ written directly) and more (accumulated), next to
+    sequences that the one-CTA kernel takes."""
+    check_full(lengths, 3, d, causal, seed=300 + len(lengths))
+
+
 def test_inconsistent_boundaries_are_reported_not_used():
     """cu_seqlens is device data the host never reads; the work-list kernels check it (starts at 0,
     never decreases, ends at total_tokens, fits the per-tile storage that max_seqlen promised) and, if
