@@ -463,8 +463,8 @@ static int attn_bwd_impl(const char* fn, const void* q, const void* k, const voi
 
     {
         ScopedTimer t(DCP_KERNEL_BWD_POST, stream);
-        e = launch_bwd_post(dq_acc, static_cast<__nv_bfloat16*>(dq), vcu, sched, n_heads, head_dim, token_stride, p.scale,
-                            direct_len, dev.sm_count, stream);
+        e = launch_bwd_post(dq_acc, static_cast<__nv_bfloat16*>(dq), vcu, sched, total_tokens, n_heads, head_dim, token_stride,
+                            p.scale, direct_len, dev.sm_count, stream);
     }
     if (e != cudaSuccess) return fail(DCP_ERR_CUDA, "%s: post kernel: %s", fn, cudaGetErrorString(e));
     g_launches.fetch_add(1);

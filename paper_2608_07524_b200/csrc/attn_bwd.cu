@@ -48,6 +48,7 @@
 #include <cuda_runtime.h>
 
 #include "attn_kernels.h"
+#include "launch.h"
 #include "sched.cuh"
 #include "sm100_ptx.cuh"
 
@@ -251,6 +252,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);     // via a shuffle: provably uniform within the warp
     const int lane = tid & 31;
     const WaitGuard guard{&sh.abort_flag, &p.sched.hdr->status};
+    grid_trigger();
 
     if (tid == 0) {
         for (int i = 0; i < 2; ++i) {
@@ -284,10 +286,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         sh.abort_flag = 0;
         fence_mbar_init();
         // the swizzled tile layout needs a 1024-byte aligned base; refuse to run otherwise
-        if ((smem_u32(smem) & 1023u) != 0) {
-            sh.abort_flag = 1;
-            atomicMax(&p.sched.hdr->status, (uint32_t)kStatusBadSmemAlign);
-        }
+        if ((smem_u32(smem) & 1023u) != 0) sh.abort_flag = 1;
     }
     if (warp == 0) {
         tmem_alloc(&sh.tmem_base, 512);
@@ -309,6 +308,8 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = sh.tmem_base;
+    grid_wait();
+    if (tid == 0 && sh.abort_flag) atomicMax(&p.sched.hdr->status, (uint32_t)kStatusBadSmemAlign);
     // when this CTA started and (at the end) when it ran out of work: the spread over CTAs measures the balance
     const bool record = p.sched.hdr->n_pair_items == 0;      // after the pair kernel the spans are that kernel's
     if (record && tid == 0 && blockIdx.x < kMaxCtas) {
@@ -715,11 +716,9 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
 template <int D, bool CAUSAL, bool TRIM>
 static cudaError_t launch_one(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tdo,
                               const CUtensorMap& tdk, const CUtensorMap& tdv, const BwdParams& p, int n_ctas, cudaStream_t stream) {
-    auto kern = attn_bwd_kernel<D, CAUSAL, TRIM>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdCfg<D>::kSmemBytes);
-    if (e != cudaSuccess) return e;
-    kern<<<n_ctas, kBwdThreads, BwdCfg<D>::kSmemBytes, stream>>>(tq, tk, tv, tdo, tdk, tdv, p);
-    return cudaGetLastError();
+    if (cudaError_t e = allow_smem<attn_bwd_kernel<D, CAUSAL, TRIM>>(BwdCfg<D>::kSmemBytes)) return e;
+    return launch_dependent(attn_bwd_kernel<D, CAUSAL, TRIM>, n_ctas, kBwdThreads, BwdCfg<D>::kSmemBytes, stream, tq, tk, tv, tdo, tdk,
+                            tdv, p);
 }
 
 cudaError_t launch_attn_bwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tdo,

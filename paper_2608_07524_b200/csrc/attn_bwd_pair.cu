@@ -50,6 +50,7 @@
 #include <cuda_runtime.h>
 
 #include "attn_kernels.h"
+#include "launch.h"
 #include "sched.cuh"
 #include "sm100_ptx.cuh"
 
@@ -153,6 +154,7 @@ attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constan
     // shared::cluster address of a barrier in the leader
     auto at_leader = [&](const uint64_t* bar) { return map_to_rank(smem_u32(bar), 0); };
 
+    grid_trigger();
     if (tid == 0) {
         for (int i = 0; i < kRing; ++i) {
             mbar_init(&sh.work_full[i], 1);
@@ -168,10 +170,7 @@ attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constan
         sh.abort_flag = 0;
         fence_mbar_init();
         mbar_expect_tx(&sh.ds_recv, kBoxBytes);          // armed one tile ahead by whoever waits on it
-        if ((smem_u32(smem) & 1023u) != 0) {             // the swizzled layouts need an aligned base; refuse to run otherwise
-            sh.abort_flag = 1;
-            atomicMax(&p.sched.hdr->status, (uint32_t)kStatusBadSmemAlign);
-        }
+        if ((smem_u32(smem) & 1023u) != 0) sh.abort_flag = 1;      // the swizzled layouts need an aligned base; refuse to run otherwise
     }
     {   // A operands of the rank-1 products, [128 keys x 16] in 8x8 core matrices, the two column halves 2 KB apart:
         // ones in columns 0-2 and nothing else (adds the lse term) starts at the first block, ones in columns 8-10 at the second
@@ -193,6 +192,8 @@ attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constan
     cluster_sync();                                      // the products write both CTAs' tensor memory
     tc_fence_after();
     const uint32_t tmem = sh.tmem_base;
+    grid_wait();
+    if (tid == 0 && sh.abort_flag) atomicMax(&p.sched.hdr->status, (uint32_t)kStatusBadSmemAlign);
     if (tid == 0 && blockIdx.x < kMaxCtas) {
         p.sched.spans[1 * kMaxCtas + blockIdx.x].begin_ns = global_timer_ns();
         if (blockIdx.x == 0) p.sched.hdr->n_ctas[1] = gridDim.x < kMaxCtas ? gridDim.x : kMaxCtas;
@@ -619,11 +620,8 @@ attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constan
 
 template <bool CAUSAL, bool TRIM>
 cudaError_t launch_one(const PairMaps& maps, const BwdParams& p, int n_ctas, cudaStream_t stream) {
-    auto kern = attn_bwd_pair_kernel<CAUSAL, TRIM>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-    if (e != cudaSuccess) return e;
-    kern<<<n_ctas & ~1, kPairThreads, kSmemBytes, stream>>>(maps, p);
-    return cudaGetLastError();
+    if (cudaError_t e = allow_smem<attn_bwd_pair_kernel<CAUSAL, TRIM>>(kSmemBytes)) return e;
+    return launch_dependent(attn_bwd_pair_kernel<CAUSAL, TRIM>, n_ctas & ~1, kPairThreads, kSmemBytes, stream, maps, p);
 }
 
 }  // namespace

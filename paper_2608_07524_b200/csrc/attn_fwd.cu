@@ -22,6 +22,7 @@
 #include <cuda_runtime.h>
 
 #include "attn_kernels.h"
+#include "launch.h"
 #include "sched.cuh"
 #include "sm100_ptx.cuh"
 
@@ -275,6 +276,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);     // via a shuffle: provably uniform within the warp
     const int lane = tid & 31;
     const WaitGuard guard{&sh.abort_flag, &p.sched.hdr->status};
+    grid_trigger();
 
     if (tid == 0) {
         for (int i = 0; i < 2; ++i) {
@@ -304,6 +306,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = sh.tmem_base;
+    grid_wait();
     // when this CTA started and (at the end) when it ran out of work: the spread over CTAs measures the balance
     if (tid == 0 && blockIdx.x < kMaxCtas) {
         p.sched.spans[0 * kMaxCtas + blockIdx.x].begin_ns = global_timer_ns();
@@ -626,11 +629,9 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
 template <int D, bool CAUSAL, bool EARLY_Q, bool TRIM>
 static cudaError_t launch_one(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& to,
                               const FwdParams& p, int n_ctas, cudaStream_t stream) {
-    auto kern = attn_fwd_kernel<D, CAUSAL, EARLY_Q, TRIM>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdCfg<D>::kSmemBytes);
-    if (e != cudaSuccess) return e;
-    kern<<<n_ctas, kFwdThreads, FwdCfg<D>::kSmemBytes, stream>>>(tq, tk, tv, to, p);
-    return cudaGetLastError();
+    if (cudaError_t e = allow_smem<attn_fwd_kernel<D, CAUSAL, EARLY_Q, TRIM>>(FwdCfg<D>::kSmemBytes)) return e;
+    return launch_dependent(attn_fwd_kernel<D, CAUSAL, EARLY_Q, TRIM>, n_ctas, kFwdThreads, FwdCfg<D>::kSmemBytes, stream, tq, tk, tv,
+                            to, p);
 }
 
 template <int D, bool TRIM>

@@ -98,8 +98,8 @@ cudaError_t launch_attn_bwd(const CUtensorMap& tq, const CUtensorMap& tk, const 
 
 // dq[T, H, d] = bf16(scale * dq_acc), undoing the tile-blocked layout
 cudaError_t launch_bwd_post(const float* dq_acc, __nv_bfloat16* dq, const int32_t* cu_seqlens, const SchedView& sched,
-                            int32_t n_heads, int32_t head_dim, int64_t row_stride, float scale, int32_t direct_len, int n_sms,
-                            cudaStream_t stream);
+                            int32_t total_tokens, int32_t n_heads, int32_t head_dim, int64_t row_stride, float scale,
+                            int32_t direct_len, int n_sms, cudaStream_t stream);
 
 // Batches in which no sequence exceeds kSmallSeqMaxLen tokens (the declared max_seqlen says so) skip the work list
 // and the 128-row tile kernels, see attn_small.cu.  The check kernel is the first of such a call (boundaries

@@ -31,6 +31,7 @@
 #include <cuda_runtime.h>
 
 #include "attn_kernels.h"
+#include "launch.h"
 #include "sm100_ptx.cuh"
 
 namespace dcp {
@@ -797,7 +798,16 @@ template <int DT, int NB, bool BWD>
 __global__ void __launch_bounds__(512, 1) small_attn_kernel(const SmallParams p) {
     extern __shared__ __align__(128) uint8_t smem[];
     constexpr int N_TILES = BWD ? 4 : 3;
-    if (p.hdr->call_bad) return;
+    grid_trigger();
+    grid_wait();
+    // one word per CTA of the check kernel; this is the first kernel that sees all of them
+    if (__syncthreads_or(threadIdx.x < kCheckCtas && p.hdr->check_bad[threadIdx.x] != 0)) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            p.hdr->call_bad = 1u;
+            atomicMax(&p.hdr->status, (uint32_t)kStatusBadLengths);
+        }
+        return;
+    }
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warps = blockDim.x >> 5;
     const StageLayout l = stage_layout(N_TILES, 16 * NB, DT ? DT : p.head_dim, BWD);
     const uint32_t zero = smem_u32(smem);
@@ -863,27 +873,31 @@ __global__ void __launch_bounds__(512, 1) small_attn_kernel(const SmallParams p)
 // never decrease, and no sequence may exceed the declared maximum; otherwise the status word says so and the
 // attention kernel computes nothing.  Then first_seq[c] = first sequence that starts at or after position
 // c * chunk, for c = 0 .. n_chunks.  `which` = 0 forward, 1 backward: no CTA time spans are recorded here.
+// Up to kCheckCtas CTAs (one CTA took 15 us on 20384 sequences): each leaves its finding in a word of its own, which the
+// attention kernel reads; where that does not run (no tokens) there is one CTA, which reports by itself.
 __global__ void __launch_bounds__(1024) small_check_kernel(const int32_t* __restrict__ cu, int32_t n_seqs, int32_t total_tokens,
                                                            int32_t max_len, int32_t chunk, int32_t n_chunks, int32_t* first_seq,
                                                            WorkspaceHeader* hdr, int which) {
-    int bad = (threadIdx.x == 0 && (cu[0] != 0 || cu[n_seqs] != total_tokens)) ? 1 : 0;
-    for (int i = threadIdx.x; i < n_seqs; i += 1024) {
-        const int32_t len = cu[i + 1] - cu[i];
-        bad |= (len < 0 || len > max_len) ? 1 : 0;
-    }
-    bad = __syncthreads_or(bad);
-    if (threadIdx.x == 0) {
-        header_begin_call(hdr, bad != 0);
-        hdr->n_ctas[which] = 0;
-    }
-    if (bad) return;
-    for (int i = threadIdx.x; i <= n_seqs; i += 1024) {
-        const int32_t here = cu[i], before = i > 0 ? cu[i - 1] : -1;
+    grid_trigger();
+    grid_wait();
+    int bad = (blockIdx.x == 0 && threadIdx.x == 0 && (cu[0] != 0 || cu[n_seqs] != total_tokens)) ? 1 : 0;
+    for (int i = blockIdx.x * 1024 + threadIdx.x; i <= n_seqs; i += gridDim.x * 1024) {
+        const int32_t before = i > 0 ? cu[i - 1] : -1, here = cu[i];
+        if (i > 0 && (here < before || here - before > max_len)) bad = 1;
+        if (before < -1 || here < before || here > total_tokens) continue;      // inconsistent, and not to be divided into chunks
         const int c_hi = min(here / chunk, n_chunks);
         for (int c = before < 0 ? 0 : before / chunk + 1; c <= c_hi; ++c) first_seq[c] = i;
     }
-    if (threadIdx.x == 0)
-        for (int c = total_tokens / chunk + 1; c <= n_chunks; ++c) first_seq[c] = n_seqs;
+    bad = __syncthreads_or(bad);
+    if (threadIdx.x == 0) {
+        hdr->check_bad[blockIdx.x] = bad ? 1u : 0u;
+        if (blockIdx.x == 0) {
+            for (int i = gridDim.x; i < kCheckCtas; ++i) hdr->check_bad[i] = 0u;
+            header_begin_call(hdr, bad != 0);
+            hdr->n_ctas[which] = 0;
+            for (int c = total_tokens / chunk + 1; c <= n_chunks; ++c) first_seq[c] = n_seqs;
+        }
+    }
 }
 
 // Token positions per chunk: 64, less for small batches so that every warp of the grid still gets a few items
@@ -912,9 +926,9 @@ bool small_path_fits(int32_t n_seqs, int32_t total_tokens, int32_t max_seqlen) {
 cudaError_t launch_small_check(bool backward, const int32_t* cu_seqlens, int32_t n_seqs, int32_t total_tokens, int32_t max_seqlen,
                                int32_t n_heads, WorkspaceHeader* hdr, int32_t* first_seq, int n_sms, cudaStream_t stream) {
     const int chunk = pick_chunk(total_tokens, n_heads, n_sms);
-    small_check_kernel<<<1, 1024, 0, stream>>>(cu_seqlens, n_seqs, total_tokens, max_seqlen, chunk, (total_tokens + chunk - 1) / chunk,
-                                               first_seq, hdr, backward ? 1 : 0);
-    return cudaGetLastError();
+    const int ctas = total_tokens == 0 ? 1 : n_seqs / 1024 + 1;
+    return launch_dependent(small_check_kernel, ctas < kCheckCtas ? ctas : kCheckCtas, 1024, 0, stream, cu_seqlens, n_seqs, total_tokens,
+                            max_seqlen, chunk, (total_tokens + chunk - 1) / chunk, first_seq, hdr, backward ? 1 : 0);
 }
 
 cudaError_t launch_small_attn(bool backward, const __nv_bfloat16* q, const __nv_bfloat16* k, const __nv_bfloat16* v,
@@ -954,20 +968,23 @@ cudaError_t launch_small_attn(bool backward, const __nv_bfloat16* q, const __nv_
     const size_t smem = kSmallHeaderBytes + (size_t)warps * p.stages * stage_layout(n_tiles, rows, head_dim, backward).stage_bytes;
     const long long n_items = (long long)p.n_chunks * n_heads;
     const unsigned grid = (unsigned)(n_items < (long long)n_sms * warps ? (n_items + warps - 1) / warps : n_sms);
-    auto launch = [&](auto kern) {
-        cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (err != cudaSuccess) return err;
-        kern<<<grid, 32 * warps, smem, stream>>>(p);
-        return cudaGetLastError();
-    };
-    const bool one = max_seqlen <= 16;
-#define DCP_SMALL_DISPATCH(DT)                                                                                      \
-    return backward ? (one ? launch(small_attn_kernel<DT, 1, true>) : launch(small_attn_kernel<DT, 2, true>))      \
-                    : (one ? launch(small_attn_kernel<DT, 1, false>) : launch(small_attn_kernel<DT, 2, false>))
-    if (head_dim == 128) { DCP_SMALL_DISPATCH(128); }
-    if (head_dim == 64) { DCP_SMALL_DISPATCH(64); }
-    if (head_dim == 72) { DCP_SMALL_DISPATCH(72); }      // the paper's 2-D model (Section 4.1)
+#define DCP_SMALL_LAUNCH(DT, NB, BWD)                                                                              \
+    do {                                                                                                          \
+        if (cudaError_t e = allow_smem<small_attn_kernel<DT, NB, BWD>>((int)kSmallSmemBudget)) return e;          \
+        return launch_dependent(small_attn_kernel<DT, NB, BWD>, grid, 32 * warps, smem, stream, p);               \
+    } while (0)
+#define DCP_SMALL_DISPATCH(DT)                                                                                     \
+    do {                                                                                                          \
+        if (rows == 16 && backward) DCP_SMALL_LAUNCH(DT, 1, true);                                                \
+        if (rows == 16) DCP_SMALL_LAUNCH(DT, 1, false);                                                           \
+        if (backward) DCP_SMALL_LAUNCH(DT, 2, true);                                                              \
+        DCP_SMALL_LAUNCH(DT, 2, false);                                                                           \
+    } while (0)
+    if (head_dim == 128) DCP_SMALL_DISPATCH(128);
+    if (head_dim == 64) DCP_SMALL_DISPATCH(64);
+    if (head_dim == 72) DCP_SMALL_DISPATCH(72);      // the paper's 2-D model (Section 4.1)
     DCP_SMALL_DISPATCH(0);
+#undef DCP_SMALL_LAUNCH
 #undef DCP_SMALL_DISPATCH
 }
 

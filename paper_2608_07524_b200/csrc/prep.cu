@@ -3,15 +3,18 @@
 #include <cuda_runtime.h>
 
 #include "attn_kernels.h"
+#include "launch.h"
 #include "sched.cuh"
+#include "sm100_ptx.cuh"
 
 namespace dcp {
 
-constexpr int kPrepThreads = 1024;
 constexpr int kRankInKernelMax = 256;     // above this many sequences the rank sort runs over several CTAs (rank_kernel)
+// The one-CTA kernels below have NT threads: 256 for batches of at most 256 sequences, whose time is the barriers and
+// dependent loads of a CTA (fewer warps, cheaper barriers), 1024 for larger ones.
 
-__device__ inline uint32_t block_exclusive_scan(uint32_t v, uint32_t* scratch, uint32_t* total);
-__device__ inline int block_exclusive_max_scan(int v, int* scratch);
+template <int NT> __device__ inline uint32_t block_exclusive_scan(uint32_t v, uint32_t* scratch, uint32_t* total);
+template <int NT> __device__ inline int block_exclusive_max_scan(int v, int* scratch);
 
 // Merging of short sequences into virtual sequences of at most 128 tokens.  One CTA.
 //
@@ -42,12 +45,14 @@ __device__ __forceinline__ bool merge_is_head(const int32_t* __restrict__ cu, in
     return cu[i - 1] / kTile != (cu[i + 1] - 1) / kTile;
 }
 
-__global__ void __launch_bounds__(kPrepThreads) merge_kernel(const int32_t* __restrict__ cu, int32_t n_seqs,
-                                                             int32_t total_tokens, int32_t max_short,
-                                                             WorkspaceHeader* hdr, int32_t* vcu, int32_t* vstart) {
+template <int NT>
+__global__ void __launch_bounds__(NT) merge_kernel(const int32_t* __restrict__ cu, int32_t n_seqs, int32_t total_tokens,
+                                                   int32_t max_short, WorkspaceHeader* hdr, int32_t* vcu, int32_t* vstart) {
     __shared__ uint32_t scratch[33];
+    grid_trigger();
+    grid_wait();
     const int tid = threadIdx.x;
-    const int per = (n_seqs + kPrepThreads - 1) / kPrepThreads;
+    const int per = (n_seqs + NT - 1) / NT;
     const int begin = min(tid * per, n_seqs), end = min(begin + per, n_seqs);
     // The boundaries come from the caller and index everything that follows: they must start at 0, never
     // decrease and end at total_tokens.  If not, the status word says so and every sequence is made empty,
@@ -57,7 +62,7 @@ __global__ void __launch_bounds__(kPrepThreads) merge_kernel(const int32_t* __re
     bad = __syncthreads_or(bad);
     if (tid == 0) header_begin_call(hdr, bad != 0);
     if (bad) {
-        for (int i = tid; i <= n_seqs; i += kPrepThreads) vcu[i] = 0;
+        for (int i = tid; i <= n_seqs; i += NT) vcu[i] = 0;
         if (tid == 0) hdr->n_vseq = 0;
         return;
     }
@@ -69,8 +74,8 @@ __global__ void __launch_bounds__(kPrepThreads) merge_kernel(const int32_t* __re
         empty |= cu[i + 1] == cu[i] ? 1 : 0;
     }
     empty = __syncthreads_or(empty);
-    const uint32_t run0 = block_exclusive_scan(local0, scratch, &n_v0);
-    const uint32_t run1 = block_exclusive_scan(local1, scratch, &n_v1);
+    const uint32_t run0 = block_exclusive_scan<NT>(local0, scratch, &n_v0);
+    const uint32_t run1 = block_exclusive_scan<NT>(local1, scratch, &n_v1);
     const uint32_t rule = (!empty && n_v1 < n_v0) ? 1u : 0u;
     const uint32_t n_v = rule ? n_v1 : n_v0;
     uint32_t run = rule ? run1 : run0;
@@ -84,9 +89,9 @@ __global__ void __launch_bounds__(kPrepThreads) merge_kernel(const int32_t* __re
             vcu[run++] = cu[i];
             last_head = i;
         }
-    for (uint32_t i = n_v + tid; i <= (uint32_t)n_seqs; i += kPrepThreads) vcu[i] = total_tokens;
+    for (uint32_t i = n_v + tid; i <= (uint32_t)n_seqs; i += NT) vcu[i] = total_tokens;
     // head of the run each sequence belongs to: the last head at or before it (sequence 0 is always one)
-    int cur = block_exclusive_max_scan(last_head, reinterpret_cast<int*>(scratch));
+    int cur = block_exclusive_max_scan<NT>(last_head, reinterpret_cast<int*>(scratch));
     for (int i = begin; i < end; ++i) {
         if (merge_is_head(cu, i, max_short, rule)) cur = i;
         vstart[i] = cu[cur];
@@ -99,6 +104,8 @@ __global__ void __launch_bounds__(kPrepThreads) merge_kernel(const int32_t* __re
 __global__ void __launch_bounds__(256) bounds_kernel(const int32_t* __restrict__ cu, int32_t n_seqs,
                                                      const WorkspaceHeader* __restrict__ hdr,
                                                      const int32_t* __restrict__ vstart, uint16_t* __restrict__ bounds) {
+    grid_trigger();
+    grid_wait();
     const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (i >= n_seqs || hdr->call_bad) return;      // merge_kernel found the boundaries inconsistent
     const int32_t a = cu[i], b = cu[i + 1];
@@ -117,6 +124,8 @@ __global__ void __launch_bounds__(256) bounds_kernel(const int32_t* __restrict__
 __global__ void __launch_bounds__(256) rank_kernel(const int32_t* __restrict__ cu, int32_t n_seqs,
                                                    const uint32_t* __restrict__ n_live_ptr, int32_t* order) {
     __shared__ int32_t len_tile[256];
+    grid_trigger();
+    grid_wait();
     const int n_live = n_live_ptr ? min((int)*n_live_ptr, n_seqs) : n_seqs;
     const int i = blockIdx.x * 256 + threadIdx.x;
     if ((int)blockIdx.x * 256 >= n_live) {             // a whole block of padding
@@ -139,8 +148,9 @@ __global__ void __launch_bounds__(256) rank_kernel(const int32_t* __restrict__ c
     if (i < n_seqs) order[rank] = i;
 }
 
-// Exclusive prefix sum of one value per thread over a CTA of kPrepThreads threads; *total receives
+// Exclusive prefix sum of one value per thread over a CTA of NT threads; *total receives
 // the sum.  scratch holds 33 words.
+template <int NT>
 __device__ inline uint32_t block_exclusive_scan(uint32_t v, uint32_t* scratch, uint32_t* total) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t incl = v;
@@ -153,7 +163,7 @@ __device__ inline uint32_t block_exclusive_scan(uint32_t v, uint32_t* scratch, u
     if (lane == 31) scratch[warp] = incl;
     __syncthreads();
     if (warp == 0) {
-        const uint32_t w = scratch[lane];
+        const uint32_t w = lane < NT / 32 ? scratch[lane] : 0u;
         uint32_t wi = w;
 #pragma unroll
         for (int s = 1; s < 32; s <<= 1) {
@@ -168,8 +178,9 @@ __device__ inline uint32_t block_exclusive_scan(uint32_t v, uint32_t* scratch, u
     return scratch[warp] + incl - v;
 }
 
-// Exclusive running maximum of one value per thread (in thread order) over a CTA of kPrepThreads
+// Exclusive running maximum of one value per thread (in thread order) over a CTA of NT
 // threads; -1 where nothing precedes.  scratch holds 33 words.
+template <int NT>
 __device__ inline int block_exclusive_max_scan(int v, int* scratch) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int incl = v;
@@ -182,7 +193,7 @@ __device__ inline int block_exclusive_max_scan(int v, int* scratch) {
     if (lane == 31) scratch[warp] = incl;
     __syncthreads();
     if (warp == 0) {
-        int wi = scratch[lane];
+        int wi = lane < NT / 32 ? scratch[lane] : -1;
 #pragma unroll
         for (int s = 1; s < 32; s <<= 1) {
             const int t = __shfl_up_sync(0xffffffffu, wi, s);
@@ -203,39 +214,40 @@ __device__ inline int block_exclusive_max_scan(int v, int* scratch) {
 // ceil(L / rows_per_block) * n_heads items; tile_prefix[b] = 128-row tiles before sequence b.
 // Sequences from *n_live_ptr on (if given) are empty padding and sorted last: only the live ones
 // are scanned, the rest get the totals.
-__global__ void __launch_bounds__(kPrepThreads) prep_kernel(const int32_t* __restrict__ cu, int32_t n_seqs,
-                                                            const uint32_t* __restrict__ n_live_ptr,
-                                                            int32_t rows_per_block, int32_t n_heads,
-                                                            WorkspaceHeader* hdr, int32_t* order, uint32_t* prefix,
-                                                            uint32_t* tile_prefix, int ranked, int32_t total_tokens,
-                                                            uint32_t tile_capacity, int32_t pair_min_len) {
+template <int NT>
+__global__ void __launch_bounds__(NT) prep_kernel(const int32_t* __restrict__ cu, int32_t n_seqs,
+                                                  const uint32_t* __restrict__ n_live_ptr, int32_t rows_per_block, int32_t n_heads,
+                                                  WorkspaceHeader* hdr, int32_t* order, uint32_t* prefix, uint32_t* tile_prefix,
+                                                  int ranked, int32_t total_tokens, uint32_t tile_capacity, int32_t pair_min_len) {
     __shared__ uint32_t scratch[33];
-    __shared__ int32_t len_sh[kPrepThreads];
+    __shared__ int32_t len_sh[NT];
+    grid_trigger();
+    grid_wait();
     const int tid = threadIdx.x;
     const int n_live = n_live_ptr ? min((int)*n_live_ptr, n_seqs) : n_seqs;
     if (!n_live_ptr) {
         // no merge_kernel ran before: check the caller's boundaries here (see merge_kernel)
         int bad = (tid == 0 && (cu[0] != 0 || cu[n_seqs] != total_tokens)) ? 1 : 0;
-        for (int i = tid; i < n_seqs; i += kPrepThreads) bad |= cu[i + 1] < cu[i] ? 1 : 0;
+        for (int i = tid; i < n_seqs; i += NT) bad |= cu[i + 1] < cu[i] ? 1 : 0;
         bad = __syncthreads_or(bad);
         if (tid == 0) header_begin_call(hdr, bad != 0);
         if (bad) {
-            for (int i = tid; i <= n_seqs; i += kPrepThreads) { prefix[i] = 0; tile_prefix[i] = 0; }
-            for (int i = tid; i < n_seqs; i += kPrepThreads) order[i] = i;
+            for (int i = tid; i <= n_seqs; i += NT) { prefix[i] = 0; tile_prefix[i] = 0; }
+            for (int i = tid; i < n_seqs; i += NT) order[i] = i;
             if (tid == 0) hdr->n_items = hdr->n_pair_items = hdr->work_counter = hdr->pair_counter = 0;
             return;
         }
     }
     if (ranked == 2) {
         // input order, those of the pair kernel first
-        const int chunk = (n_live + kPrepThreads - 1) / kPrepThreads;
+        const int chunk = (n_live + NT - 1) / NT;
         const int from = min(tid * chunk, n_live), to = min(from + chunk, n_live);
         uint32_t n_long = 0, all_long = 0;
         for (int i = from; i < to; ++i) n_long += cu[i + 1] - cu[i] >= pair_min_len ? 1u : 0u;
-        uint32_t at_long = block_exclusive_scan(n_long, scratch, &all_long);
+        uint32_t at_long = block_exclusive_scan<NT>(n_long, scratch, &all_long);
         uint32_t at_short = all_long + (uint32_t)from - at_long;
         for (int i = from; i < to; ++i) order[cu[i + 1] - cu[i] >= pair_min_len ? at_long++ : at_short++] = i;
-        for (int i = n_live + tid; i < n_seqs; i += kPrepThreads) order[i] = i;
+        for (int i = n_live + tid; i < n_seqs; i += NT) order[i] = i;
     } else if (!ranked) {                             // n_seqs <= kRankInKernelMax: one sequence per thread
         len_sh[tid] = tid < n_seqs ? cu[tid + 1] - cu[tid] : -1;
         __syncthreads();
@@ -251,7 +263,7 @@ __global__ void __launch_bounds__(kPrepThreads) prep_kernel(const int32_t* __res
     }
     __syncthreads();
     // exclusive scan of item counts over the sorted order: contiguous chunk per thread
-    const int per = (n_live + kPrepThreads - 1) / kPrepThreads;
+    const int per = (n_live + NT - 1) / NT;
     const int begin = min(tid * per, n_live), end = min(begin + per, n_live);
     auto items_of = [&](int pos) -> uint32_t {
         const int s = order[pos];
@@ -260,7 +272,7 @@ __global__ void __launch_bounds__(kPrepThreads) prep_kernel(const int32_t* __res
     };
     uint32_t local = 0, total = 0;
     for (int i = begin; i < end; ++i) local += items_of(i);
-    uint32_t run = block_exclusive_scan(local, scratch, &total);
+    uint32_t run = block_exclusive_scan<NT>(local, scratch, &total);
     if (tid == 0) {
         hdr->n_items = total;
         hdr->work_counter = hdr->pair_counter = 0;
@@ -273,16 +285,16 @@ __global__ void __launch_bounds__(kPrepThreads) prep_kernel(const int32_t* __res
         run += items_of(i);
         if (in_pair(i) && !in_pair(i + 1)) hdr->n_pair_items = run;      // they come first in the order
     }
-    for (int i = n_live + tid; i <= n_seqs; i += kPrepThreads) prefix[i] = total;
+    for (int i = n_live + tid; i <= n_seqs; i += NT) prefix[i] = total;
     // tile_prefix[b] = number of 128-row tiles of sequences 0..b-1 (input order): same two-level scan
     auto tiles_of = [&](int b) -> uint32_t { return (uint32_t)((cu[b + 1] - cu[b] + kTile - 1) / kTile); };
     local = 0;
     for (int i = begin; i < end; ++i) local += tiles_of(i);
-    run = block_exclusive_scan(local, scratch, &total);
+    run = block_exclusive_scan<NT>(local, scratch, &total);
     if (total > tile_capacity) {
         // more tiles than the workspace was sized for: max_seqlen was understated (the bound on merged runs
         // relies on it).  Nothing may index the per-tile storage: no items, no tiles.
-        for (int i = tid; i <= n_seqs; i += kPrepThreads) tile_prefix[i] = 0;
+        for (int i = tid; i <= n_seqs; i += NT) tile_prefix[i] = 0;
         if (tid == 0) {
             hdr->n_items = hdr->n_pair_items = 0;
             atomicMax(&hdr->status, (uint32_t)kStatusBadLengths);
@@ -293,7 +305,7 @@ __global__ void __launch_bounds__(kPrepThreads) prep_kernel(const int32_t* __res
         tile_prefix[i] = run;
         run += tiles_of(i);
     }
-    for (int i = n_live + tid; i <= n_seqs; i += kPrepThreads) tile_prefix[i] = total;
+    for (int i = n_live + tid; i <= n_seqs; i += NT) tile_prefix[i] = total;
 }
 
 int prep_launches(int32_t n_seqs, bool merge, bool input_order) {
@@ -305,28 +317,29 @@ cudaError_t launch_prep(const int32_t* cu_seqlens, int32_t n_seqs, int32_t total
                         uint32_t tile_capacity, bool input_order, int32_t pair_min_len, cudaStream_t stream) {
     const int32_t* cu = cu_seqlens;
     const uint32_t* n_live = nullptr;
+    const bool small = n_seqs <= 256;
     if (bounds) {                                       // merge short sequences; everything below sees vcu
         const int32_t max_short = max_seqlen < kMergeMaxLen ? (max_seqlen > 0 ? max_seqlen : 1) : kMergeMaxLen;
         // order[] is not needed until the ranking below: until then it carries each sequence's run start
-        merge_kernel<<<1, kPrepThreads, 0, stream>>>(cu_seqlens, n_seqs, total_tokens, max_short, sched.hdr,
-                                                     const_cast<int32_t*>(sched.vcu), const_cast<int32_t*>(sched.order));
-        if (cudaError_t e = cudaGetLastError()) return e;
+        int32_t* vstart = const_cast<int32_t*>(sched.order);
+        if (cudaError_t e = launch_dependent(small ? merge_kernel<256> : merge_kernel<1024>, 1, small ? 256 : 1024, 0, stream, cu_seqlens,
+                                             n_seqs, total_tokens, max_short, sched.hdr, const_cast<int32_t*>(sched.vcu), vstart))
+            return e;
         if (n_seqs > 0)
-            bounds_kernel<<<(n_seqs + 7) / 8, 256, 0, stream>>>(cu_seqlens, n_seqs, sched.hdr, sched.order, bounds);
-        if (cudaError_t e = cudaGetLastError()) return e;
+            if (cudaError_t e = launch_dependent(bounds_kernel, (n_seqs + 7) / 8, 256, 0, stream, cu_seqlens, n_seqs, sched.hdr, vstart,
+                                                 bounds))
+                return e;
         cu = sched.vcu;
         n_live = &sched.hdr->n_vseq;
     }
     const int ranked = input_order ? 2 : (n_seqs > kRankInKernelMax ? 1 : 0);
-    if (ranked == 1) {
-        rank_kernel<<<(n_seqs + 255) / 256, 256, 0, stream>>>(cu, n_seqs, n_live, const_cast<int32_t*>(sched.order));
-        if (cudaError_t e = cudaGetLastError()) return e;
-    }
-    prep_kernel<<<1, kPrepThreads, 0, stream>>>(cu, n_seqs, n_live, rows_per_block, n_heads, sched.hdr,
-                                                const_cast<int32_t*>(sched.order), const_cast<uint32_t*>(sched.prefix),
-                                                const_cast<uint32_t*>(sched.tile_prefix), ranked, total_tokens, tile_capacity,
-                                                pair_min_len);
-    return cudaGetLastError();
+    if (ranked == 1)
+        if (cudaError_t e = launch_dependent(rank_kernel, (n_seqs + 255) / 256, 256, 0, stream, cu, n_seqs, n_live,
+                                             const_cast<int32_t*>(sched.order)))
+            return e;
+    return launch_dependent(small ? prep_kernel<256> : prep_kernel<1024>, 1, small ? 256 : 1024, 0, stream, cu, n_seqs, n_live,
+                            rows_per_block, n_heads, sched.hdr, const_cast<int32_t*>(sched.order), const_cast<uint32_t*>(sched.prefix),
+                            const_cast<uint32_t*>(sched.tile_prefix), ranked, total_tokens, tile_capacity, pair_min_len);
 }
 
 // The sequence that owns 128-row tile t: (sequence, first row of the tile inside it, its length, its first token).
@@ -374,6 +387,8 @@ __global__ void __launch_bounds__(256) bwd_pre_kernel(const __nv_bfloat16* __res
                                                       float* __restrict__ dq_acc, size_t dq_acc_vec4,
                                                       int32_t total_tokens, int32_t n_heads, int32_t head_dim,
                                                       int64_t row_stride, float inv_scale, int32_t direct_len) {
+    grid_trigger();
+    grid_wait();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t n_blocks = tile_prefix[n_seqs] * (uint32_t)n_heads;
     for (uint32_t blk = blockIdx.x; blk < n_blocks; blk += gridDim.x) {
@@ -462,16 +477,12 @@ cudaError_t launch_bwd_pre(const __nv_bfloat16* o, const __nv_bfloat16* d_o, con
                            const SchedView& sched, __nv_bfloat16* stats, float* dq_acc, size_t dq_acc_elems,
                            int32_t total_tokens, int32_t n_heads, int32_t head_dim, int64_t row_stride, float scale,
                            int32_t direct_len, int n_sms, cudaStream_t stream) {
-    const int blocks = n_sms * 8;
-    if (head_dim > 64)
-        bwd_pre_kernel<128><<<blocks, 256, 0, stream>>>(o, d_o, lse, cu_seqlens, sched.tile_prefix, sched.n_seqs, stats,
-                                                        dq_acc, dq_acc_elems / 4, total_tokens, n_heads, head_dim,
-                                                        row_stride, 1.0f / scale, direct_len);
-    else
-        bwd_pre_kernel<64><<<blocks, 256, 0, stream>>>(o, d_o, lse, cu_seqlens, sched.tile_prefix, sched.n_seqs, stats,
-                                                       dq_acc, dq_acc_elems / 4, total_tokens, n_heads, head_dim,
-                                                       row_stride, 1.0f / scale, direct_len);
-    return cudaGetLastError();
+    // no more CTAs than (tile, head) blocks the batch can have
+    const size_t most = max_tiles(total_tokens, sched.n_seqs) * (size_t)n_heads;
+    const unsigned blocks = most < (size_t)n_sms * 8 ? (unsigned)most : (unsigned)n_sms * 8;
+    return launch_dependent(head_dim > 64 ? bwd_pre_kernel<128> : bwd_pre_kernel<64>, blocks, 256, 0, stream, o, d_o, lse, cu_seqlens,
+                            sched.tile_prefix, sched.n_seqs, stats, dq_acc, dq_acc_elems / 4, total_tokens, n_heads, head_dim, row_stride,
+                            1.0f / scale, direct_len);
 }
 
 // Backward helper 2: dq[T, H, d] = bf16(scale * dq_acc).  dq_acc holds, per (tile, head), a block
@@ -485,6 +496,8 @@ __global__ void __launch_bounds__(256) bwd_post_kernel(const float* __restrict__
                                                        float scale, int32_t direct_len) {
     constexpr int kRowBytes = D * 2 + 16;                    // padded row of bf16
     __shared__ __align__(16) uint8_t tile[kTile * kRowBytes];
+    grid_trigger();
+    grid_wait();
     const uint32_t n_blocks = tile_prefix[n_seqs] * (uint32_t)n_heads;
     if (blockIdx.x >= n_blocks) return;
     TileRef ref = find_tile(cu, tile_prefix, n_seqs, blockIdx.x / n_heads), ref_next = ref;
@@ -530,16 +543,12 @@ __global__ void __launch_bounds__(256) bwd_post_kernel(const float* __restrict__
 }
 
 cudaError_t launch_bwd_post(const float* dq_acc, __nv_bfloat16* dq, const int32_t* cu_seqlens, const SchedView& sched,
-                            int32_t n_heads, int32_t head_dim, int64_t row_stride, float scale, int32_t direct_len, int n_sms,
-                            cudaStream_t stream) {
-    const int blocks = n_sms * 6;
-    if (head_dim > 64)
-        bwd_post_kernel<128><<<blocks, 256, 0, stream>>>(dq_acc, dq, cu_seqlens, sched.tile_prefix, sched.n_seqs, n_heads,
-                                                         head_dim, row_stride, scale, direct_len);
-    else
-        bwd_post_kernel<64><<<blocks, 256, 0, stream>>>(dq_acc, dq, cu_seqlens, sched.tile_prefix, sched.n_seqs, n_heads,
-                                                        head_dim, row_stride, scale, direct_len);
-    return cudaGetLastError();
+                            int32_t total_tokens, int32_t n_heads, int32_t head_dim, int64_t row_stride, float scale,
+                            int32_t direct_len, int n_sms, cudaStream_t stream) {
+    const size_t most = max_tiles(total_tokens, sched.n_seqs) * (size_t)n_heads;
+    const unsigned blocks = most < (size_t)n_sms * 6 ? (unsigned)most : (unsigned)n_sms * 6;
+    return launch_dependent(head_dim > 64 ? bwd_post_kernel<128> : bwd_post_kernel<64>, blocks, 256, 0, stream, dq_acc, dq, cu_seqlens,
+                            sched.tile_prefix, sched.n_seqs, n_heads, head_dim, row_stride, scale, direct_len);
 }
 
 }  // namespace dcp

@@ -34,6 +34,7 @@ enum : uint32_t {
 // initialisation by the caller: the first kernel of a call that does not find `magic` treats the
 // header as fresh memory and clears the status word itself.
 constexpr uint32_t kHeaderMagic0 = 0x64637031u, kHeaderMagic1 = 0x9e3779b9u;
+constexpr int kCheckCtas = 16;        // CTAs of the short-sequence path's check kernel, at most
 constexpr int kMaxCtas = 256;         // persistent CTAs whose time span the header area can record
 struct WorkspaceHeader {
     uint32_t status;        // 0 = ok, else the highest kStatus* code a kernel has left since the last query
@@ -46,7 +47,8 @@ struct WorkspaceHeader {
     uint32_t n_ctas[2];     // CTAs of the last forward / backward main launch that recorded a span
     uint32_t n_pair_items;  // the first items of the list, which the pair kernel takes (0 where it does not run)
     uint32_t pair_counter;  // next unclaimed one of those
-    uint32_t pad[52];
+    uint32_t check_bad[16]; // short-sequence path: whether a CTA of the check kernel found this call's boundaries inconsistent
+    uint32_t pad[36];
 };
 static_assert(sizeof(WorkspaceHeader) == 256, "header is 256 bytes");
 
