@@ -209,6 +209,13 @@ bool short_sequence_path(int32_t n_seqs, int32_t total_tokens, int32_t max_seqle
 // Batches whose longest sequence has at most this many tokens (64 key tiles) run the forward variant for short items.
 constexpr int32_t kShortItemMaxLen = 8192;
 
+// Whether a call's single-tile work items (after merging) run on the kernels of attn_tile.cu, beside the multi-tile kernel
+// if there may be longer sequences.  A second launch costs 3 us, so it takes more of those items than the multi-tile
+// kernel's CTAs can have in flight anyway, and a batch that is mostly such items as far as the sizes tell.
+bool split_tiles(int32_t n_seqs, int32_t total_tokens, int32_t max_seqlen, int32_t n_heads, int n_sms) {
+    return max_seqlen <= kTile || ((int64_t)n_seqs * n_heads >= 2 * n_sms && total_tokens <= (int64_t)n_seqs * 4 * kTile);
+}
+
 // The kernels work on 64 or 128 columns per head; other head dimensions run zero-padded to the next of the two.
 size_t padded_dim(int32_t head_dim) { return head_dim <= 64 ? 64 : 128; }
 
@@ -283,10 +290,11 @@ static int attn_fwd_impl(const char* fn, bool merge, const void* q, const void* 
         return DCP_OK;
     }
     const bool input_order = g_input_order.load() != 0;
+    const bool split = split_tiles(n_seqs, total_tokens, max_seqlen, n_heads, dev.sm_count);
     {
         ScopedTimer t(DCP_KERNEL_PREP, stream);
         e = launch_prep(cu_seqlens, n_seqs, total_tokens, max_seqlen, kFwdRowsPerItem, n_heads, sched, bounds, UINT32_MAX,
-                        input_order, INT32_MAX, stream);
+                        input_order, split ? kTile + 1 : INT32_MAX, max_seqlen <= kTile, stream);
     }
     if (e != cudaSuccess) return fail(DCP_ERR_CUDA, "%s: work-list kernel: %s", fn, cudaGetErrorString(e));
     g_launches.fetch_add(prep_launches(n_seqs, merge, input_order));
@@ -310,12 +318,20 @@ static int attn_fwd_impl(const char* fn, bool merge, const void* q, const void* 
     p.row_stride = token_stride;
     p.scale = scale;
     p.scale_log2 = p.scale * 1.4426950408889634f;
+    p.split = split;
     {
         ScopedTimer t(DCP_KERNEL_FWD, stream);
-        e = launch_attn_fwd(tq, tk, tv, to, p, head_dim, causal != 0, max_seqlen <= kShortItemMaxLen, dev.sm_count, stream);
+        if (max_seqlen > kTile || !split) {
+            e = launch_attn_fwd(tq, tk, tv, to, p, head_dim, causal != 0, max_seqlen <= kShortItemMaxLen, dev.sm_count, stream);
+            if (e != cudaSuccess) return fail(DCP_ERR_CUDA, "%s: attention kernel: %s", fn, cudaGetErrorString(e));
+            g_launches.fetch_add(1);
+        }
+        if (split) {
+            e = launch_tile_fwd(tq, tk, tv, p, causal != 0, dev.sm_count, stream);
+            if (e != cudaSuccess) return fail(DCP_ERR_CUDA, "%s: single-tile kernel: %s", fn, cudaGetErrorString(e));
+            g_launches.fetch_add(1);
+        }
     }
-    if (e != cudaSuccess) return fail(DCP_ERR_CUDA, "%s: attention kernel: %s", fn, cudaGetErrorString(e));
-    g_launches.fetch_add(1);
     return DCP_OK;
 }
 
@@ -393,12 +409,14 @@ static int attn_bwd_impl(const char* fn, const void* q, const void* k, const voi
         return DCP_OK;
     }
     const bool input_order = g_input_order.load() != 0;
-    const bool pair = pair_path(head_dim, max_seqlen);
+    const bool pair = pair_path(head_dim);
     const int32_t direct_len = pair ? kPairDirectLen : kTile;      // longest sequence that is a single key block
+    const bool split = pair || split_tiles(n_seqs, total_tokens, max_seqlen, n_heads, dev.sm_count);
+    const bool multi = max_seqlen > kTile || !split;               // there may be items for the multi-tile kernel
     {
         ScopedTimer t(DCP_KERNEL_PREP, stream);
         e = launch_prep(cu_seqlens, n_seqs, total_tokens, max_seqlen, pair ? 2 * kTile : kTile, n_heads, sched, bounds,
-                        (uint32_t)max_tiles(total_tokens, n_seqs), input_order, pair ? kTile + 1 : INT32_MAX, stream);
+                        (uint32_t)max_tiles(total_tokens, n_seqs), input_order, split ? kTile + 1 : INT32_MAX, !multi, stream);
     }
     if (e != cudaSuccess) return fail(DCP_ERR_CUDA, "%s: work-list kernel: %s", fn, cudaGetErrorString(e));
     g_launches.fetch_add(prep_launches(n_seqs, true, input_order));
@@ -410,19 +428,16 @@ static int attn_bwd_impl(const char* fn, const void* q, const void* k, const voi
     if (int rc = make_map(&tk, k, total_tokens, n_heads, head_dim, token_stride)) return rc;
     if (int rc = make_map(&tv, v, total_tokens, n_heads, head_dim, token_stride)) return rc;
     if (int rc = make_map(&tg, d_o, total_tokens, n_heads, head_dim, token_stride)) return rc;
-    CUtensorMap tdk, tdv;
-    if (int rc = make_map(&tdk, dk, total_tokens, n_heads, head_dim, token_stride)) return rc;
-    if (int rc = make_map(&tdv, dv, total_tokens, n_heads, head_dim, token_stride)) return rc;
+    const float scale = softmax_scale > 0.f ? softmax_scale : 1.0f / std::sqrt((float)head_dim);
 
-    {
+    if (multi) {
         ScopedTimer t(DCP_KERNEL_BWD_PRE, stream);
         e = launch_bwd_pre(static_cast<const __nv_bfloat16*>(o), static_cast<const __nv_bfloat16*>(d_o), lse, vcu,
                            sched, stats, dq_acc, max_tiles(total_tokens, n_seqs) * kTile * n_heads * padded_dim(head_dim),
-                           total_tokens, n_heads, head_dim, token_stride,
-                           softmax_scale > 0.f ? softmax_scale : 1.0f / std::sqrt((float)head_dim), direct_len, dev.sm_count, stream);
+                           total_tokens, n_heads, head_dim, token_stride, scale, split ? kTile : 0, direct_len, dev.sm_count, stream);
+        if (e != cudaSuccess) return fail(DCP_ERR_CUDA, "%s: pre kernel: %s", fn, cudaGetErrorString(e));
+        g_launches.fetch_add(1);
     }
-    if (e != cudaSuccess) return fail(DCP_ERR_CUDA, "%s: pre kernel: %s", fn, cudaGetErrorString(e));
-    g_launches.fetch_add(1);
 
     BwdParams p;
     p.cu_seqlens = vcu;
@@ -437,37 +452,43 @@ static int attn_bwd_impl(const char* fn, const void* q, const void* k, const voi
     p.head_dim = head_dim;
     p.total_tokens = total_tokens;
     p.row_stride = token_stride;
-    p.scale = softmax_scale > 0.f ? softmax_scale : 1.0f / std::sqrt((float)head_dim);
-    p.scale_log2 = p.scale * 1.4426950408889634f;
-    PairMaps maps;
-    if (pair) {
-        maps.q = tq;
-        maps.k = tk;
-        maps.v = tv;
-        maps.d_o = tg;
-        if (int rc = make_map(&maps.q_rows, q, total_tokens, n_heads, head_dim, token_stride, 64)) return rc;
-        if (int rc = make_map(&maps.do_rows, d_o, total_tokens, n_heads, head_dim, token_stride, 64)) return rc;
-        if (int rc = make_stats_map(&maps.stats, stats, max_tiles(total_tokens, n_seqs) * n_heads)) return rc;
-    }
+    p.scale = scale;
+    p.scale_log2 = scale * 1.4426950408889634f;
+    p.lse = lse;
+    p.split = split;
     {
         ScopedTimer t(DCP_KERNEL_BWD_MAIN, stream);
-        if (pair) {
+        if (multi && pair) {
+            PairMaps maps;
+            maps.q = tq;
+            maps.k = tk;
+            maps.v = tv;
+            maps.d_o = tg;
+            if (int rc = make_map(&maps.q_rows, q, total_tokens, n_heads, head_dim, token_stride, 64)) return rc;
+            if (int rc = make_map(&maps.do_rows, d_o, total_tokens, n_heads, head_dim, token_stride, 64)) return rc;
+            if (int rc = make_stats_map(&maps.stats, stats, max_tiles(total_tokens, n_seqs) * n_heads)) return rc;
             e = launch_attn_bwd_pair(maps, p, head_dim, causal != 0, dev.sm_count, stream);
             if (e != cudaSuccess) return fail(DCP_ERR_CUDA, "%s: pair kernel: %s", fn, cudaGetErrorString(e));
             g_launches.fetch_add(1);
+        } else if (multi) {
+            e = launch_attn_bwd(tq, tk, tv, tg, p, causal != 0, dev.sm_count, stream);
+            if (e != cudaSuccess) return fail(DCP_ERR_CUDA, "%s: main kernel: %s", fn, cudaGetErrorString(e));
+            g_launches.fetch_add(1);
         }
-        e = launch_attn_bwd(tq, tk, tv, tg, tdk, tdv, p, head_dim, causal != 0, dev.sm_count, stream);
+        if (split) {
+            e = launch_tile_bwd(tq, tk, tv, tg, p, causal != 0, dev.sm_count, stream);
+            if (e != cudaSuccess) return fail(DCP_ERR_CUDA, "%s: single-tile kernel: %s", fn, cudaGetErrorString(e));
+            g_launches.fetch_add(1);
+        }
     }
-    if (e != cudaSuccess) return fail(DCP_ERR_CUDA, "%s: main kernel: %s", fn, cudaGetErrorString(e));
-    g_launches.fetch_add(1);
 
-    {
+    if (multi) {
         ScopedTimer t(DCP_KERNEL_BWD_POST, stream);
         e = launch_bwd_post(dq_acc, static_cast<__nv_bfloat16*>(dq), vcu, sched, total_tokens, n_heads, head_dim, token_stride,
-                            p.scale, direct_len, dev.sm_count, stream);
+                            scale, direct_len, dev.sm_count, stream);
+        if (e != cudaSuccess) return fail(DCP_ERR_CUDA, "%s: post kernel: %s", fn, cudaGetErrorString(e));
+        g_launches.fetch_add(1);
     }
-    if (e != cudaSuccess) return fail(DCP_ERR_CUDA, "%s: post kernel: %s", fn, cudaGetErrorString(e));
-    g_launches.fetch_add(1);
     return DCP_OK;
 }
 

@@ -96,7 +96,6 @@ struct BwdControl {
     uint64_t kv_full, kv_empty;
     uint64_t q_full[2], q_empty[2], do_full, do_empty, stat_full[2], stat_empty[2];
     uint64_t s_full, p_half, p_full, dp_full, ds_full, ds_free, dq_full, dq_free, dkv_full, dkv_free;
-    uint64_t stage_ready[2], stage_full[2];   // dK / dV staging (the dS^T buffer at the end of an item), per column half
     WorkItem work[2];
     uint32_t tmem_base;
     uint32_t abort_flag;
@@ -183,66 +182,10 @@ __device__ __noinline__ void compute_single_tile_item(BwdControl& sh, const BwdP
     if (lane == 0) mbar_arrive(&sh.ds_full);
 }
 
-// Item epilogue for a key block whose 128 rows all belong to the sequence (head_dim > 64): dV, then dK, leave
-// tensor memory through shared memory and TMA stores.  A thread owns a key row, so storing it directly sends 16-byte
-// pieces of 32 different rows per instruction: 4096 requests per item through the SM's outbound port, which the dQ
-// reductions already keep busy (without these stores the main kernel is 7 % faster on config 2 and the spatial
-// axis, measured).  The staging area is the dS^T buffer, idle between the last product of an item and the first
-// dS^T of the next: each group of four warps (one 64-column half = one TMA box) fills its 16 KB, its first thread
-// stores the box and the group waits until the store has read the buffer.  Out of line, so that the per-tile loop
-// of the compute warps is compiled as it would be without it.  n_staged = boxes this group has staged so far.
-template <int D>
-__device__ __noinline__ void store_dkv_staged(BwdControl& sh, const CUtensorMap* tmap_dk, const CUtensorMap* tmap_dv, uint8_t* stage,
-                                              uint32_t tmem_row, int half, int head, int tok_row0, float scale, uint32_t n_staged,
-                                              const WaitGuard guard) {
-    using Cfg = BwdCfg<D>;
-    const int lane = threadIdx.x & 31, key_in_tile = threadIdx.x & 127;
-    const bool issuer = key_in_tile == 0;
-#pragma unroll
-    for (int which = 0; which < 2; ++which, ++n_staged) {
-        const uint32_t src = tmem_row + (which == 0 ? Cfg::kDv : Cfg::kDk) + half * 64;
-        const float mul = which == 0 ? 1.0f : scale;
-        uint32_t acc[64];
-        tmem_ld_x32(src, *reinterpret_cast<uint32_t(*)[32]>(&acc[0]));
-        tmem_ld_x32(src + 32, *reinterpret_cast<uint32_t(*)[32]>(&acc[32]));
-        tmem_wait_ld();
-        if (which == 1) {               // dV and dK have left tensor memory: the next item may accumulate
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&sh.dkv_free);
-        }
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            uint4 val;
-            val.x = pack_bf16x2(__uint_as_float(acc[c * 8 + 0]) * mul, __uint_as_float(acc[c * 8 + 1]) * mul);
-            val.y = pack_bf16x2(__uint_as_float(acc[c * 8 + 2]) * mul, __uint_as_float(acc[c * 8 + 3]) * mul);
-            val.z = pack_bf16x2(__uint_as_float(acc[c * 8 + 4]) * mul, __uint_as_float(acc[c * 8 + 5]) * mul);
-            val.w = pack_bf16x2(__uint_as_float(acc[c * 8 + 6]) * mul, __uint_as_float(acc[c * 8 + 7]) * mul);
-            *reinterpret_cast<uint4*>(stage + sw128_offset((uint32_t)key_in_tile, (uint32_t)c)) = val;
-        }
-        fence_async_smem();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&sh.stage_full[half]);
-        if (issuer) {
-            if (mbar_wait(&sh.stage_full[half], n_staged & 1u, guard))
-                tma_store_3d(which == 0 ? tmap_dv : tmap_dk, stage, half * 64, head, tok_row0);
-            bulk_store_commit();
-            bulk_store_wait_read();      // the store has read the buffer: dK, or the next item's dS^T, may overwrite it
-        }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&sh.stage_ready[half]);
-        mbar_wait(&sh.stage_ready[half], n_staged & 1u, guard);
-    }
-}
-
-// TRIM: head_dim is at most D - 16, so the products skip the zero-padded columns: S^T and dP^T sum over
-// ceil(head_dim / 16) steps instead of D / 16; dV, dK and dQ are 16 * ceil(head_dim / 16) columns wide, and so
-// is what the drain warps add to the accumulator.
-template <int D, bool CAUSAL, bool TRIM>
+template <int D, bool CAUSAL>
 __global__ void __launch_bounds__(kBwdThreads, 1)
 attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k,
                 const __grid_constant__ CUtensorMap tmap_v, const __grid_constant__ CUtensorMap tmap_do,
-                const __grid_constant__ CUtensorMap tmap_dk, const __grid_constant__ CUtensorMap tmap_dv,
                 const __grid_constant__ BwdParams p) {
     using Cfg = BwdCfg<D>;
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -279,10 +222,6 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         mbar_init(&sh.dq_free, 4);
         mbar_init(&sh.dkv_full, 1);
         mbar_init(&sh.dkv_free, 8);
-        for (int i = 0; i < 2; ++i) {
-            mbar_init(&sh.stage_ready[i], 4);   // one arrival per warp of the half
-            mbar_init(&sh.stage_full[i], 4);
-        }
         sh.abort_flag = 0;
         fence_mbar_init();
         // the swizzled tile layout needs a 1024-byte aligned base; refuse to run otherwise
@@ -311,8 +250,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     grid_wait();
     if (tid == 0 && sh.abort_flag) atomicMax(&p.sched.hdr->status, (uint32_t)kStatusBadSmemAlign);
     // when this CTA started and (at the end) when it ran out of work: the spread over CTAs measures the balance
-    const bool record = p.sched.hdr->n_pair_items == 0;      // after the pair kernel the spans are that kernel's
-    if (record && tid == 0 && blockIdx.x < kMaxCtas) {
+    if (tid == 0 && blockIdx.x < kMaxCtas) {
         p.sched.spans[1 * kMaxCtas + blockIdx.x].begin_ns = global_timer_ns();
         if (blockIdx.x == 0) p.sched.hdr->n_ctas[1] = gridDim.x < kMaxCtas ? gridDim.x : kMaxCtas;
     }
@@ -333,14 +271,14 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             tma_prefetch_desc(&tmap_v);
             tma_prefetch_desc(&tmap_do);
         }
-        const uint32_t n_items = p.sched.hdr->n_items, item0 = p.sched.hdr->n_pair_items;     // items before item0: the pair kernel
+        const uint32_t n_items = p.split ? p.sched.hdr->n_long_items : p.sched.hdr->n_items;
         uint32_t n_work = 0, g = 0;
         while (true) {
             const uint32_t slot = n_work & 1u;
             WorkItem w;
             if (lane == 0) {
                 if (n_work >= 2) mbar_wait(&sh.work_empty[slot], ((n_work >> 1) - 1) & 1u, guard);
-                const uint32_t item = item0 + atomicAdd(&p.sched.hdr->work_counter, 1u);
+                const uint32_t item = atomicAdd(&p.sched.hdr->work_counter, 1u);
                 if (item < n_items && !sh.abort_flag) {
                     w = decode_item(p.sched, p.cu_seqlens, item, kTile, p.n_heads, false);
                 } else {
@@ -392,9 +330,8 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             // Shared-memory descriptors are built once; a k-step only adds a constant to the address
             // field (the issuing thread is on the critical path: MMA issue blocks while the pipe is busy).
             constexpr uint32_t idesc_abt = make_idesc_bf16(128, 128, false, false);  // both operands K-contiguous
-            const int n_ks = TRIM ? (p.head_dim + 15) >> 4 : D / 16;                // steps of 16 head_dim columns that hold data
-            const uint32_t idesc_nd_kb = make_idesc_bf16(128, TRIM ? n_ks * 16 : D, false, true);   // A K-contig / tmem, B N-contig
-            const uint32_t idesc_nd_mm = make_idesc_bf16(128, TRIM ? n_ks * 16 : D, true, true);    // A M-contig, B N-contig
+            constexpr uint32_t idesc_nd_kb = make_idesc_bf16(128, D, false, true);   // A K-contig / tmem, B N-contig
+            constexpr uint32_t idesc_nd_mm = make_idesc_bf16(128, D, true, true);    // A M-contig, B N-contig
             constexpr uint32_t kStageStep = Cfg::kTileBytes >> 4;
             const uint64_t k_km = make_sdesc_sw128(smem_u32(smem + Cfg::kOffK), 16, 1024);
             const uint64_t k_mn = make_sdesc_sw128(smem_u32(smem + Cfg::kOffK), Cfg::kBoxBytes, 1024);
@@ -416,7 +353,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             auto issue_abt = [&](uint32_t d_tmem, uint64_t a, uint64_t b) {
 #pragma unroll
                 for (int ks = 0; ks < D / 16; ++ks)
-                    if (leader && (!TRIM || ks < n_ks))
+                    if (leader)
                         tc_mma_ss(d_tmem, a + km_step(ks, Cfg::kBoxBytes), b + km_step(ks, Cfg::kBoxBytes), idesc_abt, ks > 0);
             };
             uint32_t n_work = 0, g = 0;
@@ -519,7 +456,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         const uint32_t pt_tmem = tmem + lane_base + Cfg::kSt + half * 64;   // bf16 pairs, inside this group's own S^T columns
         const uint32_t dp_tmem = tmem + lane_base + Cfg::kDp + half * 64;
         uint8_t* ds_row = smem + Cfg::kOffDs + half * 16384;
-        uint32_t n_work = 0, g = 0, n_staged = 0;
+        uint32_t n_work = 0, g = 0;
         while (true) {
             const uint32_t slot = n_work & 1u;
             const bool got = mbar_wait(&sh.work_full[slot], (n_work >> 1) & 1u, guard);
@@ -607,13 +544,6 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             // item epilogue: dV and dK rows of this key block (each group writes half the columns)
             mbar_wait(&sh.dkv_full, n_work & 1u, guard);
             tc_fence_after();
-            if (D == 128 && w.blk * kTile + kTile <= w.len) {
-                store_dkv_staged<D>(sh, &tmap_dk, &tmap_dv, smem + Cfg::kOffDs + half * 16384, tmem + lane_base, half, w.head,
-                                    w.tok0 + w.blk * kTile, p.scale, n_staged, guard);
-                n_staged += 2;
-                ++n_work;
-                continue;
-            }
             const size_t tok = (size_t)w.tok0 + (size_t)key;
             const size_t out_off = tok * p.row_stride + w.head * p.head_dim + half * (D / 2);
 #pragma unroll
@@ -694,10 +624,8 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                 } else {
                     const bool live = qrow < w.len;
                     if ((warp & 3) > 0) __nanosleep((warp & 3) * kRedStaggerNs + 64);
-                    const int n_c4 = TRIM ? ((p.head_dim + 15) >> 4) * 4 : D / 4;     // groups of four columns that hold data
 #pragma unroll
                     for (int c = 0; c < D / 4; ++c) {
-                        if (TRIM && c >= n_c4) break;
                         if (live) red_add_v4(dst + c * (kTile * 4), __uint_as_float(acc[c * 4]), __uint_as_float(acc[c * 4 + 1]),
                                    __uint_as_float(acc[c * 4 + 2]), __uint_as_float(acc[c * 4 + 3]));
                         if ((c % kRedGroup) == kRedGroup - 1) __nanosleep(kRedSleepNs);
@@ -709,29 +637,20 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
 
     tc_fence_before();
     __syncthreads();
-    if (record && tid == 0 && blockIdx.x < kMaxCtas) p.sched.spans[1 * kMaxCtas + blockIdx.x].end_ns = global_timer_ns();
+    if (tid == 0 && blockIdx.x < kMaxCtas) p.sched.spans[1 * kMaxCtas + blockIdx.x].end_ns = global_timer_ns();
     if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
-template <int D, bool CAUSAL, bool TRIM>
+template <bool CAUSAL>
 static cudaError_t launch_one(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tdo,
-                              const CUtensorMap& tdk, const CUtensorMap& tdv, const BwdParams& p, int n_ctas, cudaStream_t stream) {
-    if (cudaError_t e = allow_smem<attn_bwd_kernel<D, CAUSAL, TRIM>>(BwdCfg<D>::kSmemBytes)) return e;
-    return launch_dependent(attn_bwd_kernel<D, CAUSAL, TRIM>, n_ctas, kBwdThreads, BwdCfg<D>::kSmemBytes, stream, tq, tk, tv, tdo, tdk,
-                            tdv, p);
+                              const BwdParams& p, int n_ctas, cudaStream_t stream) {
+    if (cudaError_t e = allow_smem<attn_bwd_kernel<64, CAUSAL>>(BwdCfg<64>::kSmemBytes)) return e;
+    return launch_dependent(attn_bwd_kernel<64, CAUSAL>, n_ctas, kBwdThreads, BwdCfg<64>::kSmemBytes, stream, tq, tk, tv, tdo, p);
 }
 
 cudaError_t launch_attn_bwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tdo,
-                            const CUtensorMap& tdk, const CUtensorMap& tdv, const BwdParams& p, int head_dim, bool causal,
-                            int n_ctas, cudaStream_t stream) {
-    if (head_dim > 112)
-        return causal ? launch_one<128, true, false>(tq, tk, tv, tdo, tdk, tdv, p, n_ctas, stream)
-                      : launch_one<128, false, false>(tq, tk, tv, tdo, tdk, tdv, p, n_ctas, stream);
-    if (head_dim > 64)
-        return causal ? launch_one<128, true, true>(tq, tk, tv, tdo, tdk, tdv, p, n_ctas, stream)
-                      : launch_one<128, false, true>(tq, tk, tv, tdo, tdk, tdv, p, n_ctas, stream);
-    return causal ? launch_one<64, true, false>(tq, tk, tv, tdo, tdk, tdv, p, n_ctas, stream)
-                  : launch_one<64, false, false>(tq, tk, tv, tdo, tdk, tdv, p, n_ctas, stream);
+                            const BwdParams& p, bool causal, int n_ctas, cudaStream_t stream) {
+    return causal ? launch_one<true>(tq, tk, tv, tdo, p, n_ctas, stream) : launch_one<false>(tq, tk, tv, tdo, p, n_ctas, stream);
 }
 
 }  // namespace dcp

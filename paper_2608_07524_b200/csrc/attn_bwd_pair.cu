@@ -222,11 +222,11 @@ attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constan
     if (warp == 11) {
         // ------------------------------------------------- scheduler (leader): items of the list to both CTAs
         if (lead && lane == 0) {
-            const uint32_t n_items = p.sched.hdr->n_pair_items;
+            const uint32_t n_items = p.sched.hdr->n_long_items;
             for (uint32_t n = 0;; ++n) {
                 const uint32_t slot = n % kRing;
                 if (n >= kRing) mbar_wait_cluster(&sh.work_empty[slot], (n / kRing - 1) & 1u, guard);
-                const uint32_t item = atomicAdd(&p.sched.hdr->pair_counter, 1u);
+                const uint32_t item = atomicAdd(&p.sched.hdr->work_counter, 1u);
                 WorkItem w{0, -1, 0, 0, 0};
                 if (item < n_items && !sh.abort_flag) w = decode_item(p.sched, p.cu_seqlens, item, 2 * kTile, p.n_heads, false);
 #pragma unroll

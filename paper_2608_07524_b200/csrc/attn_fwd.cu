@@ -321,7 +321,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             tma_prefetch_desc(&tmap_q);
             tma_prefetch_desc(&tmap_k);
             tma_prefetch_desc(&tmap_v);
-            const uint32_t n_items = p.sched.hdr->n_items;
+            const uint32_t n_items = p.split ? p.sched.hdr->n_long_items : p.sched.hdr->n_items;
             uint32_t n_work = 0, kv_count = 0, q_use[2] = {0, 0};
             while (true) {
                 const uint32_t slot = n_work & 1u;

@@ -21,6 +21,7 @@ struct FwdParams {
     int64_t row_stride; // elements between consecutive tokens of q, k, v, o (n_heads * head_dim when contiguous)
     float scale;        // softmax scale
     float scale_log2;   // scale * log2(e)
+    bool split;         // the single-tile items are for launch_tile_fwd
 };
 
 struct BwdParams {
@@ -40,6 +41,8 @@ struct BwdParams {
     int64_t row_stride;   // as in FwdParams; the same for q, k, v, dO, dq, dk, dv
     float scale;
     float scale_log2;
+    const float* lse;     // [H, T]: read by launch_tile_bwd (the other kernels take it from `stats`)
+    bool split;           // the single-tile items are for launch_tile_bwd
 };
 
 // Tensor maps of the pair kernel: boxes of 64 columns x 128 rows, of 64 rows for the `_rows` maps; `stats` views the
@@ -51,7 +54,13 @@ struct PairMaps {
 // Sequences longer than one tile of a backward call whose head dimension is above 64 go to the pair kernel; a
 // sequence of at most kPairDirectLen tokens is a single work item there, which writes dQ itself.
 constexpr int kPairDirectLen = 2 * kTile;
-inline bool pair_path(int32_t head_dim, int32_t max_seqlen) { return head_dim > 64 && max_seqlen > kTile; }
+inline bool pair_path(int32_t head_dim) { return head_dim > 64; }
+
+// Single-tile work items (virtual sequences of at most 128 tokens) on kernels of their own, see attn_tile.cu.
+cudaError_t launch_tile_fwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const FwdParams& p, bool causal,
+                            int n_sms, cudaStream_t stream);
+cudaError_t launch_tile_bwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tdo,
+                            const BwdParams& p, bool causal, int n_sms, cudaStream_t stream);
 
 // Builds the work list (longest sequence first) and resets the work counter and status word.
 // With `bounds` non-null, short sequences are first merged into virtual sequences: sched.vcu and
@@ -61,11 +70,12 @@ int prep_launches(int32_t n_seqs, bool merge, bool input_order);   // kernels la
 // tile_capacity = number of 128-row tiles the per-tile storage of the workspace holds (UINT32_MAX if the
 // call uses none).  Inconsistent boundaries or more tiles than that leave an empty work list and
 // kStatusBadLengths in the status word.  input_order = true lists the sequences as they come instead of
-// longest first (a measurement aid: it shows what the ordering is worth).  Sequences of at least pair_min_len
-// tokens come first in either order, and their items are counted in the header (n_pair_items).
+// longest first (a measurement aid: it shows what the ordering is worth).  Sequences of at least long_min_len
+// tokens come first in either order and empty ones last; the header counts the first and their items (n_long_seqs, n_long_items);
+// no_long: max_seqlen promises that there are none.
 cudaError_t launch_prep(const int32_t* cu_seqlens, int32_t n_seqs, int32_t total_tokens, int32_t max_seqlen,
                         int32_t rows_per_block, int32_t n_heads, const SchedView& sched, uint16_t* bounds,
-                        uint32_t tile_capacity, bool input_order, int32_t pair_min_len, cudaStream_t stream);
+                        uint32_t tile_capacity, bool input_order, int32_t long_min_len, bool no_long, cudaStream_t stream);
 
 // One CTA that waits, with the kernels' own bounded wait and the given poll limit, on a barrier nobody
 // arrives at, and leaves through the same abort path (status word raised, no trap).
@@ -84,17 +94,17 @@ cudaError_t launch_attn_fwd(const CUtensorMap& tq, const CUtensorMap& tk, const 
 
 // Tile-aligned row statistics for the backward kernel (see BwdParams::stats) and dq_acc = 0.  Sequences of at most
 // direct_len tokens get their dQ written by the main kernel: here and in the post kernel they have no accumulator.
+// Those of at most skip_len tokens are not the main kernel's at all.
 cudaError_t launch_bwd_pre(const __nv_bfloat16* o, const __nv_bfloat16* d_o, const float* lse, const int32_t* cu_seqlens,
                            const SchedView& sched, __nv_bfloat16* stats, float* dq_acc, size_t dq_acc_elems,
                            int32_t total_tokens, int32_t n_heads, int32_t head_dim, int64_t row_stride, float scale,
-                           int32_t direct_len, int n_sms, cudaStream_t stream);
+                           int32_t skip_len, int32_t direct_len, int n_sms, cudaStream_t stream);
 
 cudaError_t launch_attn_bwd_pair(const PairMaps& maps, const BwdParams& p, int head_dim, bool causal, int n_ctas, cudaStream_t stream);
 
-// tdk, tdv = maps over dk and dv: whole key blocks leave through shared memory and TMA stores.
+// Main kernel for head dimensions up to 64 (above: the pair kernel).
 cudaError_t launch_attn_bwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tdo,
-                            const CUtensorMap& tdk, const CUtensorMap& tdv, const BwdParams& p, int head_dim, bool causal,
-                            int n_ctas, cudaStream_t stream);
+                            const BwdParams& p, bool causal, int n_ctas, cudaStream_t stream);
 
 // dq[T, H, d] = bf16(scale * dq_acc), undoing the tile-blocked layout
 cudaError_t launch_bwd_post(const float* dq_acc, __nv_bfloat16* dq, const int32_t* cu_seqlens, const SchedView& sched,

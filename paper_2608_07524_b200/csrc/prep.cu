@@ -218,7 +218,7 @@ template <int NT>
 __global__ void __launch_bounds__(NT) prep_kernel(const int32_t* __restrict__ cu, int32_t n_seqs,
                                                   const uint32_t* __restrict__ n_live_ptr, int32_t rows_per_block, int32_t n_heads,
                                                   WorkspaceHeader* hdr, int32_t* order, uint32_t* prefix, uint32_t* tile_prefix,
-                                                  int ranked, int32_t total_tokens, uint32_t tile_capacity, int32_t pair_min_len) {
+                                                  int ranked, int32_t total_tokens, uint32_t tile_capacity, int32_t long_min_len, bool no_long) {
     __shared__ uint32_t scratch[33];
     __shared__ int32_t len_sh[NT];
     grid_trigger();
@@ -234,19 +234,23 @@ __global__ void __launch_bounds__(NT) prep_kernel(const int32_t* __restrict__ cu
         if (bad) {
             for (int i = tid; i <= n_seqs; i += NT) { prefix[i] = 0; tile_prefix[i] = 0; }
             for (int i = tid; i < n_seqs; i += NT) order[i] = i;
-            if (tid == 0) hdr->n_items = hdr->n_pair_items = hdr->work_counter = hdr->pair_counter = 0;
+            if (tid == 0) hdr->n_items = hdr->n_long_items = hdr->n_long_seqs = hdr->work_counter = 0;
             return;
         }
     }
     if (ranked == 2) {
-        // input order, those of the pair kernel first
+        // input order: the long sequences, the others, the empty ones
         const int chunk = (n_live + NT - 1) / NT;
         const int from = min(tid * chunk, n_live), to = min(from + chunk, n_live);
-        uint32_t n_long = 0, all_long = 0;
-        for (int i = from; i < to; ++i) n_long += cu[i + 1] - cu[i] >= pair_min_len ? 1u : 0u;
-        uint32_t at_long = block_exclusive_scan<NT>(n_long, scratch, &all_long);
-        uint32_t at_short = all_long + (uint32_t)from - at_long;
-        for (int i = from; i < to; ++i) order[cu[i + 1] - cu[i] >= pair_min_len ? at_long++ : at_short++] = i;
+        auto kind = [&](int i) { const int32_t len = cu[i + 1] - cu[i]; return len >= long_min_len ? 0 : len > 0 ? 1 : 2; };
+        uint32_t cnt[2] = {0, 0}, all[2], at[3];
+        for (int i = from; i < to; ++i)
+            if (kind(i) < 2) ++cnt[kind(i)];
+        at[0] = block_exclusive_scan<NT>(cnt[0], scratch, &all[0]);
+        at[1] = block_exclusive_scan<NT>(cnt[1], scratch, &all[1]);
+        at[2] = all[0] + all[1] + (uint32_t)from - at[0] - at[1];
+        at[1] += all[0];
+        for (int i = from; i < to; ++i) order[at[kind(i)]++] = i;
         for (int i = n_live + tid; i < n_seqs; i += NT) order[i] = i;
     } else if (!ranked) {                             // n_seqs <= kRankInKernelMax: one sequence per thread
         len_sh[tid] = tid < n_seqs ? cu[tid + 1] - cu[tid] : -1;
@@ -275,15 +279,18 @@ __global__ void __launch_bounds__(NT) prep_kernel(const int32_t* __restrict__ cu
     uint32_t run = block_exclusive_scan<NT>(local, scratch, &total);
     if (tid == 0) {
         hdr->n_items = total;
-        hdr->work_counter = hdr->pair_counter = 0;
-        hdr->n_pair_items = 0;
+        hdr->work_counter = 0;
+        hdr->n_long_items = hdr->n_long_seqs = 0;
     }
     __syncthreads();
-    auto in_pair = [&](int pos) { return pos < n_live && cu[order[pos] + 1] - cu[order[pos]] >= pair_min_len; };
+    auto is_long = [&](int pos) { return pos < n_live && cu[order[pos] + 1] - cu[order[pos]] >= long_min_len; };
     for (int i = begin; i < end; ++i) {
         prefix[i] = run;
         run += items_of(i);
-        if (in_pair(i) && !in_pair(i + 1)) hdr->n_pair_items = run;      // they come first in the order
+        if (is_long(i) && !is_long(i + 1)) {              // they come first in the order
+            hdr->n_long_items = run;
+            hdr->n_long_seqs = i + 1;
+        }
     }
     for (int i = n_live + tid; i <= n_seqs; i += NT) prefix[i] = total;
     // tile_prefix[b] = number of 128-row tiles of sequences 0..b-1 (input order): same two-level scan
@@ -291,12 +298,14 @@ __global__ void __launch_bounds__(NT) prep_kernel(const int32_t* __restrict__ cu
     local = 0;
     for (int i = begin; i < end; ++i) local += tiles_of(i);
     run = block_exclusive_scan<NT>(local, scratch, &total);
-    if (total > tile_capacity) {
-        // more tiles than the workspace was sized for: max_seqlen was understated (the bound on merged runs
-        // relies on it).  Nothing may index the per-tile storage: no items, no tiles.
+    const bool unforeseen = __syncthreads_or(no_long && begin < end && is_long(begin));
+    if (total > tile_capacity || unforeseen) {
+        // more tiles than the workspace was sized for, or a sequence of more than one tile where no kernel for such was
+        // launched: max_seqlen was understated (the bound on merged runs relies on it).  Nothing may index the per-tile
+        // storage: no items, no tiles.
         for (int i = tid; i <= n_seqs; i += NT) tile_prefix[i] = 0;
         if (tid == 0) {
-            hdr->n_items = hdr->n_pair_items = 0;
+            hdr->n_items = hdr->n_long_items = 0;
             atomicMax(&hdr->status, (uint32_t)kStatusBadLengths);
         }
         return;
@@ -314,7 +323,7 @@ int prep_launches(int32_t n_seqs, bool merge, bool input_order) {
 
 cudaError_t launch_prep(const int32_t* cu_seqlens, int32_t n_seqs, int32_t total_tokens, int32_t max_seqlen,
                         int32_t rows_per_block, int32_t n_heads, const SchedView& sched, uint16_t* bounds,
-                        uint32_t tile_capacity, bool input_order, int32_t pair_min_len, cudaStream_t stream) {
+                        uint32_t tile_capacity, bool input_order, int32_t long_min_len, bool no_long, cudaStream_t stream) {
     const int32_t* cu = cu_seqlens;
     const uint32_t* n_live = nullptr;
     const bool small = n_seqs <= 256;
@@ -339,7 +348,7 @@ cudaError_t launch_prep(const int32_t* cu_seqlens, int32_t n_seqs, int32_t total
             return e;
     return launch_dependent(small ? prep_kernel<256> : prep_kernel<1024>, 1, small ? 256 : 1024, 0, stream, cu, n_seqs, n_live,
                             rows_per_block, n_heads, sched.hdr, const_cast<int32_t*>(sched.order), const_cast<uint32_t*>(sched.prefix),
-                            const_cast<uint32_t*>(sched.tile_prefix), ranked, total_tokens, tile_capacity, pair_min_len);
+                            const_cast<uint32_t*>(sched.tile_prefix), ranked, total_tokens, tile_capacity, long_min_len, no_long);
 }
 
 // The sequence that owns 128-row tile t: (sequence, first row of the tile inside it, its length, its first token).
@@ -386,7 +395,7 @@ __global__ void __launch_bounds__(256) bwd_pre_kernel(const __nv_bfloat16* __res
                                                       int32_t n_seqs, __nv_bfloat16* __restrict__ stats,
                                                       float* __restrict__ dq_acc, size_t dq_acc_vec4,
                                                       int32_t total_tokens, int32_t n_heads, int32_t head_dim,
-                                                      int64_t row_stride, float inv_scale, int32_t direct_len) {
+                                                      int64_t row_stride, float inv_scale, int32_t skip_len, int32_t direct_len) {
     grid_trigger();
     grid_wait();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -397,6 +406,7 @@ __global__ void __launch_bounds__(256) bwd_pre_kernel(const __nv_bfloat16* __res
         // this kernel slower: 0.39 -> 0.44 ms on 131072 tokens x 16 heads)
         const TileRef ref = find_tile(cu, tile_prefix, n_seqs, t);
         const int row0 = ref.row0, len = ref.len, tok0 = ref.tok0;
+        if (len <= skip_len) continue;
         if (len > direct_len) {
             // this (tile, head) block of the dQ accumulator; a sequence of a single key block needs none (the main
             // kernel holds its whole dQ and writes it directly)
@@ -476,13 +486,13 @@ __global__ void __launch_bounds__(256) bwd_pre_kernel(const __nv_bfloat16* __res
 cudaError_t launch_bwd_pre(const __nv_bfloat16* o, const __nv_bfloat16* d_o, const float* lse, const int32_t* cu_seqlens,
                            const SchedView& sched, __nv_bfloat16* stats, float* dq_acc, size_t dq_acc_elems,
                            int32_t total_tokens, int32_t n_heads, int32_t head_dim, int64_t row_stride, float scale,
-                           int32_t direct_len, int n_sms, cudaStream_t stream) {
+                           int32_t skip_len, int32_t direct_len, int n_sms, cudaStream_t stream) {
     // no more CTAs than (tile, head) blocks the batch can have
     const size_t most = max_tiles(total_tokens, sched.n_seqs) * (size_t)n_heads;
     const unsigned blocks = most < (size_t)n_sms * 8 ? (unsigned)most : (unsigned)n_sms * 8;
     return launch_dependent(head_dim > 64 ? bwd_pre_kernel<128> : bwd_pre_kernel<64>, blocks, 256, 0, stream, o, d_o, lse, cu_seqlens,
                             sched.tile_prefix, sched.n_seqs, stats, dq_acc, dq_acc_elems / 4, total_tokens, n_heads, head_dim, row_stride,
-                            1.0f / scale, direct_len);
+                            1.0f / scale, skip_len, direct_len);
 }
 
 // Backward helper 2: dq[T, H, d] = bf16(scale * dq_acc).  dq_acc holds, per (tile, head), a block

@@ -45,8 +45,8 @@ struct WorkspaceHeader {
     uint32_t call_bad;      // this call's boundaries were inconsistent (reset by every call)
     uint32_t magic[2];      // kHeaderMagic0/1 once the header has been initialised
     uint32_t n_ctas[2];     // CTAs of the last forward / backward main launch that recorded a span
-    uint32_t n_pair_items;  // the first items of the list, which the pair kernel takes (0 where it does not run)
-    uint32_t pair_counter;  // next unclaimed one of those
+    uint32_t n_long_items;  // items of the sequences of more than one tile, which come first in the list; the single-tile
+    uint32_t n_long_seqs;   // kernels take the rest.  (Both 0 where one kernel takes the whole list.)  And those sequences
     uint32_t check_bad[16]; // short-sequence path: whether a CTA of the check kernel found this call's boundaries inconsistent
     uint32_t pad[36];
 };

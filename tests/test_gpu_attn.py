@@ -396,6 +396,33 @@ def test_backward_on_cta_pairs(causal, d, lengths):
     check_full(lengths, 3, d, causal, seed=300 + len(lengths))
 
 
+@pytest.mark.parametrize("causal", [False, True])
+@pytest.mark.parametrize("d", [8, 64, 72, 128])
+@pytest.mark.parametrize("longest", [128, 300])
+def test_single_tile_kernels(causal, d, longest):
+    """Work items of at most 128 tokens on their own kernels: alone (nothing longer declared) and beside the multi-tile
+    kernels, several items per CTA, sequences that share a tile, fill it, or leave one row; empty ones in between."""
+    rng = np.random.default_rng(d + longest)
+    lengths = [int(x) for x in rng.choice([0, 1, 2, 13, 31, 32, 33, 64, 65, 96, 127, 128], size=180)]
+    if longest > 128:
+        for pos in (0, 50, 179):
+            lengths[pos] = longest - pos
+    check_full(lengths, 8, d, causal, seed=400 + d)
+
+
+def test_a_sequence_longer_than_a_declared_tile_is_refused():
+    # max_seqlen <= 128 promises that no sequence needs the multi-tile kernels, which are then not launched
+    dev = "cuda"
+    cu = torch.tensor([0, 100, 300], dtype=torch.int32, device=dev)
+    q, k, v, g = (x.to(dev) for x in inputs.make_qkvg(300, 2, 64, 5))
+    ws = B.alloc_workspace(300, 2, 2, 64, True, dev)
+    o = torch.full_like(q, 7.0)
+    B.dcp_varlen_attn_fwd(q, k, v, cu, 128, False, out=o, workspace=ws)
+    with pytest.raises(B.DcpError) as e:
+        B.dcp_query_status(ws)
+    assert e.value.code == B.DCP_ERR_INVALID_ARG and bool((o == 7.0).all())
+
+
 def test_inconsistent_boundaries_are_reported_not_used():
     """cu_seqlens is device data the host never reads; the work-list kernels check it (starts at 0,
     never decreases, ends at total_tokens, fits the per-tile storage that max_seqlen promised) and, if
