@@ -121,12 +121,13 @@ struct WorkItem {
     int32_t tile0;  // index of the sequence's first 128-row tile among all tiles of the batch
 };
 
-// Map item index -> (sequence, head, block).  Within a sequence, blocks vary fastest so that CTAs
-// running at the same time share one head's K and V in L2; under a causal mask the heaviest
-// blocks come first (forward: last rows see the most keys; backward: first keys are seen by the
-// most rows).
+// Map item index -> (sequence, head, block).  Without a mask the items of a sequence are alike and blocks vary fastest, so
+// that CTAs running at the same time share one head's K and V in L2.  Under a causal mask the heaviest blocks come first
+// (forward, heavy_is_last: last rows see the most keys; backward: first keys are seen by the most rows), of all heads:
+// with the heads one after the other the last head's heaviest block, up to a hundred times the lightest, started when
+// most of the work was done (one 15904-token sequence beside nine short ones, 4 heads: backward main kernel 813 us).
 __device__ inline WorkItem decode_item(const SchedView& s, const int32_t* cu_seqlens, uint32_t item, int rows_per_blk,
-                                       int n_heads, bool heavy_is_last) {
+                                       int n_heads, bool causal, bool heavy_is_last) {
     int lo = 0, hi = s.n_seqs;              // largest i with prefix[i] <= item
     while (hi - lo > 1) {
         int mid = (lo + hi) >> 1;
@@ -139,10 +140,9 @@ __device__ inline WorkItem decode_item(const SchedView& s, const int32_t* cu_seq
     w.tile0 = (int32_t)s.tile_prefix[seq];
     const uint32_t local = item - s.prefix[lo];
     const uint32_t nblk = (uint32_t)(w.len + rows_per_blk - 1) / (uint32_t)rows_per_blk;
-    w.head = (int32_t)(local / nblk);
-    const uint32_t b = local % nblk;
+    w.head = (int32_t)(causal ? local % (uint32_t)n_heads : local / nblk);
+    const uint32_t b = causal ? local / (uint32_t)n_heads : local % nblk;
     w.blk = (int32_t)(heavy_is_last ? nblk - 1 - b : b);
-    (void)n_heads;
     return w;
 }
 
