@@ -27,7 +27,7 @@
 // outer ones).  Every operand tile is used by exactly one product (Q and dO are loaded twice, as rows for S and dP
 // and as columns for dK and dV, since a CTA supplies half of B's columns), which leaves each single-buffered load
 // most of a period.  Between items nothing drains: the first S of an item follows the last dV of the previous one,
-// and dV and dK of an item are written while the next item's first tile is in flight.
+// and the drain warps write dV and dK of an item while the next one is under way.
 //
 // The issuing warp paces the pipe (an MMA issue blocks while the pipe is busy, so what it does between two products
 // is idle time of the tensor cores; a barrier poll takes 100-250 cycles under load).  So there is one commit per
@@ -75,7 +75,8 @@ constexpr int kOffOnes = 212992;                         // ones, zeros, ones (2
 constexpr int kStatBytes = 2048;                         // per-query terms of this CTA's 64 queries
 constexpr int kOffStat = kOffOnes + 6144;
 constexpr int kOffCtl = kOffStat + 2 * kStatBytes;
-constexpr int kSmemBytes = kOffCtl + 512;
+constexpr int kOffStage = kOffCtl + 512;                  // 2 KB per drain warp, for dV and dK on their way out
+constexpr int kSmemBytes = kOffStage + 8192;
 static_assert(kSmemBytes <= 232448, "exceeds the 227 KB a CTA may use");
 // tensor-memory columns.  P^T (dS^T) overwrites S^T (dP^T) packed: group 0's 64 columns go to the first 32, group
 // 1's to the last 32, which leaves 64 adjacent ones in the middle of S^T for dQ.
@@ -97,43 +98,43 @@ __device__ __forceinline__ void red_add_v4(float* addr, float a, float b, float 
     asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(addr), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
 }
 
-// dV or dK of a warp's 32 keys and 64 columns: tensor memory -> bf16 -> this warp's 4 KB of staging (128-byte swizzled
-// rows) -> full 128-byte lines of global memory, four rows per instruction.  By TMA store the wait for the staging
-// buffer to be read costs 2500 cycles a block, because the reductions of dQ fill the way out of the SM; ordinary stores
-// need no wait.  Inlined: the caller holds 64 probabilities in registers meanwhile.
-__device__ __forceinline__ void store_block(__nv_bfloat16* out, const BwdParams& p, uint8_t* stage_warp, uint32_t src_tmem,
-                                            uint32_t free_bar, float mul, int half, int head, int tok_row0, int rows_left) {
+// dV or dK of a drain warp's 32 keys, all columns: tensor memory -> bf16 in registers (the accumulator is free again),
+// then 32 columns at a time through 2 KB of staging (rows of 64 bytes, 16-byte chunks swizzled) to global memory, eight
+// rows per instruction.
+__device__ __forceinline__ void store_block(__nv_bfloat16* out, const BwdParams& p, uint8_t* stage, uint32_t src_tmem, uint32_t free_bar,
+                                            float mul, int head, int tok_row0, int rows_left) {
     const int lane = threadIdx.x & 31;
+    uint32_t pk[64];
 #pragma unroll
-    for (int c = 0; c < 2; ++c) {
+    for (int c = 0; c < 4; ++c) {
         uint32_t acc[32];
         tmem_ld_x32(src_tmem + c * 32, acc);
         tmem_wait_ld();
-        if (c == 1) {                                    // the accumulator has left tensor memory
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive_at(free_bar);
-        }
 #pragma unroll
-        for (int v4 = 0; v4 < 4; ++v4) {
-            uint4 val;
-            val.x = pack_bf16x2(__uint_as_float(acc[v4 * 8 + 0]) * mul, __uint_as_float(acc[v4 * 8 + 1]) * mul);
-            val.y = pack_bf16x2(__uint_as_float(acc[v4 * 8 + 2]) * mul, __uint_as_float(acc[v4 * 8 + 3]) * mul);
-            val.z = pack_bf16x2(__uint_as_float(acc[v4 * 8 + 4]) * mul, __uint_as_float(acc[v4 * 8 + 5]) * mul);
-            val.w = pack_bf16x2(__uint_as_float(acc[v4 * 8 + 6]) * mul, __uint_as_float(acc[v4 * 8 + 7]) * mul);
-            *reinterpret_cast<uint4*>(stage_warp + sw128_offset((uint32_t)lane, (uint32_t)(c * 4 + v4))) = val;
-        }
+        for (int e = 0; e < 16; ++e) pk[c * 16 + e] = pack_bf16x2(__uint_as_float(acc[2 * e]) * mul, __uint_as_float(acc[2 * e + 1]) * mul);
     }
+    tc_fence_before();
     __syncwarp();
-    const int chunk = lane & 7, col = half * 64 + chunk * 8;
-    __nv_bfloat16* dst = out + ((size_t)tok_row0 + (lane >> 3)) * p.row_stride + head * p.head_dim + col;
+    if (lane == 0) mbar_arrive_at(free_bar);
+    const int sub = lane >> 2, chunk = lane & 3;
+    __nv_bfloat16* dst = out + ((size_t)tok_row0 + sub) * p.row_stride + head * p.head_dim + chunk * 8;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int row = i * 4 + (lane >> 3);
-        const uint4 val = *reinterpret_cast<const uint4*>(stage_warp + sw128_offset((uint32_t)row, (uint32_t)chunk));
-        if (row < rows_left && col < p.head_dim) *reinterpret_cast<uint4*>(dst + (size_t)(i * 4) * p.row_stride) = val;
+    for (int c = 0; c < 4; ++c) {
+        if (c * 32 >= p.head_dim) break;
+#pragma unroll
+        for (int v4 = 0; v4 < 4; ++v4)
+            *reinterpret_cast<uint4*>(stage + lane * 64 + ((v4 ^ ((lane >> 1) & 3)) << 4)) =
+                make_uint4(pk[c * 16 + v4 * 4], pk[c * 16 + v4 * 4 + 1], pk[c * 16 + v4 * 4 + 2], pk[c * 16 + v4 * 4 + 3]);
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int row = i * 8 + sub;
+            const uint4 val = *reinterpret_cast<const uint4*>(stage + row * 64 + ((chunk ^ ((row >> 1) & 3)) << 4));
+            if (row < rows_left && c * 32 + chunk * 8 < p.head_dim)
+                *reinterpret_cast<uint4*>(dst + c * 32 + (size_t)(i * 8) * p.row_stride) = val;
+        }
+        __syncwarp();                                    // the staging rows have been read
     }
-    __syncwarp();                                        // the staging rows have been read
 }
 
 // TRIM: head_dim is at most 112, so S and dP sum over ceil(head_dim / 16) steps instead of 8.  dV, dK and dQ keep their
@@ -163,10 +164,9 @@ attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constan
         for (uint64_t* b : {&sh.ld_s, &sh.ld_p, &sh.ld_k, &sh.ld_v, &sh.s_done, &sh.dp_done, &sh.dk_done, &sh.dq_done, &sh.dv_done,
                             &sh.ds_recv})
             mbar_init(b, 1);
-        for (uint64_t* b : {&sh.s_read, &sh.p_full, &sh.ds_tmem, &sh.dv_free, &sh.dk_free})
-            mbar_init(b, 16);                            // the compute warps of both CTAs
+        for (uint64_t* b : {&sh.s_read, &sh.p_full, &sh.ds_tmem}) mbar_init(b, 16);      // the compute warps of both CTAs
         mbar_init(&sh.ds_smem, 9);                       // the four warps of each CTA that keep their dS^T, and the relay
-        mbar_init(&sh.dq_free, 8);
+        for (uint64_t* b : {&sh.dq_free, &sh.dv_free, &sh.dk_free}) mbar_init(b, 8);      // the drain warps of both CTAs
         sh.abort_flag = 0;
         fence_mbar_init();
         mbar_expect_tx(&sh.ds_recv, kBoxBytes);          // armed one tile ahead by whoever waits on it
@@ -430,7 +430,7 @@ attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constan
         }
     }
     } else if (warp < 8) {
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 152;");
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 136;");
         // ------------------------------------------------- compute: P^T, dS^T, and dK / dV of the previous item
         const int half = warp >> 2;                                  // which 64 query columns
         const int key_in_tile = (warp & 3) * 32 + lane;              // tensor-memory lane = key
@@ -448,20 +448,7 @@ attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constan
                        bar_ds_smem = at_leader(&sh.ds_smem);
         const uint64_t sc2 = pack_f32x2(p.scale_log2, p.scale_log2);
         uint32_t n_work = 0, k = 0;
-        WorkItem w, done{0, 0, 0, 0, 0};
-        bool pending = false;                            // `done` is an item whose dV and dK are still in tensor memory
-        auto finish = [&](uint32_t last) {               // last = the item's last tile
-            const int key0 = done.blk * 2 * kTile + (int)rank * kTile + (warp & 3) * 32;
-            // the staging buffers are this warp's dS^T rows, read by dQ of the item's last tile
-            mbar_wait(&sh.dq_done, last & 1u, guard);
-            __syncwarp();
-            tc_fence_after();                            // dV and dK were issued before that dQ
-#pragma unroll 1
-            for (int which = 0; which < 2; ++which)
-                store_block(which == 0 ? p.dv : p.dk, p, ds_box + (warp & 3) * 4096,
-                            tmem + lane_base + (which == 0 ? kColDv : kColDk) + half * 64, at_leader(which == 0 ? &sh.dv_free : &sh.dk_free),
-                            which == 0 ? 1.0f : p.scale, half, done.head, done.tok0 + key0, done.len - key0);
-        };
+        WorkItem w;
         while (take_item(n_work, w)) {
             const int key0 = w.blk * 2 * kTile + (int)rank * kTile, key = key0 + key_in_tile;
             const bool key_valid = key < w.len, key_tail = key0 + kTile > w.len;
@@ -505,12 +492,6 @@ attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constan
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive_at(bar_p);
-                __syncwarp();
-
-                if (pending) {
-                    finish(k - 1);
-                    pending = false;
-                }
 
                 // dS^T = P^T o (dP^T - D)
                 mbar_wait(&sh.dp_done, k & 1u, guard);
@@ -548,25 +529,33 @@ attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constan
                     else mbar_arrive_at(bar_ds_smem);
                 }
             }
-            pending = true;
-            done = w;
             ++n_work;
         }
-        if (pending) finish(k - 1);
     } else {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 104;");
-        // ------------------------------------------------- dQ drain: 64 queries of the tile, half of the columns per warp pair
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 136;");
+        // ------------------------------------------------- drain: dQ (64 queries of the tile, half of the columns per warp
+        // pair) and, after an item's last tile, its dV and dK: the stores wait for the way out of the SM, 5000 cycles per
+        // item, which the compute warps cannot afford on short items and these can
         const int q_in_half = (warp & 1) * 32 + lane;
         const int col0 = ((warp >> 1) & 1) * 64;
         const int n_c4 = min(64, p.head_dim - col0) / 4;             // groups of four columns that hold data
-        const uint32_t dq_tmem = tmem + ((uint32_t)((warp & 3) * 32) << 16) + kColDq;
+        const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
+        const uint32_t dq_tmem = tmem + lane_base + kColDq;
+        uint8_t* stage = smem + kOffStage + (warp & 3) * 2048;
         const uint32_t bar_free = at_leader(&sh.dq_free);
         uint32_t n_work = 0, k = 0;
         WorkItem w;
         while (take_item(n_work, w)) {
             ++n_work;
             const int n_q = n_q_of(w);
+            const int key0 = w.blk * 2 * kTile + (int)rank * kTile + (warp & 3) * 32;
             for (int i = first_q_of(w); i < n_q; ++i, ++k) {
+                if (i == n_q - 1) {                      // dV is complete before the last dQ
+                    mbar_wait(&sh.dv_done, k & 1u, guard);
+                    __syncwarp();
+                    tc_fence_after();
+                    store_block(p.dv, p, stage, tmem + lane_base + kColDv, at_leader(&sh.dv_free), 1.0f, w.head, w.tok0 + key0, w.len - key0);
+                }
                 mbar_wait(&sh.dq_done, k & 1u, guard);
                 __syncwarp();
                 tc_fence_after();
@@ -601,6 +590,8 @@ attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constan
                                        __uint_as_float(acc[c * 4 + 2]), __uint_as_float(acc[c * 4 + 3]));
                 }
             }
+            // dK was issued before the last dQ
+            store_block(p.dk, p, stage, tmem + lane_base + kColDk, at_leader(&sh.dk_free), p.scale, w.head, w.tok0 + key0, w.len - key0);
         }
     }
 
