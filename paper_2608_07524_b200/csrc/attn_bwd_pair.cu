@@ -137,10 +137,11 @@ __device__ __forceinline__ void store_block(__nv_bfloat16* out, const BwdParams&
     }
 }
 
-// TRIM: head_dim is at most 112, so S and dP sum over ceil(head_dim / 16) steps instead of 8.  dV, dK and dQ keep their
+// KS = ceil(head_dim / 16), the steps S and dP sum over (5 to 8; a template parameter, because a step count that the issuing
+// warp reads at run time costs it 650 of 4500 cycles per tile, more than the skipped steps save).  dV, dK and dQ keep their
 // 128 columns, so that consecutive products have one shape: only then are they ordered among themselves, which S(k+1)
 // overwriting the P^T that dV(k) reads, and dP(k+1) the dS^T that dK(k) reads, rely on.
-template <bool CAUSAL, bool TRIM>
+template <bool CAUSAL, int KS>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
 attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constant__ BwdParams p) {
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -325,7 +326,6 @@ attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constan
     } else if (warp == 8) {
         // ------------------------------------------------- MMA issue (all lanes in lock step, one elected lane issues)
         const bool leader = elect_one();
-        const int n_ks = TRIM ? (p.head_dim + 15) >> 4 : 8;                      // steps of 16 columns that hold data
         constexpr uint32_t idesc_abt = make_idesc_bf16(256, 128, false, false);  // S^T, dP^T: both operands K-contiguous
         constexpr uint32_t idesc_acc = make_idesc_bf16(256, 128, false, true);   // dV, dK: A in tensor memory, B N-contiguous
         constexpr uint32_t idesc_dq = make_idesc_bf16(128, 128, true, true);     // dQ: A M-contiguous, B N-contiguous
@@ -343,8 +343,8 @@ attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constan
         // D[256 x 128] = A B^T over head_dim: A in two boxes of 128 rows, B in two boxes of 64 rows; then the per-query terms
         auto issue_abt = [&](uint32_t d_tmem, uint64_t a, uint64_t b, uint64_t ones, uint64_t stat) {
 #pragma unroll
-            for (int ks = 0; ks < 8; ++ks)
-                if (leader && (!TRIM || ks < n_ks))
+            for (int ks = 0; ks < KS; ++ks)
+                if (leader)
                     tc_mma_ss_pair(d_tmem, a + (uint64_t)(((ks / 4) * kBoxBytes + (ks % 4) * 32) >> 4),
                                    b + (uint64_t)(((ks / 4) * 8192 + (ks % 4) * 32) >> 4), idesc_abt, ks > 0);
             if (leader) tc_mma_ss_pair(d_tmem, ones, stat, idesc_abt, true);
@@ -609,17 +609,26 @@ attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constan
     cluster_sync();                                      // neither CTA leaves while the other may still address it
 }
 
-template <bool CAUSAL, bool TRIM>
-cudaError_t launch_one(const PairMaps& maps, const BwdParams& p, int n_ctas, cudaStream_t stream) {
-    if (cudaError_t e = allow_smem<attn_bwd_pair_kernel<CAUSAL, TRIM>>(kSmemBytes)) return e;
-    return launch_dependent(attn_bwd_pair_kernel<CAUSAL, TRIM>, n_ctas & ~1, kPairThreads, kSmemBytes, stream, maps, p);
+template <int KS>
+cudaError_t launch_one(const PairMaps& maps, const BwdParams& p, bool causal, int n_ctas, cudaStream_t stream) {
+    auto launch = [&](auto kern) { return launch_dependent(kern, n_ctas & ~1, kPairThreads, kSmemBytes, stream, maps, p); };
+    if (causal) {
+        if (cudaError_t e = allow_smem<attn_bwd_pair_kernel<true, KS>>(kSmemBytes)) return e;
+        return launch(attn_bwd_pair_kernel<true, KS>);
+    }
+    if (cudaError_t e = allow_smem<attn_bwd_pair_kernel<false, KS>>(kSmemBytes)) return e;
+    return launch(attn_bwd_pair_kernel<false, KS>);
 }
 
 }  // namespace
 
 cudaError_t launch_attn_bwd_pair(const PairMaps& maps, const BwdParams& p, int head_dim, bool causal, int n_ctas, cudaStream_t stream) {
-    if (head_dim > 112) return causal ? launch_one<true, false>(maps, p, n_ctas, stream) : launch_one<false, false>(maps, p, n_ctas, stream);
-    return causal ? launch_one<true, true>(maps, p, n_ctas, stream) : launch_one<false, true>(maps, p, n_ctas, stream);
+    switch ((head_dim + 15) / 16) {
+        case 5: return launch_one<5>(maps, p, causal, n_ctas, stream);
+        case 6: return launch_one<6>(maps, p, causal, n_ctas, stream);
+        case 7: return launch_one<7>(maps, p, causal, n_ctas, stream);
+        default: return launch_one<8>(maps, p, causal, n_ctas, stream);
+    }
 }
 
 }  // namespace dcp
