@@ -280,7 +280,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                 if (n_work >= 2) mbar_wait(&sh.work_empty[slot], ((n_work >> 1) - 1) & 1u, guard);
                 const uint32_t item = atomicAdd(&p.sched.hdr->work_counter, 1u);
                 if (item < n_items && !sh.abort_flag) {
-                    w = decode_item(p.sched, p.cu_seqlens, item, kTile, p.n_heads, CAUSAL, false);
+                    w = decode_item(p.sched, p.cu_seqlens, item, kTile, p.n_heads, gridDim.x, CAUSAL, false);
                 } else {
                     w.tok0 = 0; w.len = -1; w.head = 0; w.blk = 0; w.tile0 = 0;
                 }

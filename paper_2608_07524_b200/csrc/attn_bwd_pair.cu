@@ -229,7 +229,7 @@ attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constan
                 if (n >= kRing) mbar_wait_cluster(&sh.work_empty[slot], (n / kRing - 1) & 1u, guard);
                 const uint32_t item = atomicAdd(&p.sched.hdr->work_counter, 1u);
                 WorkItem w{0, -1, 0, 0, 0};
-                if (item < n_items && !sh.abort_flag) w = decode_item(p.sched, p.cu_seqlens, item, 2 * kTile, p.n_heads, CAUSAL, false);
+                if (item < n_items && !sh.abort_flag) w = decode_item(p.sched, p.cu_seqlens, item, 2 * kTile, p.n_heads, gridDim.x / 2, CAUSAL, false);
 #pragma unroll
                 for (uint32_t r = 0; r < 2; ++r) {
                     const uint32_t dst = map_to_rank(smem_u32(&sh.work[slot][0]), r);

@@ -327,7 +327,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                 const uint32_t item = atomicAdd(&p.sched.hdr->work_counter, 1u);
                 WorkItem w;
                 if (item < n_items && !sh.abort_flag) {
-                    w = decode_item(p.sched, p.cu_seqlens, item, kFwdRowsPerItem, p.n_heads, CAUSAL, CAUSAL);
+                    w = decode_item(p.sched, p.cu_seqlens, item, kFwdRowsPerItem, p.n_heads, gridDim.x, CAUSAL, CAUSAL);
                 } else {
                     w.tok0 = 0; w.len = -1; w.head = 0; w.blk = 0; w.tile0 = 0;
                 }
