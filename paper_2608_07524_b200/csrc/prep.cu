@@ -115,37 +115,39 @@ __global__ void __launch_bounds__(256) bounds_kernel(const int32_t* __restrict__
     for (int32_t t = a + lane; t < b; t += 32) bounds[t] = packed;
 }
 
-// Rank sort, one thread per sequence over as many CTAs as needed: order[] = sequence ids sorted by
+// Rank sort, eight threads per sequence over as many CTAs as needed: order[] = sequence ids sorted by
 // (length descending, id ascending).  Used on its own for batches of more than kRankInKernelMax
-// sequences (one CTA doing it for a thousand sequences takes 37 us, eight CTAs 4 us); small batches do the
-// same loop inside prep_kernel and save the launch.  Sequences
+// sequences (one CTA doing it for a thousand sequences takes 37 us, one thread per sequence 13 us, this 5 us); small
+// batches do the same loop inside prep_kernel and save the launch.  Sequences
 // from *n_live on (if given) are empty padding: they keep their own index as rank and are not
 // compared against.
+constexpr int kRankPerCta = 32, kRankSlices = 8;
 __global__ void __launch_bounds__(256) rank_kernel(const int32_t* __restrict__ cu, int32_t n_seqs,
-                                                   const uint32_t* __restrict__ n_live_ptr, int32_t* order) {
-    __shared__ int32_t len_tile[256];
+                                                  const uint32_t* __restrict__ n_live_ptr, int32_t* order) {
+    __shared__ int32_t len_tile[1024];
     grid_trigger();
     grid_wait();
     const int n_live = n_live_ptr ? min((int)*n_live_ptr, n_seqs) : n_seqs;
-    const int i = blockIdx.x * 256 + threadIdx.x;
-    if ((int)blockIdx.x * 256 >= n_live) {             // a whole block of padding
-        if (i < n_seqs) order[i] = i;
+    const int slice = threadIdx.x & (kRankSlices - 1), i = blockIdx.x * kRankPerCta + threadIdx.x / kRankSlices;
+    if ((int)blockIdx.x * kRankPerCta >= n_live) {     // a whole block of padding
+        if (slice == 0 && i < n_seqs) order[i] = i;
         return;
     }
     const int32_t len_i = i < n_seqs ? cu[i + 1] - cu[i] : 0;
-    int rank = i > n_live ? i - n_live : 0;             // padding before i, all of length 0 like i itself
-    for (int j0 = 0; j0 < n_live; j0 += 256) {
-        const int j = j0 + threadIdx.x;
+    int rank = slice == 0 && i > n_live ? i - n_live : 0;      // padding before i, all of length 0 like i itself
+    for (int j0 = 0; j0 < n_live; j0 += 1024) {
+        const int cnt = min(1024, n_live - j0);
         __syncthreads();
-        len_tile[threadIdx.x] = j < n_live ? cu[j + 1] - cu[j] : -1;     // -1 never outranks anything
+        for (int t = threadIdx.x; t < cnt; t += 256) len_tile[t] = cu[j0 + t + 1] - cu[j0 + t];
         __syncthreads();
-        const int cnt = min(256, n_live - j0);
-        for (int t = 0; t < cnt; ++t) {
+        for (int t = slice; t < cnt; t += kRankSlices) {
             const int32_t len_j = len_tile[t];
             rank += (len_j > len_i) || (len_j == len_i && j0 + t < i);
         }
     }
-    if (i < n_seqs) order[rank] = i;
+#pragma unroll
+    for (int s = 1; s < kRankSlices; s <<= 1) rank += __shfl_xor_sync(0xffffffffu, rank, s);
+    if (slice == 0 && i < n_seqs) order[rank] = i;
 }
 
 // Exclusive prefix sum of one value per thread over a CTA of NT threads; *total receives
@@ -343,7 +345,7 @@ cudaError_t launch_prep(const int32_t* cu_seqlens, int32_t n_seqs, int32_t total
     }
     const int ranked = input_order ? 2 : (n_seqs > kRankInKernelMax ? 1 : 0);
     if (ranked == 1)
-        if (cudaError_t e = launch_dependent(rank_kernel, (n_seqs + 255) / 256, 256, 0, stream, cu, n_seqs, n_live,
+        if (cudaError_t e = launch_dependent(rank_kernel, (n_seqs + kRankPerCta - 1) / kRankPerCta, 256, 0, stream, cu, n_seqs, n_live,
                                              const_cast<int32_t*>(sched.order)))
             return e;
     return launch_dependent(small ? prep_kernel<256> : prep_kernel<1024>, 1, small ? 256 : 1024, 0, stream, cu, n_seqs, n_live,
@@ -352,25 +354,22 @@ cudaError_t launch_prep(const int32_t* cu_seqlens, int32_t n_seqs, int32_t total
 }
 
 // The sequence that owns 128-row tile t: (sequence, first row of the tile inside it, its length, its first token).
-// A binary search of dependent loads, a few microseconds when they miss L1: the helper kernels below look up the
-// NEXT block's tile while the current block's loads are in flight.
+// Called by converged warps: the lanes probe 32 places at a time, two rounds of loads for a thousand sequences where a
+// binary search by every thread took ten dependent ones (512 sequences of 16-200 tokens: pre kernel 55 -> 18 us, post
+// 41 -> 14).  The post kernel looks the NEXT block's tile up while the current block's loads are in flight.
 struct TileRef {
     int seq, row0, len, tok0;
 };
 __device__ __forceinline__ TileRef find_tile(const int32_t* __restrict__ cu, const uint32_t* __restrict__ tile_prefix, int32_t n_seqs,
                                              uint32_t t) {
-    int lo = 0, hi = n_seqs;
-    // when every sequence so far has exactly one tile (batches of merged short sequences), tile t belongs
-    // to sequence t: check that before paying for the search
-    if ((int)t < n_seqs && tile_prefix[t] <= t && tile_prefix[t + 1] > t) {
-        lo = (int)t;
-        hi = lo + 1;
-    }
+    const int lane = threadIdx.x & 31;
+    int lo = 0, hi = n_seqs;                // the last sequence before hi whose tiles start at or before t: never an empty one
     while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (tile_prefix[mid] <= t) lo = mid; else hi = mid;
+        const int step = (hi - lo + 31) >> 5, probe = lo + lane * step;
+        const uint32_t below = __ballot_sync(0xffffffffu, probe < hi && tile_prefix[probe] <= t);
+        lo += (__popc(below) - 1) * step;   // lane 0 probes lo itself, which is below
+        hi = min(lo + step, hi);
     }
-    while (lo + 1 < n_seqs && tile_prefix[lo + 1] <= t) ++lo;   // skip empty sequences
     TileRef r;
     r.seq = lo;
     r.row0 = (int)(t - tile_prefix[lo]) * kTile;
