@@ -566,6 +566,9 @@ attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constan
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive_at(bar_free);
+                // the reductions go out half a tile later: sent at once they delay the exchange of the next dS^T, which the next
+                // dQ waits for (3510 -> 3447 cycles per tile; 500 ns had no effect)
+                __nanosleep(900);
                 const int row_in_tile = (int)rank * 64 + q_in_half, qrow = i * kTile + row_in_tile;
                 const bool live = qrow < w.len;
                 if (w.len <= 2 * kTile) {
