@@ -273,24 +273,22 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         }
         const uint32_t n_items = p.split ? p.sched.hdr->n_long_items : p.sched.hdr->n_items;
         uint32_t n_work = 0, g = 0;
+        SeqCursor cur;
         while (true) {
             const uint32_t slot = n_work & 1u;
-            WorkItem w;
+            uint32_t item = 0;
             if (lane == 0) {
                 if (n_work >= 2) mbar_wait(&sh.work_empty[slot], ((n_work >> 1) - 1) & 1u, guard);
-                const uint32_t item = atomicAdd(&p.sched.hdr->work_counter, 1u);
-                if (item < n_items && !sh.abort_flag) {
-                    w = decode_item(p.sched, p.cu_seqlens, item, kTile, p.n_heads, gridDim.x, CAUSAL, false);
-                } else {
-                    w.tok0 = 0; w.len = -1; w.head = 0; w.blk = 0; w.tile0 = 0;
-                }
+                item = claim_item(p.sched.hdr, n_work, blockIdx.x, gridDim.x, sh.abort_flag);
+            }
+            item = __shfl_sync(0xffffffffu, item, 0);
+            WorkItem w{0, -1, 0, 0, 0};
+            if (item < n_items) w = decode_item(p.sched, p.cu_seqlens, item, kTile, p.n_heads, gridDim.x, CAUSAL, false, cur);
+            if (lane == 0) {
                 sh.work[slot] = w;
                 mbar_arrive(&sh.work_full[slot]);
             }
-            w.tok0 = __shfl_sync(0xffffffffu, w.tok0, 0);
-            w.len = __shfl_sync(0xffffffffu, w.len, 0);
-            w.head = __shfl_sync(0xffffffffu, w.head, 0);
-            w.blk = __shfl_sync(0xffffffffu, w.blk, 0);
+            __syncwarp();
             if (w.len < 0) break;
             int first_q, n_q;
             q_range(w, first_q, n_q);

@@ -222,21 +222,24 @@ attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constan
     asm volatile("setmaxnreg.dec.sync.aligned.u32 104;");
     if (warp == 11) {
         // ------------------------------------------------- scheduler (leader): items of the list to both CTAs
-        if (lead && lane == 0) {
+        if (lead) {
             const uint32_t n_items = p.sched.hdr->n_long_items;
+            SeqCursor cur;
             for (uint32_t n = 0;; ++n) {
                 const uint32_t slot = n % kRing;
                 if (n >= kRing) mbar_wait_cluster(&sh.work_empty[slot], (n / kRing - 1) & 1u, guard);
-                const uint32_t item = atomicAdd(&p.sched.hdr->work_counter, 1u);
+                uint32_t item = 0;
+                if (lane == 0) item = claim_item(p.sched.hdr, n, blockIdx.x / 2, gridDim.x / 2, sh.abort_flag);
+                item = __shfl_sync(0xffffffffu, item, 0);
                 WorkItem w{0, -1, 0, 0, 0};
-                if (item < n_items && !sh.abort_flag) w = decode_item(p.sched, p.cu_seqlens, item, 2 * kTile, p.n_heads, gridDim.x / 2, CAUSAL, false);
-#pragma unroll
-                for (uint32_t r = 0; r < 2; ++r) {
-                    const uint32_t dst = map_to_rank(smem_u32(&sh.work[slot][0]), r);
+                if (item < n_items) w = decode_item(p.sched, p.cu_seqlens, item, 2 * kTile, p.n_heads, gridDim.x / 2, CAUSAL, false, cur);
+                if (lane < 2) {                     // a lane for each CTA
+                    const uint32_t dst = map_to_rank(smem_u32(&sh.work[slot][0]), (uint32_t)lane);
                     st_cluster_v4(dst, (uint32_t)w.tok0, (uint32_t)w.len, (uint32_t)w.head, (uint32_t)w.blk);
                     st_cluster_v4(dst + 16, (uint32_t)w.tile0, 0u, 0u, 0u);
-                    mbar_arrive_release_at(map_to_rank(smem_u32(&sh.work_full[slot]), r));
+                    mbar_arrive_release_at(map_to_rank(smem_u32(&sh.work_full[slot]), (uint32_t)lane));
                 }
+                __syncwarp();
                 if (w.len < 0) break;
             }
         }

@@ -285,7 +285,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             mbar_init(&sh.o_full[i], 1);
             mbar_init(&sh.o_free[i], 4);
             mbar_init(&sh.work_full[i], 1);
-            mbar_init(&sh.work_empty[i], 9);   // 8 softmax warps + the MMA thread
+            mbar_init(&sh.work_empty[i], 9);   // 8 softmax warps + the MMA warp
             mbar_init(&sh.stage_ready[i], 1);
             mbar_init(&sh.stage_full[i], 4);   // one arrival per warp of the group
         }
@@ -319,22 +319,24 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             tma_prefetch_desc(&tmap_q);
             tma_prefetch_desc(&tmap_k);
             tma_prefetch_desc(&tmap_v);
-            const uint32_t n_items = p.split ? p.sched.hdr->n_long_items : p.sched.hdr->n_items;
-            uint32_t n_work = 0, kv_count = 0, q_use[2] = {0, 0};
-            while (true) {
-                const uint32_t slot = n_work & 1u;
+        }
+        const uint32_t n_items = p.split ? p.sched.hdr->n_long_items : p.sched.hdr->n_items;
+        uint32_t n_work = 0, kv_count = 0, q_use[2] = {0, 0};
+        SeqCursor cur;
+        while (true) {
+            const uint32_t slot = n_work & 1u;
+            uint32_t item = 0;
+            if (lane == 0) {
                 if (n_work >= 2) mbar_wait(&sh.work_empty[slot], ((n_work >> 1) - 1) & 1u, guard);
-                const uint32_t item = atomicAdd(&p.sched.hdr->work_counter, 1u);
-                WorkItem w;
-                if (item < n_items && !sh.abort_flag) {
-                    w = decode_item(p.sched, p.cu_seqlens, item, kFwdRowsPerItem, p.n_heads, gridDim.x, CAUSAL, CAUSAL);
-                } else {
-                    w.tok0 = 0; w.len = -1; w.head = 0; w.blk = 0; w.tile0 = 0;
-                }
+                item = claim_item(p.sched.hdr, n_work, blockIdx.x, gridDim.x, sh.abort_flag);
+            }
+            item = __shfl_sync(0xffffffffu, item, 0);
+            WorkItem w{0, -1, 0, 0, 0};
+            if (item < n_items) w = decode_item(p.sched, p.cu_seqlens, item, kFwdRowsPerItem, p.n_heads, gridDim.x, CAUSAL, CAUSAL, cur);
+            ++n_work;
+            if (lane == 0) {
                 sh.work[slot] = w;
                 mbar_arrive(&sh.work_full[slot]);
-                ++n_work;
-                if (w.len < 0) break;
 
                 const int r0 = w.blk * kFwdRowsPerItem;
                 const int nkv_t[2] = {kv_tiles_for<CAUSAL>(r0, w.len), kv_tiles_for<CAUSAL>(r0 + kTile, w.len)};
@@ -357,6 +359,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                     }
                 }
             }
+            __syncwarp();
+            if (w.len < 0) break;
         }
     } else if (warp == 8) {
         // ---------------------------------------------------------------- MMA issue

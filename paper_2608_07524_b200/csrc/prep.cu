@@ -355,8 +355,8 @@ cudaError_t launch_prep(const int32_t* cu_seqlens, int32_t n_seqs, int32_t total
 
 // The sequence that owns 128-row tile t: (sequence, first row of the tile inside it, its length, its first token).
 // Called by converged warps: the lanes probe 32 places at a time, two rounds of loads for a thousand sequences where a
-// binary search by every thread took ten dependent ones (512 sequences of 16-200 tokens: pre kernel 55 -> 18 us, post
-// 41 -> 14).  The post kernel looks the NEXT block's tile up while the current block's loads are in flight.
+// binary search by every thread took ten dependent ones (512 sequences of 16-200 tokens: pre kernel 55 -> 47 us, post
+// 41 -> 30).  The post kernel looks the NEXT block's tile up while the current block's loads are in flight.
 struct TileRef {
     int seq, row0, len, tok0;
 };
