@@ -35,12 +35,13 @@ namespace dcp {
 constexpr int kPolyEveryFull = 4, kPolyEveryCausal = 8;
 constexpr int kFwdThreads = 384;   // 8 softmax warps + a 4-warp control group (MMA, producer, 2 idle)
 constexpr int kKvStages = 4;
+constexpr int kPParts = 2;         // the PV product of a tile starts with the first 128 / kPParts keys of P (see issue_pv)
 constexpr float kRescaleThreshold = 8.0f;   // in log2 units
 
 struct FwdShared {
     uint64_t q_full[2], q_empty[2];
     uint64_t kv_full[kKvStages], kv_empty[kKvStages];
-    uint64_t s_full[2], p_part[2][4], o_full[2], o_free[2];
+    uint64_t s_full[2], p_part[2][kPParts], o_full[2], o_free[2];
     uint64_t work_full[2], work_empty[2];
     uint64_t stage_ready[2], stage_full[2];    // output staging buffer of a softmax group: free to write / written
     WorkItem work[2];
@@ -96,15 +97,18 @@ __device__ __forceinline__ void issue_qk(uint32_t d_tmem, uint64_t q_desc, uint6
 }
 
 // O (+)= P V: P from tensor memory (bf16 pairs per column), V with head_dim contiguous.
-// `part` selects 32 of the tile's 128 keys: the product starts on the first part of P while the softmax
+// `part` selects 128 / kPParts of the tile's 128 keys: the product starts on the first part of P while the softmax
 // group is still producing the rest, which shortens the chain S -> softmax -> PV -> next S.
+// Two parts: the MMA warp pays about 90 cycles for each wait, the softmax warps a store wait and a fence for each
+// arrival (300 causal sequences of 200 tokens, head_dim 64, with four parts 191 us, two 179, one 178; 150 of 520,
+// head_dim 128: 663, 623, 621; two of 16384: 3.44 ms, 3.41, 3.55).
 // Only the first 16 * KS columns of O are computed.
 template <int KS>
 __device__ __forceinline__ void issue_pv(uint32_t d_tmem, uint32_t p_tmem, uint64_t v_desc, bool accumulate, bool leader, int part) {
     constexpr uint32_t idesc = make_idesc_bf16(128, KS * 16, false, true);
 #pragma unroll
-    for (int k4 = 0; k4 < 2; ++k4) {
-        const int ks = part * 2 + k4;
+    for (int k = 0; k < 8 / kPParts; ++k) {
+        const int ks = part * (8 / kPParts) + k;
         if (leader) tc_mma_ts(d_tmem, p_tmem + ks * 8, v_desc + (uint64_t)((ks * 2048) >> 4), idesc, accumulate || ks > 0);
     }
 }
@@ -166,10 +170,12 @@ __device__ __noinline__ void softmax_single_tile_item(FwdShared& sh, const FwdPa
             pk[i] = pack_bf16x2(p0, p1);
         }
         tmem_st_x16(s_tmem + c * 16, pk);
-        tmem_wait_st();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&sh.p_part[0][c]);
+        if ((c + 1) % (4 / kPParts) == 0) {
+            tmem_wait_st();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sh.p_part[0][c / (4 / kPParts)]);
+        }
     }
     float l;
     {
@@ -281,7 +287,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             mbar_init(&sh.q_full[i], 1);
             mbar_init(&sh.q_empty[i], 1);
             mbar_init(&sh.s_full[i], 1);
-            for (int k = 0; k < 4; ++k) mbar_init(&sh.p_part[i][k], 4);   // one arrival per softmax warp per 32 keys of P
+            for (int k = 0; k < kPParts; ++k) mbar_init(&sh.p_part[i][k], 4);   // one arrival per softmax warp
             mbar_init(&sh.o_full[i], 1);
             mbar_init(&sh.o_free[i], 4);
             mbar_init(&sh.work_full[i], 1);
@@ -427,7 +433,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                         if (j < nkv_t[t]) {
                             if (j == 0 && use[t] >= 1) mbar_wait(&sh.o_free[t], (use[t] - 1) & 1u, guard);
 #pragma unroll
-                            for (int part = 0; part < 4; ++part) {
+                            for (int part = 0; part < kPParts; ++part) {
                                 mbar_wait(&sh.p_part[t][part], n_p[t] & 1u, guard);
                                 tc_fence_after();
                                 issue_pv<KS>(o_tmem[t], s_tmem[t], kv_mn0 + st_v * kStageStep, j > 0, leader, part);
@@ -565,11 +571,12 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                         pk[i] = pack_bf16x2(p0, p1);
                     }
                     tmem_st_x16(s_tmem + c * 16, pk);
-                    // these 32 keys of P are in tensor memory: the PV product may use them
-                    tmem_wait_st();
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&sh.p_part[t][c]);
+                    if ((c + 1) % (4 / kPParts) == 0) {     // a part of P is in tensor memory: the PV product may use it
+                        tmem_wait_st();
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(&sh.p_part[t][c / (4 / kPParts)]);
+                    }
                 }
                 {
                     float a0, a1, b0, b1;
