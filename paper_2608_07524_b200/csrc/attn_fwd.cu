@@ -420,10 +420,22 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                     const uint32_t iv = kv_base + 2 * j + 1, ik = kv_base + 2 * j + 2;
                     const uint32_t st_v = iv % kKvStages, st_k = ik % kKvStages;
                     const bool has_next = j + 1 < nkv;
-                    kv_wait(iv);
+                    if (EARLY_Q) {
+                        // Short items: V of this pass, K of the next and the first part of P_0 in one wait, a barrier
+                        // per lane, instead of three waits of about 90 cycles each (the 200-token batch above 179 ->
+                        // 173 us, 520 tokens 623 -> 608).  On long items the three come apart, and waiting for the
+                        // last of them loses what the tests gain (two of 16384: 3.41 -> 3.50 ms).
+                        uint64_t* bar = &sh.kv_full[st_v];
+                        uint32_t par = (iv / kKvStages) & 1u;
+                        if (lane == 1 && has_next) { bar = &sh.kv_full[st_k]; par = (ik / kKvStages) & 1u; }
+                        if (lane >= 2 && j < nkv_t[0]) { bar = &sh.p_part[0][0]; par = n_p[0] & 1u; }
+                        mbar_wait_all(bar, par, guard);
+                    } else {
+                        kv_wait(iv);
+                    }
 #pragma unroll
                     for (int t = 0; t < 2; ++t) {
-                        if (t == 1 && has_next) kv_wait(ik);
+                        if (!EARLY_Q && t == 1 && has_next) kv_wait(ik);
                         if (t == 1 && j + 1 < nkv_t[0]) {      // S_0(j+1) goes between the two PV products
                             tc_fence_after();
                             issue_qk<D, KS>(s_tmem[0], q_desc[0], kv_km0 + st_k * kStageStep, leader);
@@ -434,7 +446,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                             if (j == 0 && use[t] >= 1) mbar_wait(&sh.o_free[t], (use[t] - 1) & 1u, guard);
 #pragma unroll
                             for (int part = 0; part < kPParts; ++part) {
-                                mbar_wait(&sh.p_part[t][part], n_p[t] & 1u, guard);
+                                if (!EARLY_Q || t == 1 || part > 0) mbar_wait(&sh.p_part[t][part], n_p[t] & 1u, guard);
                                 tc_fence_after();
                                 issue_pv<KS>(o_tmem[t], s_tmem[t], kv_mn0 + st_v * kStageStep, j > 0, leader, part);
                             }
