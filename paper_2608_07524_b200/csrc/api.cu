@@ -412,6 +412,7 @@ static int attn_bwd_impl(const char* fn, const void* q, const void* k, const voi
     const bool pair = pair_path(head_dim);
     const int32_t direct_len = pair ? kPairDirectLen : kTile;      // longest sequence that is a single key block
     const bool split = pair || split_tiles(n_seqs, total_tokens, max_seqlen, n_heads, dev.sm_count);
+    const int32_t tiles_per_item = !split ? 0 : pair ? 2 : 1;      // of the main kernel, for the helpers' block list
     const bool multi = max_seqlen > kTile || !split;               // there may be items for the multi-tile kernel
     {
         ScopedTimer t(DCP_KERNEL_PREP, stream);
@@ -434,7 +435,7 @@ static int attn_bwd_impl(const char* fn, const void* q, const void* k, const voi
         ScopedTimer t(DCP_KERNEL_BWD_PRE, stream);
         e = launch_bwd_pre(static_cast<const __nv_bfloat16*>(o), static_cast<const __nv_bfloat16*>(d_o), lse, vcu,
                            sched, stats, dq_acc, max_tiles(total_tokens, n_seqs) * kTile * n_heads * padded_dim(head_dim),
-                           total_tokens, n_heads, head_dim, token_stride, scale, split ? kTile : 0, direct_len, dev.sm_count, stream);
+                           total_tokens, n_heads, head_dim, token_stride, scale, tiles_per_item, direct_len, dev.sm_count, stream);
         if (e != cudaSuccess) return fail(DCP_ERR_CUDA, "%s: pre kernel: %s", fn, cudaGetErrorString(e));
         g_launches.fetch_add(1);
     }
@@ -485,7 +486,7 @@ static int attn_bwd_impl(const char* fn, const void* q, const void* k, const voi
     if (multi) {
         ScopedTimer t(DCP_KERNEL_BWD_POST, stream);
         e = launch_bwd_post(dq_acc, static_cast<__nv_bfloat16*>(dq), vcu, sched, total_tokens, n_heads, head_dim, token_stride,
-                            scale, direct_len, dev.sm_count, stream);
+                            scale, tiles_per_item, direct_len, dev.sm_count, stream);
         if (e != cudaSuccess) return fail(DCP_ERR_CUDA, "%s: post kernel: %s", fn, cudaGetErrorString(e));
         g_launches.fetch_add(1);
     }

@@ -94,11 +94,12 @@ cudaError_t launch_attn_fwd(const CUtensorMap& tq, const CUtensorMap& tk, const 
 
 // Tile-aligned row statistics for the backward kernel (see BwdParams::stats) and dq_acc = 0.  Sequences of at most
 // direct_len tokens get their dQ written by the main kernel: here and in the post kernel they have no accumulator.
-// Those of at most skip_len tokens are not the main kernel's at all.
+// tiles_per_item: 128-row tiles of an item of the work list when the single-tile kernel takes part of the batch (both
+// helpers then see the rest only), else 0.
 cudaError_t launch_bwd_pre(const __nv_bfloat16* o, const __nv_bfloat16* d_o, const float* lse, const int32_t* cu_seqlens,
                            const SchedView& sched, __nv_bfloat16* stats, float* dq_acc, size_t dq_acc_elems,
                            int32_t total_tokens, int32_t n_heads, int32_t head_dim, int64_t row_stride, float scale,
-                           int32_t skip_len, int32_t direct_len, int n_sms, cudaStream_t stream);
+                           int32_t tiles_per_item, int32_t direct_len, int n_sms, cudaStream_t stream);
 
 cudaError_t launch_attn_bwd_pair(const PairMaps& maps, const BwdParams& p, int head_dim, bool causal, int n_ctas, cudaStream_t stream);
 
@@ -109,7 +110,7 @@ cudaError_t launch_attn_bwd(const CUtensorMap& tq, const CUtensorMap& tk, const 
 // dq[T, H, d] = bf16(scale * dq_acc), undoing the tile-blocked layout
 cudaError_t launch_bwd_post(const float* dq_acc, __nv_bfloat16* dq, const int32_t* cu_seqlens, const SchedView& sched,
                             int32_t total_tokens, int32_t n_heads, int32_t head_dim, int64_t row_stride, float scale,
-                            int32_t direct_len, int n_sms, cudaStream_t stream);
+                            int32_t tiles_per_item, int32_t direct_len, int n_sms, cudaStream_t stream);
 
 // Batches in which no sequence exceeds kSmallSeqMaxLen tokens (the declared max_seqlen says so) skip the work list
 // and the 128-row tile kernels, see attn_small.cu.  The check kernel is the first of such a call (boundaries

@@ -353,30 +353,54 @@ cudaError_t launch_prep(const int32_t* cu_seqlens, int32_t n_seqs, int32_t total
                             const_cast<uint32_t*>(sched.tile_prefix), ranked, total_tokens, tile_capacity, long_min_len, no_long);
 }
 
-// The sequence that owns 128-row tile t: (sequence, first row of the tile inside it, its length, its first token).
-// Called by converged warps: the lanes probe 32 places at a time, two rounds of loads for a thousand sequences where a
-// binary search by every thread took ten dependent ones (512 sequences of 16-200 tokens: pre kernel 55 -> 47 us, post
-// 41 -> 30).  The post kernel looks the NEXT block's tile up while the current block's loads are in flight.
-struct TileRef {
-    int seq, row0, len, tok0;
+// A (128-row tile, head) block of the backward helpers.
+struct BlockRef {
+    uint32_t tile, head;
+    int row0, len, tok0;        // first row inside the sequence, the sequence's length and first token
 };
-__device__ __forceinline__ TileRef find_tile(const int32_t* __restrict__ cu, const uint32_t* __restrict__ tile_prefix, int32_t n_seqs,
-                                             uint32_t t) {
-    const int lane = threadIdx.x & 31;
-    int lo = 0, hi = n_seqs;                // the last sequence before hi whose tiles start at or before t: never an empty one
-    while (hi - lo > 1) {
-        const int step = (hi - lo + 31) >> 5, probe = lo + lane * step;
-        const uint32_t below = __ballot_sync(0xffffffffu, probe < hi && tile_prefix[probe] <= t);
-        lo += (__popc(below) - 1) * step;   // lane 0 probes lo itself, which is below
-        hi = min(lo + step, hi);
+
+// Where the helpers find their blocks.  tiles_per_item > 0: in the work list's sequences of more than one tile, which come
+// first in it, tiles_per_item tiles to an item; heads vary fastest, so that CTAs running at the same time share memory
+// pages.  0: in all tiles of the batch, in input order.  Going through all tiles of a batch of short sequences, nine
+// tenths of them to be skipped after a search, took longer than the work (512 sequences of 16-200 tokens, head_dim 64: pre
+// kernel 51 -> 40 us, post 33 -> 29; with only the rows inside the sequences zeroed and read, 35 and 25).
+struct BlockList {
+    const int32_t* cu;
+    const int32_t* order;
+    const uint32_t* prefix;
+    const uint32_t* tile_prefix;
+    const WorkspaceHeader* hdr;
+    int32_t n_seqs, n_heads, tiles_per_item;
+
+    __device__ __forceinline__ uint32_t size() const {
+        return tiles_per_item > 0 ? hdr->n_long_items * (uint32_t)tiles_per_item : tile_prefix[n_seqs] * (uint32_t)n_heads;
     }
-    TileRef r;
-    r.seq = lo;
-    r.row0 = (int)(t - tile_prefix[lo]) * kTile;
-    r.tok0 = cu[lo];
-    r.len = cu[lo + 1] - r.tok0;
-    return r;
-}
+    // Called by converged warps: the lanes probe 32 places at a time, two rounds of loads for a thousand sequences where a
+    // binary search by every thread took ten dependent ones (512 sequences of 16-200 tokens: pre kernel 55 -> 47 us, post
+    // 41 -> 30).  The post kernel looks the NEXT block up while the current block's loads are in flight.
+    __device__ __forceinline__ BlockRef find(uint32_t idx) const {
+        const int lane = threadIdx.x & 31;
+        const bool listed = tiles_per_item > 0;
+        const uint32_t* const start = listed ? prefix : tile_prefix;
+        const uint32_t scale = listed ? (uint32_t)tiles_per_item : (uint32_t)n_heads;
+        int lo = 0, hi = listed ? (int)hdr->n_long_seqs : n_seqs;   // the last place whose blocks start at or before idx
+        while (hi - lo > 1) {
+            const int step = (hi - lo + 31) >> 5, probe = lo + lane * step;
+            const uint32_t below = __ballot_sync(0xffffffffu, probe < hi && start[probe] * scale <= idx);
+            lo += (__popc(below) - 1) * step;   // lane 0 probes lo itself, which is below
+            hi = min(lo + step, hi);
+        }
+        const int seq = listed ? order[lo] : lo;
+        const uint32_t local = idx - start[lo] * scale, in_seq = local / (uint32_t)n_heads;
+        BlockRef r;
+        r.head = local % (uint32_t)n_heads;
+        r.tile = tile_prefix[seq] + in_seq;
+        r.row0 = (int)in_seq * kTile;
+        r.tok0 = cu[seq];
+        r.len = cu[seq + 1] - r.tok0;
+        return r;
+    }
+};
 
 // ---------------------------------------------------------------------------------------------
 // Backward helper 1.  For every (128-row tile, head) it writes a [128 rows x 16] bf16 tile holding,
@@ -390,28 +414,28 @@ __device__ __forceinline__ TileRef find_tile(const int32_t* __restrict__ cu, con
 template <int D>
 __global__ void __launch_bounds__(256) bwd_pre_kernel(const __nv_bfloat16* __restrict__ o,
                                                       const __nv_bfloat16* __restrict__ d_o, const float* __restrict__ lse,
-                                                      const int32_t* __restrict__ cu, const uint32_t* __restrict__ tile_prefix,
-                                                      int32_t n_seqs, __nv_bfloat16* __restrict__ stats,
+                                                      const BlockList list, __nv_bfloat16* __restrict__ stats,
                                                       float* __restrict__ dq_acc, size_t dq_acc_vec4,
                                                       int32_t total_tokens, int32_t n_heads, int32_t head_dim,
-                                                      int64_t row_stride, float inv_scale, int32_t skip_len, int32_t direct_len) {
+                                                      int64_t row_stride, float inv_scale, int32_t direct_len) {
     grid_trigger();
     grid_wait();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t n_blocks = tile_prefix[n_seqs] * (uint32_t)n_heads;
-    for (uint32_t blk = blockIdx.x; blk < n_blocks; blk += gridDim.x) {
-        const uint32_t t = blk / n_heads, h = blk % n_heads;
+    const uint32_t n_blocks = list.size();
+    for (uint32_t idx = blockIdx.x; idx < n_blocks; idx += gridDim.x) {
         // (looking the next block's tile up while this block's loads are in flight, as the post kernel does, made
         // this kernel slower: 0.39 -> 0.44 ms on 131072 tokens x 16 heads)
-        const TileRef ref = find_tile(cu, tile_prefix, n_seqs, t);
+        const BlockRef ref = list.find(idx);
         const int row0 = ref.row0, len = ref.len, tok0 = ref.tok0;
-        if (len <= skip_len) continue;
+        if (row0 >= len) continue;                       // an item's second tile may lie past the end
+        const uint32_t t = ref.tile, h = ref.head, blk = t * (uint32_t)n_heads + h;
         if (len > direct_len) {
             // this (tile, head) block of the dQ accumulator; a sequence of a single key block needs none (the main
             // kernel holds its whole dQ and writes it directly)
             float4* acc_blk = reinterpret_cast<float4*>(dq_acc) + (size_t)blk * (kTile * D / 4);
             if ((size_t)(blk + 1) * (kTile * D / 4) <= dq_acc_vec4)
-                for (int e = threadIdx.x; e < kTile * D / 4; e += blockDim.x) acc_blk[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int e = threadIdx.x; e < kTile * D / 4; e += blockDim.x)      // the main kernel adds to no other rows
+                    if (e % kTile < len - row0) acc_blk[e] = make_float4(0.f, 0.f, 0.f, 0.f);
         }
         {
         uint8_t* out = reinterpret_cast<uint8_t*>(stats) + ((size_t)t * n_heads + h) * (kTile * 16 * 2);
@@ -485,13 +509,13 @@ __global__ void __launch_bounds__(256) bwd_pre_kernel(const __nv_bfloat16* __res
 cudaError_t launch_bwd_pre(const __nv_bfloat16* o, const __nv_bfloat16* d_o, const float* lse, const int32_t* cu_seqlens,
                            const SchedView& sched, __nv_bfloat16* stats, float* dq_acc, size_t dq_acc_elems,
                            int32_t total_tokens, int32_t n_heads, int32_t head_dim, int64_t row_stride, float scale,
-                           int32_t skip_len, int32_t direct_len, int n_sms, cudaStream_t stream) {
+                           int32_t tiles_per_item, int32_t direct_len, int n_sms, cudaStream_t stream) {
     // no more CTAs than (tile, head) blocks the batch can have
     const size_t most = max_tiles(total_tokens, sched.n_seqs) * (size_t)n_heads;
     const unsigned blocks = most < (size_t)n_sms * 8 ? (unsigned)most : (unsigned)n_sms * 8;
-    return launch_dependent(head_dim > 64 ? bwd_pre_kernel<128> : bwd_pre_kernel<64>, blocks, 256, 0, stream, o, d_o, lse, cu_seqlens,
-                            sched.tile_prefix, sched.n_seqs, stats, dq_acc, dq_acc_elems / 4, total_tokens, n_heads, head_dim, row_stride,
-                            1.0f / scale, skip_len, direct_len);
+    const BlockList list{cu_seqlens, sched.order, sched.prefix, sched.tile_prefix, sched.hdr, sched.n_seqs, n_heads, tiles_per_item};
+    return launch_dependent(head_dim > 64 ? bwd_pre_kernel<128> : bwd_pre_kernel<64>, blocks, 256, 0, stream, o, d_o, lse, list, stats,
+                            dq_acc, dq_acc_elems / 4, total_tokens, n_heads, head_dim, row_stride, 1.0f / scale, direct_len);
 }
 
 // Backward helper 2: dq[T, H, d] = bf16(scale * dq_acc).  dq_acc holds, per (tile, head), a block
@@ -500,24 +524,22 @@ cudaError_t launch_bwd_pre(const __nv_bfloat16* o, const __nv_bfloat16* d_o, con
 // sequences of a single tile, whose dQ the main kernel has already written.
 template <int D>
 __global__ void __launch_bounds__(256) bwd_post_kernel(const float* __restrict__ dq_acc, __nv_bfloat16* __restrict__ dq,
-                                                       const int32_t* __restrict__ cu, const uint32_t* __restrict__ tile_prefix,
-                                                       int32_t n_seqs, int32_t n_heads, int32_t head_dim, int64_t row_stride,
+                                                       const BlockList list, int32_t n_heads, int32_t head_dim, int64_t row_stride,
                                                        float scale, int32_t direct_len) {
     constexpr int kRowBytes = D * 2 + 16;                    // padded row of bf16
     __shared__ __align__(16) uint8_t tile[kTile * kRowBytes];
     grid_trigger();
     grid_wait();
-    const uint32_t n_blocks = tile_prefix[n_seqs] * (uint32_t)n_heads;
+    const uint32_t n_blocks = list.size();
     if (blockIdx.x >= n_blocks) return;
-    TileRef ref = find_tile(cu, tile_prefix, n_seqs, blockIdx.x / n_heads), ref_next = ref;
-    for (uint32_t blk = blockIdx.x; blk < n_blocks; blk += gridDim.x, ref = ref_next) {
-        const uint32_t t = blk / n_heads, h = blk % n_heads;
-        const bool more = blk + gridDim.x < n_blocks;
-        const uint32_t t_next = (blk + gridDim.x) / n_heads;
+    BlockRef ref = list.find(blockIdx.x), ref_next = ref;
+    for (uint32_t idx = blockIdx.x; idx < n_blocks; idx += gridDim.x, ref = ref_next) {
+        const uint32_t t = ref.tile, h = ref.head;
+        const bool more = idx + gridDim.x < n_blocks;
         const int row0 = ref.row0, len = ref.len;
         const int rows = min(kTile, len - row0);
-        if (len <= direct_len) {          // a single key block: the main kernel has written dq itself
-            if (more) ref_next = find_tile(cu, tile_prefix, n_seqs, t_next);
+        if (len <= direct_len || row0 >= len) {          // a single key block: the main kernel has written dq itself
+            if (more) ref_next = list.find(idx + gridDim.x);
             continue;
         }
         const float4* src = reinterpret_cast<const float4*>(dq_acc + ((size_t)t * n_heads + h) * (kTile * D));
@@ -526,11 +548,13 @@ __global__ void __launch_bounds__(256) bwd_post_kernel(const float* __restrict__
         for (int e0 = threadIdx.x; e0 < kTile * D / 4; e0 += 8 * 256) {
             float4 v[8];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) v[u] = src[e0 + u * 256];
-            if (e0 == (int)threadIdx.x && more) ref_next = find_tile(cu, tile_prefix, n_seqs, t_next);
+            for (int u = 0; u < 8; ++u)
+                if ((e0 + u * 256) % kTile < rows) v[u] = src[e0 + u * 256];
+            if (e0 == (int)threadIdx.x && more) ref_next = list.find(idx + gridDim.x);
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
                 const int e = e0 + u * 256, c4 = e / kTile, r = e % kTile;
+                if (r >= rows) continue;
                 __nv_bfloat162 lo2 = __floats2bfloat162_rn(v[u].x * scale, v[u].y * scale);
                 __nv_bfloat162 hi2 = __floats2bfloat162_rn(v[u].z * scale, v[u].w * scale);
                 uint2 pk;
@@ -553,11 +577,12 @@ __global__ void __launch_bounds__(256) bwd_post_kernel(const float* __restrict__
 
 cudaError_t launch_bwd_post(const float* dq_acc, __nv_bfloat16* dq, const int32_t* cu_seqlens, const SchedView& sched,
                             int32_t total_tokens, int32_t n_heads, int32_t head_dim, int64_t row_stride, float scale,
-                            int32_t direct_len, int n_sms, cudaStream_t stream) {
+                            int32_t tiles_per_item, int32_t direct_len, int n_sms, cudaStream_t stream) {
     const size_t most = max_tiles(total_tokens, sched.n_seqs) * (size_t)n_heads;
     const unsigned blocks = most < (size_t)n_sms * 6 ? (unsigned)most : (unsigned)n_sms * 6;
-    return launch_dependent(head_dim > 64 ? bwd_post_kernel<128> : bwd_post_kernel<64>, blocks, 256, 0, stream, dq_acc, dq, cu_seqlens,
-                            sched.tile_prefix, sched.n_seqs, n_heads, head_dim, row_stride, scale, direct_len);
+    const BlockList list{cu_seqlens, sched.order, sched.prefix, sched.tile_prefix, sched.hdr, sched.n_seqs, n_heads, tiles_per_item};
+    return launch_dependent(head_dim > 64 ? bwd_post_kernel<128> : bwd_post_kernel<64>, blocks, 256, 0, stream, dq_acc, dq, list,
+                            n_heads, head_dim, row_stride, scale, direct_len);
 }
 
 }  // namespace dcp
