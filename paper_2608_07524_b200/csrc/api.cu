@@ -195,6 +195,7 @@ SchedView carve_sched(void* workspace, int32_t n_seqs) {
     s.prefix = reinterpret_cast<const uint32_t*>(base + sizeof(int32_t) * (size_t)n_seqs);
     s.tile_prefix = s.prefix + (size_t)n_seqs + 1;
     s.vcu = reinterpret_cast<const int32_t*>(s.tile_prefix + (size_t)n_seqs + 1);
+    s.vfirst = s.vcu + (size_t)n_seqs + 1;
     s.n_seqs = n_seqs;
     return s;
 }
@@ -265,7 +266,9 @@ static int attn_fwd_impl(const char* fn, bool merge, const void* q, const void* 
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
 
     const SchedView sched = carve_sched(workspace, n_seqs);
-    uint16_t* bounds = merge ? reinterpret_cast<uint16_t*>(static_cast<uint8_t*>(workspace) + sched_bytes(n_seqs)) : nullptr;
+    const bool split = split_tiles(n_seqs, total_tokens, max_seqlen, n_heads, dev.sm_count);
+    // the per-token table is read by the multi-tile kernel where that takes the merged sequences
+    uint16_t* bounds = merge && !split ? reinterpret_cast<uint16_t*>(static_cast<uint8_t*>(workspace) + sched_bytes(n_seqs)) : nullptr;
     cudaError_t e;
     const float scale = softmax_scale > 0.f ? softmax_scale : 1.0f / std::sqrt((float)head_dim);
     if (short_sequence_path(n_seqs, total_tokens, max_seqlen)) {
@@ -290,14 +293,13 @@ static int attn_fwd_impl(const char* fn, bool merge, const void* q, const void* 
         return DCP_OK;
     }
     const bool input_order = g_input_order.load() != 0;
-    const bool split = split_tiles(n_seqs, total_tokens, max_seqlen, n_heads, dev.sm_count);
     {
         ScopedTimer t(DCP_KERNEL_PREP, stream);
-        e = launch_prep(cu_seqlens, n_seqs, total_tokens, max_seqlen, kFwdRowsPerItem, n_heads, sched, bounds, UINT32_MAX,
+        e = launch_prep(cu_seqlens, n_seqs, total_tokens, max_seqlen, kFwdRowsPerItem, n_heads, sched, merge, bounds, UINT32_MAX,
                         input_order, split ? kTile + 1 : INT32_MAX, max_seqlen <= kTile, stream);
     }
     if (e != cudaSuccess) return fail(DCP_ERR_CUDA, "%s: work-list kernel: %s", fn, cudaGetErrorString(e));
-    g_launches.fetch_add(prep_launches(n_seqs, merge, input_order));
+    g_launches.fetch_add(prep_launches(n_seqs, merge, bounds != nullptr, input_order));
     if (total_tokens == 0 || n_seqs == 0) return DCP_OK;
 
     CUtensorMap tq, tk, tv, to;
@@ -308,6 +310,7 @@ static int attn_fwd_impl(const char* fn, bool merge, const void* q, const void* 
 
     FwdParams p;
     p.cu_seqlens = merge ? sched.vcu : cu_seqlens;
+    p.members = merge ? cu_seqlens : nullptr;
     p.bounds = bounds;
     p.o = static_cast<__nv_bfloat16*>(o);
     p.lse = lse;
@@ -379,7 +382,9 @@ static int attn_bwd_impl(const char* fn, const void* q, const void* k, const voi
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
 
     const SchedView sched = carve_sched(workspace, n_seqs);
-    uint16_t* bounds = reinterpret_cast<uint16_t*>(static_cast<uint8_t*>(workspace) + sched_bytes(n_seqs));
+    const bool pair = pair_path(head_dim);
+    const bool split = pair || split_tiles(n_seqs, total_tokens, max_seqlen, n_heads, dev.sm_count);
+    uint16_t* bounds = split ? nullptr : reinterpret_cast<uint16_t*>(static_cast<uint8_t*>(workspace) + sched_bytes(n_seqs));
     uint8_t* base = static_cast<uint8_t*>(workspace) + sched_bytes(n_seqs) + bounds_bytes(total_tokens);
     __nv_bfloat16* stats = reinterpret_cast<__nv_bfloat16*>(base);
     float* dq_acc = reinterpret_cast<float*>(base + align256(max_tiles(total_tokens, n_seqs) * n_heads * (size_t)(kTile * 16 * 2)));
@@ -409,18 +414,16 @@ static int attn_bwd_impl(const char* fn, const void* q, const void* k, const voi
         return DCP_OK;
     }
     const bool input_order = g_input_order.load() != 0;
-    const bool pair = pair_path(head_dim);
     const int32_t direct_len = pair ? kPairDirectLen : kTile;      // longest sequence that is a single key block
-    const bool split = pair || split_tiles(n_seqs, total_tokens, max_seqlen, n_heads, dev.sm_count);
     const int32_t tiles_per_item = !split ? 0 : pair ? 2 : 1;      // of the main kernel, for the helpers' block list
     const bool multi = max_seqlen > kTile || !split;               // there may be items for the multi-tile kernel
     {
         ScopedTimer t(DCP_KERNEL_PREP, stream);
-        e = launch_prep(cu_seqlens, n_seqs, total_tokens, max_seqlen, pair ? 2 * kTile : kTile, n_heads, sched, bounds,
+        e = launch_prep(cu_seqlens, n_seqs, total_tokens, max_seqlen, pair ? 2 * kTile : kTile, n_heads, sched, true, bounds,
                         (uint32_t)max_tiles(total_tokens, n_seqs), input_order, split ? kTile + 1 : INT32_MAX, !multi, stream);
     }
     if (e != cudaSuccess) return fail(DCP_ERR_CUDA, "%s: work-list kernel: %s", fn, cudaGetErrorString(e));
-    g_launches.fetch_add(prep_launches(n_seqs, true, input_order));
+    g_launches.fetch_add(prep_launches(n_seqs, true, bounds != nullptr, input_order));
     const int32_t* vcu = sched.vcu;      // every later kernel works on the virtual sequences
     if (total_tokens == 0 || n_seqs == 0) return DCP_OK;
 
@@ -442,6 +445,7 @@ static int attn_bwd_impl(const char* fn, const void* q, const void* k, const voi
 
     BwdParams p;
     p.cu_seqlens = vcu;
+    p.members = cu_seqlens;
     p.bounds = bounds;
     p.stats = stats;
     p.dq_acc = dq_acc;

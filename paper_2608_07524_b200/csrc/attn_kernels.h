@@ -10,7 +10,8 @@ namespace dcp {
 
 struct FwdParams {
     const int32_t* cu_seqlens;    // boundaries of the (virtual) sequences the work list was built over
-    const uint16_t* bounds;       // per-token table of the merged path (see sched.cuh), or null
+    const int32_t* members;       // the caller's boundaries where sequences have been merged (launch_tile_fwd), or null
+    const uint16_t* bounds;       // per-token table of the merged path (launch_attn_fwd, see sched.cuh), or null
     __nv_bfloat16* o;
     float* lse;
     SchedView sched;
@@ -26,6 +27,7 @@ struct FwdParams {
 
 struct BwdParams {
     const int32_t* cu_seqlens;    // as in FwdParams
+    const int32_t* members;
     const uint16_t* bounds;
     const __nv_bfloat16* stats;   // per (tile, head) a [128 queries x 16] bf16 tile in the layout the MMA reads:
                                   // columns 0-2 = -lse/scale split in three bf16 parts, 8-10 = -D likewise
@@ -63,10 +65,10 @@ cudaError_t launch_tile_bwd(const CUtensorMap& tq, const CUtensorMap& tk, const 
                             const BwdParams& p, bool causal, int n_sms, cudaStream_t stream);
 
 // Builds the work list (longest sequence first) and resets the work counter and status word.
-// With `bounds` non-null, short sequences are first merged into virtual sequences: sched.vcu and
-// `bounds` are written and the list is built over sched.vcu, which the later kernels must then be
-// given as their boundary array; with `bounds` null the list is built over cu_seqlens itself.
-int prep_launches(int32_t n_seqs, bool merge, bool input_order);   // kernels launch_prep enqueues (1 to 4)
+// With `merge`, short sequences are first merged into virtual sequences: sched.vcu and sched.vfirst
+// (and `bounds`, unless it is null) are written and the list is built over sched.vcu, which the later kernels must then be
+// given as their boundary array; without, the list is built over cu_seqlens itself.
+int prep_launches(int32_t n_seqs, bool merge, bool table, bool input_order);   // kernels launch_prep enqueues (1 to 4)
 // tile_capacity = number of 128-row tiles the per-tile storage of the workspace holds (UINT32_MAX if the
 // call uses none).  Inconsistent boundaries or more tiles than that leave an empty work list and
 // kStatusBadLengths in the status word.  input_order = true lists the sequences as they come instead of
@@ -74,7 +76,7 @@ int prep_launches(int32_t n_seqs, bool merge, bool input_order);   // kernels la
 // tokens come first in either order and empty ones last; the header counts the first and their items (n_long_seqs, n_long_items);
 // no_long: max_seqlen promises that there are none.
 cudaError_t launch_prep(const int32_t* cu_seqlens, int32_t n_seqs, int32_t total_tokens, int32_t max_seqlen,
-                        int32_t rows_per_block, int32_t n_heads, const SchedView& sched, uint16_t* bounds,
+                        int32_t rows_per_block, int32_t n_heads, const SchedView& sched, bool merge, uint16_t* bounds,
                         uint32_t tile_capacity, bool input_order, int32_t long_min_len, bool no_long, cudaStream_t stream);
 
 // One CTA that waits, with the kernels' own bounded wait and the given poll limit, on a barrier nobody

@@ -13,7 +13,7 @@
 // registers (it equals sum_c dO_ic O_ic because O = P V), so these items need no pass over O, no per-query tiles, no fp32
 // accumulator and no conversion pass: q, k, v, dO in, dq, dk, dv out.
 //
-// Several short sequences may share the tile: row i sees the keys [first, end) of its own sequence (per-token table), and
+// Several short sequences may share the tile: row i sees the keys [first, end) of its own sequence, and
 // a warp skips the 32-key chunks that none of its rows sees.
 //
 // Roles (192 threads): warps 0-3 compute, warp 4 TMA producer, warp 5 MMA issue.  Items are dealt round robin: they cost
@@ -38,28 +38,38 @@ constexpr int kTileThreads = 192;
 constexpr int kBoxBytes = kTile * 128;               // 128 rows of 64 bf16 columns
 
 struct TileItem {
-    int tok0, len, head;
+    int tok0, len, head, seq;
 };
 
 // Item i of the single-tile part of the work list: its sequences come after the longer ones, n_heads items each.
 __device__ __forceinline__ TileItem tile_item(const SchedView& s, const int32_t* cu, uint32_t first_seq, uint32_t i, int n_heads) {
-    const int seq = s.order[first_seq + i / (uint32_t)n_heads];
     TileItem w;
+    w.seq = s.order[first_seq + i / (uint32_t)n_heads];
     w.head = (int)(i % (uint32_t)n_heads);
-    w.tok0 = cu[seq];
-    w.len = cu[seq + 1] - w.tok0;
+    w.tok0 = cu[w.seq];
+    w.len = cu[w.seq + 1] - w.tok0;
     return w;
 }
 
-// Keys [lo, hi) that a row sees; none for rows past the end.
-__device__ __forceinline__ void row_keys(const TileItem& w, int row, const uint16_t* bounds, bool causal, int& lo, int& hi) {
+// Keys [lo, hi) that a row sees; none for rows past the end.  A row of a merged sequence (`members` = the caller's
+// boundaries) finds its own sequence by bisection among the members: a few cached loads while the item's products run.
+// (A table of every token's range, as the multi-tile kernels read it, takes a launch to fill.)
+__device__ __forceinline__ void row_keys(const TileItem& w, int row, const SchedView& s, const int32_t* __restrict__ members, bool causal,
+                                         int& lo, int& hi) {
     lo = hi = 0;
     if (row < w.len) {
         hi = w.len;
-        if (bounds) {
-            const uint32_t b = bounds[(size_t)w.tok0 + row];
-            lo = (int)(b & 0xffu);
-            hi = (int)(b >> 8);
+        if (members) {
+            int a = s.vfirst[w.seq], b = s.vfirst[w.seq + 1];
+            if (b - a > 1) {                         // the last member that starts at or before this token: it is not empty
+                while (b - a > 1) {
+                    const int mid = (a + b) >> 1;
+                    if (members[mid] <= w.tok0 + row) a = mid;
+                    else b = mid;
+                }
+                lo = members[a] - w.tok0;
+                hi = members[a + 1] - w.tok0;
+            }
         }
         if (causal && hi > row + 1) hi = row + 1;
     }
@@ -196,11 +206,11 @@ tile_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         const uint32_t my = tmem + ((uint32_t)(warp * 32) << 16);
         const int row = tid;                                         // query row
         const uint64_t sc2 = pack_f32x2(p.scale_log2, p.scale_log2);
-        TileItem w{0, 0, 0};
+        TileItem w{0, 0, 0, 0};
         int lo = 0, hi = 0;
         if (blockIdx.x < n) {
             w = tile_item(p.sched, p.cu_seqlens, first_seq, blockIdx.x, p.n_heads);
-            row_keys(w, row, p.bounds, causal, lo, hi);
+            row_keys(w, row, p.sched, p.members, causal, lo, hi);
         }
         uint32_t k = 0;
         for (uint32_t i = blockIdx.x; i < n; i += gridDim.x, ++k) {
@@ -264,7 +274,7 @@ tile_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             if (valid) p.lse[(size_t)cur.head * p.total_tokens + cur.tok0 + row] = m * p.scale + __logf(l);
             if (i + gridDim.x < n) {                 // the next item's keys, while the product runs
                 w = tile_item(p.sched, p.cu_seqlens, first_seq, i + gridDim.x, p.n_heads);
-                row_keys(w, row, p.bounds, causal, lo, hi);
+                row_keys(w, row, p.sched, p.members, causal, lo, hi);
             }
             mbar_wait(&sh.o_full, k & 1u, guard);
             __syncwarp();
@@ -431,12 +441,12 @@ tile_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         const int row = tid;                                 // query row
         uint8_t *p_row = smem + Cfg::kOffP, *ds_row = smem + Cfg::kOffDs, *stage = smem + Cfg::kOffP + warp * 4096;
         const uint64_t sc2 = pack_f32x2(p.scale_log2, p.scale_log2);
-        TileItem w{0, 0, 0};
+        TileItem w{0, 0, 0, 0};
         int lo = 0, hi = 0;
         float lse = 0.f;
         auto fetch = [&](uint32_t i) {
             w = tile_item(p.sched, p.cu_seqlens, first_seq, i, p.n_heads);
-            row_keys(w, row, p.bounds, causal, lo, hi);
+            row_keys(w, row, p.sched, p.members, causal, lo, hi);
             lse = row < w.len ? p.lse[(size_t)w.head * p.total_tokens + w.tok0 + row] : 0.f;
         };
         if (blockIdx.x < n) fetch(blockIdx.x);

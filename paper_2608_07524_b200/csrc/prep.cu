@@ -33,9 +33,10 @@ template <int NT> __device__ inline int block_exclusive_max_scan(int v, int* scr
 // bound on the number of tiles that sizes the workspace: it is derived for rule 0).
 // Outputs: vcu[0..n_v] = boundaries of the virtual sequences, vcu[n_v+1..n_seqs] = total_tokens
 // (empty padding, so that vcu is a valid boundary array of n_seqs sequences); hdr->n_vseq = n_v;
-// hdr->merge_rule = the rule used; vstart[i] = first token of the virtual sequence that input
-// sequence i belongs to (read by bounds_kernel, so that no thread there has to walk back over a run,
-// which under rule 0 may hold any number of empty sequences).
+// hdr->merge_rule = the rule used; vfirst[v] = first input sequence of virtual sequence v, vfirst[n_v] = n_seqs;
+// vstart[i] (unless null) = first token of the virtual sequence that input sequence i belongs to (read by
+// bounds_kernel, so that no thread there has to walk back over a run, which under rule 0 may hold any number of
+// empty sequences).
 __device__ __forceinline__ bool merge_is_head(const int32_t* __restrict__ cu, int i, int32_t max_short, uint32_t rule) {
     if (i == 0 || cu[i + 1] - cu[i] > max_short || cu[i] - cu[i - 1] > max_short) return true;
     if (rule == 0) {
@@ -47,7 +48,7 @@ __device__ __forceinline__ bool merge_is_head(const int32_t* __restrict__ cu, in
 
 template <int NT>
 __global__ void __launch_bounds__(NT) merge_kernel(const int32_t* __restrict__ cu, int32_t n_seqs, int32_t total_tokens,
-                                                   int32_t max_short, WorkspaceHeader* hdr, int32_t* vcu, int32_t* vstart) {
+                                                   int32_t max_short, WorkspaceHeader* hdr, int32_t* vcu, int32_t* vfirst, int32_t* vstart) {
     __shared__ uint32_t scratch[33];
     grid_trigger();
     grid_wait();
@@ -82,14 +83,17 @@ __global__ void __launch_bounds__(NT) merge_kernel(const int32_t* __restrict__ c
     if (tid == 0) {
         hdr->n_vseq = n_v;
         hdr->merge_rule = rule;
+        vfirst[n_v] = n_seqs;
     }
     int last_head = -1;
     for (int i = begin; i < end; ++i)
         if (merge_is_head(cu, i, max_short, rule)) {
-            vcu[run++] = cu[i];
+            vcu[run] = cu[i];
+            vfirst[run++] = i;
             last_head = i;
         }
     for (uint32_t i = n_v + tid; i <= (uint32_t)n_seqs; i += NT) vcu[i] = total_tokens;
+    if (!vstart) return;
     // head of the run each sequence belongs to: the last head at or before it (sequence 0 is always one)
     int cur = block_exclusive_max_scan<NT>(last_head, reinterpret_cast<int*>(scratch));
     for (int i = begin; i < end; ++i) {
@@ -319,24 +323,26 @@ __global__ void __launch_bounds__(NT) prep_kernel(const int32_t* __restrict__ cu
     for (int i = n_live + tid; i <= n_seqs; i += NT) tile_prefix[i] = total;
 }
 
-int prep_launches(int32_t n_seqs, bool merge, bool input_order) {
-    return (n_seqs > kRankInKernelMax && !input_order ? 2 : 1) + (merge ? (n_seqs > 0 ? 2 : 1) : 0);
+int prep_launches(int32_t n_seqs, bool merge, bool table, bool input_order) {
+    return (n_seqs > kRankInKernelMax && !input_order ? 2 : 1) + (merge ? 1 : 0) + (merge && table && n_seqs > 0 ? 1 : 0);
 }
 
 cudaError_t launch_prep(const int32_t* cu_seqlens, int32_t n_seqs, int32_t total_tokens, int32_t max_seqlen,
-                        int32_t rows_per_block, int32_t n_heads, const SchedView& sched, uint16_t* bounds,
+                        int32_t rows_per_block, int32_t n_heads, const SchedView& sched, bool merge, uint16_t* bounds,
                         uint32_t tile_capacity, bool input_order, int32_t long_min_len, bool no_long, cudaStream_t stream) {
     const int32_t* cu = cu_seqlens;
     const uint32_t* n_live = nullptr;
     const bool small = n_seqs <= 256;
-    if (bounds) {                                       // merge short sequences; everything below sees vcu
+    if (merge) {                                        // merge short sequences; everything below sees vcu
         const int32_t max_short = max_seqlen < kMergeMaxLen ? (max_seqlen > 0 ? max_seqlen : 1) : kMergeMaxLen;
-        // order[] is not needed until the ranking below: until then it carries each sequence's run start
-        int32_t* vstart = const_cast<int32_t*>(sched.order);
+        // order[] is not needed until the ranking below: until then it carries each sequence's run start, which the
+        // table's kernel reads.  That launch is 4 us of a call's chain, so only calls whose kernels read the table have it
+        int32_t* vstart = bounds ? const_cast<int32_t*>(sched.order) : nullptr;
         if (cudaError_t e = launch_dependent(small ? merge_kernel<256> : merge_kernel<1024>, 1, small ? 256 : 1024, 0, stream, cu_seqlens,
-                                             n_seqs, total_tokens, max_short, sched.hdr, const_cast<int32_t*>(sched.vcu), vstart))
+                                             n_seqs, total_tokens, max_short, sched.hdr, const_cast<int32_t*>(sched.vcu),
+                                             const_cast<int32_t*>(sched.vfirst), vstart))
             return e;
-        if (n_seqs > 0)
+        if (bounds && n_seqs > 0)
             if (cudaError_t e = launch_dependent(bounds_kernel, (n_seqs + 7) / 8, 256, 0, stream, cu_seqlens, n_seqs, sched.hdr, vstart,
                                                  bounds))
                 return e;

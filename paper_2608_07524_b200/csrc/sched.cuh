@@ -10,7 +10,8 @@
 // "virtual sequences" of at most 128 tokens that the kernels treat as one tile with a
 // block-diagonal mask: the work list is built over the virtual boundaries `vcu` (a subsequence of
 // cu_seqlens, padded with empty sequences), and a per-token table gives, for tokens of virtual
-// sequences of at most 128 tokens, the range of positions the token's own sequence covers.
+// sequences of at most 128 tokens, the range of positions the token's own sequence covers.  (Only the multi-tile
+// kernels read that table, and only when they take such items: the single-tile kernels search cu_seqlens, see attn_tile.cu.)
 #pragma once
 #include <cstdint>
 
@@ -79,7 +80,8 @@ constexpr size_t kSpanBytes = 2 * kMaxCtas * sizeof(CtaSpan);      // 8 KB right
 // After the header and the span table: int32 order[n_seqs] (sequence ids, longest first, ties by id),
 // uint32 prefix[n_seqs + 1] (items before the i-th sequence of `order`),
 // uint32 tile_prefix[n_seqs + 1] (128-row tiles before sequence b, in input order) and
-// int32 vcu[n_seqs + 1] (virtual sequence boundaries; unused when sequences are not merged).
+// int32 vcu[n_seqs + 1] (virtual sequence boundaries) and int32 vfirst[n_seqs + 1] (first input sequence of each virtual
+// one); the last two are unused when sequences are not merged.
 // All of these are indexed by VIRTUAL sequence; `cu` is the boundary array the kernels read
 // (vcu, or the caller's cu_seqlens when merging is off).
 struct SchedView {
@@ -89,12 +91,13 @@ struct SchedView {
     const uint32_t* prefix;
     const uint32_t* tile_prefix;
     const int32_t* vcu;
+    const int32_t* vfirst;
     int32_t n_seqs;
 };
 
 __host__ __device__ constexpr size_t sched_bytes(int32_t n_seqs) {
     return (sizeof(WorkspaceHeader) + kSpanBytes + sizeof(int32_t) * (size_t)n_seqs +
-            2 * sizeof(uint32_t) * ((size_t)n_seqs + 1) + sizeof(int32_t) * ((size_t)n_seqs + 1) + 255) & ~(size_t)255;
+            4 * sizeof(uint32_t) * ((size_t)n_seqs + 1) + 255) & ~(size_t)255;
 }
 
 // Per-token table of the merged path: low byte = first position, high byte = one past the last
