@@ -3,7 +3,7 @@
 // Such an item is a chain (load, S, softmax, product, store) with nothing to overlap inside it, a few microseconds long
 // for 0.1-0.2 us of memory traffic per SM: what it needs is other items in flight on the same SM.  The multi-tile kernels
 // hold one CTA per SM (all of tensor memory, 200 KB of shared memory), so they ran such items one after the other.
-// Here a CTA is small: 128 compute threads, one thread per row; tensor memory is reused within the item, so that
+// Here a CTA is small: one compute thread per row (two in the backward); tensor memory is reused within the item, so that
 //
 //     forward,  head_dim <= 64:   128 columns,  48 KB  -> 4 CTAs per SM         head_dim > 64:  256 columns,  96 KB -> 2 CTAs
 //     backward, head_dim <= 64:   256 columns, 112 KB  -> 2 CTAs per SM         head_dim > 64:  512 columns, 160 KB -> 1 CTA
@@ -16,8 +16,8 @@
 // Several short sequences may share the tile: row i sees the keys [first, end) of its own sequence, and
 // a warp skips the 32-key chunks that none of its rows sees.
 //
-// Roles (192 threads): warps 0-3 compute, warp 4 TMA producer, warp 5 MMA issue.  Items are dealt round robin: they cost
-// about the same, the longest first.
+// Roles (forward, 192 threads): warps 0-3 compute, warp 4 TMA producer, warp 5 MMA issue; backward: see there.  Items are
+// dealt round robin: they cost about the same, the longest first.
 //
 // Backward in tensor memory: S and dP (128 columns each); pass A writes P back over S in fp32 and to shared memory in
 // bf16 and sums D; pass B forms dS = P o (dP - D) -> shared memory; then dV = P^T dO, dK = dS^T Q, dQ = dS K overwrite S and
@@ -86,38 +86,36 @@ __device__ __forceinline__ void load_tile(uint8_t* dst, const CUtensorMap* map, 
     for (int b = 0; b < D / 64; ++b) tma_load_3d(dst + b * kBoxBytes, map, bar, b * 64, head, row);
 }
 
-// 32 rows of an accumulator (this warp's lanes), D columns: tensor memory -> x mul -> bf16 -> 4 KB of staging in shared
-// memory (128-byte swizzled rows) -> whole rows of global memory.  The accumulator has been read when it returns.
-template <int D>
-__device__ __forceinline__ void store_rows(__nv_bfloat16* out, int64_t row_stride, int head_dim, uint8_t* stage, uint32_t tmem,
-                                           float mul, int rows_left) {
+// 32 rows of an accumulator (this warp's lanes), W columns: tensor memory -> x mul -> bf16 -> 2 KB of staging in shared
+// memory (rows of 64 bytes, 16-byte chunks swizzled) -> global memory, eight rows per instruction.  The accumulator has
+// been read when it returns.
+template <int W>
+__device__ __forceinline__ void store_rows(__nv_bfloat16* out, int64_t row_stride, int cols, uint8_t* stage, uint32_t tmem, float mul,
+                                           int rows_left) {
     const int lane = threadIdx.x & 31;
-    const int chunk = lane & 7;
+    const int sub = lane >> 2, chunk = lane & 3;
 #pragma unroll
-    for (int half = 0; half < D / 64; ++half) {
+    for (int c = 0; c < W / 32; ++c) {
+        uint32_t acc[32];
+        tmem_ld_x32(tmem + c * 32, acc);
+        tmem_wait_ld();
 #pragma unroll
-        for (int c = 0; c < 2; ++c) {
-            uint32_t acc[32];
-            tmem_ld_x32(tmem + half * 64 + c * 32, acc);
-            tmem_wait_ld();
-#pragma unroll
-            for (int v4 = 0; v4 < 4; ++v4) {
-                uint4 val;
-                val.x = pack_bf16x2(__uint_as_float(acc[v4 * 8 + 0]) * mul, __uint_as_float(acc[v4 * 8 + 1]) * mul);
-                val.y = pack_bf16x2(__uint_as_float(acc[v4 * 8 + 2]) * mul, __uint_as_float(acc[v4 * 8 + 3]) * mul);
-                val.z = pack_bf16x2(__uint_as_float(acc[v4 * 8 + 4]) * mul, __uint_as_float(acc[v4 * 8 + 5]) * mul);
-                val.w = pack_bf16x2(__uint_as_float(acc[v4 * 8 + 6]) * mul, __uint_as_float(acc[v4 * 8 + 7]) * mul);
-                *reinterpret_cast<uint4*>(stage + sw128_offset((uint32_t)lane, (uint32_t)(c * 4 + v4))) = val;
-            }
+        for (int v4 = 0; v4 < 4; ++v4) {
+            uint4 val;
+            val.x = pack_bf16x2(__uint_as_float(acc[v4 * 8 + 0]) * mul, __uint_as_float(acc[v4 * 8 + 1]) * mul);
+            val.y = pack_bf16x2(__uint_as_float(acc[v4 * 8 + 2]) * mul, __uint_as_float(acc[v4 * 8 + 3]) * mul);
+            val.z = pack_bf16x2(__uint_as_float(acc[v4 * 8 + 4]) * mul, __uint_as_float(acc[v4 * 8 + 5]) * mul);
+            val.w = pack_bf16x2(__uint_as_float(acc[v4 * 8 + 6]) * mul, __uint_as_float(acc[v4 * 8 + 7]) * mul);
+            *reinterpret_cast<uint4*>(stage + lane * 64 + ((v4 ^ ((lane >> 1) & 3)) << 4)) = val;
         }
         __syncwarp();
-        const int col = half * 64 + chunk * 8;
-        __nv_bfloat16* dst = out + (size_t)(lane >> 3) * row_stride + col;
+        const int col = c * 32 + chunk * 8;
+        __nv_bfloat16* dst = out + (size_t)sub * row_stride + col;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int row = i * 4 + (lane >> 3);
-            const uint4 val = *reinterpret_cast<const uint4*>(stage + sw128_offset((uint32_t)row, (uint32_t)chunk));
-            if (row < rows_left && col < head_dim) *reinterpret_cast<uint4*>(dst + (size_t)(i * 4) * row_stride) = val;
+        for (int i = 0; i < 4; ++i) {
+            const int row = i * 8 + sub;
+            const uint4 val = *reinterpret_cast<const uint4*>(stage + row * 64 + ((chunk ^ ((row >> 1) & 3)) << 4));
+            if (row < rows_left && col < cols) *reinterpret_cast<uint4*>(dst + (size_t)(i * 8) * row_stride) = val;
         }
         __syncwarp();                                // the staging rows have been read
     }
@@ -326,6 +324,13 @@ tile_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
 }
 
 // ------------------------------------------------------------------------------------------------- backward
+// 320 threads: warps 0-3 take the keys (and output columns) of the first half, warps 4-7 those of the second, so that a
+// thread holds half a row; warp 8 TMA producer, warp 9 MMA issue.  An item is one chain per CTA, and tensor memory allows
+// two CTAs per SM: with whole rows and four warps it took 10 us, half of it in this arithmetic and in the stores, and V,
+// loaded only after the stores had staged through its buffer, another 1.5 us (512 texts of 16-200 tokens, 16 heads of 64:
+// this kernel 124 -> 101 us, the training step 441 -> 422).
+constexpr int kTileBwdThreads = 320;
+
 struct BwdTileShared {
     uint64_t in_full, s_full, ds_full, dv_full, dk_full, dq_full, item_free;
     uint32_t tmem_base, abort_flag;
@@ -335,8 +340,8 @@ template <int D>
 struct BwdTileCfg {
     static constexpr int kTileBytes = kTile * D * 2;
     static constexpr int kOffQ = 0, kOffK = kTileBytes, kOffDo = 2 * kTileBytes;
-    static constexpr int kOffP = 3 * kTileBytes;             // V until dP is there, then P (32 KB), then staging
-    static constexpr int kOffDs = kOffP + 32768;
+    static constexpr int kOffP = 3 * kTileBytes;             // V until dP is there, then P (32 KB)
+    static constexpr int kOffDs = kOffP + 32768;             // partial sums of D, then dS, then staging (2 KB per warp)
     static constexpr int kOffCtl = kOffDs + 32768;
     static constexpr int kSmemBytes = kOffCtl + 128;
     static constexpr uint32_t kCols = D == 64 ? 256 : 512;
@@ -345,7 +350,7 @@ struct BwdTileCfg {
 static_assert(sizeof(BwdTileShared) <= 128, "control block must fit its slot");
 
 template <int D>
-__global__ void __launch_bounds__(kTileThreads, D == 64 ? 2 : 1)
+__global__ void __launch_bounds__(kTileBwdThreads, D == 64 ? 2 : 1)
 tile_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k,
                 const __grid_constant__ CUtensorMap tmap_v, const __grid_constant__ CUtensorMap tmap_do,
                 const __grid_constant__ BwdParams p, bool causal) {
@@ -358,11 +363,11 @@ tile_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     grid_trigger();
     if (tid == 0) {
         for (uint64_t* b : {&sh.in_full, &sh.s_full, &sh.dv_full, &sh.dk_full, &sh.dq_full}) mbar_init(b, 1);
-        for (uint64_t* b : {&sh.ds_full, &sh.item_free}) mbar_init(b, 4);
+        for (uint64_t* b : {&sh.ds_full, &sh.item_free}) mbar_init(b, 8);
         sh.abort_flag = (smem_u32(smem) & 1023u) != 0 ? 1u : 0u;
         fence_mbar_init();
     }
-    if (warp == 4) {
+    if (warp == 8) {
         tmem_alloc(&sh.tmem_base, Cfg::kCols);
         tmem_relinquish();
     }
@@ -376,7 +381,7 @@ tile_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     const uint32_t n = sh.abort_flag ? 0u : p.sched.hdr->n_items - p.sched.hdr->n_long_items;
     if (blockIdx.x == 0 && tid == 0 && p.sched.hdr->n_long_items == 0) p.sched.hdr->n_ctas[1] = 0;
 
-    if (warp == 4) {
+    if (warp == 8) {
         if (lane == 0) {
             uint32_t k = 0;
             for (uint32_t i = blockIdx.x; i < n; i += gridDim.x, ++k) {
@@ -384,15 +389,14 @@ tile_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                 if (k >= 1) mbar_wait(&sh.dv_full, (k - 1) & 1u, guard);     // (and the previous item's loads have completed)
                 mbar_expect_tx(&sh.in_full, 4 * Cfg::kTileBytes);
                 load_tile<D>(smem + Cfg::kOffDo, &tmap_do, &sh.in_full, w.head, w.tok0);
+                load_tile<D>(smem + Cfg::kOffP, &tmap_v, &sh.in_full, w.head, w.tok0);      // the product has read P
                 if (k >= 1) mbar_wait(&sh.dk_full, (k - 1) & 1u, guard);
                 load_tile<D>(smem + Cfg::kOffQ, &tmap_q, &sh.in_full, w.head, w.tok0);
                 if (k >= 1) mbar_wait(&sh.dq_full, (k - 1) & 1u, guard);
                 load_tile<D>(smem + Cfg::kOffK, &tmap_k, &sh.in_full, w.head, w.tok0);
-                if (k >= 1) mbar_wait(&sh.item_free, (k - 1) & 1u, guard);
-                load_tile<D>(smem + Cfg::kOffP, &tmap_v, &sh.in_full, w.head, w.tok0);
             }
         }
-    } else if (warp == 5) {
+    } else if (warp == 9) {
         const bool leader = elect_one();
         const int n_ks = (p.head_dim + 15) >> 4;
         constexpr uint32_t idesc_s = make_idesc_bf16(128, 128, false, false);
@@ -412,7 +416,8 @@ tile_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         auto mn_step = [](int ks) -> uint64_t { return (uint64_t)((ks * 2048) >> 4); };
         uint32_t k = 0;
         for (uint32_t i = blockIdx.x; i < n; i += gridDim.x, ++k) {
-            mbar_wait_all(&sh.in_full, k & 1u, guard);       // V was loaded after item_free: the accumulators have been read
+            mbar_wait_all(&sh.in_full, k & 1u, guard);
+            if (k >= 1) mbar_wait_all(&sh.item_free, (k - 1) & 1u, guard);       // the accumulators have been read
             tc_fence_after();
 #pragma unroll
             for (int ks = 0; ks < D / 16; ++ks)
@@ -437,9 +442,12 @@ tile_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             if (leader) tc_commit(&sh.dq_full);
         }
     } else {
-        const uint32_t my = tmem + ((uint32_t)(warp * 32) << 16);
-        const int row = tid;                                 // query row
-        uint8_t *p_row = smem + Cfg::kOffP, *ds_row = smem + Cfg::kOffDs, *stage = smem + Cfg::kOffP + warp * 4096;
+        const int half = warp >> 2, quarter = warp & 3;      // of the columns, of the rows
+        const uint32_t my = tmem + ((uint32_t)(quarter * 32) << 16);
+        const int row = quarter * 32 + lane;                 // query row
+        uint8_t *p_row = smem + Cfg::kOffP + half * kBoxBytes, *ds_row = smem + Cfg::kOffDs + half * kBoxBytes;
+        uint8_t* stage = smem + Cfg::kOffDs + warp * 2048;
+        float* sums = reinterpret_cast<float*>(smem + Cfg::kOffDs + quarter * 4096);     // in rows only these two warps write
         const uint64_t sc2 = pack_f32x2(p.scale_log2, p.scale_log2);
         TileItem w{0, 0, 0, 0};
         int lo = 0, hi = 0;
@@ -460,7 +468,8 @@ tile_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             tc_fence_after();
             float sum = 0.f;                                 // D_i
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
+            for (int u = 0; u < 2; ++u) {
+                const int c = half * 2 + u;
                 const bool seen = c * 32 < whi && c * 32 + 32 > wlo;
                 uint32_t pk[16];
                 if (seen) {
@@ -490,12 +499,19 @@ tile_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                 }
 #pragma unroll
                 for (int v4 = 0; v4 < 4; ++v4)
-                    *reinterpret_cast<uint4*>(p_row + (c / 2) * kBoxBytes + sw128_offset((uint32_t)row, (uint32_t)((c & 1) * 4 + v4))) =
+                    *reinterpret_cast<uint4*>(p_row + sw128_offset((uint32_t)row, (uint32_t)(u * 4 + v4))) =
                         make_uint4(pk[v4 * 4], pk[v4 * 4 + 1], pk[v4 * 4 + 2], pk[v4 * 4 + 3]);
             }
             tmem_wait_st();
+            // D of the whole row: the two warps that share it exchange their halves (in dS's buffer, which is idle until both
+            // have read)
+            sums[half * 32 + lane] = sum;
+            bar_sync(1 + quarter, 64);
+            sum += sums[(half ^ 1) * 32 + lane];
+            bar_sync(1 + quarter, 64);
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
+            for (int u = 0; u < 2; ++u) {
+                const int c = half * 2 + u;
                 const bool seen = c * 32 < whi && c * 32 + 32 > wlo;
                 uint32_t pk[16];
                 if (seen) {
@@ -513,7 +529,7 @@ tile_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                 }
 #pragma unroll
                 for (int v4 = 0; v4 < 4; ++v4)
-                    *reinterpret_cast<uint4*>(ds_row + (c / 2) * kBoxBytes + sw128_offset((uint32_t)row, (uint32_t)((c & 1) * 4 + v4))) =
+                    *reinterpret_cast<uint4*>(ds_row + sw128_offset((uint32_t)row, (uint32_t)(u * 4 + v4))) =
                         make_uint4(pk[v4 * 4], pk[v4 * 4 + 1], pk[v4 * 4 + 2], pk[v4 * 4 + 3]);
             }
             fence_async_smem();
@@ -522,22 +538,17 @@ tile_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             if (lane == 0) mbar_arrive(&sh.ds_full);
             const TileItem cur = w;
             if (i + gridDim.x < n) fetch(i + gridDim.x);
-            const int rows_left = cur.len - warp * 32;
-            const size_t off = ((size_t)cur.tok0 + warp * 32) * p.row_stride + (size_t)cur.head * p.head_dim;
-            // (dV: rows are keys.)  P has been read when dV is there, so its buffer stages what leaves.
-            mbar_wait(&sh.dv_full, k & 1u, guard);
-            __syncwarp();
-            tc_fence_after();
-            store_rows<D>(p.dv + off, p.row_stride, p.head_dim, stage, my + Cfg::kColDv, 1.0f, rows_left);
-            mbar_wait(&sh.dk_full, k & 1u, guard);
-            __syncwarp();
-            tc_fence_after();
-            store_rows<D>(p.dk + off, p.row_stride, p.head_dim, stage, my + Cfg::kColDk, p.scale, rows_left);
+            constexpr int W = D / 2;                         // output columns of this warp
+            const int rows_left = cur.len - quarter * 32, cols = p.head_dim - half * W;
+            const size_t off = ((size_t)cur.tok0 + quarter * 32) * p.row_stride + (size_t)cur.head * p.head_dim + half * W;
+            // (dV, dK: rows are keys.)  dS has been read when dQ is there, so its buffer stages what leaves; the next item's
+            // operands are on their way meanwhile.
             mbar_wait(&sh.dq_full, k & 1u, guard);
             __syncwarp();
             tc_fence_after();
-            store_rows<D>(p.dq + off, p.row_stride, p.head_dim, stage, my + Cfg::kColDq, p.scale, rows_left);
-            fence_async_smem();
+            store_rows<W>(p.dv + off, p.row_stride, cols, stage, my + Cfg::kColDv + half * W, 1.0f, rows_left);
+            store_rows<W>(p.dk + off, p.row_stride, cols, stage, my + Cfg::kColDk + half * W, p.scale, rows_left);
+            store_rows<W>(p.dq + off, p.row_stride, cols, stage, my + Cfg::kColDq + half * W, p.scale, rows_left);
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&sh.item_free);
@@ -546,7 +557,7 @@ tile_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     __syncwarp();
     tc_fence_before();
     __syncthreads();
-    if (warp == 4) tmem_dealloc(tmem, Cfg::kCols);
+    if (warp == 8) tmem_dealloc(tmem, Cfg::kCols);
 }
 
 template <int D>
@@ -560,7 +571,7 @@ template <int D>
 cudaError_t launch_bwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tdo, const BwdParams& p,
                        bool causal, unsigned n_ctas, cudaStream_t stream) {
     if (cudaError_t e = allow_smem<tile_bwd_kernel<D>>(BwdTileCfg<D>::kSmemBytes)) return e;
-    return launch_dependent(tile_bwd_kernel<D>, n_ctas, kTileThreads, BwdTileCfg<D>::kSmemBytes, stream, tq, tk, tv, tdo, p, causal);
+    return launch_dependent(tile_bwd_kernel<D>, n_ctas, kTileBwdThreads, BwdTileCfg<D>::kSmemBytes, stream, tq, tk, tv, tdo, p, causal);
 }
 
 unsigned tile_grid(int n_sms, int per_sm, int32_t n_seqs, int32_t n_heads) {
