@@ -296,7 +296,7 @@ static int attn_fwd_impl(const char* fn, bool merge, const void* q, const void* 
     {
         ScopedTimer t(DCP_KERNEL_PREP, stream);
         e = launch_prep(cu_seqlens, n_seqs, total_tokens, max_seqlen, kFwdRowsPerItem, n_heads, sched, merge, bounds, UINT32_MAX,
-                        input_order, split ? kTile + 1 : INT32_MAX, max_seqlen <= kTile, stream);
+                        input_order, split ? kTile + 1 : INT32_MAX, max_seqlen <= kTile ? kTile : INT32_MAX, stream);
     }
     if (e != cudaSuccess) return fail(DCP_ERR_CUDA, "%s: work-list kernel: %s", fn, cudaGetErrorString(e));
     g_launches.fetch_add(prep_launches(n_seqs, merge, bounds != nullptr, input_order));
@@ -417,10 +417,11 @@ static int attn_bwd_impl(const char* fn, const void* q, const void* k, const voi
     const int32_t direct_len = pair ? kPairDirectLen : kTile;      // longest sequence that is a single key block
     const int32_t tiles_per_item = !split ? 0 : pair ? 2 : 1;      // of the main kernel, for the helpers' block list
     const bool multi = max_seqlen > kTile || !split;               // there may be items for the multi-tile kernel
+    const bool all_direct = max_seqlen <= direct_len && split;     // no dQ goes through the accumulator
     {
         ScopedTimer t(DCP_KERNEL_PREP, stream);
         e = launch_prep(cu_seqlens, n_seqs, total_tokens, max_seqlen, pair ? 2 * kTile : kTile, n_heads, sched, true, bounds,
-                        (uint32_t)max_tiles(total_tokens, n_seqs), input_order, split ? kTile + 1 : INT32_MAX, !multi, stream);
+                        (uint32_t)max_tiles(total_tokens, n_seqs), input_order, split ? kTile + 1 : INT32_MAX, !multi ? kTile : all_direct ? direct_len : INT32_MAX, stream);
     }
     if (e != cudaSuccess) return fail(DCP_ERR_CUDA, "%s: work-list kernel: %s", fn, cudaGetErrorString(e));
     g_launches.fetch_add(prep_launches(n_seqs, true, bounds != nullptr, input_order));
@@ -487,7 +488,7 @@ static int attn_bwd_impl(const char* fn, const void* q, const void* k, const voi
         }
     }
 
-    if (multi) {
+    if (multi && !all_direct) {
         ScopedTimer t(DCP_KERNEL_BWD_POST, stream);
         e = launch_bwd_post(dq_acc, static_cast<__nv_bfloat16*>(dq), vcu, sched, total_tokens, n_heads, head_dim, token_stride,
                             scale, tiles_per_item, direct_len, dev.sm_count, stream);

@@ -224,7 +224,7 @@ template <int NT>
 __global__ void __launch_bounds__(NT) prep_kernel(const int32_t* __restrict__ cu, int32_t n_seqs,
                                                   const uint32_t* __restrict__ n_live_ptr, int32_t rows_per_block, int32_t n_heads,
                                                   WorkspaceHeader* hdr, int32_t* order, uint32_t* prefix, uint32_t* tile_prefix,
-                                                  int ranked, int32_t total_tokens, uint32_t tile_capacity, int32_t long_min_len, bool no_long) {
+                                                  int ranked, int32_t total_tokens, uint32_t tile_capacity, int32_t long_min_len, int32_t max_len) {
     __shared__ uint32_t scratch[33];
     __shared__ int32_t len_sh[NT];
     grid_trigger();
@@ -281,7 +281,11 @@ __global__ void __launch_bounds__(NT) prep_kernel(const int32_t* __restrict__ cu
         return (uint32_t)((len + rows_per_block - 1) / rows_per_block) * (uint32_t)n_heads;
     };
     uint32_t local = 0, total = 0;
-    for (int i = begin; i < end; ++i) local += items_of(i);
+    int unforeseen = 0;
+    for (int i = begin; i < end; ++i) {
+        local += items_of(i);
+        unforeseen |= cu[order[i] + 1] - cu[order[i]] > max_len ? 1 : 0;
+    }
     uint32_t run = block_exclusive_scan<NT>(local, scratch, &total);
     if (tid == 0) {
         hdr->n_items = total;
@@ -304,10 +308,9 @@ __global__ void __launch_bounds__(NT) prep_kernel(const int32_t* __restrict__ cu
     local = 0;
     for (int i = begin; i < end; ++i) local += tiles_of(i);
     run = block_exclusive_scan<NT>(local, scratch, &total);
-    const bool unforeseen = __syncthreads_or(no_long && begin < end && is_long(begin));
+    unforeseen = __syncthreads_or(unforeseen);
     if (total > tile_capacity || unforeseen) {
-        // more tiles than the workspace was sized for, or a sequence of more than one tile where no kernel for such was
-        // launched: max_seqlen was understated (the bound on merged runs relies on it).  Nothing may index the per-tile
+        // more tiles than the workspace was sized for, or a sequence longer than the launched kernels take: max_seqlen was understated (the bound on merged runs relies on it).  Nothing may index the per-tile
         // storage: no items, no tiles.
         for (int i = tid; i <= n_seqs; i += NT) tile_prefix[i] = 0;
         if (tid == 0) {
@@ -329,7 +332,7 @@ int prep_launches(int32_t n_seqs, bool merge, bool table, bool input_order) {
 
 cudaError_t launch_prep(const int32_t* cu_seqlens, int32_t n_seqs, int32_t total_tokens, int32_t max_seqlen,
                         int32_t rows_per_block, int32_t n_heads, const SchedView& sched, bool merge, uint16_t* bounds,
-                        uint32_t tile_capacity, bool input_order, int32_t long_min_len, bool no_long, cudaStream_t stream) {
+                        uint32_t tile_capacity, bool input_order, int32_t long_min_len, int32_t max_len, cudaStream_t stream) {
     const int32_t* cu = cu_seqlens;
     const uint32_t* n_live = nullptr;
     const bool small = n_seqs <= 256;
@@ -356,7 +359,7 @@ cudaError_t launch_prep(const int32_t* cu_seqlens, int32_t n_seqs, int32_t total
             return e;
     return launch_dependent(small ? prep_kernel<256> : prep_kernel<1024>, 1, small ? 256 : 1024, 0, stream, cu, n_seqs, n_live,
                             rows_per_block, n_heads, sched.hdr, const_cast<int32_t*>(sched.order), const_cast<uint32_t*>(sched.prefix),
-                            const_cast<uint32_t*>(sched.tile_prefix), ranked, total_tokens, tile_capacity, long_min_len, no_long);
+                            const_cast<uint32_t*>(sched.tile_prefix), ranked, total_tokens, tile_capacity, long_min_len, max_len);
 }
 
 // A (128-row tile, head) block of the backward helpers.

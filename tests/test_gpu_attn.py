@@ -396,6 +396,32 @@ def test_backward_on_cta_pairs(causal, d, lengths):
     check_full(lengths, 3, d, causal, seed=300 + len(lengths))
 
 
+@pytest.mark.parametrize("d", [72, 128])
+@pytest.mark.parametrize("longest", [129, 256, 257])
+def test_backward_around_one_pair_item(d, longest):
+    """Up to 256 tokens every sequence is one item of the pair kernel, dQ needs no accumulator and nothing converts one
+    (129: the item's second half has one row; 256: full); at 257 the accumulator is back."""
+    rng = np.random.default_rng(d + longest)
+    lengths = [int(x) for x in rng.choice([0, 1, 64, 65, 128, 129, 192, 193, 255], size=30) if x <= longest] + [longest, longest]
+    check_full(lengths, 3, d, True, seed=500 + d)
+
+
+def test_a_sequence_longer_than_a_declared_pair_item_is_refused():
+    # max_seqlen <= 256 promises that no dQ needs the accumulator, whose kernels are then not launched
+    dev = "cuda"
+    lengths = [200] * 39 + [257]
+    T = sum(lengths)
+    cu = torch.tensor(np.concatenate([[0], np.cumsum(lengths)]), dtype=torch.int32, device=dev)
+    q, k, v, g = (x.to(dev) for x in inputs.make_qkvg(T, 8, 72, 6))
+    ws = B.alloc_workspace(T, len(lengths), 8, 72, True, dev)
+    o, lse = B.dcp_varlen_attn_fwd(q, k, v, cu, 257, False, workspace=ws)
+    dq = torch.full_like(q, 7.0)
+    B.dcp_varlen_attn_bwd(q, k, v, o, g, lse, cu, 256, False, dq=dq, dk=torch.empty_like(q), dv=torch.empty_like(q), workspace=ws)
+    with pytest.raises(B.DcpError) as e:
+        B.dcp_query_status(ws)
+    assert e.value.code == B.DCP_ERR_INVALID_ARG and bool((dq == 7.0).all())
+
+
 @pytest.mark.parametrize("causal", [False, True])
 @pytest.mark.parametrize("d", [8, 64, 72, 128])
 @pytest.mark.parametrize("longest", [128, 300])
