@@ -306,7 +306,7 @@ static int attn_fwd_impl(const char* fn, bool merge, const void* q, const void* 
     if (int rc = make_map(&tq, q, total_tokens, n_heads, head_dim, token_stride)) return rc;
     if (int rc = make_map(&tk, k, total_tokens, n_heads, head_dim, token_stride)) return rc;
     if (int rc = make_map(&tv, v, total_tokens, n_heads, head_dim, token_stride)) return rc;
-    if (int rc = make_map(&to, o, total_tokens, n_heads, head_dim, token_stride)) return rc;
+    if (int rc = make_map(&to, o, total_tokens, n_heads, head_dim, token_stride, 32)) return rc;
 
     FwdParams p;
     p.cu_seqlens = merge ? sched.vcu : cu_seqlens;

@@ -43,7 +43,6 @@ struct FwdShared {
     uint64_t kv_full[kKvStages], kv_empty[kKvStages];
     uint64_t s_full[2], p_part[2][kPParts], o_full[2], o_free[2];
     uint64_t work_full[2], work_empty[2];
-    uint64_t stage_ready[2], stage_full[2];    // output staging buffer of a softmax group: free to write / written
     WorkItem work[2];
     uint32_t tmem_base;
     uint32_t abort_flag;
@@ -54,8 +53,8 @@ struct FwdCfg {
     static constexpr int kTileBytes = kTile * D * 2;   // one Q, K or V tile
     static constexpr int kBoxes = D / 64;               // TMA boxes per tile (64 columns = 128 bytes each)
     static constexpr int kBoxBytes = kTile * 128;
-    static constexpr int kStageBytes = kTile * 128;     // 128 rows of 64 bf16 columns: what one TMA store box holds
-    static constexpr int kOffStage = (2 + kKvStages) * kTileBytes;   // one staging buffer per softmax group
+    static constexpr int kStageBytes = kTile * 128;     // 128 rows of 64 bf16 columns
+    static constexpr int kOffStage = (2 + kKvStages) * kTileBytes;   // of O: 4 KB (one TMA store box) per softmax warp
     static constexpr int kSmemBytes = kOffStage + 2 * kStageBytes + 1024;
     static constexpr uint32_t kS0 = 0, kS1 = 128, kO0 = 256, kO1 = 256 + D;   // tensor-memory columns
 };
@@ -212,21 +211,22 @@ __device__ __noinline__ void softmax_single_tile_item(FwdShared& sh, const FwdPa
     if (lane == 0) mbar_arrive(&sh.o_free[0]);
 }
 
-// Epilogue of a Q tile whose 128 rows all belong to the sequence: O = acc / l leaves tensor memory through a
-// staging buffer in shared memory and TMA stores, 64 columns (one box) at a time.  A thread owns a row, so storing
-// it directly costs 16 instructions of 32 scattered 16-byte pieces each, about a microsecond of the load/store
-// unit per tile: as much as a key tile's softmax, which is what short work items cannot afford (uniform batches
-// of 256-token sequences: forward 0.41 -> 0.36 ms).  Kept out of line so that the loop over key tiles is compiled
-// exactly as it would be without it (inlined it cost the long-sequence forward 6 %).  Called by the 128 threads
-// of a softmax group; n_staged = boxes this group has stored so far (the parity of its two barriers).
+// Epilogue of a warp's 32 rows of a Q tile, all of which belong to the sequence: O = acc / l leaves tensor memory through
+// 4 KB of staging per warp and TMA stores, 64 columns (one box) at a time.  A thread owns a row, so storing it directly
+// costs 16 instructions of 32 scattered 16-byte pieces each, about a microsecond of the load/store unit per tile: as much
+// as a key tile's softmax, which is what short work items cannot afford.  Warps do not wait for one another, and of a
+// sequence's last tile only the warp that its end cuts stores directly.  Kept out of line so that the loop over key tiles
+// is compiled exactly as it would be without it (inlined it cost the long-sequence forward 6 %).
+// Against one store of 128 rows per group, for which four warps waited twice per box (uniform batches, 16 heads of 128, ns per
+// 128 x 128 tile and SM, the causal ones in brackets): 256 tokens 1644 -> 1604 (2220 -> 2082), 300: 1692 -> 1629 (2368 ->
+// 1991), 512: 1255 -> 1212 (1757 -> 1655), 1200: 1030 -> 1005 (1236 -> 1196), 4096: 909 -> 900 (993 -> 977).  Ordinary stores
+// of whole 128-byte lines from the same staging rows instead: 256 tokens + 8 %, 4096 equal.
 template <int D>
-__device__ __noinline__ void store_whole_tile(FwdShared& sh, const CUtensorMap* tmap_o, uint8_t* stage, uint32_t o_tmem,
-                                              float inv_l, int t, int head, int tok_row0, uint32_t n_staged,
-                                              const WaitGuard guard) {
-    const int lane = threadIdx.x & 31, row_in_tile = threadIdx.x & 127;
-    const bool issuer = row_in_tile == 0;
+__device__ __noinline__ void store_whole_rows(FwdShared& sh, const CUtensorMap* tmap_o, uint8_t* stage, uint32_t o_tmem,
+                                              float inv_l, int t, int head, int tok_row0) {
+    const int lane = threadIdx.x & 31;
 #pragma unroll
-    for (int half = 0; half < D / 64; ++half, ++n_staged) {
+    for (int half = 0; half < D / 64; ++half) {
         uint32_t acc[64];
         tmem_ld_x32(o_tmem + half * 64, *reinterpret_cast<uint32_t(*)[32]>(&acc[0]));
         tmem_ld_x32(o_tmem + half * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(&acc[32]));
@@ -236,11 +236,8 @@ __device__ __noinline__ void store_whole_tile(FwdShared& sh, const CUtensorMap* 
             __syncwarp();
             if (lane == 0) mbar_arrive(&sh.o_free[t]);
         }
-        if (issuer) {
-            bulk_store_wait_read();              // the previous store has read the staging buffer
-            mbar_arrive(&sh.stage_ready[t]);
-        }
-        mbar_wait(&sh.stage_ready[t], n_staged & 1u, guard);
+        if (lane == 0) bulk_store_wait_read();       // the previous store has read the staging rows
+        __syncwarp();
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
             uint4 val;
@@ -248,13 +245,12 @@ __device__ __noinline__ void store_whole_tile(FwdShared& sh, const CUtensorMap* 
             val.y = pack_bf16x2(__uint_as_float(acc[c * 8 + 2]) * inv_l, __uint_as_float(acc[c * 8 + 3]) * inv_l);
             val.z = pack_bf16x2(__uint_as_float(acc[c * 8 + 4]) * inv_l, __uint_as_float(acc[c * 8 + 5]) * inv_l);
             val.w = pack_bf16x2(__uint_as_float(acc[c * 8 + 6]) * inv_l, __uint_as_float(acc[c * 8 + 7]) * inv_l);
-            *reinterpret_cast<uint4*>(stage + sw128_offset((uint32_t)row_in_tile, (uint32_t)c)) = val;
+            *reinterpret_cast<uint4*>(stage + sw128_offset((uint32_t)lane, (uint32_t)c)) = val;
         }
         fence_async_smem();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&sh.stage_full[t]);
-        if (issuer) {
-            if (mbar_wait(&sh.stage_full[t], n_staged & 1u, guard)) tma_store_3d(tmap_o, stage, half * 64, head, tok_row0);
+        if (lane == 0) {
+            tma_store_3d(tmap_o, stage, half * 64, head, tok_row0);
             bulk_store_commit();
         }
     }
@@ -292,8 +288,6 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             mbar_init(&sh.o_free[i], 4);
             mbar_init(&sh.work_full[i], 1);
             mbar_init(&sh.work_empty[i], 9);   // 8 softmax warps + the MMA warp
-            mbar_init(&sh.stage_ready[i], 1);
-            mbar_init(&sh.stage_full[i], 4);   // one arrival per warp of the group
         }
         for (int i = 0; i < kKvStages; ++i) {
             mbar_init(&sh.kv_full[i], 1);
@@ -480,7 +474,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
         const uint32_t s_tmem = tmem + lane_base + (t == 0 ? Cfg::kS0 : Cfg::kS1);
         const uint32_t o_tmem = tmem + lane_base + (t == 0 ? Cfg::kO0 : Cfg::kO1);
-        uint32_t n_work = 0, n_s = 0, use = 0, n_staged = 0;
+        uint32_t n_work = 0, n_s = 0, use = 0;
         while (true) {
             const uint32_t slot = n_work & 1u;
             const bool got = mbar_wait(&sh.work_full[slot], (n_work >> 1) & 1u, guard);
@@ -605,11 +599,9 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             const float inv_l = 1.0f / l;
             const bool valid = row < w.len;
             const size_t tok = (size_t)w.tok0 + (size_t)row;
-            if (r_tile + kTile <= w.len) {
-                // every row of the tile belongs to the sequence: it leaves through shared memory and TMA stores
-                store_whole_tile<D>(sh, &tmap_o, smem + Cfg::kOffStage + t * Cfg::kStageBytes, o_tmem, inv_l, t, w.head,
-                                    w.tok0 + r_tile, n_staged, guard);
-                n_staged += D / 64;
+            const int row0 = r_tile + (warp & 3) * 32;
+            if (row0 + 32 <= w.len) {
+                store_whole_rows<D>(sh, &tmap_o, smem + Cfg::kOffStage + warp * 4096, o_tmem, inv_l, t, w.head, w.tok0 + row0);
                 p.lse[(size_t)w.head * p.total_tokens + tok] = m * p.scale + __logf(l);
                 continue;
             }
@@ -636,7 +628,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             __syncwarp();
             if (lane == 0) mbar_arrive(&sh.o_free[t]);
         }
-        if ((tid & 127) == 0) bulk_store_wait_all();     // this group's stores are complete before the CTA ends
+        if (lane == 0) bulk_store_wait_all();            // this warp's stores are complete before the CTA ends
     }
 
     tc_fence_before();
