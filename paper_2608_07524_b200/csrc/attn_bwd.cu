@@ -59,7 +59,7 @@ namespace dcp {
 // requests and shared-memory stores of the other warps wait behind them; short sleeps (which, unlike
 // a spin on the clock, take no issue slots) let those through.  __nanosleep rounds down to steps of
 // about 128 ns here (100 ns had no effect, 150-250 ns the same effect), so the values sit in the
-// middle of a step.  Backward main kernel alone on config 3: 60.2 ms without any pause, 58.3 with the
+// middle of a step.  Backward main kernel alone on the video batch: 60.2 ms without any pause, 58.3 with the
 // pauses, 55.8 with the stagger as well; two steps per pause or per stagger, or a pause after every
 // second atomic, cost 57-85 ms.  In the power-capped bench loop: 61.7 -> 58.1 ms.
 constexpr int kRedGroup = 4;

@@ -37,7 +37,9 @@
 // Measured (16 heads of 128, fwd + bwd in turn under the power cap; the one-CTA kernel in brackets): two sequences of
 // 16384 tokens 9.1 ms = 1200 TFLOP/s (10.5 ms = 1046), 3770 cycles per Q tile and pair (4850 per 128 keys); the video
 // batch's step 69.8 ms (75.2), the 2-D model's spatial axis 8.31 (8.83), at head_dim 72 7.90 (8.16), causal text 4.99
-// (5.08).  Without the reductions the first is 8.7 ms: what is left is the compute warps' chain S -> P -> dS per tile.
+// (5.08).  Without the reductions the first is 8.7 ms.  The products need 3300 cycles per tile (dQ 1024 of them: M = 128 on
+// a pair runs at half the rate of M = 256), barrier latency the rest; an item's first tile takes 3200 more, most of it waiting
+// for the drain warps to have read the previous dK and dQ.
 //
 // Sequences of one block (at most 256 tokens) write dQ directly; longer ones add it to the fp32 accumulator that
 // the pre kernel zeroes and the post kernel converts (layout as in the one-CTA kernel).

@@ -29,9 +29,9 @@
 namespace dcp {
 
 // One pair of exponentials in this many is computed on the FMA pipe instead of the special-function
-// unit (0: none).  Measured on the forward kernel alone: bidirectional config 3, 18.2 ms with none,
+// unit (0: none).  Measured on the forward kernel alone: the video batch (bidirectional), 18.2 ms with none,
 // 17.8 with packed arithmetic only, 17.5 / 17.1 / 17.1 with every 8th / 4th / 3rd pair, 18.7 with every
-// 2nd; causal config 2, 1.23 / 1.17 / 1.17 / 1.23 / 1.23 ms.
+// 2nd; the causal text batch, 1.23 / 1.17 / 1.17 / 1.23 / 1.23 ms.
 constexpr int kPolyEveryFull = 4, kPolyEveryCausal = 8;
 constexpr int kFwdThreads = 384;   // 8 softmax warps + a 4-warp control group (MMA, producer, 2 idle)
 constexpr int kKvStages = 4;
@@ -402,9 +402,9 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                     commit(&sh.s_full[t]);
                     // When items are short (a query block sees a few key tiles: causal masks, batches of short
                     // sequences) a Q tile is released as soon as its last S product is issued, so that the next
-                    // item's Q load runs while this item's last PV products do instead of after them (config 2
+                    // item's Q load runs while this item's last PV products do instead of after them (text batch
                     // forward 1.05 -> 1.01 ms, spatial axis of the 2-D workload 1.97 -> 1.84 ms).  On long items the
-                    // two extra tests per key step cost the MMA warp more than the early load gains (config 3
+                    // two extra tests per key step cost the MMA warp more than the early load gains (video batch
                     // forward 16.4 -> 16.9 ms), so the host picks the variant by mask and longest sequence.
                     if (EARLY_Q && nkv_t[t] == 1) commit(&sh.q_empty[t]);
                 }
