@@ -461,6 +461,7 @@ static int attn_bwd_impl(const char* fn, const void* q, const void* k, const voi
     p.scale = scale;
     p.scale_log2 = scale * 1.4426950408889634f;
     p.lse = lse;
+    p.inv_scale = 1.0f / scale;
     p.split = split;
     {
         ScopedTimer t(DCP_KERNEL_BWD_MAIN, stream);
@@ -482,7 +483,9 @@ static int attn_bwd_impl(const char* fn, const void* q, const void* k, const voi
             g_launches.fetch_add(1);
         }
         if (split) {
-            e = launch_tile_bwd(tq, tk, tv, tg, p, causal != 0, dev.sm_count, stream);
+            CUtensorMap to;
+            if (int rc = make_map(&to, o, total_tokens, n_heads, head_dim, token_stride)) return rc;
+            e = launch_tile_bwd(tq, tk, tv, to, tg, p, causal != 0, dev.sm_count, stream);
             if (e != cudaSuccess) return fail(DCP_ERR_CUDA, "%s: single-tile kernel: %s", fn, cudaGetErrorString(e));
             g_launches.fetch_add(1);
         }

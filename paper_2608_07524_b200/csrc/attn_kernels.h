@@ -43,7 +43,9 @@ struct BwdParams {
     int64_t row_stride;   // as in FwdParams; the same for q, k, v, dO, dq, dk, dv
     float scale;
     float scale_log2;
-    const float* lse;     // [H, T]: read by launch_tile_bwd (the other kernels take it from `stats`)
+    // read by launch_tile_bwd, which forms the per-query terms itself (the other kernels take them from `stats`)
+    const float* lse;     // [H, T]
+    float inv_scale;      // 1 / scale
     bool split;           // the single-tile items are for launch_tile_bwd
 };
 
@@ -63,8 +65,8 @@ inline bool pair_path(int32_t head_dim) { return head_dim > 64; }
 // Single-tile work items (virtual sequences of at most 128 tokens) on kernels of their own, see attn_tile.cu.
 cudaError_t launch_tile_fwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const FwdParams& p, bool causal,
                             int n_sms, cudaStream_t stream);
-cudaError_t launch_tile_bwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tdo,
-                            const BwdParams& p, bool causal, int n_sms, cudaStream_t stream);
+cudaError_t launch_tile_bwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& to,
+                            const CUtensorMap& tdo, const BwdParams& p, bool causal, int n_sms, cudaStream_t stream);
 
 // Builds the work list (longest sequence first) and resets the work counter and status word.
 // With `merge`, short sequences are first merged into virtual sequences: sched.vcu and sched.vfirst

@@ -6,12 +6,15 @@
 // Here a CTA is small: one compute thread per row (two in the backward); tensor memory is reused within the item, so that
 //
 //     forward,  head_dim <= 64:   128 columns,  48 KB  -> 4 CTAs per SM         head_dim > 64:  256 columns,  96 KB -> 2 CTAs
-//     backward, head_dim <= 64:   256 columns, 112 KB  -> 2 CTAs per SM         head_dim > 64:  512 columns, 160 KB -> 1 CTA
+//     backward, head_dim <= 64:   256 columns, 112 KB  -> 2 CTAs per SM         head_dim > 64:  512 columns, 192 KB -> 1 CTA
 //
 // and the next item's loads start as soon as an operand's buffer is free.  Queries are rows (lanes) in both directions.
-// That makes the backward's per-query terms scalars of a thread: lse_i is read, and D_i = sum_j P_ij dP_ij is summed in
-// registers (it equals sum_c dO_ic O_ic because O = P V), so these items need no pass over O, no per-query tiles, no fp32
-// accumulator and no conversion pass: q, k, v, dO in, dq, dk, dv out.
+// The backward's per-query terms, -lse/scale and -D_i = -sum_c dO_ic O_ic, enter S and dP as in the multi-tile kernels: by
+// a K = 16 product of a [128 x 16] tile of bf16 parts with a tile of ones.  The compute warps form that tile from O and dO in
+// shared memory while the products that S and dP begin with run, so these items need no pre kernel, no fp32 accumulator
+// and no conversion pass: q, k, v, o, dO in, dq, dk, dv out.  (D_i = sum_j P_ij dP_ij from registers would save reading o: 512
+// texts of 16-200 tokens, 16 heads of 64, training step 417 us instead of 427.  But it is another number wherever o
+// is not this call's own P V: rounded to bf16, or the output over more keys than these, with the lse to match.)
 //
 // Several short sequences may share the tile: row i sees the keys [first, end) of its own sequence, and
 // a warp skips the 32-key chunks that none of its rows sees.
@@ -19,15 +22,19 @@
 // Roles (forward, 192 threads): warps 0-3 compute, warp 4 TMA producer, warp 5 MMA issue; backward: see there.  Items are
 // dealt round robin: they cost about the same, the longest first.
 //
-// Backward in tensor memory: S and dP (128 columns each); pass A writes P back over S in fp32 and to shared memory in
-// bf16 and sums D; pass B forms dS = P o (dP - D) -> shared memory; then dV = P^T dO, dK = dS^T Q, dQ = dS K overwrite S and
-// dP (P^T and dS^T are the same bytes read with keys contiguous as the M dimension).
+// Backward in tensor memory: S and dP (128 columns each); one pass over both gives P and dS -> shared memory; then
+// dV = P^T dO, dK = dS^T Q, dQ = dS K overwrite S and dP (P^T and dS^T are the same bytes read with keys contiguous as the
+// M dimension).
+//
+// Every sum here has the order that the multi-tile kernels give it, so an item's results are the same bits whichever kernel
+// the batch sends it to.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
 #include "attn_kernels.h"
 #include "launch.h"
+#include "row_terms.cuh"
 #include "sched.cuh"
 #include "sm100_ptx.cuh"
 
@@ -235,7 +242,7 @@ tile_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             if (hi <= lo) m = 0.f;
             const float neg_m = -m * p.scale_log2;
             const uint64_t nm2 = pack_f32x2(neg_m, neg_m);
-            float l = 0.f;
+            uint64_t sum2[2] = {0ull, 0ull};         // keys 0, 4, .. | 1, 5, .. and 2, 6, .. | 3, 7, ..
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
                 uint32_t pk[16];
@@ -244,18 +251,15 @@ tile_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                     tmem_ld_x32(my + c * 32, s);
                     tmem_wait_ld();
                     const uint32_t bits = chunk_bits(lo, hi, c);
-                    float l0 = 0.f, l1 = 0.f;
 #pragma unroll
                     for (int e = 0; e < 16; ++e) {
                         float x0, x1;
                         unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(s[2 * e]), __uint_as_float(s[2 * e + 1])), sc2, nm2), x0, x1);
                         const float p0 = bits & (1u << (2 * e)) ? fast_exp2(x0) : 0.f;
                         const float p1 = bits & (2u << (2 * e)) ? fast_exp2(x1) : 0.f;
-                        l0 += p0;
-                        l1 += p1;
+                        sum2[e & 1] = add_f32x2(sum2[e & 1], pack_f32x2(p0, p1));
                         pk[e] = pack_bf16x2(p0, p1);
                     }
-                    l += l0 + l1;
                 } else {
 #pragma unroll
                     for (int e = 0; e < 16; ++e) pk[e] = 0u;
@@ -268,6 +272,13 @@ tile_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             if (lane == 0) mbar_arrive(&sh.p_full);
             const TileItem cur = w;
             const bool valid = row < cur.len;
+            float l;
+            {
+                float a0, a1, b0, b1;
+                unpack_f32x2(sum2[0], a0, a1);
+                unpack_f32x2(sum2[1], b0, b1);
+                l = (a0 + a1) + (b0 + b1);
+            }
             const float inv_l = l > 0.f ? 1.0f / l : 0.f;
             if (valid) p.lse[(size_t)cur.head * p.total_tokens + cur.tok0 + row] = m * p.scale + __logf(l);
             if (i + gridDim.x < n) {                 // the next item's keys, while the product runs
@@ -328,11 +339,11 @@ tile_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
 // thread holds half a row; warp 8 TMA producer, warp 9 MMA issue.  An item is one chain per CTA, and tensor memory allows
 // two CTAs per SM: with whole rows and four warps it took 10 us, half of it in this arithmetic and in the stores, and V,
 // loaded only after the stores had staged through its buffer, another 1.5 us (512 texts of 16-200 tokens, 16 heads of 64:
-// this kernel 124 -> 101 us, the training step 441 -> 422).
+// this kernel 124 -> 101 us, the training step 441 -> 422; 112 and 427 since it reads o).
 constexpr int kTileBwdThreads = 320;
 
 struct BwdTileShared {
-    uint64_t in_full, s_full, ds_full, dv_full, dk_full, dq_full, item_free;
+    uint64_t in_full, o_full, terms_full, s_full, ds_full, dv_full, dk_full, dq_full, item_free;
     uint32_t tmem_base, abort_flag;
 };
 
@@ -340,9 +351,14 @@ template <int D>
 struct BwdTileCfg {
     static constexpr int kTileBytes = kTile * D * 2;
     static constexpr int kOffQ = 0, kOffK = kTileBytes, kOffDo = 2 * kTileBytes;
-    static constexpr int kOffP = 3 * kTileBytes;             // V until dP is there, then P (32 KB)
-    static constexpr int kOffDs = kOffP + 32768;             // partial sums of D, then dS, then staging (2 KB per warp)
-    static constexpr int kOffCtl = kOffDs + 32768;
+    static constexpr int kOffP = 3 * kTileBytes;             // V (and O) until dP is there, then P (32 KB)
+    static constexpr int kOffDs = kOffP + 32768;             // dS, then staging (2 KB per warp)
+    // until S and dP are there, dS's buffer holds the per-query terms and the ones beside the staging
+    static constexpr int kOffTerms = kOffDs + 16384;
+    static constexpr int kOffOnes = kOffTerms + kTermTileBytes;      // ones, zeros, ones (2 KB each), see the pair kernel
+    // O: in the half of P's buffer that V leaves free (two CTAs per SM have no other room), or beside
+    static constexpr int kOffO = D == 64 ? kOffP + kTileBytes : kOffDs + 32768;
+    static constexpr int kOffCtl = kOffDs + 32768 + (D == 64 ? 0 : kTileBytes);
     static constexpr int kSmemBytes = kOffCtl + 128;
     static constexpr uint32_t kCols = D == 64 ? 256 : 512;
     static constexpr uint32_t kColS = 0, kColDp = 128, kColDv = 0, kColDk = D, kColDq = 2 * D;
@@ -352,8 +368,8 @@ static_assert(sizeof(BwdTileShared) <= 128, "control block must fit its slot");
 template <int D>
 __global__ void __launch_bounds__(kTileBwdThreads, D == 64 ? 2 : 1)
 tile_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k,
-                const __grid_constant__ CUtensorMap tmap_v, const __grid_constant__ CUtensorMap tmap_do,
-                const __grid_constant__ BwdParams p, bool causal) {
+                const __grid_constant__ CUtensorMap tmap_v, const __grid_constant__ CUtensorMap tmap_o,
+                const __grid_constant__ CUtensorMap tmap_do, const __grid_constant__ BwdParams p, bool causal) {
     using Cfg = BwdTileCfg<D>;
     extern __shared__ __align__(1024) uint8_t smem[];
     BwdTileShared& sh = *reinterpret_cast<BwdTileShared*>(smem + Cfg::kOffCtl);
@@ -362,8 +378,8 @@ tile_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     const WaitGuard guard{&sh.abort_flag, &p.sched.hdr->status};
     grid_trigger();
     if (tid == 0) {
-        for (uint64_t* b : {&sh.in_full, &sh.s_full, &sh.dv_full, &sh.dk_full, &sh.dq_full}) mbar_init(b, 1);
-        for (uint64_t* b : {&sh.ds_full, &sh.item_free}) mbar_init(b, 8);
+        for (uint64_t* b : {&sh.in_full, &sh.o_full, &sh.s_full, &sh.dv_full, &sh.dk_full, &sh.dq_full}) mbar_init(b, 1);
+        for (uint64_t* b : {&sh.terms_full, &sh.ds_full, &sh.item_free}) mbar_init(b, 8);
         sh.abort_flag = (smem_u32(smem) & 1023u) != 0 ? 1u : 0u;
         fence_mbar_init();
     }
@@ -387,8 +403,10 @@ tile_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             for (uint32_t i = blockIdx.x; i < n; i += gridDim.x, ++k) {
                 const TileItem w = tile_item(p.sched, p.cu_seqlens, first_seq, i, p.n_heads);
                 if (k >= 1) mbar_wait(&sh.dv_full, (k - 1) & 1u, guard);     // (and the previous item's loads have completed)
-                mbar_expect_tx(&sh.in_full, 4 * Cfg::kTileBytes);
-                load_tile<D>(smem + Cfg::kOffDo, &tmap_do, &sh.in_full, w.head, w.tok0);
+                mbar_expect_tx(&sh.o_full, 2 * Cfg::kTileBytes);
+                load_tile<D>(smem + Cfg::kOffO, &tmap_o, &sh.o_full, w.head, w.tok0);
+                load_tile<D>(smem + Cfg::kOffDo, &tmap_do, &sh.o_full, w.head, w.tok0);
+                mbar_expect_tx(&sh.in_full, 3 * Cfg::kTileBytes);
                 load_tile<D>(smem + Cfg::kOffP, &tmap_v, &sh.in_full, w.head, w.tok0);      // the product has read P
                 if (k >= 1) mbar_wait(&sh.dk_full, (k - 1) & 1u, guard);
                 load_tile<D>(smem + Cfg::kOffQ, &tmap_q, &sh.in_full, w.head, w.tok0);
@@ -412,11 +430,15 @@ tile_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         const uint64_t p_mn = make_sdesc_sw128(smem_u32(smem + Cfg::kOffP), kBoxBytes, 1024);
         const uint64_t ds_mn = make_sdesc_sw128(smem_u32(smem + Cfg::kOffDs), kBoxBytes, 1024);
         const uint64_t ds_km = make_sdesc_sw128(smem_u32(smem + Cfg::kOffDs), 16, 1024);
+        const uint64_t terms = make_sdesc_nosw(smem_u32(smem + Cfg::kOffTerms), 2048, 128);
+        const uint64_t ones_s = make_sdesc_nosw(smem_u32(smem + Cfg::kOffOnes), 2048, 128);
+        const uint64_t ones_d = make_sdesc_nosw(smem_u32(smem + Cfg::kOffOnes + 2048), 2048, 128);
         auto km_step = [](int ks) -> uint64_t { return (uint64_t)(((ks / 4) * kBoxBytes + (ks % 4) * 32) >> 4); };
         auto mn_step = [](int ks) -> uint64_t { return (uint64_t)((ks * 2048) >> 4); };
         uint32_t k = 0;
         for (uint32_t i = blockIdx.x; i < n; i += gridDim.x, ++k) {
             mbar_wait_all(&sh.in_full, k & 1u, guard);
+            mbar_wait_all(&sh.o_full, k & 1u, guard);            // (dO)
             if (k >= 1) mbar_wait_all(&sh.item_free, (k - 1) & 1u, guard);       // the accumulators have been read
             tc_fence_after();
 #pragma unroll
@@ -425,12 +447,17 @@ tile_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
 #pragma unroll
             for (int ks = 0; ks < D / 16; ++ks)
                 if (leader && ks < n_ks) tc_mma_ss(tmem + Cfg::kColDp, do_km + km_step(ks), v_km + km_step(ks), idesc_s, ks > 0);
+            mbar_wait_all(&sh.terms_full, k & 1u, guard);
+            if (leader) tc_mma_ss(tmem + Cfg::kColS, terms, ones_s, idesc_s, true);
+            if (leader) tc_mma_ss(tmem + Cfg::kColDp, terms, ones_d, idesc_s, true);
             if (leader) tc_commit(&sh.s_full);
             mbar_wait_all(&sh.ds_full, k & 1u, guard);
             tc_fence_after();
 #pragma unroll
-            for (int ks = 0; ks < 8; ++ks)
-                if (leader) tc_mma_ss(tmem + Cfg::kColDv, p_mn + mn_step(ks), do_mn + mn_step(ks), idesc_mm, ks > 0);
+            for (int k8 = 0; k8 < 8; ++k8) {                 // k-steps {0,1,4,5} then {2,3,6,7}, as the multi-tile kernel adds them
+                const int ks = (k8 / 2 % 2) * 4 + (k8 / 4) * 2 + k8 % 2;
+                if (leader) tc_mma_ss(tmem + Cfg::kColDv, p_mn + mn_step(ks), do_mn + mn_step(ks), idesc_mm, k8 > 0);
+            }
             if (leader) tc_commit(&sh.dv_full);
 #pragma unroll
             for (int ks = 0; ks < 8; ++ks)
@@ -447,90 +474,87 @@ tile_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         const int row = quarter * 32 + lane;                 // query row
         uint8_t *p_row = smem + Cfg::kOffP + half * kBoxBytes, *ds_row = smem + Cfg::kOffDs + half * kBoxBytes;
         uint8_t* stage = smem + Cfg::kOffDs + warp * 2048;
-        float* sums = reinterpret_cast<float*>(smem + Cfg::kOffDs + quarter * 4096);     // in rows only these two warps write
         const uint64_t sc2 = pack_f32x2(p.scale_log2, p.scale_log2);
+        const int t_row = warp * 16 + (lane & 15), t_role = lane >> 4;   // the row and which of its terms this thread stores
         TileItem w{0, 0, 0, 0};
         int lo = 0, hi = 0;
-        float lse = 0.f;
+        float lse = 0.f;                                     // of t_row
         auto fetch = [&](uint32_t i) {
             w = tile_item(p.sched, p.cu_seqlens, first_seq, i, p.n_heads);
             row_keys(w, row, p.sched, p.members, causal, lo, hi);
-            lse = row < w.len ? p.lse[(size_t)w.head * p.total_tokens + w.tok0 + row] : 0.f;
+            lse = t_row < w.len ? p.lse[(size_t)w.head * p.total_tokens + w.tok0 + t_row] : 0.f;
         };
         if (blockIdx.x < n) fetch(blockIdx.x);
         uint32_t k = 0;
         for (uint32_t i = blockIdx.x; i < n; i += gridDim.x, ++k) {
+            // The buffer of dS is free here: this thread has seen dQ of the item before, the last product that reads it.
+            for (int c = tid; c < 6144 / 16; c += 256)
+                *reinterpret_cast<uint4*>(smem + Cfg::kOffOnes + c * 16) =
+                    c / 128 == 1 ? make_uint4(0u, 0u, 0u, 0u) : make_uint4(0x3f803f80u, 0x00003f80u, 0u, 0u);   // 1,1 | 1,0 | 0..
+            mbar_wait(&sh.o_full, k & 1u, guard);
+            __syncwarp();
+            {
+                // the even (odd) chunks of eight columns of this row, added as the pre kernel's lanes add theirs
+                float part[D / 16];
+#pragma unroll
+                for (int c = 0; c < D / 16; ++c) {
+                    const int chunk = 2 * c + t_role;
+                    const uint32_t at = (uint32_t)(chunk / 8) * kBoxBytes + sw128_offset((uint32_t)t_row, (uint32_t)(chunk % 8));
+                    part[c] = chunk_dot(*reinterpret_cast<const uint4*>(smem + Cfg::kOffO + at),
+                                        *reinterpret_cast<const uint4*>(smem + Cfg::kOffDo + at));
+                }
+#pragma unroll
+                for (int s = D / 32; s > 0; s >>= 1) {
+#pragma unroll
+                    for (int c = 0; c < s; ++c) part[c] += part[c + s];
+                }
+                const float sum = part[0] + __shfl_xor_sync(0xffffffffu, part[0], 16);
+                const bool live = t_row < w.len;
+                const float none = t_role == 0 ? kNoRow : 0.f;
+                store_term(smem + Cfg::kOffTerms, t_row, t_role, !live ? none : t_role == 0 ? -lse * p.inv_scale : -sum);
+            }
+            fence_async_smem();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sh.terms_full);
             const int wlo = __reduce_min_sync(0xffffffffu, hi > lo ? lo : kTile), whi = __reduce_max_sync(0xffffffffu, hi);
-            const float nl = -lse * 1.4426950408889634f;
-            const uint64_t nl2 = pack_f32x2(nl, nl);
-            mbar_wait(&sh.s_full, k & 1u, guard);
+            mbar_wait(&sh.s_full, k & 1u, guard);            // (the products have read V, the terms and the ones)
             __syncwarp();
             tc_fence_after();
-            float sum = 0.f;                                 // D_i
-#pragma unroll
+#pragma unroll 1
             for (int u = 0; u < 2; ++u) {
                 const int c = half * 2 + u;
                 const bool seen = c * 32 < whi && c * 32 + 32 > wlo;
-                uint32_t pk[16];
+                auto put = [&](int v4, const uint32_t (&pk)[4], const uint32_t (&ds)[4]) {
+                    const uint32_t at = sw128_offset((uint32_t)row, (uint32_t)(u * 4 + v4));
+                    *reinterpret_cast<uint4*>(p_row + at) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+                    *reinterpret_cast<uint4*>(ds_row + at) = make_uint4(ds[0], ds[1], ds[2], ds[3]);
+                };
                 if (seen) {
                     uint32_t s[32], dp[32];
                     tmem_ld_x32(my + Cfg::kColS + c * 32, s);
                     tmem_ld_x32(my + Cfg::kColDp + c * 32, dp);
                     tmem_wait_ld();
                     const uint32_t bits = chunk_bits(lo, hi, c);
-                    float s0 = 0.f, s1 = 0.f;
 #pragma unroll
-                    for (int e = 0; e < 16; ++e) {
-                        float x0, x1;
-                        unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(s[2 * e]), __uint_as_float(s[2 * e + 1])), sc2, nl2), x0, x1);
-                        const float p0 = bits & (1u << (2 * e)) ? fast_exp2(x0) : 0.f;
-                        const float p1 = bits & (2u << (2 * e)) ? fast_exp2(x1) : 0.f;
-                        s0 += p0 * __uint_as_float(dp[2 * e]);
-                        s1 += p1 * __uint_as_float(dp[2 * e + 1]);
-                        s[2 * e] = __float_as_uint(p0);
-                        s[2 * e + 1] = __float_as_uint(p1);
-                        pk[e] = pack_bf16x2(p0, p1);
+                    for (int v4 = 0; v4 < 4; ++v4) {
+                        uint32_t pk[4], ds[4];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            const int j = v4 * 8 + 2 * e;
+                            float x0, x1;
+                            unpack_f32x2(mul_f32x2(pack_f32x2(__uint_as_float(s[j]), __uint_as_float(s[j + 1])), sc2), x0, x1);
+                            const float p0 = bits & (1u << j) ? fast_exp2(x0) : 0.f;
+                            const float p1 = bits & (2u << j) ? fast_exp2(x1) : 0.f;
+                            pk[e] = pack_bf16x2(p0, p1);
+                            ds[e] = pack_bf16x2(p0 * __uint_as_float(dp[j]), p1 * __uint_as_float(dp[j + 1]));
+                        }
+                        put(v4, pk, ds);
                     }
-                    sum += s0 + s1;
-                    tmem_st_x32(my + Cfg::kColS + c * 32, s);
                 } else {
+                    const uint32_t zero[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
-                    for (int e = 0; e < 16; ++e) pk[e] = 0u;
+                    for (int v4 = 0; v4 < 4; ++v4) put(v4, zero, zero);
                 }
-#pragma unroll
-                for (int v4 = 0; v4 < 4; ++v4)
-                    *reinterpret_cast<uint4*>(p_row + sw128_offset((uint32_t)row, (uint32_t)(u * 4 + v4))) =
-                        make_uint4(pk[v4 * 4], pk[v4 * 4 + 1], pk[v4 * 4 + 2], pk[v4 * 4 + 3]);
-            }
-            tmem_wait_st();
-            // D of the whole row: the two warps that share it exchange their halves (in dS's buffer, which is idle until both
-            // have read)
-            sums[half * 32 + lane] = sum;
-            bar_sync(1 + quarter, 64);
-            sum += sums[(half ^ 1) * 32 + lane];
-            bar_sync(1 + quarter, 64);
-#pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                const int c = half * 2 + u;
-                const bool seen = c * 32 < whi && c * 32 + 32 > wlo;
-                uint32_t pk[16];
-                if (seen) {
-                    uint32_t s[32], dp[32];
-                    tmem_ld_x32(my + Cfg::kColS + c * 32, s);
-                    tmem_ld_x32(my + Cfg::kColDp + c * 32, dp);
-                    tmem_wait_ld();
-#pragma unroll
-                    for (int e = 0; e < 16; ++e)
-                        pk[e] = pack_bf16x2(__uint_as_float(s[2 * e]) * (__uint_as_float(dp[2 * e]) - sum),
-                                            __uint_as_float(s[2 * e + 1]) * (__uint_as_float(dp[2 * e + 1]) - sum));
-                } else {
-#pragma unroll
-                    for (int e = 0; e < 16; ++e) pk[e] = 0u;
-                }
-#pragma unroll
-                for (int v4 = 0; v4 < 4; ++v4)
-                    *reinterpret_cast<uint4*>(ds_row + sw128_offset((uint32_t)row, (uint32_t)(u * 4 + v4))) =
-                        make_uint4(pk[v4 * 4], pk[v4 * 4 + 1], pk[v4 * 4 + 2], pk[v4 * 4 + 3]);
             }
             fence_async_smem();
             tc_fence_before();
@@ -568,10 +592,11 @@ cudaError_t launch_fwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUten
     return launch_dependent(tile_fwd_kernel<D>, n_ctas, kTileThreads, kSmem, stream, tq, tk, tv, p, causal);
 }
 template <int D>
-cudaError_t launch_bwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tdo, const BwdParams& p,
-                       bool causal, unsigned n_ctas, cudaStream_t stream) {
+cudaError_t launch_bwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& to,
+                       const CUtensorMap& tdo, const BwdParams& p, bool causal, unsigned n_ctas, cudaStream_t stream) {
     if (cudaError_t e = allow_smem<tile_bwd_kernel<D>>(BwdTileCfg<D>::kSmemBytes)) return e;
-    return launch_dependent(tile_bwd_kernel<D>, n_ctas, kTileBwdThreads, BwdTileCfg<D>::kSmemBytes, stream, tq, tk, tv, tdo, p, causal);
+    return launch_dependent(tile_bwd_kernel<D>, n_ctas, kTileBwdThreads, BwdTileCfg<D>::kSmemBytes, stream, tq, tk, tv, to, tdo, p,
+                            causal);
 }
 
 unsigned tile_grid(int n_sms, int per_sm, int32_t n_seqs, int32_t n_heads) {
@@ -587,10 +612,10 @@ cudaError_t launch_tile_fwd(const CUtensorMap& tq, const CUtensorMap& tk, const 
                            : launch_fwd<64>(tq, tk, tv, p, causal, tile_grid(n_sms, 4, p.sched.n_seqs, p.n_heads), stream);
 }
 
-cudaError_t launch_tile_bwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tdo,
-                            const BwdParams& p, bool causal, int n_sms, cudaStream_t stream) {
-    return p.head_dim > 64 ? launch_bwd<128>(tq, tk, tv, tdo, p, causal, tile_grid(n_sms, 1, p.sched.n_seqs, p.n_heads), stream)
-                           : launch_bwd<64>(tq, tk, tv, tdo, p, causal, tile_grid(n_sms, 2, p.sched.n_seqs, p.n_heads), stream);
+cudaError_t launch_tile_bwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& to,
+                            const CUtensorMap& tdo, const BwdParams& p, bool causal, int n_sms, cudaStream_t stream) {
+    return p.head_dim > 64 ? launch_bwd<128>(tq, tk, tv, to, tdo, p, causal, tile_grid(n_sms, 1, p.sched.n_seqs, p.n_heads), stream)
+                           : launch_bwd<64>(tq, tk, tv, to, tdo, p, causal, tile_grid(n_sms, 2, p.sched.n_seqs, p.n_heads), stream);
 }
 
 }  // namespace dcp

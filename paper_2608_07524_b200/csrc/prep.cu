@@ -4,6 +4,7 @@
 
 #include "attn_kernels.h"
 #include "launch.h"
+#include "row_terms.cuh"
 #include "sched.cuh"
 #include "sm100_ptx.cuh"
 
@@ -447,7 +448,7 @@ __global__ void __launch_bounds__(256) bwd_pre_kernel(const __nv_bfloat16* __res
                     if (e % kTile < len - row0) acc_blk[e] = make_float4(0.f, 0.f, 0.f, 0.f);
         }
         {
-        uint8_t* out = reinterpret_cast<uint8_t*>(stats) + ((size_t)t * n_heads + h) * (kTile * 16 * 2);
+        uint8_t* out = reinterpret_cast<uint8_t*>(stats) + ((size_t)t * n_heads + h) * kTermTileBytes;
         // Half a warp reads a row with 16-byte loads (D = 128; a quarter warp for D = 64), so that a warp
         // instruction covers 2 (4) rows; a warp takes 16 rows per pass with eight loads of 16 bytes in flight per
         // lane (the kernel waits on HBM latency: bytes in flight are what it runs on).
@@ -465,7 +466,7 @@ __global__ void __launch_bounds__(256) bwd_pre_kernel(const __nv_bfloat16* __res
                 const int r = r0 + u * kRowsPerInst + sub;
                 a[u] = make_uint4(0u, 0u, 0u, 0u);
                 b[u] = make_uint4(0u, 0u, 0u, 0u);
-                nl[u] = -1e30f;
+                nl[u] = kNoRow;
                 if (row0 + r < len) {
                     const size_t tok = (size_t)tok0 + row0 + r;
                     // rows hold head_dim <= D columns; lanes past them re-read column 0 and drop it, so that the
@@ -479,14 +480,7 @@ __global__ void __launch_bounds__(256) bwd_pre_kernel(const __nv_bfloat16* __res
             }
 #pragma unroll
             for (int u = 0; u < kU; ++u) {
-                const uint32_t aw[4] = {a[u].x, a[u].y, a[u].z, a[u].w}, bw[4] = {b[u].x, b[u].y, b[u].z, b[u].w};
-                float sum = 0.f;
-#pragma unroll
-                for (int w = 0; w < 4; ++w) {
-                    const float2 x = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&aw[w]));
-                    const float2 y = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&bw[w]));
-                    sum += x.x * y.x + x.y * y.y;
-                }
+                float sum = chunk_dot(a[u], b[u]);
 #pragma unroll
                 for (int sft = kLanesPerRow / 2; sft > 0; sft >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, sft);
                 acc[u] = sum;
@@ -497,17 +491,7 @@ __global__ void __launch_bounds__(256) bwd_pre_kernel(const __nv_bfloat16* __res
 #pragma unroll
                 for (int u = 0; u < kU; ++u) {
                     const int r = r0 + u * kRowsPerInst + sub;
-                    const float x = role == 0 ? nl[u] : -acc[u];      // every lane of the group holds the row's sum
-                    const __nv_bfloat16 b0 = __float2bfloat16(x);
-                    const float r1 = x - __bfloat162float(b0);
-                    const __nv_bfloat16 b1 = __float2bfloat16(r1);
-                    const __nv_bfloat16 b2 = __float2bfloat16(r1 - __bfloat162float(b1));
-                    uint4 v;
-                    v.x = (uint32_t)__bfloat16_as_ushort(b0) | ((uint32_t)__bfloat16_as_ushort(b1) << 16);
-                    v.y = (uint32_t)__bfloat16_as_ushort(b2);
-                    v.z = 0u;
-                    v.w = 0u;
-                    *reinterpret_cast<uint4*>(out + role * 2048 + (r / 8) * 128 + (r % 8) * 16) = v;
+                    store_term(out, r, role, role == 0 ? nl[u] : -acc[u]);     // every lane of the group holds the row's sum
                 }
             }
         }

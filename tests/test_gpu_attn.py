@@ -436,6 +436,70 @@ def test_single_tile_kernels(causal, d, longest):
     check_full(lengths, 8, d, causal, seed=400 + d)
 
 
+def backward_with_given_terms(q, k, v, g, o, lse, cu, causal):
+    """fp64 gradients from the caller's own o and lse: P = exp(S - lse), D = sum_c dO O, dS = P (dP - D)."""
+    scale = q.shape[2] ** -0.5
+    q, k, v, g, o, lse = (x.double().cpu() for x in (q, k, v, g, o, lse))
+    dq, dk, dv = torch.zeros_like(q), torch.zeros_like(k), torch.zeros_like(v)
+    for a, b in zip(cu[:-1], cu[1:]):
+        s = torch.einsum("ihc,jhc->hij", q[a:b], k[a:b]) * scale
+        p = torch.exp(s - lse[:, a:b, None])
+        if causal:
+            p = p.tril()
+        d = (g[a:b] * o[a:b]).sum(-1).t()[..., None]
+        ds = p * (torch.einsum("ihc,jhc->hij", g[a:b], v[a:b]) - d) * scale
+        dq[a:b] = torch.einsum("hij,jhc->ihc", ds, k[a:b])
+        dk[a:b] = torch.einsum("hij,ihc->jhc", ds, q[a:b])
+        dv[a:b] = torch.einsum("hij,ihc->jhc", p, g[a:b])
+    return (x.numpy() for x in (dq, dk, dv))
+
+
+@pytest.mark.parametrize("causal", [False, True])
+@pytest.mark.parametrize("d", [40, 64, 72, 128])
+@pytest.mark.parametrize("lengths", [[100, 128, 33, 20, 1, 65], [100, 128, 33, 20, 1, 65] * 10, [300, 17, 90, 256, 129]],
+                         ids=["few", "many", "with longer ones"])
+def test_backward_takes_its_terms_from_the_callers_o_and_lse(causal, d, lengths):
+    """Attention over part of the keys: o and lse come from all of them (half as many again for every sequence), and the
+    backward of the part must use them as they are, whichever kernels the batch goes to."""
+    H = 8
+    rng = np.random.default_rng(d)
+    cu = [0] + [int(x) for x in np.cumsum(lengths)]
+    q, k, v, g = inputs.make_qkvg(cu[-1], H, d, 700 + d)
+    extra = torch.from_numpy(rng.standard_normal((2, H, 40, d))).float()
+    o, lse = torch.empty_like(q), torch.empty((H, cu[-1]))
+    for a, b in zip(cu[:-1], cu[1:]):
+        s = torch.einsum("ihc,jhc->hij", q[a:b].float(), k[a:b].float()) * d ** -0.5
+        if causal:
+            s = s.masked_fill(torch.ones(b - a, b - a).triu(1).bool(), float("-inf"))
+        s = torch.cat([s, torch.einsum("ihc,hjc->hij", q[a:b].float(), extra[0]) * d ** -0.5], -1)
+        values = torch.cat([v[a:b].float().transpose(0, 1), extra[1]], 1)
+        o[a:b] = torch.einsum("hij,hjc->ihc", s.softmax(-1), values).to(torch.bfloat16)
+        lse[:, a:b] = s.logsumexp(-1)
+    _, _, dq, dk, dv = run_gpu(q, k, v, g, cu, causal, o_override=o, lse_override=lse)
+    for name, got, ref in zip(("dq", "dk", "dv"), (dq, dk, dv), backward_with_given_terms(q, k, v, g, o, lse, cu, causal)):
+        assert_close(name, got, ref)
+
+
+@pytest.mark.parametrize("causal", [False, True])
+@pytest.mark.parametrize("d", [40, 64, 72, 128])
+def test_single_tile_results_do_not_depend_on_the_rest_of_the_batch(causal, d):
+    """A sequence of at most 128 tokens goes to the single-tile or to the multi-tile kernels, by the batch around it: the
+    same sums in the same order, hence the same bits."""
+    head = [100, 128, 65, 127]
+    n, H = sum(head), 2
+    out = []
+    for rest in ([300], [100] * 200):                # few items: multi-tile kernels (above d = 64 the forward only); many: single-tile
+        lengths = head + rest
+        cu = np.concatenate([[0], np.cumsum(lengths)]).astype(np.int32)
+        q, k, v, g = inputs.make_qkvg(int(cu[-1]), H, d, 800)
+        for i, x in enumerate((q, k, v, g)):
+            x[:n] = inputs.make_qkvg(n, H, d, 810 + i)[0]
+        out.append(run_gpu(q, k, v, g, cu, causal))
+    for name, a, b in zip(("o", "lse", "dq", "dk", "dv"), *out):
+        same = torch.equal(a[:, :n], b[:, :n]) if name == "lse" else torch.equal(a[:n], b[:n])
+        assert same, name
+
+
 def test_a_sequence_longer_than_a_declared_tile_is_refused():
     # max_seqlen <= 128 promises that no sequence needs the multi-tile kernels, which are then not launched
     dev = "cuda"
