@@ -195,7 +195,6 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);     // via a shuffle: provably uniform within the warp
     const int lane = tid & 31;
     const WaitGuard guard{&sh.abort_flag, &p.sched.hdr->status};
-    grid_trigger();
 
     if (tid == 0) {
         for (int i = 0; i < 2; ++i) {
@@ -247,6 +246,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = sh.tmem_base;
+    grid_trigger();
     grid_wait();
     if (tid == 0 && sh.abort_flag) atomicMax(&p.sched.hdr->status, (uint32_t)kStatusBadSmemAlign);
     // when this CTA started and (at the end) when it ran out of work: the spread over CTAs measures the balance

@@ -158,7 +158,6 @@ attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constan
     // shared::cluster address of a barrier in the leader
     auto at_leader = [&](const uint64_t* bar) { return map_to_rank(smem_u32(bar), 0); };
 
-    grid_trigger();
     if (tid == 0) {
         for (int i = 0; i < kRing; ++i) {
             mbar_init(&sh.work_full[i], 1);
@@ -195,6 +194,7 @@ attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constan
     cluster_sync();                                      // the products write both CTAs' tensor memory
     tc_fence_after();
     const uint32_t tmem = sh.tmem_base;
+    grid_trigger();
     grid_wait();
     if (tid == 0 && sh.abort_flag) atomicMax(&p.sched.hdr->status, (uint32_t)kStatusBadSmemAlign);
     if (tid == 0 && blockIdx.x < kMaxCtas) {

@@ -146,7 +146,6 @@ tile_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     const int tid = threadIdx.x, lane = tid & 31;
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
     const WaitGuard guard{&sh.abort_flag, &p.sched.hdr->status};
-    grid_trigger();
     if (tid == 0) {
         for (uint64_t* b : {&sh.qk_full, &sh.v_full, &sh.s_full, &sh.o_full}) mbar_init(b, 1);
         for (uint64_t* b : {&sh.p_full, &sh.v_free, &sh.o_free}) mbar_init(b, 4);
@@ -161,6 +160,7 @@ tile_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = sh.tmem_base;
+    grid_trigger();
     grid_wait();
     if (tid == 0 && sh.abort_flag) atomicMax(&p.sched.hdr->status, (uint32_t)kStatusBadSmemAlign);
     const uint32_t first_seq = p.sched.hdr->n_long_seqs;
@@ -376,7 +376,6 @@ tile_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     const int tid = threadIdx.x, lane = tid & 31;
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
     const WaitGuard guard{&sh.abort_flag, &p.sched.hdr->status};
-    grid_trigger();
     if (tid == 0) {
         for (uint64_t* b : {&sh.in_full, &sh.o_full, &sh.s_full, &sh.dv_full, &sh.dk_full, &sh.dq_full}) mbar_init(b, 1);
         for (uint64_t* b : {&sh.terms_full, &sh.ds_full, &sh.item_free}) mbar_init(b, 8);
@@ -391,6 +390,7 @@ tile_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = sh.tmem_base;
+    grid_trigger();
     grid_wait();
     if (tid == 0 && sh.abort_flag) atomicMax(&p.sched.hdr->status, (uint32_t)kStatusBadSmemAlign);
     const uint32_t first_seq = p.sched.hdr->n_long_seqs;

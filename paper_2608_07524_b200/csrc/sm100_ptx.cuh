@@ -15,7 +15,9 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
 }
 
 // Dependent launches (launch.h): the next kernel of the stream may start its CTAs, / everything the kernels before this
-// one wrote is visible.  Every thread of every kernel launched that way waits before it touches global memory.
+// one wrote is visible.  Every thread of every kernel launched that way waits before it touches global memory.  A kernel that
+// allocates tensor memory triggers after the allocation and a barrier: the next kernel's CTAs hold what they allocate until
+// this grid has ended, and an allocation waits without limit, so what this grid needs must be its own before they start.
 __device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
