@@ -132,7 +132,7 @@ __device__ __noinline__ void compute_single_tile_item(BwdControl& sh, const BwdP
     }
     if (CAUSAL && key_in_tile > q_lo) q_lo = key_in_tile;     // a key is seen from its own position on
     float pf[64];
-    mbar_wait(&sh.s_full, g & 1u, guard);
+    mbar_wait_warp(&sh.s_full, g & 1u, guard);
     tc_fence_after();
     {
         uint32_t sr[64];
@@ -158,8 +158,8 @@ __device__ __noinline__ void compute_single_tile_item(BwdControl& sh, const BwdP
             if (lane == 0) mbar_arrive(c == 0 ? &sh.p_half : &sh.p_full);
         }
     }
-    mbar_wait(&sh.dp_full, g & 1u, guard);
-    if (g >= 1) mbar_wait(&sh.ds_free, (g - 1) & 1u, guard);
+    mbar_wait_warp(&sh.dp_full, g & 1u, guard);
+    if (g >= 1) mbar_wait_warp(&sh.ds_free, (g - 1) & 1u, guard);
     tc_fence_after();
     {
         uint32_t dr[64];
@@ -226,6 +226,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         // the swizzled tile layout needs a 1024-byte aligned base; refuse to run otherwise
         if ((smem_u32(smem) & 1023u) != 0) sh.abort_flag = 1;
     }
+    __syncwarp();
     if (warp == 0) {
         tmem_alloc(&sh.tmem_base, 512);
         tmem_relinquish();
@@ -357,7 +358,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             uint32_t n_work = 0, g = 0;
             while (true) {
                 const uint32_t slot = n_work & 1u;
-                const bool got = mbar_wait(&sh.work_full[slot], (n_work >> 1) & 1u, guard);
+                const bool got = mbar_wait_warp(&sh.work_full[slot], (n_work >> 1) & 1u, guard);
                 if (!__all_sync(0xffffffffu, got)) break;
                 const WorkItem w = sh.work[slot];
                 __syncwarp();
@@ -366,17 +367,17 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                 int first_q, n_q;
                 q_range(w, first_q, n_q);
                 const int N = n_q - first_q;
-                mbar_wait(&sh.kv_full, n_work & 1u, guard);
+                mbar_wait_warp(&sh.kv_full, n_work & 1u, guard);
                 // S^T and dP^T of the first tile
                 uint32_t stage = g % Cfg::kQStages;
-                mbar_wait(&sh.q_full[stage], (g / Cfg::kQStages) & 1u, guard);
+                mbar_wait_warp(&sh.q_full[stage], (g / Cfg::kQStages) & 1u, guard);
                 tc_fence_after();
-                mbar_wait(&sh.stat_full[g & 1u], (g >> 1) & 1u, guard);
+                mbar_wait_warp(&sh.stat_full[g & 1u], (g >> 1) & 1u, guard);
                 issue_abt(tmem + Cfg::kSt, k_km, q_km0 + stage * kStageStep);
                 if (leader) tc_mma_ss(tmem + Cfg::kSt, ones_s, stat0 + (g & 1u) * kStatStep, idesc_abt, true);
                 if (leader) tc_commit(&sh.s_full);
-                mbar_wait(&sh.do_full, g & 1u, guard);
-                if (g >= 1) mbar_wait(&sh.dq_free, (g - 1) & 1u, guard);
+                mbar_wait_warp(&sh.do_full, g & 1u, guard);
+                if (g >= 1) mbar_wait_warp(&sh.dq_free, (g - 1) & 1u, guard);
                 tc_fence_after();
                 issue_abt(tmem + Cfg::kDp, v_km, do_km);
                 if (leader) tc_mma_ss(tmem + Cfg::kDp, ones_d, stat0 + (g & 1u) * kStatStep, idesc_abt, true);
@@ -386,13 +387,13 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                     const uint32_t nstage = stage + 1 == Cfg::kQStages ? 0 : stage + 1;
                     const bool has_next = n + 1 < N;
                     // dV += P^T dO
-                    mbar_wait(&sh.p_half, g & 1u, guard);
-                    if (n == 0 && n_work >= 1) mbar_wait(&sh.dkv_free, (n_work - 1) & 1u, guard);
+                    mbar_wait_warp(&sh.p_half, g & 1u, guard);
+                    if (n == 0 && n_work >= 1) mbar_wait_warp(&sh.dkv_free, (n_work - 1) & 1u, guard);
                     tc_fence_after();
 #pragma unroll
                     for (int part = 0; part < 2; ++part) {
                         if (part == 1) {
-                            mbar_wait(&sh.p_full, g & 1u, guard);
+                            mbar_wait_warp(&sh.p_full, g & 1u, guard);
                             tc_fence_after();
                         }
 #pragma unroll
@@ -405,15 +406,15 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                     if (leader) tc_commit(&sh.do_empty);
                     // S^T of the next tile
                     if (has_next) {
-                        mbar_wait(&sh.q_full[nstage], ((g + 1) / Cfg::kQStages) & 1u, guard);
-                        mbar_wait(&sh.stat_full[(g + 1) & 1u], ((g + 1) >> 1) & 1u, guard);
+                        mbar_wait_warp(&sh.q_full[nstage], ((g + 1) / Cfg::kQStages) & 1u, guard);
+                        mbar_wait_warp(&sh.stat_full[(g + 1) & 1u], ((g + 1) >> 1) & 1u, guard);
                         tc_fence_after();
                         issue_abt(tmem + Cfg::kSt, k_km, q_km0 + nstage * kStageStep);
                         if (leader) tc_mma_ss(tmem + Cfg::kSt, ones_s, stat0 + ((g + 1) & 1u) * kStatStep, idesc_abt, true);
                         if (leader) tc_commit(&sh.s_full);
                     }
                     // dQ tile = dS K  (A: dS^T read M-contiguous; B: K with head_dim contiguous)
-                    mbar_wait(&sh.ds_full, g & 1u, guard);
+                    mbar_wait_warp(&sh.ds_full, g & 1u, guard);
                     tc_fence_after();
 #pragma unroll
                     for (int ks = 0; ks < kTile / 16; ++ks)
@@ -428,8 +429,8 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                     if (leader) tc_commit(&sh.ds_free);
                     // dP^T of the next tile (its columns hold dQ until the drain warps have read it)
                     if (has_next) {
-                        mbar_wait(&sh.do_full, (g + 1) & 1u, guard);
-                        mbar_wait(&sh.dq_free, g & 1u, guard);
+                        mbar_wait_warp(&sh.do_full, (g + 1) & 1u, guard);
+                        mbar_wait_warp(&sh.dq_free, g & 1u, guard);
                         tc_fence_after();
                         issue_abt(tmem + Cfg::kDp, v_km, do_km);
                         if (leader) tc_mma_ss(tmem + Cfg::kDp, ones_d, stat0 + ((g + 1) & 1u) * kStatStep, idesc_abt, true);
@@ -457,7 +458,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         uint32_t n_work = 0, g = 0;
         while (true) {
             const uint32_t slot = n_work & 1u;
-            const bool got = mbar_wait(&sh.work_full[slot], (n_work >> 1) & 1u, guard);
+            const bool got = mbar_wait_warp(&sh.work_full[slot], (n_work >> 1) & 1u, guard);
             if (!__all_sync(0xffffffffu, got)) break;
             const WorkItem w = sh.work[slot];
             __syncwarp();
@@ -477,7 +478,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             for (int i = first_q; i < n_q; ++i, ++g) {
                 const bool diag = CAUSAL && i == w.blk;
                 float pf[64];
-                mbar_wait(&sh.s_full, g & 1u, guard);
+                mbar_wait_warp(&sh.s_full, g & 1u, guard);
                 tc_fence_after();
                 {
                     // all 64 scores of this thread's key row are requested before the single wait
@@ -515,8 +516,8 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                 if (lane == 0) mbar_arrive(&sh.p_full);
 
                 // dS^T = P^T o (dP^T - D)
-                mbar_wait(&sh.dp_full, g & 1u, guard);
-                if (g >= 1) mbar_wait(&sh.ds_free, (g - 1) & 1u, guard);
+                mbar_wait_warp(&sh.dp_full, g & 1u, guard);
+                if (g >= 1) mbar_wait_warp(&sh.ds_free, (g - 1) & 1u, guard);
                 tc_fence_after();
                 {
                     uint32_t dr[64];
@@ -540,7 +541,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             }
 
             // item epilogue: dV and dK rows of this key block (each group writes half the columns)
-            mbar_wait(&sh.dkv_full, n_work & 1u, guard);
+            mbar_wait_warp(&sh.dkv_full, n_work & 1u, guard);
             tc_fence_after();
             const size_t tok = (size_t)w.tok0 + (size_t)key;
             const size_t out_off = tok * p.row_stride + w.head * p.head_dim + half * (D / 2);
@@ -565,6 +566,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                             if (half * (D / 2) + c * 32 + v4 * 8 < p.head_dim) *reinterpret_cast<uint4*>(dst + c * 32 + v4 * 8) = val;
                         }
                     }
+                    __syncwarp();    // the next load is warp-wide
                 }
             }
             tc_fence_before();
@@ -580,7 +582,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         uint32_t n_work = 0, g = 0;
         while (true) {
             const uint32_t slot = n_work & 1u;
-            const bool got = mbar_wait(&sh.work_full[slot], (n_work >> 1) & 1u, guard);
+            const bool got = mbar_wait_warp(&sh.work_full[slot], (n_work >> 1) & 1u, guard);
             if (!__all_sync(0xffffffffu, got)) break;
             const WorkItem w = sh.work[slot];
             __syncwarp();
@@ -590,7 +592,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             int first_q, n_q;
             q_range(w, first_q, n_q);
             for (int i = first_q; i < n_q; ++i, ++g) {
-                mbar_wait(&sh.dq_full, g & 1u, guard);
+                mbar_wait_warp(&sh.dq_full, g & 1u, guard);
                 tc_fence_after();
                 // accumulator block of (tile, head) is [D/4][128 rows][4]: the 32 rows of a warp are
                 // contiguous for a fixed column group, so each vector atomic covers whole sectors
@@ -636,6 +638,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     tc_fence_before();
     __syncthreads();
     if (tid == 0 && blockIdx.x < kMaxCtas) p.sched.spans[1 * kMaxCtas + blockIdx.x].end_ns = global_timer_ns();
+    __syncwarp();
     if (warp == 0) tmem_dealloc(tmem, 512);
 }
 

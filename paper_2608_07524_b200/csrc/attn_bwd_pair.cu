@@ -461,8 +461,7 @@ attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constan
             for (int i = first_q_of(w); i < n_q; ++i, ++k) {
                 const bool diag = CAUSAL && i * kTile < key0 + kTile;
                 float pf[64];
-                mbar_wait(&sh.s_done, k & 1u, guard);
-                __syncwarp();
+                mbar_wait_warp(&sh.s_done, k & 1u, guard);
                 tc_fence_after();
                 {
                     uint32_t sr[64];
@@ -499,8 +498,7 @@ attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constan
                 if (lane == 0) mbar_arrive_at(bar_p);
 
                 // dS^T = P^T o (dP^T - D)
-                mbar_wait(&sh.dp_done, k & 1u, guard);
-                __syncwarp();
+                mbar_wait_warp(&sh.dp_done, k & 1u, guard);
                 tc_fence_after();
                 uint32_t ds[32];
                 {
@@ -522,7 +520,7 @@ attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constan
                 __syncwarp();
                 if (lane == 0) mbar_arrive_at(bar_ds_tmem);
                 // shared memory: dQ of the previous tile, which read it (in both CTAs), was issued before dV of this one
-                if (k >= 1) mbar_wait(&sh.dq_done, (k - 1) & 1u, guard);
+                if (k >= 1) mbar_wait_warp(&sh.dq_done, (k - 1) & 1u, guard);
 #pragma unroll
                 for (int c = 0; c < 8; ++c)
                     *reinterpret_cast<uint4*>(ds_box + sw128_offset(key_in_tile, c)) =
@@ -556,13 +554,11 @@ attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constan
             const int key0 = w.blk * 2 * kTile + (int)rank * kTile + (warp & 3) * 32;
             for (int i = first_q_of(w); i < n_q; ++i, ++k) {
                 if (i == n_q - 1) {                      // dV is complete before the last dQ
-                    mbar_wait(&sh.dv_done, k & 1u, guard);
-                    __syncwarp();
+                    mbar_wait_warp(&sh.dv_done, k & 1u, guard);
                     tc_fence_after();
                     store_block(p.dv, p, stage, tmem + lane_base + kColDv, at_leader(&sh.dv_free), 1.0f, w.head, w.tok0 + key0, w.len - key0);
                 }
-                mbar_wait(&sh.dq_done, k & 1u, guard);
-                __syncwarp();
+                mbar_wait_warp(&sh.dq_done, k & 1u, guard);
                 tc_fence_after();
                 uint32_t acc[64];
                 tmem_ld_x32(dq_tmem, *reinterpret_cast<uint32_t(*)[32]>(&acc[0]));

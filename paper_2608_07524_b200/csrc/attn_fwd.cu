@@ -131,7 +131,7 @@ __device__ __noinline__ void softmax_single_tile_item(FwdShared& sh, const FwdPa
         end_key = (int)(b >> 8);
     }
     const int last_key = CAUSAL ? (row < end_key - 1 ? row : end_key - 1) : end_key - 1;
-    mbar_wait(&sh.s_full[0], s_parity, guard);
+    mbar_wait_warp(&sh.s_full[0], s_parity, guard);
     tc_fence_after();
     uint32_t s[128];
 #pragma unroll
@@ -183,7 +183,7 @@ __device__ __noinline__ void softmax_single_tile_item(FwdShared& sh, const FwdPa
         unpack_f32x2(sum2[1], b0, b1);
         l = (a0 + a1) + (b0 + b1);
     }
-    mbar_wait(&sh.o_full[0], o_parity, guard);
+    mbar_wait_warp(&sh.o_full[0], o_parity, guard);
     tc_fence_after();
     const float inv_l = 1.0f / l;
     const size_t tok = (size_t)w.tok0 + (size_t)row;
@@ -204,6 +204,7 @@ __device__ __noinline__ void softmax_single_tile_item(FwdShared& sh, const FwdPa
                 if (c * 32 + v4 * 8 < p.head_dim) *reinterpret_cast<uint4*>(out + c * 32 + v4 * 8) = val;
             }
         }
+        __syncwarp();                // the next load is warp-wide
     }
     if (valid) p.lse[(size_t)w.head * p.total_tokens + tok] = m * p.scale + __logf(l);
     tc_fence_before();
@@ -253,6 +254,7 @@ __device__ __noinline__ void store_whole_rows(FwdShared& sh, const CUtensorMap* 
             tma_store_3d(tmap_o, stage, half * 64, head, tok_row0);
             bulk_store_commit();
         }
+        __syncwarp();
     }
 }
 
@@ -295,6 +297,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         sh.abort_flag = 0;
         fence_mbar_init();
     }
+    __syncwarp();
     if (warp == 0) {
         tmem_alloc(&sh.tmem_base, 512);
         tmem_relinquish();
@@ -375,12 +378,12 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             const uint32_t s_tmem[2] = {tmem + Cfg::kS0, tmem + Cfg::kS1};
             const uint32_t o_tmem[2] = {tmem + Cfg::kO0, tmem + Cfg::kO1};
             auto kv_wait = [&](uint32_t idx) {
-                mbar_wait(&sh.kv_full[idx % kKvStages], (idx / kKvStages) & 1u, guard);
+                mbar_wait_warp(&sh.kv_full[idx % kKvStages], (idx / kKvStages) & 1u, guard);
             };
             auto commit = [&](uint64_t* bar) { if (leader) tc_commit(bar); };
             while (true) {
                 const uint32_t slot = n_work & 1u;
-                const bool got = mbar_wait(&sh.work_full[slot], (n_work >> 1) & 1u, guard);
+                const bool got = mbar_wait_warp(&sh.work_full[slot], (n_work >> 1) & 1u, guard);
                 if (!__all_sync(0xffffffffu, got)) break;
                 const WorkItem w = sh.work[slot];
                 __syncwarp();
@@ -396,7 +399,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
 #pragma unroll
                 for (int t = 0; t < 2; ++t) {
                     if (nkv_t[t] == 0) continue;
-                    mbar_wait(&sh.q_full[t], use[t] & 1u, guard);
+                    mbar_wait_warp(&sh.q_full[t], use[t] & 1u, guard);
                     tc_fence_after();
                     issue_qk<D, KS>(s_tmem[t], q_desc[t], kv_km0 + (kv_base % kKvStages) * kStageStep, leader);
                     commit(&sh.s_full[t]);
@@ -437,10 +440,10 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                             if (EARLY_Q && j + 2 == nkv_t[0]) commit(&sh.q_empty[0]);
                         }
                         if (j < nkv_t[t]) {
-                            if (j == 0 && use[t] >= 1) mbar_wait(&sh.o_free[t], (use[t] - 1) & 1u, guard);
+                            if (j == 0 && use[t] >= 1) mbar_wait_warp(&sh.o_free[t], (use[t] - 1) & 1u, guard);
 #pragma unroll
                             for (int part = 0; part < kPParts; ++part) {
-                                if (!EARLY_Q || t == 1 || part > 0) mbar_wait(&sh.p_part[t][part], n_p[t] & 1u, guard);
+                                if (!EARLY_Q || t == 1 || part > 0) mbar_wait_warp(&sh.p_part[t][part], n_p[t] & 1u, guard);
                                 tc_fence_after();
                                 issue_pv<KS>(o_tmem[t], s_tmem[t], kv_mn0 + st_v * kStageStep, j > 0, leader, part);
                             }
@@ -477,7 +480,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         uint32_t n_work = 0, n_s = 0, use = 0;
         while (true) {
             const uint32_t slot = n_work & 1u;
-            const bool got = mbar_wait(&sh.work_full[slot], (n_work >> 1) & 1u, guard);
+            const bool got = mbar_wait_warp(&sh.work_full[slot], (n_work >> 1) & 1u, guard);
             if (!__all_sync(0xffffffffu, got)) break;
             const WorkItem w = sh.work[slot];
             __syncwarp();
@@ -499,7 +502,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
 
             float m = -INFINITY, l = 0.f;
             for (int j = 0; j < nkv; ++j) {
-                mbar_wait(&sh.s_full[t], n_s & 1u, guard);
+                mbar_wait_warp(&sh.s_full[t], n_s & 1u, guard);
                 ++n_s;
                 tc_fence_after();
                 uint32_t s[128];
@@ -593,7 +596,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             }
 
             // epilogue: O = acc / l, lse = m*scale + ln l
-            mbar_wait(&sh.o_full[t], use & 1u, guard);
+            mbar_wait_warp(&sh.o_full[t], use & 1u, guard);
             ++use;
             tc_fence_after();
             const float inv_l = 1.0f / l;
@@ -607,19 +610,21 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             }
             __nv_bfloat16* out = p.o + tok * p.row_stride + w.head * p.head_dim;
 #pragma unroll
-            for (int c = 0; c < D / 32; ++c) {
-                uint32_t acc[32];
-                tmem_ld_x32(o_tmem + c * 32, acc);
+            for (int c = 0; c < D / 64; ++c) {
+                uint32_t acc[64];
+                if (c > 0) __syncwarp();             // the load is warp-wide, the stores before it are not
+                tmem_ld_x32(o_tmem + c * 64, *reinterpret_cast<uint32_t(*)[32]>(&acc[0]));
+                tmem_ld_x32(o_tmem + c * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(&acc[32]));
                 tmem_wait_ld();
                 if (valid) {
 #pragma unroll
-                    for (int v4 = 0; v4 < 4; ++v4) {
+                    for (int v4 = 0; v4 < 8; ++v4) {
                         uint4 val;
                         val.x = pack_bf16x2(__uint_as_float(acc[v4 * 8 + 0]) * inv_l, __uint_as_float(acc[v4 * 8 + 1]) * inv_l);
                         val.y = pack_bf16x2(__uint_as_float(acc[v4 * 8 + 2]) * inv_l, __uint_as_float(acc[v4 * 8 + 3]) * inv_l);
                         val.z = pack_bf16x2(__uint_as_float(acc[v4 * 8 + 4]) * inv_l, __uint_as_float(acc[v4 * 8 + 5]) * inv_l);
                         val.w = pack_bf16x2(__uint_as_float(acc[v4 * 8 + 6]) * inv_l, __uint_as_float(acc[v4 * 8 + 7]) * inv_l);
-                        if (c * 32 + v4 * 8 < p.head_dim) *reinterpret_cast<uint4*>(out + c * 32 + v4 * 8) = val;
+                        if (c * 64 + v4 * 8 < p.head_dim) *reinterpret_cast<uint4*>(out + c * 64 + v4 * 8) = val;
                     }
                 }
             }
@@ -634,6 +639,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     tc_fence_before();
     __syncthreads();
     if (tid == 0 && blockIdx.x < kMaxCtas) p.sched.spans[0 * kMaxCtas + blockIdx.x].end_ns = global_timer_ns();
+    __syncwarp();
     if (warp == 0) tmem_dealloc(tmem, 512);
 }
 

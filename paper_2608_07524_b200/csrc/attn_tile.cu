@@ -221,8 +221,7 @@ tile_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         for (uint32_t i = blockIdx.x; i < n; i += gridDim.x, ++k) {
             // chunks that some row of the warp sees
             const int wlo = __reduce_min_sync(0xffffffffu, hi > lo ? lo : kTile), whi = __reduce_max_sync(0xffffffffu, hi);
-            mbar_wait(&sh.s_full, k & 1u, guard);
-            __syncwarp();
+            mbar_wait_warp(&sh.s_full, k & 1u, guard);
             tc_fence_after();
             float m = -INFINITY;
 #pragma unroll
@@ -285,8 +284,7 @@ tile_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                 w = tile_item(p.sched, p.cu_seqlens, first_seq, i + gridDim.x, p.n_heads);
                 row_keys(w, row, p.sched, p.members, causal, lo, hi);
             }
-            mbar_wait(&sh.o_full, k & 1u, guard);
-            __syncwarp();
+            mbar_wait_warp(&sh.o_full, k & 1u, guard);
             tc_fence_after();
             // a row's 1 / l goes with its thread: scaled here, so the rows leave unscaled from the staging buffer
             uint8_t* stage = sV + warp * 4096;       // V has been read by the product
@@ -491,8 +489,7 @@ tile_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             for (int c = tid; c < 6144 / 16; c += 256)
                 *reinterpret_cast<uint4*>(smem + Cfg::kOffOnes + c * 16) =
                     c / 128 == 1 ? make_uint4(0u, 0u, 0u, 0u) : make_uint4(0x3f803f80u, 0x00003f80u, 0u, 0u);   // 1,1 | 1,0 | 0..
-            mbar_wait(&sh.o_full, k & 1u, guard);
-            __syncwarp();
+            mbar_wait_warp(&sh.o_full, k & 1u, guard);
             {
                 // the even (odd) chunks of eight columns of this row, added as the pre kernel's lanes add theirs
                 float part[D / 16];
@@ -517,8 +514,7 @@ tile_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             __syncwarp();
             if (lane == 0) mbar_arrive(&sh.terms_full);
             const int wlo = __reduce_min_sync(0xffffffffu, hi > lo ? lo : kTile), whi = __reduce_max_sync(0xffffffffu, hi);
-            mbar_wait(&sh.s_full, k & 1u, guard);            // (the products have read V, the terms and the ones)
-            __syncwarp();
+            mbar_wait_warp(&sh.s_full, k & 1u, guard);            // (the products have read V, the terms and the ones)
             tc_fence_after();
 #pragma unroll 1
             for (int u = 0; u < 2; ++u) {
@@ -567,8 +563,7 @@ tile_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             const size_t off = ((size_t)cur.tok0 + quarter * 32) * p.row_stride + (size_t)cur.head * p.head_dim + half * W;
             // (dV, dK: rows are keys.)  dS has been read when dQ is there, so its buffer stages what leaves; the next item's
             // operands are on their way meanwhile.
-            mbar_wait(&sh.dq_full, k & 1u, guard);
-            __syncwarp();
+            mbar_wait_warp(&sh.dq_full, k & 1u, guard);
             tc_fence_after();
             store_rows<W>(p.dv + off, p.row_stride, cols, stage, my + Cfg::kColDv + half * W, 1.0f, rows_left);
             store_rows<W>(p.dk + off, p.row_stride, cols, stage, my + Cfg::kColDk + half * W, p.scale, rows_left);

@@ -83,6 +83,15 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, const 
     return mbar_wait_limited(bar, parity, g, kSpinLimit);
 }
 
+// The same for a converged warp, which it leaves converged: the lanes give up polling one by one, and what follows a wait is
+// warp-wide (tensor-memory accesses, an elected lane's products whose operands the warp shares).  mbar_wait itself is for
+// code that a single lane runs.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, const WaitGuard& g) {
+    const bool got = mbar_wait(bar, parity, g);
+    __syncwarp();
+    return got;
+}
+
 // The same for a converged warp whose lanes may wait on different barriers: all lanes leave the loop together.
 __device__ __forceinline__ bool mbar_wait_all(uint64_t* bar, uint32_t parity, const WaitGuard& g) {
     for (uint32_t spin = 0; spin < kSpinLimit; ++spin) {
@@ -202,7 +211,7 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t pa
         : "memory");
     return done != 0;
 }
-__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity, const WaitGuard& g) {
+__device__ __forceinline__ bool mbar_poll_cluster(uint64_t* bar, uint32_t parity, const WaitGuard& g) {
     for (uint32_t spin = 0; spin < kSpinLimit; ++spin) {
         if (mbar_try_wait_cluster(bar, parity)) return true;
         if ((spin & 1023u) == 1023u && *g.abort_flag) return false;
@@ -210,6 +219,12 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity
     *g.abort_flag = 1u;
     if (g.status) atomicMax(g.status, (uint32_t)kStatusWaitTimeout);
     return false;
+}
+// for a converged warp, which it leaves converged
+__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity, const WaitGuard& g) {
+    const bool got = mbar_poll_cluster(bar, parity, g);
+    __syncwarp();
+    return got;
 }
 __device__ __forceinline__ void st_cluster_v4(uint32_t cluster_addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
     asm volatile("st.shared::cluster.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(cluster_addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
