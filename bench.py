@@ -242,8 +242,8 @@ class Job:
         return tokens, flops
 
     def sm_busy(self):
-        """Per persistent CTA, how long it was busy in the last forward and backward main launch: the spread
-        is the single-GPU imbalance (max / mean = 1 means every SM worked until the end)."""
+        """Per SM (one persistent CTA each on long sequences), how long the main kernels of the last forward and backward kept
+        it busy: the spread is the single-GPU imbalance (max / mean = 1 means every SM worked until the end)."""
         from paper_2608_07524_b200 import binding as B
         out = {}
         for which, key in ((0, "fwd"), (1, "bwd_main")):

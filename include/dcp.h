@@ -310,9 +310,11 @@ int dcp_selftest_wait_timeout(void* workspace, uint32_t spin_limit, void* cuda_s
  * Section 2.3's imbalance, which on one GPU shows as SMs idling while one long sequence finishes).
  * dcp_set_work_order(1) makes later calls list sequences as they come instead of longest first;
  * dcp_set_work_order(0) restores the default.  Process-wide.
- * dcp_read_cta_spans synchronises `cuda_stream` and returns, for the last forward (which = 0) or
- * backward main (which = 1) launch on `workspace`, when each persistent CTA started and when it ran
- * out of work, in nanoseconds of the GPU's global timer: begin_ns, end_ns [256] (host), *n_ctas valid. */
+ * dcp_read_cta_spans synchronises `cuda_stream` and returns, for the last forward (which = 0) or backward
+ * (which = 1) on `workspace`, when the first of the call's persistent CTAs on an SM started and when the last one
+ * there ran out of work (all main kernels of the call; a call of long sequences has one CTA per SM), in nanoseconds of the
+ * GPU's global timer: begin_ns, end_ns [256] (host), one entry per SM that had a CTA, *n_ctas entries valid (0 after a call that
+ * took the short-sequence kernels). */
 int dcp_set_work_order(int input_order);
 
 /* Batches of very short sequences (Section 4.1: the temporal axis of a 2-D model has sequences of a handful

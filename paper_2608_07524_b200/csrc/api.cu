@@ -189,7 +189,7 @@ SchedView carve_sched(void* workspace, int32_t n_seqs) {
     SchedView s;
     uint8_t* base = static_cast<uint8_t*>(workspace);
     s.hdr = reinterpret_cast<WorkspaceHeader*>(base);
-    s.spans = reinterpret_cast<CtaSpan*>(base + sizeof(WorkspaceHeader));
+    s.spans = reinterpret_cast<SmSpan*>(base + sizeof(WorkspaceHeader));
     base += sizeof(WorkspaceHeader) + kSpanBytes;
     s.order = reinterpret_cast<const int32_t*>(base);
     s.prefix = reinterpret_cast<const uint32_t*>(base + sizeof(int32_t) * (size_t)n_seqs);
@@ -296,7 +296,8 @@ static int attn_fwd_impl(const char* fn, bool merge, const void* q, const void* 
     {
         ScopedTimer t(DCP_KERNEL_PREP, stream);
         e = launch_prep(cu_seqlens, n_seqs, total_tokens, max_seqlen, kFwdRowsPerItem, n_heads, sched, merge, bounds, UINT32_MAX,
-                        input_order, split ? kTile + 1 : INT32_MAX, max_seqlen <= kTile ? kTile : INT32_MAX, stream);
+                        input_order, split ? kTile + 1 : INT32_MAX, max_seqlen <= kTile ? kTile : INT32_MAX, 0,
+                        split && max_seqlen <= kTile, stream);
     }
     if (e != cudaSuccess) return fail(DCP_ERR_CUDA, "%s: work-list kernel: %s", fn, cudaGetErrorString(e));
     g_launches.fetch_add(prep_launches(n_seqs, merge, bounds != nullptr, input_order));
@@ -421,7 +422,8 @@ static int attn_bwd_impl(const char* fn, const void* q, const void* k, const voi
     {
         ScopedTimer t(DCP_KERNEL_PREP, stream);
         e = launch_prep(cu_seqlens, n_seqs, total_tokens, max_seqlen, pair ? 2 * kTile : kTile, n_heads, sched, true, bounds,
-                        (uint32_t)max_tiles(total_tokens, n_seqs), input_order, split ? kTile + 1 : INT32_MAX, !multi ? kTile : all_direct ? direct_len : INT32_MAX, stream);
+                        (uint32_t)max_tiles(total_tokens, n_seqs), input_order, split ? kTile + 1 : INT32_MAX,
+                        !multi ? kTile : all_direct ? direct_len : INT32_MAX, 1, !multi, stream);
     }
     if (e != cudaSuccess) return fail(DCP_ERR_CUDA, "%s: work-list kernel: %s", fn, cudaGetErrorString(e));
     g_launches.fetch_add(prep_launches(n_seqs, true, bounds != nullptr, input_order));
@@ -524,7 +526,7 @@ extern "C" int dcp_varlen_attn_bwd_strided(const void* q, const void* k, const v
 // ---------------------------------------------------------------------------------------------
 // Forward attention for callers that cannot allocate device memory.
 //
-// The forward kernel needs scratch for its work list (header, CTA time spans, sequence order, prefix
+// The forward kernel needs scratch for its work list (header, SM time spans, sequence order, prefix
 // sums).  Here that scratch is a fixed array in the library's own device image, so the caller passes
 // inputs and outputs only.  Every GPU that loads this library holds the array until the process exits.
 #define DCP_NOALLOC_MAX_SEQS_VALUE 4096
@@ -618,21 +620,24 @@ extern "C" int dcp_read_cta_spans(const void* workspace, int32_t which, void* cu
         return fail(DCP_ERR_INVALID_ARG, "dcp_read_cta_spans: null pointer or `which` not 0/1");
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     WorkspaceHeader hdr;
-    static_assert(sizeof(CtaSpan) == 16, "span is two 64-bit words");
-    std::vector<CtaSpan> spans(kMaxCtas);
+    static_assert(sizeof(SmSpan) == 16, "span is two 64-bit words");
+    std::vector<SmSpan> spans(kMaxSms);
     const uint8_t* base = static_cast<const uint8_t*>(workspace);
     cudaError_t e = cudaMemcpyAsync(&hdr, base, sizeof hdr, cudaMemcpyDeviceToHost, stream);
     if (e == cudaSuccess)
-        e = cudaMemcpyAsync(spans.data(), base + sizeof(WorkspaceHeader) + (size_t)which * kMaxCtas * sizeof(CtaSpan),
-                            kMaxCtas * sizeof(CtaSpan), cudaMemcpyDeviceToHost, stream);
+        e = cudaMemcpyAsync(spans.data(), base + sizeof(WorkspaceHeader) + (size_t)which * kMaxSms * sizeof(SmSpan),
+                            kMaxSms * sizeof(SmSpan), cudaMemcpyDeviceToHost, stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
     if (e != cudaSuccess) return fail(DCP_ERR_CUDA, "dcp_read_cta_spans: %s", cudaGetErrorString(e));
-    if (hdr.magic[0] != kHeaderMagic0 || hdr.magic[1] != kHeaderMagic1 || hdr.n_ctas[which] > (uint32_t)kMaxCtas)
+    if (hdr.magic[0] != kHeaderMagic0 || hdr.magic[1] != kHeaderMagic1)
         return fail(DCP_ERR_INVALID_ARG, "dcp_read_cta_spans: no attention call has run on this workspace");
-    *n_ctas = (int32_t)hdr.n_ctas[which];
-    for (int i = 0; i < *n_ctas; ++i) {
-        begin_ns[i] = (int64_t)spans[i].begin_ns;
-        end_ns[i] = (int64_t)spans[i].end_ns;
+    *n_ctas = 0;
+    for (const SmSpan& s : spans) {
+        // entries of SMs without a CTA hold an earlier call's span, what the memory held before, or (cleared) no time
+        constexpr unsigned long long kHour = 3600ull * 1000000000ull;
+        if (hdr.spans_from[which] == 0 || s.begin_ns - hdr.spans_from[which] > kHour || s.end_ns - s.begin_ns > kHour) continue;
+        begin_ns[*n_ctas] = (int64_t)s.begin_ns;
+        end_ns[(*n_ctas)++] = (int64_t)s.end_ns;
     }
     return DCP_OK;
 }

@@ -250,11 +250,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     grid_trigger();
     grid_wait();
     if (tid == 0 && sh.abort_flag) atomicMax(&p.sched.hdr->status, (uint32_t)kStatusBadSmemAlign);
-    // when this CTA started and (at the end) when it ran out of work: the spread over CTAs measures the balance
-    if (tid == 0 && blockIdx.x < kMaxCtas) {
-        p.sched.spans[1 * kMaxCtas + blockIdx.x].begin_ns = global_timer_ns();
-        if (blockIdx.x == 0) p.sched.hdr->n_ctas[1] = gridDim.x < kMaxCtas ? gridDim.x : kMaxCtas;
-    }
+    if (tid == 0) span_begin(p.sched, 1);
 
     // Q tiles that see key block `blk`: [first_q, n_q)
     auto q_range = [](const WorkItem& w, int& first_q, int& n_q) {
@@ -637,7 +633,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
 
     tc_fence_before();
     __syncthreads();
-    if (tid == 0 && blockIdx.x < kMaxCtas) p.sched.spans[1 * kMaxCtas + blockIdx.x].end_ns = global_timer_ns();
+    if (tid == 0) span_end(p.sched, 1);
     __syncwarp();
     if (warp == 0) tmem_dealloc(tmem, 512);
 }

@@ -197,10 +197,7 @@ attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constan
     grid_trigger();
     grid_wait();
     if (tid == 0 && sh.abort_flag) atomicMax(&p.sched.hdr->status, (uint32_t)kStatusBadSmemAlign);
-    if (tid == 0 && blockIdx.x < kMaxCtas) {
-        p.sched.spans[1 * kMaxCtas + blockIdx.x].begin_ns = global_timer_ns();
-        if (blockIdx.x == 0) p.sched.hdr->n_ctas[1] = gridDim.x < kMaxCtas ? gridDim.x : kMaxCtas;
-    }
+    if (tid == 0) span_begin(p.sched, 1);
 
     // Q tiles that see key block `blk`: [first_q, n_q)
     auto first_q_of = [](const WorkItem& w) { return CAUSAL ? 2 * w.blk : 0; };
@@ -602,7 +599,7 @@ attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constan
     __syncwarp();
     tc_fence_before();
     __syncthreads();
-    if (tid == 0 && blockIdx.x < kMaxCtas) p.sched.spans[1 * kMaxCtas + blockIdx.x].end_ns = global_timer_ns();
+    if (tid == 0) span_end(p.sched, 1);
     // after an abandoned wait a copy to the partner may still be under way: give it time before the CTAs leave
     if (sh.abort_flag) for (int i = 0; i < 64; ++i) __nanosleep(1000);
     __syncwarp();

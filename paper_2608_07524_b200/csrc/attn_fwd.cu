@@ -308,11 +308,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     const uint32_t tmem = sh.tmem_base;
     grid_trigger();
     grid_wait();
-    // when this CTA started and (at the end) when it ran out of work: the spread over CTAs measures the balance
-    if (tid == 0 && blockIdx.x < kMaxCtas) {
-        p.sched.spans[0 * kMaxCtas + blockIdx.x].begin_ns = global_timer_ns();
-        if (blockIdx.x == 0) p.sched.hdr->n_ctas[0] = gridDim.x < kMaxCtas ? gridDim.x : kMaxCtas;
-    }
+    if (tid == 0) span_begin(p.sched, 0);
 
     if (warp >= 8) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
@@ -638,7 +634,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
 
     tc_fence_before();
     __syncthreads();
-    if (tid == 0 && blockIdx.x < kMaxCtas) p.sched.spans[0 * kMaxCtas + blockIdx.x].end_ns = global_timer_ns();
+    if (tid == 0) span_end(p.sched, 0);
     __syncwarp();
     if (warp == 0) tmem_dealloc(tmem, 512);
 }

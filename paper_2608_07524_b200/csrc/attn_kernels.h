@@ -79,9 +79,11 @@ int prep_launches(int32_t n_seqs, bool merge, bool table, bool input_order);   /
 // longest first (a measurement aid: it shows what the ordering is worth).  Sequences of at least long_min_len
 // tokens come first in either order and empty ones last; the header counts the first and their items (n_long_seqs, n_long_items);
 // max_len: longest sequence that the call's kernels take; a longer one leaves an empty list and kStatusBadLengths as well.
+// which: 0 forward, 1 backward; clear_spans: only the single-tile kernel follows (see SmSpan).
 cudaError_t launch_prep(const int32_t* cu_seqlens, int32_t n_seqs, int32_t total_tokens, int32_t max_seqlen,
                         int32_t rows_per_block, int32_t n_heads, const SchedView& sched, bool merge, uint16_t* bounds,
-                        uint32_t tile_capacity, bool input_order, int32_t long_min_len, int32_t max_len, cudaStream_t stream);
+                        uint32_t tile_capacity, bool input_order, int32_t long_min_len, int32_t max_len, int which, bool clear_spans,
+                        cudaStream_t stream);
 
 // One CTA that waits, with the kernels' own bounded wait and the given poll limit, on a barrier nobody
 // arrives at, and leaves through the same abort path (status word raised, no trap).

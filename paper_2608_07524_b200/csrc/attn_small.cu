@@ -872,7 +872,7 @@ __global__ void __launch_bounds__(512, 1) small_attn_kernel(const SmallParams p)
 // First kernel of a call on the short-sequence path: the boundaries must start at 0, end at total_tokens,
 // never decrease, and no sequence may exceed the declared maximum; otherwise the status word says so and the
 // attention kernel computes nothing.  Then first_seq[c] = first sequence that starts at or after position
-// c * chunk, for c = 0 .. n_chunks.  `which` = 0 forward, 1 backward: no CTA time spans are recorded here.
+// c * chunk, for c = 0 .. n_chunks.  `which` = 0 forward, 1 backward: no time spans are recorded here.
 // Up to kCheckCtas CTAs (one CTA took 15 us on 20384 sequences): each leaves its finding in a word of its own, which the
 // attention kernel reads; where that does not run (no tokens) there is one CTA, which reports by itself.
 __global__ void __launch_bounds__(1024) small_check_kernel(const int32_t* __restrict__ cu, int32_t n_seqs, int32_t total_tokens,
@@ -894,7 +894,7 @@ __global__ void __launch_bounds__(1024) small_check_kernel(const int32_t* __rest
         if (blockIdx.x == 0) {
             for (int i = gridDim.x; i < kCheckCtas; ++i) hdr->check_bad[i] = 0u;
             header_begin_call(hdr, bad != 0);
-            hdr->n_ctas[which] = 0;
+            hdr->spans_from[which] = 0ull;
             for (int c = total_tokens / chunk + 1; c <= n_chunks; ++c) first_seq[c] = n_seqs;
         }
     }

@@ -165,7 +165,7 @@ tile_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     if (tid == 0 && sh.abort_flag) atomicMax(&p.sched.hdr->status, (uint32_t)kStatusBadSmemAlign);
     const uint32_t first_seq = p.sched.hdr->n_long_seqs;
     const uint32_t n = sh.abort_flag ? 0u : p.sched.hdr->n_items - p.sched.hdr->n_long_items;
-    if (blockIdx.x == 0 && tid == 0 && p.sched.hdr->n_long_items == 0) p.sched.hdr->n_ctas[0] = 0;     // no spans of this call
+    if (tid == 0) span_merge_begin(p.sched, 0);
 
     if (warp == 4) {
         if (lane == 0) {
@@ -329,6 +329,7 @@ tile_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     __syncwarp();
     tc_fence_before();
     __syncthreads();
+    if (tid == 0) span_merge_end(p.sched, 0);
     if (warp == 4) tmem_dealloc(tmem, kCols);
 }
 
@@ -393,7 +394,7 @@ tile_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     if (tid == 0 && sh.abort_flag) atomicMax(&p.sched.hdr->status, (uint32_t)kStatusBadSmemAlign);
     const uint32_t first_seq = p.sched.hdr->n_long_seqs;
     const uint32_t n = sh.abort_flag ? 0u : p.sched.hdr->n_items - p.sched.hdr->n_long_items;
-    if (blockIdx.x == 0 && tid == 0 && p.sched.hdr->n_long_items == 0) p.sched.hdr->n_ctas[1] = 0;
+    if (tid == 0) span_merge_begin(p.sched, 1);
 
     if (warp == 8) {
         if (lane == 0) {
@@ -576,6 +577,7 @@ tile_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     __syncwarp();
     tc_fence_before();
     __syncthreads();
+    if (tid == 0) span_merge_end(p.sched, 1);
     if (warp == 8) tmem_dealloc(tmem, Cfg::kCols);
 }
 

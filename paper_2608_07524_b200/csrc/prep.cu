@@ -225,13 +225,18 @@ template <int NT>
 __global__ void __launch_bounds__(NT) prep_kernel(const int32_t* __restrict__ cu, int32_t n_seqs,
                                                   const uint32_t* __restrict__ n_live_ptr, int32_t rows_per_block, int32_t n_heads,
                                                   WorkspaceHeader* hdr, int32_t* order, uint32_t* prefix, uint32_t* tile_prefix,
-                                                  int ranked, int32_t total_tokens, uint32_t tile_capacity, int32_t long_min_len, int32_t max_len) {
+                                                  int ranked, int32_t total_tokens, uint32_t tile_capacity, int32_t long_min_len, int32_t max_len,
+                                                  SmSpan* spans, int which, bool clear_spans) {
     __shared__ uint32_t scratch[33];
     __shared__ int32_t len_sh[NT];
+    unsigned long long now = 0;
+    if (threadIdx.x == 0) now = global_timer_ns();    // before the wait: reading the timer takes long enough to see in a small call
     grid_trigger();
     grid_wait();
     const int tid = threadIdx.x;
     const int n_live = n_live_ptr ? min((int)*n_live_ptr, n_seqs) : n_seqs;
+    if (clear_spans)
+        for (int i = tid; i < kMaxSms; i += NT) spans[which * kMaxSms + i] = SmSpan{~0ull, 0ull};
     if (!n_live_ptr) {
         // no merge_kernel ran before: check the caller's boundaries here (see merge_kernel)
         int bad = (tid == 0 && (cu[0] != 0 || cu[n_seqs] != total_tokens)) ? 1 : 0;
@@ -289,6 +294,7 @@ __global__ void __launch_bounds__(NT) prep_kernel(const int32_t* __restrict__ cu
     }
     uint32_t run = block_exclusive_scan<NT>(local, scratch, &total);
     if (tid == 0) {
+        hdr->spans_from[which] = now;
         hdr->n_items = total;
         hdr->work_counter = 0;
         hdr->n_long_items = hdr->n_long_seqs = 0;
@@ -333,7 +339,8 @@ int prep_launches(int32_t n_seqs, bool merge, bool table, bool input_order) {
 
 cudaError_t launch_prep(const int32_t* cu_seqlens, int32_t n_seqs, int32_t total_tokens, int32_t max_seqlen,
                         int32_t rows_per_block, int32_t n_heads, const SchedView& sched, bool merge, uint16_t* bounds,
-                        uint32_t tile_capacity, bool input_order, int32_t long_min_len, int32_t max_len, cudaStream_t stream) {
+                        uint32_t tile_capacity, bool input_order, int32_t long_min_len, int32_t max_len, int which, bool clear_spans,
+                        cudaStream_t stream) {
     const int32_t* cu = cu_seqlens;
     const uint32_t* n_live = nullptr;
     const bool small = n_seqs <= 256;
@@ -360,7 +367,8 @@ cudaError_t launch_prep(const int32_t* cu_seqlens, int32_t n_seqs, int32_t total
             return e;
     return launch_dependent(small ? prep_kernel<256> : prep_kernel<1024>, 1, small ? 256 : 1024, 0, stream, cu, n_seqs, n_live,
                             rows_per_block, n_heads, sched.hdr, const_cast<int32_t*>(sched.order), const_cast<uint32_t*>(sched.prefix),
-                            const_cast<uint32_t*>(sched.tile_prefix), ranked, total_tokens, tile_capacity, long_min_len, max_len);
+                            const_cast<uint32_t*>(sched.tile_prefix), ranked, total_tokens, tile_capacity, long_min_len, max_len,
+                            sched.spans, which, clear_spans);
 }
 
 // A (128-row tile, head) block of the backward helpers.

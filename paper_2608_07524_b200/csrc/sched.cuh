@@ -36,7 +36,7 @@ enum : uint32_t {
 // header as fresh memory and clears the status word itself.
 constexpr uint32_t kHeaderMagic0 = 0x64637031u, kHeaderMagic1 = 0x9e3779b9u;
 constexpr int kCheckCtas = 16;        // CTAs of the short-sequence path's check kernel, at most
-constexpr int kMaxCtas = 256;         // persistent CTAs whose time span the header area can record
+constexpr int kMaxSms = 256;          // SMs whose time span the header area can record
 struct WorkspaceHeader {
     uint32_t status;        // 0 = ok, else the highest kStatus* code a kernel has left since the last query
     uint32_t work_counter;  // items claimed beyond the workers' first ones
@@ -45,11 +45,11 @@ struct WorkspaceHeader {
     uint32_t merge_rule;    // which of the two merging rules built them (see merge_kernel)
     uint32_t call_bad;      // this call's boundaries were inconsistent (reset by every call)
     uint32_t magic[2];      // kHeaderMagic0/1 once the header has been initialised
-    uint32_t n_ctas[2];     // CTAs of the last forward / backward main launch that recorded a span
     uint32_t n_long_items;  // items of the sequences of more than one tile, which come first in the list; the single-tile
     uint32_t n_long_seqs;   // kernels take the rest.  (Both 0 where one kernel takes the whole list.)  And those sequences
     uint32_t check_bad[16]; // short-sequence path: whether a CTA of the check kernel found this call's boundaries inconsistent
-    uint32_t pad[36];
+    unsigned long long spans_from[2];     // when the list of the last forward / backward was built; 0: it recorded no spans
+    uint32_t pad[34];
 };
 static_assert(sizeof(WorkspaceHeader) == 256, "header is 256 bytes");
 
@@ -59,7 +59,7 @@ static_assert(sizeof(WorkspaceHeader) == 256, "header is 256 bytes");
 __device__ __forceinline__ void header_begin_call(WorkspaceHeader* hdr, bool bad) {
     if (hdr->magic[0] != kHeaderMagic0 || hdr->magic[1] != kHeaderMagic1) {
         hdr->status = kStatusOk;
-        hdr->n_ctas[0] = hdr->n_ctas[1] = 0;
+        hdr->spans_from[0] = hdr->spans_from[1] = 0ull;
         hdr->magic[0] = kHeaderMagic0;
         hdr->magic[1] = kHeaderMagic1;
     }
@@ -68,14 +68,16 @@ __device__ __forceinline__ void header_begin_call(WorkspaceHeader* hdr, bool bad
 }
 #endif
 
-// When a persistent CTA of the forward (slot 0) or backward main kernel (slot 1) started and when it
-// ran out of work, in nanoseconds of the GPU's global timer.  Their spread over the CTAs is the
-// single-GPU form of the paper's imbalance ratio (Section 2.3, Section 4.2): with a good work order
-// every CTA ends within one item of the others.
-struct CtaSpan {
+// When the first persistent CTA of the forward (slot 0) or the backward's main kernels (slot 1) on an SM started and when the
+// last one there ran out of work, in nanoseconds of the GPU's global timer (what begins before spans_from is not this
+// call's).  Their spread over the SMs is the single-GPU form of the paper's imbalance ratio (Section 2.3, Section 4.2): with
+// a good work order every SM ends within one item of the others.  By SM, because a call may have two main kernels, of one to
+// four CTAs per SM: the multi-tile kernels, one CTA on every SM, store; the single-tile kernels that follow them merge theirs
+// in, and where these are alone prep_kernel has cleared the slot.
+struct SmSpan {
     unsigned long long begin_ns, end_ns;
 };
-constexpr size_t kSpanBytes = 2 * kMaxCtas * sizeof(CtaSpan);      // 8 KB right after the header
+constexpr size_t kSpanBytes = 2 * kMaxSms * sizeof(SmSpan);      // 8 KB right after the header
 
 // After the header and the span table: int32 order[n_seqs] (sequence ids, longest first, ties by id),
 // uint32 prefix[n_seqs + 1] (items before the i-th sequence of `order`),
@@ -86,7 +88,7 @@ constexpr size_t kSpanBytes = 2 * kMaxCtas * sizeof(CtaSpan);      // 8 KB right
 // (vcu, or the caller's cu_seqlens when merging is off).
 struct SchedView {
     WorkspaceHeader* hdr;
-    CtaSpan* spans;         // [2][kMaxCtas]
+    SmSpan* spans;          // [2][kMaxSms]
     const int32_t* order;
     const uint32_t* prefix;
     const uint32_t* tile_prefix;

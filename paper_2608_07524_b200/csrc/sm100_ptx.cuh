@@ -110,6 +110,30 @@ __device__ __forceinline__ unsigned long long global_timer_ns() {
     return t;
 }
 
+// A CTA's span of the call's main kernels, as its SM's or merged into that (see SmSpan); one thread, after grid_wait / at the
+// end.
+__device__ __forceinline__ uint32_t sm_id() {
+    uint32_t id;
+    asm volatile("mov.u32 %0, %%smid;" : "=r"(id));
+    return id;
+}
+__device__ __forceinline__ void span_begin(const SchedView& s, int which) {
+    const uint32_t sm = sm_id();
+    if (sm < kMaxSms) s.spans[which * kMaxSms + sm].begin_ns = global_timer_ns();
+}
+__device__ __forceinline__ void span_end(const SchedView& s, int which) {
+    const uint32_t sm = sm_id();
+    if (sm < kMaxSms) s.spans[which * kMaxSms + sm].end_ns = global_timer_ns();
+}
+__device__ __forceinline__ void span_merge_begin(const SchedView& s, int which) {
+    const uint32_t sm = sm_id();
+    if (sm < kMaxSms) atomicMin(&s.spans[which * kMaxSms + sm].begin_ns, global_timer_ns());
+}
+__device__ __forceinline__ void span_merge_end(const SchedView& s, int which) {
+    const uint32_t sm = sm_id();
+    if (sm < kMaxSms) atomicMax(&s.spans[which * kMaxSms + sm].end_ns, global_timer_ns());
+}
+
 // Generic-proxy writes to shared memory become visible to the async proxy (TMA, tcgen05.mma).
 __device__ __forceinline__ void fence_async_smem() {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");

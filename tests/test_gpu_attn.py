@@ -653,6 +653,32 @@ def test_cta_spans_are_recorded():
         assert int(end.max() - begin.min()) < 10 ** 9          # nanoseconds: well under a second
 
 
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("lengths", [[100] * 200, [100] * 200 + [1000], [100] * 3], ids=["single tiles", "both kernels", "few"])
+def test_cta_spans_cover_every_main_kernel(lengths, d):
+    """Batches whose items go to the single-tile kernels, or to both: a span per SM that had a CTA, from the first start to
+    the last end, inside the call."""
+    dev = "cuda"
+    H = 8
+    cu = np.concatenate([[0], np.cumsum(lengths)]).astype(np.int32)
+    q, k, v, g = (x.to(dev) for x in inputs.make_qkvg(int(cu[-1]), H, d, 67))
+    cud = torch.tensor(cu, device=dev)
+    ws = B.alloc_workspace(int(cu[-1]), len(lengths), H, d, True, dev)
+    n_sms = torch.cuda.get_device_properties(0).multi_processor_count
+    last = 0
+    for _ in range(2):                               # the second call's spans replace the first's
+        o, lse = B.dcp_varlen_attn_fwd(q, k, v, cud, max(lengths), False, workspace=ws)
+        B.dcp_varlen_attn_bwd(q, k, v, o, g, lse, cud, max(lengths), False, workspace=ws)
+        spans = [B.dcp_read_cta_spans(ws, which) for which in (0, 1)]
+        for begin, end in spans:
+            assert 0 < begin.size <= n_sms
+            assert bool((end >= begin).all()) and int(begin.min()) > last and int(end.max() - begin.min()) < 10 ** 9
+        if len(lengths) > 3:
+            assert spans[0][0].size == spans[1][0].size == n_sms
+        assert int(spans[1][0].min()) >= int(spans[0][1].max())         # the backward's kernels follow the forward's
+        last = int(spans[1][1].max())
+
+
 @pytest.mark.parametrize("lengths", [[300, 5, 13, 129, 64, 700], [13, 1, 0, 7, 16, 9, 12, 3] * 40],
                          ids=["tile kernels", "short-sequence kernels"])
 @pytest.mark.parametrize("causal", [False, True])
