@@ -448,7 +448,7 @@ def run_ours(args):
     bwd_flops_per_launch = (flops / args.steps) * (2.5 / 3.5) / max(bwd_n / args.steps, 1)
     achieved = bwd_flops_per_launch / (bwd_ms / max(bwd_n, 1) * 1e-3) / 1e12 if bwd_n else None
     plain = not args.drop_longer_than and args.layers == 1 and not args.longest_last and args.order == "longest"
-    roofline = {"bound": "tensor", "kernel": "attn_bwd_kernel (backward main)", "achieved": achieved,
+    roofline = {"bound": "tensor", "kernel": ("attn_bwd_pair_kernel" if d > 64 else "attn_bwd_kernel") + " (backward main)", "achieved": achieved,
                 "peak": peaks["sustained"], "unit": UNIT, "frac": (achieved / peaks["sustained"]) if achieved else None,
                 "peak_source": f"bf16_tflops_sustained of {peaks['source']} MEASURED_PEAKS.json",
                 "traffic": load_dram_traffic(args.workload) if plain else None,

@@ -269,11 +269,11 @@ int dcp_varlen_attn_bwd_strided(const void* q, const void* k, const void* v, con
  * real-time loop, a plug-in handed fixed buffers by its host program, a process whose allocator is
  * locked down after start-up).  Same operation, arguments, layouts and error codes as
  * dcp_varlen_attn_fwd, but the work-list scratch is a fixed array inside the library's device
- * image (about 74 KB, held by every GPU that loads the library until the process exits) instead of
+ * image (about 90 KB, held by every GPU that loads the library until the process exits) instead of
  * a caller buffer.  Limits and rules:
- *   - runs of very short sequences are not merged into shared tiles here (the table that needs grows
- *     with the token count), so such batches run slower than through dcp_varlen_attn_fwd; results
- *     agree within rounding (sequences of at most 128 tokens take different code paths);
+ *   - runs of short sequences are not merged into shared tiles here (where the multi-tile kernel takes merged
+ *     runs it reads a table that grows with the token count), so such batches run slower than through
+ *     dcp_varlen_attn_fwd; results agree within rounding;
  *   - n_seqs <= DCP_NOALLOC_MAX_SEQS, else DCP_ERR_UNSUPPORTED and nothing is enqueued;
  *   - the call allocates nothing on the device and frees nothing;
  *   - the first call on each device looks up the array's device address (a synchronous runtime

@@ -587,7 +587,7 @@ extern "C" int dcp_varlen_attn_fwd_noalloc(const void* q, const void* k, const v
     if (int rc = noalloc_scratch(fn, &scratch)) return rc;
     if (sched_bytes(n_seqs) > kNoAllocScratchBytes)      // cannot happen for n_seqs <= the maximum; kept as a guard
         return fail(DCP_ERR_UNSUPPORTED, "%s: built-in scratch too small", fn);
-    // short sequences are not merged here: the table that needs is sized by the token count
+    // short sequences are not merged here: the table that the multi-tile kernel reads for them is sized by the token count
     return attn_fwd_impl(fn, false, q, k, v, cu_seqlens, n_seqs, total_tokens, max_seqlen, n_heads, head_dim,
                          (int64_t)n_heads * head_dim, causal, softmax_scale, o, lse, scratch, kNoAllocScratchBytes,
                          cuda_stream);

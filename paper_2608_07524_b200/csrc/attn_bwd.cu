@@ -19,14 +19,13 @@
 //
 // dQ tiles are added into an fp32 accumulator in global memory with vector atomics because every
 // key block of a sequence contributes to the same query rows.  The accumulator is a workspace, so
-// its layout is chosen for the atomics: per (tile, head) a block [d/4][128 rows][4 floats], which
+// its layout is chosen for the atomics: per (tile, head) a block [16][128 rows][4 floats], which
 // makes the 32 rows a warp holds contiguous (full 32-byte sectors, four 128-byte lines per
 // instruction instead of 32 scattered ones); a small kernel converts it to [T, H, d] bf16 later.
-// These 64 KB per (Q tile, K tile) pair are what bounds the kernel: the SM's path to L2 moves about
-// 15-25 bytes per clock for reductions, per-thread atomics and shared-memory bulk reductions alike,
-// and the atomics share the load/store unit with the compute warps' dS^T stores; with the atomics
-// compiled out the same kernel runs a third faster.  What helps is pausing the drain warps briefly
-// between groups of atomics (see kRedGroup).  Measured and rejected: pacing by spinning on the clock
+// These 32 KB per (Q tile, K tile) pair leave the SM at 15-25 bytes per clock, by per-thread atomics and
+// shared-memory bulk reductions alike, and the atomics share the load/store unit with the compute warps' dS^T
+// stores.  What helps is pausing the drain warps briefly between groups of atomics (see kRedGroup).  Measured and
+// rejected, all when this kernel still took head dimension 128 and 64 KB per pair: pacing by spinning on the clock
 // (the spin takes issue slots from the compute warps), bulk reductions from a 16 KB staging buffer,
 // atomics into an L2-hot block (same time, so the limit is on the SM's side), dK before dQ, and
 // staggering the Q walk of neighbouring key blocks.
@@ -55,24 +54,23 @@
 namespace dcp {
 
 // The drain warps pause after every kRedGroup vector atomics, and warp k of the four starts k pauses
-// late.  Issued back to back, a tile's 64 KB of atomics fill the SM's queue towards L2, and the TMA
+// late.  Issued back to back, a tile's atomics fill the SM's queue towards L2, and the TMA
 // requests and shared-memory stores of the other warps wait behind them; short sleeps (which, unlike
 // a spin on the clock, take no issue slots) let those through.  __nanosleep rounds down to steps of
 // about 128 ns here (100 ns had no effect, 150-250 ns the same effect), so the values sit in the
-// middle of a step.  Backward main kernel alone on the video batch: 60.2 ms without any pause, 58.3 with the
-// pauses, 55.8 with the stagger as well; two steps per pause or per stagger, or a pause after every
-// second atomic, cost 57-85 ms.  In the power-capped bench loop: 61.7 -> 58.1 ms.
+// middle of a step.  Chosen at head dimension 128, which the pair kernel has since taken over (video batch, this kernel
+// alone: 60.2 ms without any pause, 58.3 with the pauses, 55.8 with the stagger as well; two steps per pause or per
+// stagger, or a pause after every second atomic, 57-85 ms); not measured again at 64.
 constexpr int kRedGroup = 4;
 constexpr unsigned kRedSleepNs = 192;        // one step
 constexpr unsigned kRedStaggerNs = 128;      // per drain warp, plus half a step
 constexpr int kBwdThreads = 512;
 constexpr float kLog2e = 1.4426950408889634f;
 
-template <int D>
+constexpr int kD = 64;                       // columns of a tile (head dimensions above have the pair kernel)
+
 struct BwdCfg {
-    static constexpr int kTileBytes = kTile * D * 2;     // K, V, Q or dO tile
-    static constexpr int kBoxBytes = kTile * 128;
-    static constexpr int kBoxes = D / 64;
+    static constexpr int kTileBytes = kTile * kD * 2;    // K, V, Q or dO tile: one box of 64 columns
     static constexpr int kDsBytes = kTile * kTile * 2;   // dS^T tile, bf16
     // shared-memory map (offsets from a 1024-byte aligned base)
     static constexpr int kOffK = 0;
@@ -106,11 +104,8 @@ __device__ __forceinline__ void red_add_v4(float* addr, float a, float b, float 
     asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(addr), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
 }
 
-template <int D>
 __device__ __forceinline__ void bwd_load_tile(uint8_t* dst, const CUtensorMap* map, uint64_t* bar, int head, int row) {
-#pragma unroll
-    for (int b = 0; b < BwdCfg<D>::kBoxes; ++b)
-        tma_load_3d(dst + b * BwdCfg<D>::kBoxBytes, map, bar, b * 64, head, row);
+    tma_load_3d(dst, map, bar, 0, head, row);
 }
 
 // Compute-warp work of an item that is a single tile pair (a virtual sequence of at most 128 tokens,
@@ -182,12 +177,12 @@ __device__ __noinline__ void compute_single_tile_item(BwdControl& sh, const BwdP
     if (lane == 0) mbar_arrive(&sh.ds_full);
 }
 
-template <int D, bool CAUSAL>
+template <bool CAUSAL>
 __global__ void __launch_bounds__(kBwdThreads, 1)
 attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k,
                 const __grid_constant__ CUtensorMap tmap_v, const __grid_constant__ CUtensorMap tmap_do,
                 const __grid_constant__ BwdParams p) {
-    using Cfg = BwdCfg<D>;
+    using Cfg = BwdCfg;
     extern __shared__ __align__(1024) uint8_t smem[];
     BwdControl& sh = *reinterpret_cast<BwdControl*>(smem + Cfg::kOffCtl);
 
@@ -292,8 +287,8 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             if (lane == 0) {
                 if (n_work >= 1) mbar_wait(&sh.kv_empty, (n_work - 1) & 1u, guard);
                 mbar_expect_tx(&sh.kv_full, 2 * Cfg::kTileBytes);
-                bwd_load_tile<D>(smem + Cfg::kOffK, &tmap_k, &sh.kv_full, w.head, w.tok0 + w.blk * kTile);
-                bwd_load_tile<D>(smem + Cfg::kOffV, &tmap_v, &sh.kv_full, w.head, w.tok0 + w.blk * kTile);
+                bwd_load_tile(smem + Cfg::kOffK, &tmap_k, &sh.kv_full, w.head, w.tok0 + w.blk * kTile);
+                bwd_load_tile(smem + Cfg::kOffV, &tmap_v, &sh.kv_full, w.head, w.tok0 + w.blk * kTile);
             }
             ++n_work;
             for (int i = first_q; i < n_q; ++i, ++g) {
@@ -302,7 +297,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                 if (lane == 0) {
                     if (fill >= 1) mbar_wait(&sh.q_empty[stage], (fill - 1) & 1u, guard);
                     mbar_expect_tx(&sh.q_full[stage], Cfg::kTileBytes);
-                    bwd_load_tile<D>(smem + Cfg::kOffQ + stage * Cfg::kTileBytes, &tmap_q, &sh.q_full[stage], w.head, row);
+                    bwd_load_tile(smem + Cfg::kOffQ + stage * Cfg::kTileBytes, &tmap_q, &sh.q_full[stage], w.head, row);
                     // per-query terms (2 slots): slot g&1 is free once the rank-1 MMAs of tile g-2 are done.
                     // The 4 KB block of this (tile, head) comes by bulk copy in the layout the MMA reads.
                     if (g >= 2) mbar_wait(&sh.stat_empty[g & 1u], ((g >> 1) - 1) & 1u, guard);
@@ -312,7 +307,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                                   Cfg::kStatBytes, &sh.stat_full[g & 1u]);
                     if (g >= 1) mbar_wait(&sh.do_empty, (g - 1) & 1u, guard);
                     mbar_expect_tx(&sh.do_full, Cfg::kTileBytes);
-                    bwd_load_tile<D>(smem + Cfg::kOffDo, &tmap_do, &sh.do_full, w.head, row);
+                    bwd_load_tile(smem + Cfg::kOffDo, &tmap_do, &sh.do_full, w.head, row);
                 }
             }
         }
@@ -325,16 +320,16 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             // Shared-memory descriptors are built once; a k-step only adds a constant to the address
             // field (the issuing thread is on the critical path: MMA issue blocks while the pipe is busy).
             constexpr uint32_t idesc_abt = make_idesc_bf16(128, 128, false, false);  // both operands K-contiguous
-            constexpr uint32_t idesc_nd_kb = make_idesc_bf16(128, D, false, true);   // A K-contig / tmem, B N-contig
-            constexpr uint32_t idesc_nd_mm = make_idesc_bf16(128, D, true, true);    // A M-contig, B N-contig
+            constexpr uint32_t idesc_nd_kb = make_idesc_bf16(128, kD, false, true);   // A K-contig / tmem, B N-contig
+            constexpr uint32_t idesc_nd_mm = make_idesc_bf16(128, kD, true, true);    // A M-contig, B N-contig
             constexpr uint32_t kStageStep = Cfg::kTileBytes >> 4;
             const uint64_t k_km = make_sdesc_sw128(smem_u32(smem + Cfg::kOffK), 16, 1024);
-            const uint64_t k_mn = make_sdesc_sw128(smem_u32(smem + Cfg::kOffK), Cfg::kBoxBytes, 1024);
+            const uint64_t k_mn = make_sdesc_sw128(smem_u32(smem + Cfg::kOffK), Cfg::kTileBytes, 1024);
             const uint64_t v_km = make_sdesc_sw128(smem_u32(smem + Cfg::kOffV), 16, 1024);
             const uint64_t q_km0 = make_sdesc_sw128(smem_u32(smem + Cfg::kOffQ), 16, 1024);
-            const uint64_t q_mn0 = make_sdesc_sw128(smem_u32(smem + Cfg::kOffQ), Cfg::kBoxBytes, 1024);
+            const uint64_t q_mn0 = make_sdesc_sw128(smem_u32(smem + Cfg::kOffQ), Cfg::kTileBytes, 1024);
             const uint64_t do_km = make_sdesc_sw128(smem_u32(smem + Cfg::kOffDo), 16, 1024);
-            const uint64_t do_mn = make_sdesc_sw128(smem_u32(smem + Cfg::kOffDo), Cfg::kBoxBytes, 1024);
+            const uint64_t do_mn = make_sdesc_sw128(smem_u32(smem + Cfg::kOffDo), Cfg::kTileBytes, 1024);
             const uint64_t ds_km = make_sdesc_sw128(smem_u32(smem + Cfg::kOffDs), 16, 1024);
             const uint64_t ds_mn = make_sdesc_sw128(smem_u32(smem + Cfg::kOffDs), 16384, 1024);
             const uint64_t ones_s = make_sdesc_nosw(smem_u32(smem + Cfg::kOffOnes), 2048, 128);
@@ -344,12 +339,12 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             // address-field increments (16-byte units) of k-step ks
             auto km_step = [](int ks, int box_bytes) -> uint64_t { return (uint64_t)(((ks / 4) * box_bytes + (ks % 4) * 32) >> 4); };
             auto mn_step = [](int ks) -> uint64_t { return (uint64_t)((ks * 2048) >> 4); };
-            // D[128 x 128] = A B^T, both [128 x D] tiles with head_dim contiguous
+            // D[128 x 128] = A B^T, both [128 x 64] tiles with head_dim contiguous
             auto issue_abt = [&](uint32_t d_tmem, uint64_t a, uint64_t b) {
 #pragma unroll
-                for (int ks = 0; ks < D / 16; ++ks)
+                for (int ks = 0; ks < kD / 16; ++ks)
                     if (leader)
-                        tc_mma_ss(d_tmem, a + km_step(ks, Cfg::kBoxBytes), b + km_step(ks, Cfg::kBoxBytes), idesc_abt, ks > 0);
+                        tc_mma_ss(d_tmem, a + km_step(ks, Cfg::kTileBytes), b + km_step(ks, Cfg::kTileBytes), idesc_abt, ks > 0);
             };
             uint32_t n_work = 0, g = 0;
             while (true) {
@@ -540,14 +535,14 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             mbar_wait_warp(&sh.dkv_full, n_work & 1u, guard);
             tc_fence_after();
             const size_t tok = (size_t)w.tok0 + (size_t)key;
-            const size_t out_off = tok * p.row_stride + w.head * p.head_dim + half * (D / 2);
+            const size_t out_off = tok * p.row_stride + w.head * p.head_dim + half * (kD / 2);
 #pragma unroll
             for (int which = 0; which < 2; ++which) {
-                const uint32_t src = tmem + lane_base + (which == 0 ? Cfg::kDv : Cfg::kDk) + half * (D / 2);
+                const uint32_t src = tmem + lane_base + (which == 0 ? Cfg::kDv : Cfg::kDk) + half * (kD / 2);
                 __nv_bfloat16* dst = (which == 0 ? p.dv : p.dk) + out_off;
                 const float mul = which == 0 ? 1.0f : p.scale;
 #pragma unroll
-                for (int c = 0; c < D / 64; ++c) {
+                for (int c = 0; c < kD / 64; ++c) {
                     uint32_t acc[32];
                     tmem_ld_x32(src + c * 32, acc);
                     tmem_wait_ld();
@@ -559,7 +554,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                             val.y = pack_bf16x2(__uint_as_float(acc[v4 * 8 + 2]) * mul, __uint_as_float(acc[v4 * 8 + 3]) * mul);
                             val.z = pack_bf16x2(__uint_as_float(acc[v4 * 8 + 4]) * mul, __uint_as_float(acc[v4 * 8 + 5]) * mul);
                             val.w = pack_bf16x2(__uint_as_float(acc[v4 * 8 + 6]) * mul, __uint_as_float(acc[v4 * 8 + 7]) * mul);
-                            if (half * (D / 2) + c * 32 + v4 * 8 < p.head_dim) *reinterpret_cast<uint4*>(dst + c * 32 + v4 * 8) = val;
+                            if (half * (kD / 2) + c * 32 + v4 * 8 < p.head_dim) *reinterpret_cast<uint4*>(dst + c * 32 + v4 * 8) = val;
                         }
                     }
                     __syncwarp();    // the next load is warp-wide
@@ -590,15 +585,15 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             for (int i = first_q; i < n_q; ++i, ++g) {
                 mbar_wait_warp(&sh.dq_full, g & 1u, guard);
                 tc_fence_after();
-                // accumulator block of (tile, head) is [D/4][128 rows][4]: the 32 rows of a warp are
+                // accumulator block of (tile, head) is [16][128 rows][4]: the 32 rows of a warp are
                 // contiguous for a fixed column group, so each vector atomic covers whole sectors
                 const int qrow = i * kTile + q_in_tile;
-                float* dst = p.dq_acc + (((size_t)w.tile0 + i) * p.n_heads + w.head) * (size_t)(kTile * D) + q_in_tile * 4;
+                float* dst = p.dq_acc + (((size_t)w.tile0 + i) * p.n_heads + w.head) * (size_t)(kTile * kD) + q_in_tile * 4;
                 // read the whole tile first and release tensor memory at once: dP^T of the next tile waits
                 // on it, while the atomics below may take as long as they like
-                uint32_t acc[D];
+                uint32_t acc[kD];
 #pragma unroll
-                for (int c = 0; c < D / 32; ++c) tmem_ld_x32(dq_tmem + c * 32, *reinterpret_cast<uint32_t(*)[32]>(&acc[c * 32]));
+                for (int c = 0; c < kD / 32; ++c) tmem_ld_x32(dq_tmem + c * 32, *reinterpret_cast<uint32_t(*)[32]>(&acc[c * 32]));
                 tmem_wait_ld();
                 tc_fence_before();
                 __syncwarp();
@@ -608,7 +603,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                     if (qrow < w.len) {
                         __nv_bfloat16* out = p.dq + ((size_t)w.tok0 + qrow) * p.row_stride + w.head * p.head_dim;
 #pragma unroll
-                        for (int c = 0; c < D / 8; ++c) {
+                        for (int c = 0; c < kD / 8; ++c) {
                             uint4 val;
                             val.x = pack_bf16x2(__uint_as_float(acc[c * 8 + 0]) * p.scale, __uint_as_float(acc[c * 8 + 1]) * p.scale);
                             val.y = pack_bf16x2(__uint_as_float(acc[c * 8 + 2]) * p.scale, __uint_as_float(acc[c * 8 + 3]) * p.scale);
@@ -621,7 +616,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                     const bool live = qrow < w.len;
                     if ((warp & 3) > 0) __nanosleep((warp & 3) * kRedStaggerNs + 64);
 #pragma unroll
-                    for (int c = 0; c < D / 4; ++c) {
+                    for (int c = 0; c < kD / 4; ++c) {
                         if (live) red_add_v4(dst + c * (kTile * 4), __uint_as_float(acc[c * 4]), __uint_as_float(acc[c * 4 + 1]),
                                    __uint_as_float(acc[c * 4 + 2]), __uint_as_float(acc[c * 4 + 3]));
                         if ((c % kRedGroup) == kRedGroup - 1) __nanosleep(kRedSleepNs);
@@ -641,8 +636,8 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
 template <bool CAUSAL>
 static cudaError_t launch_one(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tdo,
                               const BwdParams& p, int n_ctas, cudaStream_t stream) {
-    if (cudaError_t e = allow_smem<attn_bwd_kernel<64, CAUSAL>>(BwdCfg<64>::kSmemBytes)) return e;
-    return launch_dependent(attn_bwd_kernel<64, CAUSAL>, n_ctas, kBwdThreads, BwdCfg<64>::kSmemBytes, stream, tq, tk, tv, tdo, p);
+    if (cudaError_t e = allow_smem<attn_bwd_kernel<CAUSAL>>(BwdCfg::kSmemBytes)) return e;
+    return launch_dependent(attn_bwd_kernel<CAUSAL>, n_ctas, kBwdThreads, BwdCfg::kSmemBytes, stream, tq, tk, tv, tdo, p);
 }
 
 cudaError_t launch_attn_bwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tdo,

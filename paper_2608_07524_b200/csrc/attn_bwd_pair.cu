@@ -35,11 +35,13 @@
 // lanes at the same time.
 //
 // Measured (16 heads of 128, fwd + bwd in turn under the power cap; the one-CTA kernel in brackets): two sequences of
-// 16384 tokens 9.1 ms = 1200 TFLOP/s (10.5 ms = 1046), 3770 cycles per Q tile and pair (4850 per 128 keys); the video
-// batch's step 69.8 ms (75.2), the 2-D model's spatial axis 8.31 (8.83), at head_dim 72 7.90 (8.16), causal text 4.99
-// (5.08).  Without the reductions the first is 8.7 ms.  The products need 3300 cycles per tile (dQ 1024 of them: M = 128 on
-// a pair runs at half the rate of M = 256), barrier latency the rest; an item's first tile takes 3200 more, most of it waiting
-// for the drain warps to have read the previous dK and dQ.
+// 16384 tokens 9.1 ms = 1200 TFLOP/s (10.5 ms = 1046); the video batch's step 69.8 ms (75.2), the 2-D model's spatial axis
+// 8.31 (8.83), at head_dim 72 7.90 (8.16), causal text 4.99 (5.08).  Without the reductions the first is 8.7 ms.  A Q tile
+// of the first takes 2.54 us and pair at the 1460 MHz that the power cap leaves, 3720 cycles, and 2.24 us, 4180 cycles,
+// when the kernel runs with pauses at 1870-1965 MHz (the loads, the exchange and the reductions do not get faster with the
+// clock).  The products need 3300 cycles per tile (dQ 1024 of them: M = 128 on a pair runs at half the rate of M = 256),
+// barrier latency the rest; an item's first tile takes 3200 more, most of it waiting for the drain warps to have read the
+// previous dK and dQ.
 //
 // Sequences of one block (at most 256 tokens) write dQ directly; longer ones add it to the fp32 accumulator that
 // the pre kernel zeroes and the post kernel converts (layout as in the one-CTA kernel).
@@ -433,7 +435,7 @@ attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constan
     }
     } else if (warp < 8) {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 136;");
-        // ------------------------------------------------- compute: P^T, dS^T, and dK / dV of the previous item
+        // ------------------------------------------------- compute: P^T and dS^T
         const int half = warp >> 2;                                  // which 64 query columns
         const int key_in_tile = (warp & 3) * 32 + lane;              // tensor-memory lane = key
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
@@ -565,7 +567,8 @@ attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constan
                 __syncwarp();
                 if (lane == 0) mbar_arrive_at(bar_free);
                 // the reductions go out half a tile later: sent at once they delay the exchange of the next dS^T, which the next
-                // dQ waits for (3510 -> 3447 cycles per tile; 500 ns had no effect)
+                // dQ waits for (2 % of a tile's time on long sequences, 3 % on 256-token ones, although those send none; 500 ns had
+                // no effect).  One value for head dimensions 72 to 128 and any clock.
                 __nanosleep(900);
                 const int row_in_tile = (int)rank * 64 + q_in_half, qrow = i * kTile + row_in_tile;
                 const bool live = qrow < w.len;

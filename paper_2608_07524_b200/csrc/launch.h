@@ -9,7 +9,7 @@ namespace dcp {
 
 // Launches `kern` so that its CTAs may start while the kernel before it in the stream still runs (programmatic stream
 // serialisation): what comes before its grid_wait() (barriers, tensor memory, descriptor prefetch) and the launch itself
-// then overlap that kernel.  A call is a chain of four to seven kernels, most of them a few microseconds long.
+// then overlap that kernel.  A call is a chain of two to seven kernels, most of them a few microseconds long.
 template <typename... P, typename... A>
 cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t stream, A&&... args) {
     cudaLaunchConfig_t cfg{};

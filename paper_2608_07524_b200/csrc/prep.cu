@@ -317,8 +317,8 @@ __global__ void __launch_bounds__(NT) prep_kernel(const int32_t* __restrict__ cu
     run = block_exclusive_scan<NT>(local, scratch, &total);
     unforeseen = __syncthreads_or(unforeseen);
     if (total > tile_capacity || unforeseen) {
-        // more tiles than the workspace was sized for, or a sequence longer than the launched kernels take: max_seqlen was understated (the bound on merged runs relies on it).  Nothing may index the per-tile
-        // storage: no items, no tiles.
+        // more tiles than the workspace was sized for, or a sequence longer than the launched kernels take: max_seqlen was
+        // understated (the bound on merged runs relies on it).  Nothing may index the per-tile storage: no items, no tiles.
         for (int i = tid; i <= n_seqs; i += NT) tile_prefix[i] = 0;
         if (tid == 0) {
             hdr->n_items = hdr->n_long_items = 0;
@@ -427,8 +427,8 @@ struct BlockList {
 // accumulators with a K=16 MMA against a tile of ones.  Rows past the sequence end get -1e30 and 0,
 // which makes their probabilities vanish without masking.  The tile is stored in the MMA's shared-
 // memory layout (8x8 core matrices; column halves 2048 bytes apart) and is 4 KB-aligned, so one bulk
-// copy fetches it.  Also zeroes the fp32 dQ accumulator blocks of sequences longer than one tile (a
-// sequence of a single tile gets its dQ written directly by the main kernel).  HBM-bound.
+// copy fetches it.  Also zeroes the fp32 dQ accumulator blocks of sequences longer than direct_len, one key block of the main
+// kernel (shorter ones get their dQ written directly by it).  HBM-bound.
 template <int D>
 __global__ void __launch_bounds__(256) bwd_pre_kernel(const __nv_bfloat16* __restrict__ o,
                                                       const __nv_bfloat16* __restrict__ d_o, const float* __restrict__ lse,
@@ -522,7 +522,7 @@ cudaError_t launch_bwd_pre(const __nv_bfloat16* o, const __nv_bfloat16* d_o, con
 // Backward helper 2: dq[T, H, d] = bf16(scale * dq_acc).  dq_acc holds, per (tile, head), a block
 // [d/4][128 rows][4 floats]; a CTA reads one block with coalesced 16-byte loads, transposes it in
 // shared memory as bf16 and writes whole rows.  Rows past the sequence end are skipped, and so are
-// sequences of a single tile, whose dQ the main kernel has already written.
+// sequences of at most direct_len tokens, whose dQ the main kernel has already written.
 template <int D>
 __global__ void __launch_bounds__(256) bwd_post_kernel(const float* __restrict__ dq_acc, __nv_bfloat16* __restrict__ dq,
                                                        const BlockList list, int32_t n_heads, int32_t head_dim, int64_t row_stride,

@@ -15,6 +15,8 @@
 #pragma once
 #include <cstdint>
 
+#include "item_order.h"
+
 namespace dcp {
 
 constexpr int kTile = 128;            // rows of a Q tile / keys of a K,V tile
@@ -133,13 +135,7 @@ __device__ __forceinline__ uint32_t claim_item(WorkspaceHeader* hdr, uint32_t n,
     return n == 0 ? worker : n_workers + atomicAdd(&hdr->work_counter, 1u);
 }
 
-// Map item index -> (sequence, head, block).  Without a mask the items of a sequence are alike and blocks vary fastest, so
-// that CTAs running at the same time share one head's K and V in L2.  Under a causal mask the heaviest blocks come first
-// (forward, heavy_is_last: last rows see the most keys; backward: first keys are seen by the most rows), of as many heads
-// together as give every CTA two items: one head at a time, the last head's heaviest block, up to a hundred times the
-// lightest, started when most of the work was done (one 15904-token sequence beside nine short ones, 4 heads: backward
-// main kernel 813 us, 656 with its heads together); all heads together, sequences of many blocks lose the sharing in L2
-// (131072 tokens, 8 heads: forward 28.1 ms one head at a time, 32.9 together).
+// Map item index -> (sequence, head, block); the order inside a sequence is item_place's.
 //
 // Called by a whole warp.  `cur` keeps the sequence of the item before, which the next item of a worker usually shares (a
 // sequence has n_heads or more items in a row); otherwise the lanes probe 32 places of the list at a time.  One thread's
@@ -174,22 +170,9 @@ __device__ inline WorkItem decode_item(const SchedView& s, const int32_t* cu_seq
     w.tile0 = cur.tile0;
     const uint32_t local = item - cur.begin;
     const uint32_t nblk = (uint32_t)(w.len + rows_per_blk - 1) / (uint32_t)rows_per_blk;
-    uint32_t b;
-    if (causal) {
-        // groups of `least` or more heads, as equal as they come (a small last group would be the tail all over again)
-        const uint32_t heads = (uint32_t)n_heads, least = (2u * (uint32_t)n_workers + nblk - 1) / nblk;
-        const uint32_t groups = least < heads ? heads / least : 1u, size = heads / groups, larger = heads % groups;
-        const uint32_t in_larger = larger * (size + 1) * nblk;       // items of the groups of one head more, which come first
-        const uint32_t g_size = local < in_larger ? size + 1 : size, rest = local < in_larger ? local : local - in_larger;
-        const uint32_t head0 = (local < in_larger ? 0u : larger * (size + 1)) + rest / (g_size * nblk) * g_size;
-        const uint32_t in_group = rest % (g_size * nblk);
-        w.head = (int32_t)(head0 + in_group % g_size);
-        b = in_group / g_size;
-    } else {
-        w.head = (int32_t)(local / nblk);
-        b = local % nblk;
-    }
-    w.blk = (int32_t)(heavy_is_last ? nblk - 1 - b : b);
+    const ItemPlace at = item_place(local, nblk, (uint32_t)n_heads, (uint32_t)n_workers, causal, heavy_is_last);
+    w.head = (int32_t)at.head;
+    w.blk = (int32_t)at.blk;
     return w;
 }
 
