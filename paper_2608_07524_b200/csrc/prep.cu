@@ -428,9 +428,12 @@ struct BlockList {
 // which makes their probabilities vanish without masking.  The tile is stored in the MMA's shared-
 // memory layout (8x8 core matrices; column halves 2048 bytes apart) and is 4 KB-aligned, so one bulk
 // copy fetches it.  Also zeroes the fp32 dQ accumulator blocks of sequences longer than direct_len, one key block of the main
-// kernel (shorter ones get their dQ written directly by it).  HBM-bound.
+// kernel (shorter ones get their dQ written directly by it), the columns that hold data.  HBM-bound.  Zeroing behind a
+// pass's loads and head_dim's columns instead of D (us before and after, 65536 tokens x 16 heads): 72 columns 193 -> 161,
+// 128 columns 212 -> 205; text batch 251 -> 244, 2-D model's spatial axis 386 -> 378.
+constexpr int kPreCtas = 4;      // per SM: 64 registers a thread
 template <int D>
-__global__ void __launch_bounds__(256) bwd_pre_kernel(const __nv_bfloat16* __restrict__ o,
+__global__ void __launch_bounds__(256, kPreCtas) bwd_pre_kernel(const __nv_bfloat16* __restrict__ o,
                                                       const __nv_bfloat16* __restrict__ d_o, const float* __restrict__ lse,
                                                       const BlockList list, __nv_bfloat16* __restrict__ stats,
                                                       float* __restrict__ dq_acc, size_t dq_acc_vec4,
@@ -447,14 +450,13 @@ __global__ void __launch_bounds__(256) bwd_pre_kernel(const __nv_bfloat16* __res
         const int row0 = ref.row0, len = ref.len, tok0 = ref.tok0;
         if (row0 >= len) continue;                       // an item's second tile may lie past the end
         const uint32_t t = ref.tile, h = ref.head, blk = t * (uint32_t)n_heads + h;
-        if (len > direct_len) {
-            // this (tile, head) block of the dQ accumulator; a sequence of a single key block needs none (the main
-            // kernel holds its whole dQ and writes it directly)
-            float4* acc_blk = reinterpret_cast<float4*>(dq_acc) + (size_t)blk * (kTile * D / 4);
-            if ((size_t)(blk + 1) * (kTile * D / 4) <= dq_acc_vec4)
-                for (int e = threadIdx.x; e < kTile * D / 4; e += blockDim.x)      // the main kernel adds to no other rows
-                    if (e % kTile < len - row0) acc_blk[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-        }
+        // this (tile, head) block of the dQ accumulator; a sequence of a single key block needs none (the main kernel holds
+        // its whole dQ and writes it directly).  The main kernel adds to no other rows or columns than these.
+        float4* acc_blk = reinterpret_cast<float4*>(dq_acc) + (size_t)blk * (kTile * D / 4);
+        const bool zero = len > direct_len && (size_t)(blk + 1) * (kTile * D / 4) <= dq_acc_vec4;
+        if (D == 64 && zero)
+            for (int e = threadIdx.x; e < kTile * D / 4; e += blockDim.x)
+                if (e % kTile < len - row0 && e / kTile * 4 < head_dim) acc_blk[e] = make_float4(0.f, 0.f, 0.f, 0.f);
         {
         uint8_t* out = reinterpret_cast<uint8_t*>(stats) + ((size_t)t * n_heads + h) * kTermTileBytes;
         // Half a warp reads a row with 16-byte loads (D = 128; a quarter warp for D = 64), so that a warp
@@ -486,6 +488,14 @@ __global__ void __launch_bounds__(256) bwd_pre_kernel(const __nv_bfloat16* __res
                     if (lane % kLanesPerRow == 0) nl[u] = -lse[(size_t)h * total_tokens + tok] * inv_scale;
                 }
             }
+            // Behind the loads, which would queue behind these stores.  (At 64 columns a block is one pass, and this order is
+            // 1 to 2 % slower than zeroing first.  Unrolled, the loop costs registers, and with them resident CTAs: + 70 %.)
+            if (D == 128 && zero) {
+                constexpr int kPer = 8 * kRowsPerInst * kU * D / 4;
+                const int z0 = (r0 - warp * kRowsPerInst * kU) * D / 4;
+                for (int e = z0 + threadIdx.x; e < z0 + kPer; e += blockDim.x)
+                    if (e % kTile < len - row0 && e / kTile * 4 < head_dim) acc_blk[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+            }
 #pragma unroll
             for (int u = 0; u < kU; ++u) {
                 float sum = chunk_dot(a[u], b[u]);
@@ -511,9 +521,10 @@ cudaError_t launch_bwd_pre(const __nv_bfloat16* o, const __nv_bfloat16* d_o, con
                            const SchedView& sched, __nv_bfloat16* stats, float* dq_acc, size_t dq_acc_elems,
                            int32_t total_tokens, int32_t n_heads, int32_t head_dim, int64_t row_stride, float scale,
                            int32_t tiles_per_item, int32_t direct_len, int n_sms, cudaStream_t stream) {
-    // no more CTAs than (tile, head) blocks the batch can have
-    const size_t most = max_tiles(total_tokens, sched.n_seqs) * (size_t)n_heads;
-    const unsigned blocks = most < (size_t)n_sms * 8 ? (unsigned)most : (unsigned)n_sms * 8;
+    // as many CTAs as are resident, or twice as many (ragged batches, whose blocks are not alike: text batch 0.977 -> 0.970 of
+    // the time before), no more than (tile, head) blocks the batch can have
+    const size_t most = max_tiles(total_tokens, sched.n_seqs) * (size_t)n_heads, full = (size_t)n_sms * kPreCtas * (head_dim > 64 ? 2 : 1);
+    const unsigned blocks = (unsigned)(most < full ? most : full);
     const BlockList list{cu_seqlens, sched.order, sched.prefix, sched.tile_prefix, sched.hdr, sched.n_seqs, n_heads, tiles_per_item};
     return launch_dependent(head_dim > 64 ? bwd_pre_kernel<128> : bwd_pre_kernel<64>, blocks, 256, 0, stream, o, d_o, lse, list, stats,
                             dq_acc, dq_acc_elems / 4, total_tokens, n_heads, head_dim, row_stride, 1.0f / scale, direct_len);
@@ -522,9 +533,13 @@ cudaError_t launch_bwd_pre(const __nv_bfloat16* o, const __nv_bfloat16* d_o, con
 // Backward helper 2: dq[T, H, d] = bf16(scale * dq_acc).  dq_acc holds, per (tile, head), a block
 // [d/4][128 rows][4 floats]; a CTA reads one block with coalesced 16-byte loads, transposes it in
 // shared memory as bf16 and writes whole rows.  Rows past the sequence end are skipped, and so are
-// sequences of at most direct_len tokens, whose dQ the main kernel has already written.
+// sequences of at most direct_len tokens, whose dQ the main kernel has already written.  A thread's eight loads of a pass lie
+// a constant distance apart, columns past head_dim are not read, and the grid is one wave of resident CTAs (us before and after,
+// 65536 tokens x 16 heads): 64 columns 75 -> 69, 72 columns 126 -> 92, 128 columns 147 -> 133; text batch 178 -> 160, 2-D
+// model's spatial axis 253 -> 222.
+constexpr int kPostCtas = 4;     // per SM: 64 registers a thread, 35 KB of shared memory
 template <int D>
-__global__ void __launch_bounds__(256) bwd_post_kernel(const float* __restrict__ dq_acc, __nv_bfloat16* __restrict__ dq,
+__global__ void __launch_bounds__(256, kPostCtas) bwd_post_kernel(const float* __restrict__ dq_acc, __nv_bfloat16* __restrict__ dq,
                                                        const BlockList list, int32_t n_heads, int32_t head_dim, int64_t row_stride,
                                                        float scale, int32_t direct_len) {
     constexpr int kRowBytes = D * 2 + 16;                    // padded row of bf16
@@ -545,17 +560,20 @@ __global__ void __launch_bounds__(256) bwd_post_kernel(const float* __restrict__
         }
         const float4* src = reinterpret_cast<const float4*>(dq_acc + ((size_t)t * n_heads + h) * (kTile * D));
         // eight 16-byte loads in flight per thread before the first use (the kernel waits on HBM latency), and the
-        // next block's tile is looked up while the first eight are in flight
-        for (int e0 = threadIdx.x; e0 < kTile * D / 4; e0 += 8 * 256) {
+        // next block's tile is looked up while the first eight are in flight; columns past head_dim hold nothing
+        const int r = threadIdx.x % kTile, half = threadIdx.x / kTile;
+#pragma unroll
+        for (int i0 = 0; i0 < D / 8; i0 += 8) {
+            if (i0 * 8 >= head_dim) break;
             float4 v[8];
 #pragma unroll
             for (int u = 0; u < 8; ++u)
-                if ((e0 + u * 256) % kTile < rows) v[u] = src[e0 + u * 256];
-            if (e0 == (int)threadIdx.x && more) ref_next = list.find(idx + gridDim.x);
+                if (r < rows && (2 * (i0 + u) + half) * 4 < head_dim) v[u] = src[(i0 + u) * 256 + threadIdx.x];
+            if (i0 == 0 && more) ref_next = list.find(idx + gridDim.x);
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
-                const int e = e0 + u * 256, c4 = e / kTile, r = e % kTile;
-                if (r >= rows) continue;
+                const int c4 = 2 * (i0 + u) + half;
+                if (r >= rows || c4 * 4 >= head_dim) continue;
                 __nv_bfloat162 lo2 = __floats2bfloat162_rn(v[u].x * scale, v[u].y * scale);
                 __nv_bfloat162 hi2 = __floats2bfloat162_rn(v[u].z * scale, v[u].w * scale);
                 uint2 pk;
@@ -580,7 +598,7 @@ cudaError_t launch_bwd_post(const float* dq_acc, __nv_bfloat16* dq, const int32_
                             int32_t total_tokens, int32_t n_heads, int32_t head_dim, int64_t row_stride, float scale,
                             int32_t tiles_per_item, int32_t direct_len, int n_sms, cudaStream_t stream) {
     const size_t most = max_tiles(total_tokens, sched.n_seqs) * (size_t)n_heads;
-    const unsigned blocks = most < (size_t)n_sms * 6 ? (unsigned)most : (unsigned)n_sms * 6;
+    const unsigned blocks = most < (size_t)n_sms * kPostCtas ? (unsigned)most : (unsigned)n_sms * kPostCtas;
     const BlockList list{cu_seqlens, sched.order, sched.prefix, sched.tile_prefix, sched.hdr, sched.n_seqs, n_heads, tiles_per_item};
     return launch_dependent(head_dim > 64 ? bwd_post_kernel<128> : bwd_post_kernel<64>, blocks, 256, 0, stream, dq_acc, dq, list,
                             n_heads, head_dim, row_stride, scale, direct_len);
