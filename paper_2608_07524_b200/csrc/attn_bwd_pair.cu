@@ -22,9 +22,9 @@
 //
 //     dV(k) | S(k+1) | dK(k) | dP(k+1) | dQ(k)
 //
-// so that the compute warps rarely wait: S(k+1) runs while they form dS(k), dP(k+1) while they form P(k+1).  dQ lives
-// in the middle columns of S^T, which are free once S(k+1) has been read into registers (P^T is packed into the
-// outer ones).  Every operand tile is used by exactly one product (Q and dO are loaded twice, as rows for S and dP
+// so that the compute warps rarely wait: S(k+1) runs while they form dS(k), dP(k+1) while they form P(k+1).  Above head
+// dimension 96 dQ lives in the middle columns of S^T, which are free once S(k+1) has been read into registers (P^T is packed
+// into the outer ones); up to 96 it has columns of its own, so that S(k+1) does not wait for dQ(k-1) to be drained.  Every operand tile is used by exactly one product (Q and dO are loaded twice, as rows for S and dP
 // and as columns for dK and dV, since a CTA supplies half of B's columns), which leaves each single-buffered load
 // most of a period.  Between items nothing drains: the first S of an item follows the last dV of the previous one,
 // and the drain warps write dV and dK of an item while the next one is under way.
@@ -84,7 +84,15 @@ constexpr int kSmemBytes = kOffStage + 8192;
 static_assert(kSmemBytes <= 232448, "exceeds the 227 KB a CTA may use");
 // tensor-memory columns.  P^T (dS^T) overwrites S^T (dP^T) packed: group 0's 64 columns go to the first 32, group
 // 1's to the last 32, which leaves 64 adjacent ones in the middle of S^T for dQ.
-constexpr uint32_t kColS = 0, kColDp = 128, kColDv = 256, kColDk = 384, kColDq = kColS + 32;
+// Up to head dimension 96 the three results take 96 columns (a pair's products come in steps of 32) and dQ, 48 then, has room
+// of its own.  Main kernel, 65536 tokens x 16 heads of 72, us with 128 columns and dQ in S^T: sequences of 200 tokens 477 ->
+// 445, 256: 398 -> 373, 1200: 1456 -> 1440, causal 512: 591 -> 559, causal 1200: 1011 -> 955; of 96: 300 814 -> 780.
+template <int KS>
+struct PairCols {
+    static constexpr int kW = KS <= 6 ? 96 : 128;
+    static constexpr bool kOwnDq = kW == 96;
+    static constexpr uint32_t kS = 0, kDp = 128, kDv = 256, kDk = 256 + kW, kDq = kOwnDq ? 256 + 2 * kW : kS + 32;
+};
 
 struct PairControl {
     uint64_t work_full[kRing], work_empty[kRing];
@@ -105,12 +113,13 @@ __device__ __forceinline__ void red_add_v4(float* addr, float a, float b, float 
 // dV or dK of a drain warp's 32 keys, all columns: tensor memory -> bf16 in registers (the accumulator is free again),
 // then 32 columns at a time through 2 KB of staging (rows of 64 bytes, 16-byte chunks swizzled) to global memory, eight
 // rows per instruction.
+template <int W>
 __device__ __forceinline__ void store_block(__nv_bfloat16* out, const BwdParams& p, uint8_t* stage, uint32_t src_tmem, uint32_t free_bar,
                                             float mul, int head, int tok_row0, int rows_left) {
     const int lane = threadIdx.x & 31;
-    uint32_t pk[64];
+    uint32_t pk[W / 2];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
+    for (int c = 0; c < W / 32; ++c) {
         uint32_t acc[32];
         tmem_ld_x32(src_tmem + c * 32, acc);
         tmem_wait_ld();
@@ -123,7 +132,7 @@ __device__ __forceinline__ void store_block(__nv_bfloat16* out, const BwdParams&
     const int sub = lane >> 2, chunk = lane & 3;
     __nv_bfloat16* dst = out + ((size_t)tok_row0 + sub) * p.row_stride + head * p.head_dim + chunk * 8;
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
+    for (int c = 0; c < W / 32; ++c) {
         if (c * 32 >= p.head_dim) break;
 #pragma unroll
         for (int v4 = 0; v4 < 4; ++v4)
@@ -142,12 +151,13 @@ __device__ __forceinline__ void store_block(__nv_bfloat16* out, const BwdParams&
 }
 
 // KS = ceil(head_dim / 16), the steps S and dP sum over (5 to 8; a template parameter, because a step count that the issuing
-// warp reads at run time costs it 650 of 4500 cycles per tile, more than the skipped steps save).  dV, dK and dQ keep their
-// 128 columns, so that consecutive products have one shape: only then are they ordered among themselves, which S(k+1)
-// overwriting the P^T that dV(k) reads, and dP(k+1) the dS^T that dK(k) reads, rely on.
+// warp reads at run time costs it 650 of 4500 cycles per tile, more than the skipped steps save).  dV, dK and dQ have 96 or
+// 128 columns (PairCols).  S(k+1) overwrites the P^T that dV(k) reads, and dP(k+1) the dS^T that dK(k) reads: the pipe runs the
+// products of one issuing thread in order, as the forward's S after O += P V relies on too.
 template <bool CAUSAL, int KS>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
 attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constant__ BwdParams p) {
+    using Cols = PairCols<KS>;
     extern __shared__ __align__(1024) uint8_t smem[];
     PairControl& sh = *reinterpret_cast<PairControl*>(smem + kOffCtl);
 
@@ -247,7 +257,7 @@ attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constan
     } else if (warp == 9) {
         // ------------------------------------------------- TMA producer
         // Loads are issued in the order in which the buffers come free: those of dK one tile later than those of S.
-        const int x_half = (int)rank * 64;               // columns of B this CTA supplies to dV, dK, dQ
+        const int x_half = (int)rank * (Cols::kW / 2);               // columns of B this CTA supplies to dV, dK, dQ
         if (lane == 0) {
             tma_prefetch_desc(&maps.q);
             tma_prefetch_desc(&maps.q_rows);
@@ -331,8 +341,8 @@ attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constan
         // ------------------------------------------------- MMA issue (all lanes in lock step, one elected lane issues)
         const bool leader = elect_one();
         constexpr uint32_t idesc_abt = make_idesc_bf16(256, 128, false, false);  // S^T, dP^T: both operands K-contiguous
-        constexpr uint32_t idesc_acc = make_idesc_bf16(256, 128, false, true);   // dV, dK: A in tensor memory, B N-contiguous
-        constexpr uint32_t idesc_dq = make_idesc_bf16(128, 128, true, true);     // dQ: A M-contiguous, B N-contiguous
+        constexpr uint32_t idesc_acc = make_idesc_bf16(256, Cols::kW, false, true);   // dV, dK: A in tensor memory, B N-contiguous
+        constexpr uint32_t idesc_dq = make_idesc_bf16(128, Cols::kW, true, true);     // dQ: A M-contiguous, B N-contiguous
         const uint64_t k_km = make_sdesc_sw128(smem_u32(smem + kOffK), 16, 1024);
         const uint64_t v_km = make_sdesc_sw128(smem_u32(smem + kOffV), 16, 1024);
         const uint64_t qr_km = make_sdesc_sw128(smem_u32(smem + kOffQr), 16, 1024);
@@ -382,10 +392,10 @@ attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constan
             bool first = true;
             ++n_work;
             wait1(&sh.ld_s, 0);
-            issue_abt(tmem + kColS, k_km, qr_km, ones_s, stat0);
+            issue_abt(tmem + Cols::kS, k_km, qr_km, ones_s, stat0);
             commit(&sh.s_done);
             wait1(&sh.ld_p, 0);
-            issue_abt(tmem + kColDp, v_km, dor_km, ones_d, stat0);
+            issue_abt(tmem + Cols::kDp, v_km, dor_km, ones_d, stat0);
             commit(&sh.dp_done);
             while (cur) {
                 // the tile after this one
@@ -400,30 +410,30 @@ attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constan
                 }
                 const uint64_t stat = stat0 + ((k + 1) & 1u) * (kStatBytes >> 4);
                 wait(first && item >= 1 ? 3 : 2, &sh.p_full, k, &sh.ld_v, k, &sh.dv_free, item - 1);
-                issue_acc(tmem + kColDv, tmem + kColS, doc_mn, !first);
+                issue_acc(tmem + Cols::kDv, tmem + Cols::kS, doc_mn, !first);
                 commit(&sh.dv_done);
                 if (next) {
-                    wait(k >= 1 ? 2 : 1, &sh.ld_s, k + 1, &sh.dq_free, k - 1, &sh.ld_s, k + 1);
-                    issue_abt(tmem + kColS, k_km, qr_km, ones_s, stat);
+                    wait(!Cols::kOwnDq && k >= 1 ? 2 : 1, &sh.ld_s, k + 1, &sh.dq_free, k - 1, &sh.ld_s, k + 1);
+                    issue_abt(tmem + Cols::kS, k_km, qr_km, ones_s, stat);
                     commit(&sh.s_done);
                 }
                 wait(first && item >= 1 ? 3 : 2, &sh.ds_tmem, k, &sh.ld_k, k, &sh.dk_free, item - 1);
-                issue_acc(tmem + kColDk, tmem + kColDp, qc_mn, !first);
+                issue_acc(tmem + Cols::kDk, tmem + Cols::kDp, qc_mn, !first);
                 commit(&sh.dk_done);
                 if (next) {
                     wait1(&sh.ld_p, k + 1);
-                    issue_abt(tmem + kColDp, v_km, dor_km, ones_d, stat);
+                    issue_abt(tmem + Cols::kDp, v_km, dor_km, ones_d, stat);
                     commit(&sh.dp_done);
                 }
                 // the columns of dQ: S(k+1) has been read, which was issued after the drain of dQ(k-1); for the last tile
                 // that drain itself
-                if (next) wait(3, &sh.ds_smem, k, &sh.ds_recv, k, &sh.s_read, k + 1);
+                if (next && !Cols::kOwnDq) wait(3, &sh.ds_smem, k, &sh.ds_recv, k, &sh.s_read, k + 1);
                 else wait(k >= 1 ? 3 : 2, &sh.ds_smem, k, &sh.ds_recv, k, &sh.dq_free, k - 1);
                 if (leader) mbar_expect_tx(&sh.ds_recv, kBoxBytes);
 #pragma unroll
                 for (int ks = 0; ks < 16; ++ks)
                     if (leader)
-                        tc_mma_ss_pair(tmem + kColDq, ds_mn + (uint64_t)((ks * 2048) >> 4), kx_mn + (uint64_t)((ks * 2048) >> 4),
+                        tc_mma_ss_pair(tmem + Cols::kDq, ds_mn + (uint64_t)((ks * 2048) >> 4), kx_mn + (uint64_t)((ks * 2048) >> 4),
                                        idesc_dq, ks > 0);
                 commit(&sh.dq_done);
                 cur = next;
@@ -439,10 +449,10 @@ attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constan
         const int half = warp >> 2;                                  // which 64 query columns
         const int key_in_tile = (warp & 3) * 32 + lane;              // tensor-memory lane = key
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
-        const uint32_t st_tmem = tmem + lane_base + kColS + half * 64;
-        const uint32_t dp_tmem = tmem + lane_base + kColDp + half * 64;
-        const uint32_t pt_tmem = tmem + lane_base + kColS + half * 96;       // packed: columns 0-31 or 96-127
-        const uint32_t dst_tmem = tmem + lane_base + kColDp + half * 96;
+        const uint32_t st_tmem = tmem + lane_base + Cols::kS + half * 64;
+        const uint32_t dp_tmem = tmem + lane_base + Cols::kDp + half * 64;
+        const uint32_t pt_tmem = tmem + lane_base + Cols::kS + half * 96;       // packed: columns 0-31 or 96-127
+        const uint32_t dst_tmem = tmem + lane_base + Cols::kDp + half * 96;
         // dS^T of the queries whose dQ this CTA computes stays here, the other half goes to the partner
         const bool keep = half == (int)rank;
         uint8_t* ds_box = smem + (keep ? kOffDs + (int)rank * kBoxBytes : kOffSend);
@@ -539,10 +549,10 @@ attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constan
         // pair) and, after an item's last tile, its dV and dK: the stores wait for the way out of the SM, 5000 cycles per
         // item, which the compute warps cannot afford on short items and these can
         const int q_in_half = (warp & 1) * 32 + lane;
-        const int col0 = ((warp >> 1) & 1) * 64;
-        const int n_c4 = min(64, p.head_dim - col0) / 4;             // groups of four columns that hold data
+        const int col0 = ((warp >> 1) & 1) * (Cols::kW / 2);
+        const int n_c4 = min(Cols::kW / 2, p.head_dim - col0) / 4;             // groups of four columns that hold data
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
-        const uint32_t dq_tmem = tmem + lane_base + kColDq;
+        const uint32_t dq_tmem = tmem + lane_base + Cols::kDq;
         uint8_t* stage = smem + kOffStage + (warp & 3) * 2048;
         const uint32_t bar_free = at_leader(&sh.dq_free);
         uint32_t n_work = 0, k = 0;
@@ -555,28 +565,30 @@ attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constan
                 if (i == n_q - 1) {                      // dV is complete before the last dQ
                     mbar_wait_warp(&sh.dv_done, k & 1u, guard);
                     tc_fence_after();
-                    store_block(p.dv, p, stage, tmem + lane_base + kColDv, at_leader(&sh.dv_free), 1.0f, w.head, w.tok0 + key0, w.len - key0);
+                    store_block<Cols::kW>(p.dv, p, stage, tmem + lane_base + Cols::kDv, at_leader(&sh.dv_free), 1.0f, w.head, w.tok0 + key0, w.len - key0);
                 }
                 mbar_wait_warp(&sh.dq_done, k & 1u, guard);
                 tc_fence_after();
-                uint32_t acc[64];
+                uint32_t acc[Cols::kW / 2];
                 tmem_ld_x32(dq_tmem, *reinterpret_cast<uint32_t(*)[32]>(&acc[0]));
-                tmem_ld_x32(dq_tmem + 32, *reinterpret_cast<uint32_t(*)[32]>(&acc[32]));
+                if constexpr (Cols::kW == 128) tmem_ld_x32(dq_tmem + 32, *reinterpret_cast<uint32_t(*)[32]>(&acc[32]));
+                else tmem_ld_x16(dq_tmem + 32, *reinterpret_cast<uint32_t(*)[16]>(&acc[32]));
                 tmem_wait_ld();
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive_at(bar_free);
                 // the reductions go out half a tile later: sent at once they delay the exchange of the next dS^T, which the next
                 // dQ waits for (2 % of a tile's time on long sequences, 3 % on 256-token ones, although those send none; 500 ns had
-                // no effect).  One value for head dimensions 72 to 128 and any clock.
-                __nanosleep(900);
+                // no effect).  With columns of its own a dQ may leave later still, which pays on long sequences (one pause of 900 for
+                // all costs 2 to 3 % at 8000 tokens of 72; on short ones the longer pause holds the drain up: 256 tokens + 8 %).
+                __nanosleep(Cols::kOwnDq && w.len > 2048 ? 1344 : 900);
                 const int row_in_tile = (int)rank * 64 + q_in_half, qrow = i * kTile + row_in_tile;
                 const bool live = qrow < w.len;
                 if (w.len <= 2 * kTile) {
                     // the sequence's only key block: this is the whole dQ
                     __nv_bfloat16* out = p.dq + ((size_t)w.tok0 + qrow) * p.row_stride + w.head * p.head_dim + col0;
 #pragma unroll
-                    for (int c = 0; c < 8; ++c) {
+                    for (int c = 0; c < Cols::kW / 16; ++c) {
                         uint4 val;
                         val.x = pack_bf16x2(__uint_as_float(acc[c * 8 + 0]) * p.scale, __uint_as_float(acc[c * 8 + 1]) * p.scale);
                         val.y = pack_bf16x2(__uint_as_float(acc[c * 8 + 2]) * p.scale, __uint_as_float(acc[c * 8 + 3]) * p.scale);
@@ -588,14 +600,14 @@ attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constan
                     float* dst = p.dq_acc + (((size_t)w.tile0 + i) * p.n_heads + w.head) * (size_t)(kTile * 128) + row_in_tile * 4 +
                                  (col0 / 4) * (kTile * 4);
 #pragma unroll
-                    for (int c = 0; c < 16; ++c)
+                    for (int c = 0; c < Cols::kW / 8; ++c)
                         if (live && c < n_c4)
                             red_add_v4(dst + c * (kTile * 4), __uint_as_float(acc[c * 4]), __uint_as_float(acc[c * 4 + 1]),
                                        __uint_as_float(acc[c * 4 + 2]), __uint_as_float(acc[c * 4 + 3]));
                 }
             }
             // dK was issued before the last dQ
-            store_block(p.dk, p, stage, tmem + lane_base + kColDk, at_leader(&sh.dk_free), p.scale, w.head, w.tok0 + key0, w.len - key0);
+            store_block<Cols::kW>(p.dk, p, stage, tmem + lane_base + Cols::kDk, at_leader(&sh.dk_free), p.scale, w.head, w.tok0 + key0, w.len - key0);
         }
     }
 
