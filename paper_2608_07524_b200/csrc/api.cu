@@ -217,6 +217,16 @@ bool split_tiles(int32_t n_seqs, int32_t total_tokens, int32_t max_seqlen, int32
     return max_seqlen <= kTile || ((int64_t)n_seqs * n_heads >= 2 * n_sms && total_tokens <= (int64_t)n_seqs * 4 * kTile);
 }
 
+// Query rows of a forward work item.  Two tiles share each K and V load and keep the tensor pipe busy between them, but a
+// call is over when its longest chain of key tiles is, and a tile alone gets through one in 2250 cycles, two together in
+// 3280: items of one tile where every CTA has at most one of them.  Five requests of 24-995 tokens, 8 heads of 128: 22.2 ->
+// 20.0 us; four of 50-321, 3 heads of 72: 14.6 -> 13.6.  (The bound counts a partial tile for every sequence; the list itself
+// is only known on the device.)
+int fwd_rows_per_item(int32_t n_seqs, int32_t total_tokens, int32_t n_heads, int n_sms) {
+    const int64_t most = ((int64_t)total_tokens / kTile + n_seqs) * n_heads;
+    return most <= n_sms ? kTile : kFwdRowsPerItem;
+}
+
 // The kernels work on 64 or 128 columns per head; other head dimensions run zero-padded to the next of the two.
 size_t padded_dim(int32_t head_dim) { return head_dim <= 64 ? 64 : 128; }
 
@@ -293,9 +303,10 @@ static int attn_fwd_impl(const char* fn, bool merge, const void* q, const void* 
         return DCP_OK;
     }
     const bool input_order = g_input_order.load() != 0;
+    const int rows = fwd_rows_per_item(n_seqs, total_tokens, n_heads, dev.sm_count);
     {
         ScopedTimer t(DCP_KERNEL_PREP, stream);
-        e = launch_prep(cu_seqlens, n_seqs, total_tokens, max_seqlen, kFwdRowsPerItem, n_heads, sched, merge, bounds, UINT32_MAX,
+        e = launch_prep(cu_seqlens, n_seqs, total_tokens, max_seqlen, rows, n_heads, sched, merge, bounds, UINT32_MAX,
                         input_order, split ? kTile + 1 : INT32_MAX, max_seqlen <= kTile ? kTile : INT32_MAX, 0,
                         split && max_seqlen <= kTile, stream);
     }
@@ -326,7 +337,7 @@ static int attn_fwd_impl(const char* fn, bool merge, const void* q, const void* 
     {
         ScopedTimer t(DCP_KERNEL_FWD, stream);
         if (max_seqlen > kTile || !split) {
-            e = launch_attn_fwd(tq, tk, tv, to, p, head_dim, causal != 0, max_seqlen <= kShortItemMaxLen, dev.sm_count, stream);
+            e = launch_attn_fwd(tq, tk, tv, to, p, head_dim, causal != 0, max_seqlen <= kShortItemMaxLen, rows, dev.sm_count, stream);
             if (e != cudaSuccess) return fail(DCP_ERR_CUDA, "%s: attention kernel: %s", fn, cudaGetErrorString(e));
             g_launches.fetch_add(1);
         }

@@ -262,7 +262,10 @@ __device__ __noinline__ void store_whole_rows(FwdShared& sh, const CUtensorMap* 
 // KS = ceil(head_dim / 16) <= D / 16: the products skip the zero-padded columns, S sums over KS steps and O is 16 KS
 // columns wide (head_dim 72, the width of the paper's second model, does 5/8 of the padded work).  A template parameter:
 // with the count read at run time the MMA warp, which paces the pipe, lost more than the skipped steps save.
-template <int D, bool CAUSAL, bool EARLY_Q, int KS>
+// ROWS: query rows of an item, 256 or (calls with an item for a CTA at most) 128, where the second softmax group has nothing
+// to do.  Sharing the key tiles of the one Q tile between the groups and merging their sums was no faster: five short requests of
+// up to 995 tokens 22.0 us with two tiles to an item, 20.0 with one, 19.6 shared, but three of 18-391 13.6, 13.2 and 14.3.
+template <int D, bool CAUSAL, bool EARLY_Q, int KS, int ROWS>
 __global__ void __launch_bounds__(kFwdThreads, 1)
 attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k,
                 const __grid_constant__ CUtensorMap tmap_v, const __grid_constant__ CUtensorMap tmap_o,
@@ -331,14 +334,14 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             }
             item = __shfl_sync(0xffffffffu, item, 0);
             WorkItem w{0, -1, 0, 0, 0};
-            if (item < n_items) w = decode_item(p.sched, p.cu_seqlens, item, kFwdRowsPerItem, p.n_heads, gridDim.x, CAUSAL, CAUSAL, cur);
+            if (item < n_items) w = decode_item(p.sched, p.cu_seqlens, item, ROWS, p.n_heads, gridDim.x, CAUSAL, CAUSAL, cur);
             ++n_work;
             if (lane == 0) {
                 sh.work[slot] = w;
                 mbar_arrive(&sh.work_full[slot]);
 
-                const int r0 = w.blk * kFwdRowsPerItem;
-                const int nkv_t[2] = {kv_tiles_for<CAUSAL>(r0, w.len), kv_tiles_for<CAUSAL>(r0 + kTile, w.len)};
+                const int r0 = w.blk * ROWS;
+                const int nkv_t[2] = {kv_tiles_for<CAUSAL>(r0, w.len), ROWS > kTile ? kv_tiles_for<CAUSAL>(r0 + kTile, w.len) : 0};
                 const int nkv = nkv_t[0] > nkv_t[1] ? nkv_t[0] : nkv_t[1];
 #pragma unroll
                 for (int t = 0; t < 2; ++t) {
@@ -386,8 +389,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                 if (lane == 0) mbar_arrive(&sh.work_empty[slot]);
                 ++n_work;
                 if (w.len < 0) break;
-                const int r0 = w.blk * kFwdRowsPerItem;
-                const int nkv_t[2] = {kv_tiles_for<CAUSAL>(r0, w.len), kv_tiles_for<CAUSAL>(r0 + kTile, w.len)};
+                const int r0 = w.blk * ROWS;
+                const int nkv_t[2] = {kv_tiles_for<CAUSAL>(r0, w.len), ROWS > kTile ? kv_tiles_for<CAUSAL>(r0 + kTile, w.len) : 0};
                 const int nkv = nkv_t[0] > nkv_t[1] ? nkv_t[0] : nkv_t[1];
 
                 // S_t(0) for both tiles
@@ -491,8 +494,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                 }
                 continue;
             }
-            const int r_tile = w.blk * kFwdRowsPerItem + t * kTile;
-            const int nkv = kv_tiles_for<CAUSAL>(r_tile, w.len);
+            const int r_tile = w.blk * ROWS + t * kTile;
+            const int nkv = t * kTile < ROWS ? kv_tiles_for<CAUSAL>(r_tile, w.len) : 0;
             if (nkv == 0) continue;
             const int row = r_tile + row_in_tile;       // row inside the sequence (may be >= len)
 
@@ -639,30 +642,34 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
-template <int D, bool CAUSAL, bool EARLY_Q, int KS>
+template <int D, bool CAUSAL, bool EARLY_Q, int KS, int ROWS = kFwdRowsPerItem>
 static cudaError_t launch_one(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& to,
                               const FwdParams& p, int n_ctas, cudaStream_t stream) {
-    if (cudaError_t e = allow_smem<attn_fwd_kernel<D, CAUSAL, EARLY_Q, KS>>(FwdCfg<D>::kSmemBytes)) return e;
-    return launch_dependent(attn_fwd_kernel<D, CAUSAL, EARLY_Q, KS>, n_ctas, kFwdThreads, FwdCfg<D>::kSmemBytes, stream, tq, tk, tv,
+    if (cudaError_t e = allow_smem<attn_fwd_kernel<D, CAUSAL, EARLY_Q, KS, ROWS>>(FwdCfg<D>::kSmemBytes)) return e;
+    return launch_dependent(attn_fwd_kernel<D, CAUSAL, EARLY_Q, KS, ROWS>, n_ctas, kFwdThreads, FwdCfg<D>::kSmemBytes, stream, tq, tk, tv,
                             to, p);
 }
 
 template <int D, int KS>
 static cudaError_t launch_masked(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& to,
-                                 const FwdParams& p, bool causal, bool short_items, int n_ctas, cudaStream_t stream) {
+                                 const FwdParams& p, bool causal, bool short_items, int rows, int n_ctas, cudaStream_t stream) {
+    if (rows == kTile)
+        return causal ? launch_one<D, true, true, KS, kTile>(tq, tk, tv, to, p, n_ctas, stream)
+                      : launch_one<D, false, true, KS, kTile>(tq, tk, tv, to, p, n_ctas, stream);
     if (causal) return launch_one<D, true, true, KS>(tq, tk, tv, to, p, n_ctas, stream);
     return short_items ? launch_one<D, false, true, KS>(tq, tk, tv, to, p, n_ctas, stream)
                        : launch_one<D, false, false, KS>(tq, tk, tv, to, p, n_ctas, stream);
 }
 
 cudaError_t launch_attn_fwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& to,
-                            const FwdParams& p, int head_dim, bool causal, bool short_items, int n_ctas, cudaStream_t stream) {
+                            const FwdParams& p, int head_dim, bool causal, bool short_items, int rows, int n_ctas,
+                            cudaStream_t stream) {
     switch (head_dim <= 64 ? 4 : (head_dim + 15) / 16) {
-        case 4: return launch_masked<64, 4>(tq, tk, tv, to, p, causal, short_items, n_ctas, stream);
-        case 5: return launch_masked<128, 5>(tq, tk, tv, to, p, causal, short_items, n_ctas, stream);
-        case 6: return launch_masked<128, 6>(tq, tk, tv, to, p, causal, short_items, n_ctas, stream);
-        case 7: return launch_masked<128, 7>(tq, tk, tv, to, p, causal, short_items, n_ctas, stream);
-        default: return launch_masked<128, 8>(tq, tk, tv, to, p, causal, short_items, n_ctas, stream);
+        case 4: return launch_masked<64, 4>(tq, tk, tv, to, p, causal, short_items, rows, n_ctas, stream);
+        case 5: return launch_masked<128, 5>(tq, tk, tv, to, p, causal, short_items, rows, n_ctas, stream);
+        case 6: return launch_masked<128, 6>(tq, tk, tv, to, p, causal, short_items, rows, n_ctas, stream);
+        case 7: return launch_masked<128, 7>(tq, tk, tv, to, p, causal, short_items, rows, n_ctas, stream);
+        default: return launch_masked<128, 8>(tq, tk, tv, to, p, causal, short_items, rows, n_ctas, stream);
     }
 }
 

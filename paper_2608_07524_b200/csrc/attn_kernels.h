@@ -97,9 +97,11 @@ cudaError_t launch_copy_segments(const void* src, void* dst, const int32_t* seg,
 
 // short_items: no sequence of the batch is longer than a few dozen tiles, so work items are short and the
 // variant that releases Q slots early pays (under a causal mask it always does).
+// rows: query rows of an item of the list, kFwdRowsPerItem or one tile.
 // `to` = a map over o with boxes of 32 rows: what a softmax warp stores.
 cudaError_t launch_attn_fwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& to,
-                            const FwdParams& p, int head_dim, bool causal, bool short_items, int n_ctas, cudaStream_t stream);
+                            const FwdParams& p, int head_dim, bool causal, bool short_items, int rows, int n_ctas,
+                            cudaStream_t stream);
 
 // Tile-aligned row statistics for the backward kernel (see BwdParams::stats) and dq_acc = 0.  Sequences of at most
 // direct_len tokens get their dQ written by the main kernel: here and in the post kernel they have no accumulator.
