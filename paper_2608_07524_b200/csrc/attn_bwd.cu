@@ -46,6 +46,8 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "attn_kernels.h"
 #include "launch.h"
 #include "sched.cuh"
@@ -477,29 +479,36 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                     tmem_ld_x32(st_tmem, *reinterpret_cast<uint32_t(*)[32]>(&sr[0]));
                     tmem_ld_x32(st_tmem + 32, *reinterpret_cast<uint32_t(*)[32]>(&sr[32]));
                     tmem_wait_ld();
+                    // the key is seen by the queries from `lo` of this thread's 64 on
+                    const int lo = !key_valid ? 64 : diag ? key - (i * kTile + half * 64) : -64;
+                    auto form_p = [&](auto masked) {
 #pragma unroll
-                    for (int c = 0; c < 2; ++c) {
-                        // 32 query columns at a time: the dV product starts on the first chunk while the
-                        // second is still being exponentiated
+                        for (int c = 0; c < 2; ++c) {
+                            // 32 query columns at a time: the dV product starts on the first chunk while the
+                            // second is still being exponentiated
 #pragma unroll
-                        for (int e = 0; e < 32; ++e) pf[c * 32 + e] = fast_exp2(__uint_as_float(sr[c * 32 + e]) * p.scale_log2);
-                        if (key_tail || diag) {
-                            const int q_first = i * kTile + half * 64 + c * 32;   // query index of element 0
+                            for (int e = 0; e < 32; ++e) pf[c * 32 + e] = fast_exp2(__uint_as_float(sr[c * 32 + e]) * p.scale_log2);
+                            if constexpr (decltype(masked)::value) {
 #pragma unroll
-                            for (int e = 0; e < 32; ++e)
-                                if (!key_valid || (diag && key > q_first + e)) pf[c * 32 + e] = 0.f;
+                                for (int e = 0; e < 32; ++e) pf[c * 32 + e] = c * 32 + e >= lo ? pf[c * 32 + e] : 0.f;
+                            }
+                            uint32_t pk[16];
+#pragma unroll
+                            for (int e = 0; e < 16; ++e) pk[e] = pack_bf16x2(pf[c * 32 + 2 * e], pf[c * 32 + 2 * e + 1]);
+                            tmem_st_x16(pt_tmem + c * 16, pk);
+                            if (c == 0) {
+                                tmem_wait_st();
+                                tc_fence_before();
+                                __syncwarp();
+                                if (lane == 0) mbar_arrive(&sh.p_half);
+                            }
                         }
-                        uint32_t pk[16];
-#pragma unroll
-                        for (int e = 0; e < 16; ++e) pk[e] = pack_bf16x2(pf[c * 32 + 2 * e], pf[c * 32 + 2 * e + 1]);
-                        tmem_st_x16(pt_tmem + c * 16, pk);
-                        if (c == 0) {
-                            tmem_wait_st();
-                            tc_fence_before();
-                            __syncwarp();
-                            if (lane == 0) mbar_arrive(&sh.p_half);
-                        }
-                    }
+                    };
+                    // Masked tiles have a copy of the loop, with one select per element (before: a test of (key_valid, diag, key >
+                    // query) on every element, in the one loop).  65536 tokens, 16 heads of 64: causal 300-token sequences 435 ->
+                    // 408 us, 1200 736 -> 708, 4096 1802 -> 1768; without a causal mask 1200 1201 -> 1190, 4096 3352 -> 3295.
+                    if (key_tail || diag) form_p(std::true_type{});
+                    else form_p(std::false_type{});
                 }
                 tmem_wait_st();
                 tc_fence_before();
