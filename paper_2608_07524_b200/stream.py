@@ -8,12 +8,14 @@ that batch's data):
                                forward again if its recompute count > 0 (activation recomputation
                                re-runs the layer's forward before its backward, Section 3.4);
                                backward; scatter o, lse, dq, dk, dv back to the batch's order.
-A plan with a single micro-batch runs in place, without copies.  All arithmetic happens in libdcp;
+A plan with a single micro-batch runs in place, without copies, and a micro-batch of sequences that are neighbours in the
+batch with those of lse only.  All arithmetic happens in libdcp;
 this module only owns buffers and issues calls.
 """
 from __future__ import annotations
 
 from dataclasses import dataclass, field
+from types import SimpleNamespace
 from typing import List, Optional, Sequence
 
 import numpy as np
@@ -89,7 +91,9 @@ def plan_length_group(n_seqs: int, seq_len: int, batch_size: int, recompute: int
 class _Buffers:
     """q, k, v, dO, o, dq, dk, dv [tokens, H, d] bf16 and lse [H * tokens] fp32 on the device."""
 
-    def __init__(self, tokens, n_heads, head_dim, device, value_seed=None):
+    ROWS = ("q", "k", "v", "g", "o", "dq", "dk", "dv")
+
+    def __init__(self, tokens, n_heads, head_dim, device, value_seed=None, lse=None):
         import torch
         from . import inputs
         if value_seed is None:
@@ -98,7 +102,7 @@ class _Buffers:
         else:
             self.q, self.k, self.v, self.g = inputs.make_qkvg_device(tokens, n_heads, head_dim, value_seed, device)
         self.o, self.dq, self.dk, self.dv = (torch.empty_like(self.q) for _ in range(4))
-        self.lse = torch.empty(n_heads * tokens, dtype=torch.float32, device=device)
+        self.lse = torch.empty(n_heads * tokens, dtype=torch.float32, device=device) if lse is None else lse
 
 
 class StreamRunner:
@@ -118,6 +122,7 @@ class StreamRunner:
         self.max_tokens, self.max_seqs = max_tokens, max_seqs
         self.batch = _Buffers(max_tokens, n_heads, head_dim, device, value_seed)
         self.stage: Optional[_Buffers] = None
+        self.stage_lse = None
         # the single-batch benchmarks address the batch buffers directly
         self.q, self.k, self.v, self.g = self.batch.q, self.batch.k, self.batch.v, self.batch.g
         self.o, self.dq, self.dk, self.dv, self.lse = self.batch.o, self.batch.dq, self.batch.dk, self.batch.dv, self.batch.lse
@@ -186,17 +191,28 @@ class StreamRunner:
         if mb.seg is None:
             self._attention(self.batch, cu_dev, T, max_len, mb.recompute)
             return T
-        if self.stage is None:
-            self.stage = _Buffers(self.max_tokens, self.H, self.d, self.device)
-        b, s = self.batch, self.stage
-        row_bytes = self.H * self.d * 2
-        for src, dst in ((b.q, s.q), (b.k, s.k), (b.v, s.v), (b.g, s.g)):
-            binding.dcp_copy_segments(src, dst, seg_dev, n_seg, row_bytes)
-        self._attention(s, cu_dev, T, max_len, mb.recompute)
-        for dst, src in ((b.o, s.o), (b.dq, s.dq), (b.dk, s.dk), (b.dv, s.dv)):
-            binding.dcp_copy_segments(src, dst, seg_dev, n_seg, row_bytes, reverse=True)
+        b = self.batch
+        if self.stage_lse is None:
+            self.stage_lse = self.torch.empty_like(b.lse)
+        if T and mb.seq_index is not None and bool((np.diff(mb.seq_index) == 1).all()):
+            # sequences that lie side by side in the batch (the longest, alone in its micro-batch, above all) run where they
+            # are: only lse, whose planes are as long as the call's tokens, is moved.  12 clips split into 28800 | 14400, 9600 |
+            # the rest: 0.8 ms of copies in a step of 34 become 0.5
+            row0 = int(mb.seg[0, 0])
+            view = SimpleNamespace(lse=self.stage_lse, **{n: getattr(b, n)[row0:row0 + T] for n in _Buffers.ROWS})
+            self._attention(view, cu_dev, T, max_len, mb.recompute)
+        else:
+            if self.stage is None:
+                self.stage = _Buffers(self.max_tokens, self.H, self.d, self.device, lse=self.stage_lse)
+            s = self.stage
+            row_bytes = self.H * self.d * 2
+            for src, dst in ((b.q, s.q), (b.k, s.k), (b.v, s.v), (b.g, s.g)):
+                binding.dcp_copy_segments(src, dst, seg_dev, n_seg, row_bytes)
+            self._attention(s, cu_dev, T, max_len, mb.recompute)
+            for dst, src in ((b.o, s.o), (b.dq, s.dq), (b.dk, s.dk), (b.dv, s.dv)):
+                binding.dcp_copy_segments(src, dst, seg_dev, n_seg, row_bytes, reverse=True)
         Tb = int(batch_tokens)
-        binding.dcp_copy_segments(s.lse, b.lse, seg_dev, n_seg, 4, reverse=True, n_planes=self.H,
+        binding.dcp_copy_segments(self.stage_lse, b.lse, seg_dev, n_seg, 4, reverse=True, n_planes=self.H,
                                   src_plane_bytes=4 * T, dst_plane_bytes=4 * Tb)
         return T
 
