@@ -125,6 +125,15 @@ int device_info(DeviceInfo* out) {
     return DCP_OK;
 }
 
+// How much of memory a tile's request makes L2 fetch around it.  256 bytes, except where heads start in the middle of a
+// 32-byte sector and a box of 64 columns ends well past its head (head dimensions 8, 24, 40, 72, 88, 104): there the larger
+// fetch costs the forward of single-tile items a tenth to a quarter (65536 tokens, 16 heads, us with 256 and with 128 bytes:
+// sequences of 60 tokens of 72 234 and 194, of 40 175 and 133, of 88 276 and 222; of 128 tokens of 72 134 and 126) and changes
+// nothing elsewhere.  128 bytes for all would cost the backward of 80 and 96 3 %, of 56 2 %; 64, 96 and 128 forward do not care.
+CUtensorMapL2promotion l2_promotion(int32_t head_dim) {
+    return head_dim % 16 != 0 && head_dim % 64 <= 40 ? CU_TENSOR_MAP_L2_PROMOTION_L2_128B : CU_TENSOR_MAP_L2_PROMOTION_L2_256B;
+}
+
 // [T, H, d] bf16 viewed as a 3-D tensor (d, H, T); a box is 64 columns x 1 head x 128 tokens,
 // written to shared memory as 128 rows of 128 bytes with the 128-byte swizzle.  Rows past T are
 // zero-filled.  Consecutive tokens are row_stride elements apart (n_heads * head_dim when the tensor is
@@ -139,7 +148,7 @@ int make_map(CUtensorMap* map, const void* base, int32_t total_tokens, int32_t n
     const cuuint32_t elem_strides[3] = {1, 1, 1};
     const CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box,
                            elem_strides, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                           CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+                           l2_promotion(head_dim), CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return fail(DCP_ERR_CUDA, "cuTensorMapEncodeTiled failed with CUresult %d", (int)r);
     return DCP_OK;
 }
