@@ -600,10 +600,11 @@ attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constan
                 __syncwarp();
                 if (lane == 0) mbar_arrive_at(bar_free);
                 // the reductions go out half a tile later: sent at once they delay the exchange of the next dS^T, which the next
-                // dQ waits for (2 % of a tile's time on long sequences, 3 % on 256-token ones, although those send none; 500 ns had
-                // no effect).  With columns of its own a dQ may leave later still, which pays on long sequences (one pause of 900 for
+                // dQ waits for (2 % of a tile's time on long sequences; 500 ns had no effect).  An item that writes its dQ directly
+                // sends none, and without the pause its dK is out sooner (65536 tokens, 16 heads of 128: sequences of 200 tokens
+                // 597 -> 578 us, 256: 494 -> 478, causal 598 -> 576; up to 96 columns no difference).  With columns of its own a dQ may leave later still, which pays on long sequences (one pause of 900 for
                 // all costs 2 to 3 % at 8000 tokens of 72; on short ones the longer pause holds the drain up: 256 tokens + 8 %).
-                __nanosleep(Cols::kOwnDq && w.len > 2048 ? 1344 : 900);
+                if (Cols::kOwnDq || w.len > 2 * kTile) __nanosleep(Cols::kOwnDq && w.len > 2048 ? 1344 : 900);
                 const int row_in_tile = (int)rank * 64 + q_in_half, qrow = i * kTile + row_in_tile;
                 const bool live = qrow < w.len;
                 if (w.len <= 2 * kTile) {
