@@ -429,9 +429,10 @@ struct BlockList {
 // memory layout (8x8 core matrices; column halves 2048 bytes apart) and is 4 KB-aligned, so one bulk
 // copy fetches it.  Also zeroes the fp32 dQ accumulator blocks of sequences longer than direct_len, one key block of the main
 // kernel (shorter ones get their dQ written directly by it), the columns that hold data.  HBM-bound.  Zeroing behind a
-// pass's loads and head_dim's columns instead of D (us before and after, 65536 tokens x 16 heads): 72 columns 193 -> 161,
-// 128 columns 212 -> 205; text batch 251 -> 244, 2-D model's spatial axis 386 -> 378.
-constexpr int kPreCtas = 4;      // per SM: 64 registers a thread
+// pass's loads, head_dim's columns instead of D, and the loads in flight below (us before and after, 65536 tokens x 16 heads): 64
+// columns 109 -> 97, 72 columns 193 -> 139, 128 columns 212 -> 186 (5.9 TB/s); text batch 251 -> 227, 2-D model's spatial axis
+// 386 -> 353, of 72 370 -> 267.
+constexpr int kPreCtas = 6;      // per SM: 40 registers a thread
 template <int D>
 __global__ void __launch_bounds__(256, kPreCtas) bwd_pre_kernel(const __nv_bfloat16* __restrict__ o,
                                                       const __nv_bfloat16* __restrict__ d_o, const float* __restrict__ lse,
@@ -454,17 +455,16 @@ __global__ void __launch_bounds__(256, kPreCtas) bwd_pre_kernel(const __nv_bfloa
         // its whole dQ and writes it directly).  The main kernel adds to no other rows or columns than these.
         float4* acc_blk = reinterpret_cast<float4*>(dq_acc) + (size_t)blk * (kTile * D / 4);
         const bool zero = len > direct_len && (size_t)(blk + 1) * (kTile * D / 4) <= dq_acc_vec4;
-        if (D == 64 && zero)
-            for (int e = threadIdx.x; e < kTile * D / 4; e += blockDim.x)
-                if (e % kTile < len - row0 && e / kTile * 4 < head_dim) acc_blk[e] = make_float4(0.f, 0.f, 0.f, 0.f);
         {
         uint8_t* out = reinterpret_cast<uint8_t*>(stats) + ((size_t)t * n_heads + h) * kTermTileBytes;
         // Half a warp reads a row with 16-byte loads (D = 128; a quarter warp for D = 64), so that a warp
-        // instruction covers 2 (4) rows; a warp takes 16 rows per pass with eight loads of 16 bytes in flight per
-        // lane (the kernel waits on HBM latency: bytes in flight are what it runs on).
+        // instruction covers 2 (4) rows; a warp takes 4 (8) rows per pass with four loads of 16 bytes in flight per
+        // lane.  The kernel waits on HBM latency: bytes in flight are what it runs on, and six CTAs of 40 registers have more
+        // of them than four of 64 with twice the loads per lane (eight loads, four CTAs: 7 to 14 % slower; 16, two: 38 %;
+        // two, eight: 7 %).
         constexpr int kLanesPerRow = D / 8;                 // 16 or 8
         constexpr int kRowsPerInst = 32 / kLanesPerRow;     // 2 or 4
-        constexpr int kU = 4;                               // row groups in flight per lane
+        constexpr int kU = 2;                               // row groups in flight per lane
         const int sub = lane / kLanesPerRow, col = (lane % kLanesPerRow) * 8;
         const bool lane_live = col < head_dim;
         const int lane_col = lane_live ? col : 0;
@@ -488,9 +488,9 @@ __global__ void __launch_bounds__(256, kPreCtas) bwd_pre_kernel(const __nv_bfloa
                     if (lane % kLanesPerRow == 0) nl[u] = -lse[(size_t)h * total_tokens + tok] * inv_scale;
                 }
             }
-            // Behind the loads, which would queue behind these stores.  (At 64 columns a block is one pass, and this order is
-            // 1 to 2 % slower than zeroing first.  Unrolled, the loop costs registers, and with them resident CTAs: + 70 %.)
-            if (D == 128 && zero) {
+            // Behind the loads, which would queue behind these stores.  (Unrolled, the loop costs registers, and with them
+            // resident CTAs: + 70 %.)
+            if (zero) {
                 constexpr int kPer = 8 * kRowsPerInst * kU * D / 4;
                 const int z0 = (r0 - warp * kRowsPerInst * kU) * D / 4;
                 for (int e = z0 + threadIdx.x; e < z0 + kPer; e += blockDim.x)
