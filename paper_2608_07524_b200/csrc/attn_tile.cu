@@ -535,6 +535,8 @@ tile_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                     tmem_ld_x32(my + Cfg::kColDp + c * 32, dp);
                     tmem_wait_ld();
                     const uint32_t bits = chunk_bits(lo, hi, c);
+                    // Of 64 columns every element is exponentiated and the mask selects afterwards: no branch around the
+                    // exponential (- 1 to - 3 %; of 128 columns, one CTA per SM, + 0 to 1 %: there the mask comes first).
 #pragma unroll
                     for (int v4 = 0; v4 < 4; ++v4) {
                         uint32_t pk[4], ds[4];
@@ -543,8 +545,12 @@ tile_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                             const int j = v4 * 8 + 2 * e;
                             float x0, x1;
                             unpack_f32x2(mul_f32x2(pack_f32x2(__uint_as_float(s[j]), __uint_as_float(s[j + 1])), sc2), x0, x1);
-                            const float p0 = bits & (1u << j) ? fast_exp2(x0) : 0.f;
-                            const float p1 = bits & (2u << j) ? fast_exp2(x1) : 0.f;
+                            if constexpr (D == 64) {
+                                x0 = fast_exp2(x0);
+                                x1 = fast_exp2(x1);
+                            }
+                            const float p0 = bits & (1u << j) ? (D == 64 ? x0 : fast_exp2(x0)) : 0.f;
+                            const float p1 = bits & (2u << j) ? (D == 64 ? x1 : fast_exp2(x1)) : 0.f;
                             pk[e] = pack_bf16x2(p0, p1);
                             ds[e] = pack_bf16x2(p0 * __uint_as_float(dp[j]), p1 * __uint_as_float(dp[j + 1]));
                         }
