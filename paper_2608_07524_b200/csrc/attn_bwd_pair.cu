@@ -154,8 +154,12 @@ __device__ __forceinline__ void store_block(__nv_bfloat16* out, const BwdParams&
 
 // KS = ceil(head_dim / 16), the steps S and dP sum over (5 to 8; a template parameter, because a step count that the issuing
 // warp reads at run time costs it 650 of 4500 cycles per tile, more than the skipped steps save).  dV, dK and dQ have 96 or
-// 128 columns (PairCols).  S(k+1) overwrites the P^T that dV(k) reads, and dP(k+1) the dS^T that dK(k) reads: the pipe runs the
-// products of one issuing thread in order, as the forward's S after O += P V relies on too.
+// 128 columns (PairCols).  S(k+1) overwrites the P^T that dV(k) reads, and dP(k+1) the dS^T that dK(k) reads.  With 128 columns
+// these products have one shape (256 x 128), and the pipe has always run them in the order of their issue.  Of 256 x 96 and 256 x
+// 128 nothing says so (the PTX ISA does of one accumulator and shape), so there the one waits until the other has completed.
+// S(k+1) is ready long before it is read, so that this costs little (backward, 65536 tokens x 16 heads of 72, us without and with
+// the waits: 256 tokens 476 and 474, causal 300 907 and 919, 1200 1689 and 1704, causal 1217 and 1228, 16384 16039 and 16120,
+// causal 8601 and 8634; of 88 and 96 - 3 to + 1 %).
 template <bool CAUSAL, int KS>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
 attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constant__ BwdParams p) {
@@ -415,7 +419,9 @@ attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constan
                 issue_acc(tmem + Cols::kDv, tmem + Cols::kS, doc_mn, !first);
                 commit(&sh.dv_done);
                 if (next) {
-                    wait(!Cols::kOwnDq && k >= 1 ? 2 : 1, &sh.ld_s, k + 1, &sh.dq_free, k - 1, &sh.ld_s, k + 1);
+                    // until its columns are free: of the P^T that dV(k) reads (a product of another shape), or of dQ(k-1)
+                    if (Cols::kOwnDq) wait(2, &sh.ld_s, k + 1, &sh.dv_done, k, &sh.ld_s, k + 1);
+                    else wait(k >= 1 ? 2 : 1, &sh.ld_s, k + 1, &sh.dq_free, k - 1, &sh.ld_s, k + 1);
                     issue_abt(tmem + Cols::kS, k_km, qr_km, ones_s, stat);
                     commit(&sh.s_done);
                 }
@@ -423,7 +429,7 @@ attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constan
                 issue_acc(tmem + Cols::kDk, tmem + Cols::kDp, qc_mn, !first);
                 commit(&sh.dk_done);
                 if (next) {
-                    wait1(&sh.ld_p, k + 1);
+                    wait(Cols::kOwnDq ? 2 : 1, &sh.ld_p, k + 1, &sh.dk_done, k, &sh.ld_p, k + 1);   // (dK(k) reads dS^T)
                     issue_abt(tmem + Cols::kDp, v_km, dor_km, ones_d, stat);
                     commit(&sh.dp_done);
                 }

@@ -406,6 +406,39 @@ def test_backward_around_one_pair_item(d, longest):
     check_full(lengths, 3, d, True, seed=500 + d)
 
 
+@pytest.mark.parametrize("causal", [False, True])
+@pytest.mark.parametrize("d", [40, 64, 72, 80, 88, 96])
+def test_backward_of_many_items_per_cta(d, causal):
+    """Several items of up to 15 Q tiles for every CTA or pair, one after the other through the same columns and buffers: close
+    to the oracle row by row, and dV and dK, which no atomics add up, the same bits in every run."""
+    lengths, H, dev = [129, 1900, 700, 257, 512, 1025, 383, 255, 1300, 130, 256], 16, "cuda"
+    cu = np.concatenate([[0], np.cumsum(lengths)]).astype(np.int32)
+    q, k, v, g = inputs.make_qkvg(int(cu[-1]), H, d, 600 + d)
+    o, lse, dq, dk, dv = run_gpu(q, k, v, g, cu, causal)
+    ref = oracle.attn_bwd(q, k, v, g, cu, causal)
+    # D is formed from o in bf16, off by 2^-8 |dO_i| |o_i| at most, which reaches dQ_i as that times scale sum_j P_ij k_j and dK_j
+    # as sum_i P_ij of it times scale q_i: much of a gradient where a query sees few keys.  The oracle's dV forms that last sum
+    # in one column, and in the others, of |g|, what dV is a sum of.
+    norm = lambda x: np.linalg.norm(to64(x), axis=2)
+    off = 2.0 ** -8 * norm(g) * norm(o) * d ** -0.5
+    terms = g.abs()
+    terms[:, :, -1] = torch.tensor(off * norm(q))
+    bound = oracle.attn_bwd(q, k, v, terms, cu, causal)[2]
+    for name, got, want, more in zip(("dq", "dk", "dv"), (dq, dk, dv), ref, (off * norm(k).max(), 1.01 * bound[:, :, -1], 0.0)):
+        assert_close(name, got, want)
+        err, row = np.linalg.norm(to64(got) - want, axis=2), np.linalg.norm(want, axis=2)
+        # P, dS and the results are rounded to bf16, 2^-8 of each term and of the sum at most and 2^-9 on average: a fifth of what
+        # is allowed here, where one wrong tile of the row's fifteen would be a quarter
+        assert np.all(err <= 2e-2 * row + 1e-2 * np.sqrt(np.mean(row ** 2)) + more), name
+    # dV = P^T dO: P is rounded (2^-8) and so is the sum; the exponentials and lse add less than 2^-11
+    assert np.all((np.abs(to64(dv) - ref[2]) <= (2.0 ** -7 + 2.0 ** -10) * bound)[:, :, :-1])
+    qd, kd, vd, gd = (x.to(dev) for x in (q, k, v, g))
+    cud = torch.tensor(cu, device=dev)
+    for _ in range(10):
+        _, dk2, dv2 = B.dcp_varlen_attn_bwd(qd, kd, vd, o, gd, lse, cud, max(lengths), causal)
+        assert torch.equal(dk, dk2) and torch.equal(dv, dv2)
+
+
 def test_a_sequence_longer_than_a_declared_pair_item_is_refused():
     # max_seqlen <= 256 promises that no dQ needs the accumulator, whose kernels are then not launched
     dev = "cuda"

@@ -64,3 +64,15 @@ def test_loads_after_a_rows_own_stores_follow_a_barrier():
             before_load, after_stores = loop[:loop.index("tmem_ld_x32")], text[close:].split("\n")[2]
             assert "__syncwarp();" in before_load + after_stores, f"{fn}: line {text[:m.start()].count(chr(10)) + 2}"
     assert n == 3
+
+
+def test_a_product_of_another_shape_waits_for_the_one_that_reads_what_it_overwrites():
+    """The pair backward up to 96 columns: S (256 x 128) overwrites the P^T that dV (256 x 96) reads, dP the dS^T that dK reads,
+    and only products of one shape are known to be ordered among themselves."""
+    with open(os.path.join(CSRC, "attn_bwd_pair.cu")) as f:
+        text = re.sub(r"//[^\n]*", "", f.read())
+    loop = text[text.index("while (cur) {"):]
+    for overwrites, reader in (("kS", "dv_done"), ("kDp", "dk_done")):
+        end = loop.index(f"issue_abt(tmem + Cols::{overwrites},")
+        before = loop[loop.rindex("commit(", 0, end):end]
+        assert re.search(rf"kOwnDq\) wait\(2, .*&sh\.{reader}, k,|wait\(Cols::kOwnDq \? 2 : 1, .*&sh\.{reader}, k,", before), overwrites
