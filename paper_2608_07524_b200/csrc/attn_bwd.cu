@@ -79,9 +79,9 @@ struct BwdCfg {
     static constexpr int kOffV = kTileBytes;
     static constexpr int kQStages = 2;                     // Q is needed early (S^T) and late (dK)
     // K and V have two slots: the next item's (and, behind them in the producer's order, its first Q, terms and dO) load
-    // while this item still runs; with one slot they waited for its last product, a load latency per item.  65536 tokens,
-    // 16 heads of 64: 150 tokens 477 -> 469 us, causal 443 -> 426; 256 337 -> 329; 300 489 -> 478; 4096 - 1 to 0 %; of 40: 256
-    // 394 -> 360, causal 341 -> 311, causal 16384 + 1 to 3 %.
+    // while this item still runs; with one slot they waited for its last product, a load latency per item.  Backward, 65536
+    // tokens, 16 heads, us with one slot and with two: of 64 150 tokens 738 and 730, causal 693 and 672, 256 556 and 549, 300 735
+    // and 726; of 40 256 548 and 509, causal 495 and 467; causal 16384 of 40, 56 and 64 within 0.5 %.
     static constexpr int kKvBytes = 2 * kTileBytes;
     static constexpr int kOffQ = 2 * kKvBytes;
     static constexpr int kOffDo = (4 + kQStages) * kTileBytes;          // dO lives only from dP^T to dV: one stage
@@ -644,6 +644,9 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                     if ((warp & 3) > 0) __nanosleep((warp & 3) * kRedStaggerNs + 64);
 #pragma unroll
                     for (int c = 0; c < kD / 4; ++c) {
+                        // only the columns that hold data are zeroed before and read afterwards (all 64 for head dimension 40: 1200
+                        // tokens 1372 -> 1299 us, causal 16384 7523 -> 6533; 56 7588 -> 7217; 64 unchanged)
+                        if (c * 4 >= p.head_dim) break;
                         if (live) red_add_v4(dst + c * (kTile * 4), __uint_as_float(acc[c * 4]), __uint_as_float(acc[c * 4 + 1]),
                                    __uint_as_float(acc[c * 4 + 2]), __uint_as_float(acc[c * 4 + 3]));
                         if ((c % kRedGroup) == kRedGroup - 1) __nanosleep(kRedSleepNs);

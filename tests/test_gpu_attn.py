@@ -439,6 +439,28 @@ def test_backward_of_many_items_per_cta(d, causal):
         assert torch.equal(dk, dk2) and torch.equal(dv, dv2)
 
 
+@pytest.mark.parametrize("d", [8, 40, 56, 72, 96])
+def test_the_accumulator_holds_the_columns_and_rows_that_are_zeroed(d):
+    """The fp32 accumulator of dQ is tiles of 64 or 128 columns.  Of a smaller head dimension only its columns are zeroed, added
+    to and read: an addition to any other word would turn this NaN into the canonical one."""
+    lengths, H, dev, poison = [300, 340], 3, "cuda", 0x7FA5A5A5
+    T = sum(lengths)
+    cu = torch.tensor([0, 300, 640], dtype=torch.int32, device=dev)
+    q, k, v, g = (x.to(dev) for x in inputs.make_qkvg(T, H, d, 21))
+    o, lse = B.dcp_varlen_attn_fwd(q, k, v, cu, 340, False)
+    sizes = {x: B.dcp_varlen_attn_workspace(T, 2, H, x)[1] for x in (64, 128)}
+    tiles = (sizes[128] - sizes[64]) // (H * 128 * 64 * 4)            # the accumulator is what depends on the columns, and comes last
+    cols = 64 if d <= 64 else 128
+    ws = torch.full((sizes[cols] // 4,), poison, dtype=torch.int32, device=dev)
+    dq, _, _ = B.dcp_varlen_attn_bwd(q, k, v, o, g, lse, cu, 340, False, workspace=ws.view(torch.uint8))
+    B.dcp_query_status(ws.view(torch.uint8))
+    assert bool(torch.isfinite(dq).all())
+    acc = ws[-tiles * H * 128 * cols:].view(tiles, H, cols // 4, 128, 4)
+    assert bool((acc[:6, :, : d // 4, :44] != poison).all())          # three tiles each; the last has 44 and 84 rows
+    assert bool((acc[:, :, d // 4:] == poison).all())
+    assert bool((acc[2, :, :, 44:] == poison).all()) and bool((acc[5, :, :, 84:] == poison).all()) and bool((acc[6:] == poison).all())
+
+
 def test_a_sequence_longer_than_a_declared_pair_item_is_refused():
     # max_seqlen <= 256 promises that no dQ needs the accumulator, whose kernels are then not launched
     dev = "cuda"
