@@ -92,8 +92,9 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, c
     return got;
 }
 
-// The same for a converged warp whose lanes may wait on different barriers: all lanes leave the loop together.
-__device__ __forceinline__ bool mbar_wait_all(uint64_t* bar, uint32_t parity, const WaitGuard& g) {
+// The same for a converged warp whose lanes may wait on different barriers: all lanes leave the loop together, and the barrier
+// behind it makes what one lane has acquired the others' (a vote does not order memory).
+__device__ __forceinline__ bool mbar_poll_all(uint64_t* bar, uint32_t parity, const WaitGuard& g) {
     for (uint32_t spin = 0; spin < kSpinLimit; ++spin) {
         if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
         if ((spin & 1023u) == 1023u && __any_sync(0xffffffffu, *g.abort_flag != 0u)) return false;
@@ -101,6 +102,11 @@ __device__ __forceinline__ bool mbar_wait_all(uint64_t* bar, uint32_t parity, co
     *g.abort_flag = 1u;
     if (g.status) atomicMax(g.status, (uint32_t)kStatusWaitTimeout);
     return false;
+}
+__device__ __forceinline__ bool mbar_wait_all(uint64_t* bar, uint32_t parity, const WaitGuard& g) {
+    const bool got = mbar_poll_all(bar, parity, g);
+    __syncwarp();
+    return got;
 }
 
 // Nanoseconds of the GPU-wide timer (the same clock on every SM, unlike clock64).

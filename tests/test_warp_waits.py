@@ -76,3 +76,15 @@ def test_a_product_of_another_shape_waits_for_the_one_that_reads_what_it_overwri
         end = loop.index(f"issue_abt(tmem + Cols::{overwrites},")
         before = loop[loop.rindex("commit(", 0, end):end]
         assert re.search(rf"kOwnDq\) wait\(2, .*&sh\.{reader}, k,|wait\(Cols::kOwnDq \? 2 : 1, .*&sh\.{reader}, k,", before), overwrites
+
+
+def test_a_vote_is_followed_by_a_barrier():
+    """Waits whose lanes poll different barriers: a vote does not order memory, so what one lane acquired is the others' (the one
+    that issues the product among them) only behind a warp barrier."""
+    with open(os.path.join(CSRC, "sm100_ptx.cuh")) as f:
+        text = re.sub(r"//[^\n]*", "", f.read())
+    for name in ("mbar_wait_warp", "mbar_wait_all", "mbar_wait_cluster"):
+        start = text.index(f"bool {name}(")
+        body = text[start:text.index("\n}\n", start)]
+        assert re.search(r"__syncwarp\(\);\s*return got;\s*$", body), name
+        assert body.count("return") == 1, name
