@@ -485,9 +485,11 @@ attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constan
                     tmem_ld_x32(st_tmem, *reinterpret_cast<uint32_t(*)[32]>(&sr[0]));
                     tmem_ld_x32(st_tmem + 32, *reinterpret_cast<uint32_t(*)[32]>(&sr[32]));
                     tmem_wait_ld();
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive_at(bar_s_read);
+                    if constexpr (!Cols::kOwnDq) {                   // dQ may have the columns
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive_at(bar_s_read);
+                    }
                     // the key is seen by the queries from `lo` of this thread's 64 on
                     const bool edge = key_tail || diag;
                     const int lo = !key_valid ? 64 : diag ? key - (i * kTile + half * 64) : -64;
