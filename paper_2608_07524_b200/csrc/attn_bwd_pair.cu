@@ -24,10 +24,11 @@
 //
 // so that the compute warps rarely wait: S(k+1) runs while they form dS(k), dP(k+1) while they form P(k+1).  Above head
 // dimension 96 dQ lives in the middle columns of S^T, which are free once S(k+1) has been read into registers (P^T is packed
-// into the outer ones); up to 96 it has columns of its own, so that S(k+1) does not wait for dQ(k-1) to be drained.  Every operand tile is used by exactly one product (Q and dO are loaded twice, as rows for S and dP
-// and as columns for dK and dV, since a CTA supplies half of B's columns), which leaves each single-buffered load
-// most of a period.  Between items nothing drains: the first S of an item follows the last dV of the previous one,
-// and the drain warps write dV and dK of an item while the next one is under way.
+// into the outer ones); up to 96 it has columns of its own, so that S(k+1) does not wait for dQ(k-1) to be drained.  Every
+// operand tile is used by exactly one product (Q and dO are loaded twice, as rows for S and dP and as columns for dK and dV,
+// since a CTA supplies half of B's columns), which leaves each single-buffered load most of a period.  Between items nothing
+// drains: the first S of an item follows the last dV of the previous one, and the drain warps write dV and dK of an item while
+// the next one is under way.
 //
 // The issuing warp paces the pipe (an MMA issue blocks while the pipe is busy, so what it does between two products
 // is idle time of the tensor cores; a barrier poll takes 100-250 cycles under load).  So there is one commit per
@@ -95,6 +96,15 @@ struct PairCols {
     static constexpr bool kOwnDq = kW == 96;
     static constexpr uint32_t kS = 0, kDp = 128, kDv = 256, kDk = 256 + kW, kDq = kOwnDq ? 256 + 2 * kW : kS + 32;
 };
+
+// The reductions of a dQ tile go out half a tile later: sent at once they delay the exchange of the next dS^T, which the next dQ
+// waits for (2 % of a tile's time on long sequences; 500 ns had no effect).  With columns of its own a dQ may leave later still,
+// which pays on long sequences: 65536 tokens x 16 heads of 72 and 96, without a mask, kRedDelayLongNs instead of kRedDelayNs at 384
+// tokens + 2 and + 6 %, 600 + 2 and + 4, 1000 + 1 and + 1, 2048 - 2 and - 1, 3000 - 3 and - 2, 8192 - 3 and - 3; causal 600 + 1
+// and + 3, 2048 + 1 and + 1, 8192 - 2 and - 2.  An item that writes its dQ directly sends none and does not wait: its dK is out
+// sooner (16 heads of 128: sequences of 200 tokens 597 -> 578 us, 256 494 -> 478, causal 598 -> 576; of 72 to 96 0 to - 2 %).
+constexpr unsigned kRedDelayNs = 900, kRedDelayLongNs = 1344;
+constexpr int kLongRed = 2048;
 
 struct PairControl {
     uint64_t work_full[kRing], work_empty[kRing];
@@ -369,7 +379,7 @@ attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constan
                                    b + (uint64_t)(((ks / 4) * 8192 + (ks % 4) * 32) >> 4), idesc_abt, ks > 0);
             if (leader) tc_mma_ss_pair(d_tmem, ones, stat, idesc_abt, true);
         };
-        // D[256 x 128] (+)= A B over the 128 queries; A = packed bf16 in tensor memory (columns 0-31 and 96-127 of `a_tmem`)
+        // D[256 x 96 or 128] (+)= A B over the 128 queries; A = packed bf16 in tensor memory (columns 0-31 and 96-127 of `a_tmem`)
         auto issue_acc = [&](uint32_t d_tmem, uint32_t a_tmem, uint64_t b, bool accumulate) {
 #pragma unroll
             for (int ks = 0; ks < 8; ++ks)
@@ -607,12 +617,7 @@ attn_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constan
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive_at(bar_free);
-                // the reductions go out half a tile later: sent at once they delay the exchange of the next dS^T, which the next
-                // dQ waits for (2 % of a tile's time on long sequences; 500 ns had no effect).  An item that writes its dQ directly
-                // sends none, and without the pause its dK is out sooner (65536 tokens, 16 heads of 128: sequences of 200 tokens
-                // 597 -> 578 us, 256: 494 -> 478, causal 598 -> 576; up to 96 columns no difference).  With columns of its own a dQ may leave later still, which pays on long sequences (one pause of 900 for
-                // all costs 2 to 3 % at 8000 tokens of 72; on short ones the longer pause holds the drain up: 256 tokens + 8 %).
-                if (Cols::kOwnDq || w.len > 2 * kTile) __nanosleep(Cols::kOwnDq && w.len > 2048 ? 1344 : 900);
+                if (w.len > 2 * kTile) __nanosleep(Cols::kOwnDq && w.len > kLongRed ? kRedDelayLongNs : kRedDelayNs);
                 const int row_in_tile = (int)rank * 64 + q_in_half, qrow = i * kTile + row_in_tile;
                 const bool live = qrow < w.len;
                 if (w.len <= 2 * kTile) {
