@@ -129,7 +129,9 @@ int device_info(DeviceInfo* out) {
 // 32-byte sector and a box of 64 columns ends well past its head (head dimensions 8, 24, 40, 72, 88, 104): there the larger
 // fetch costs the forward of single-tile items a tenth to a quarter (65536 tokens, 16 heads, us with 256 and with 128 bytes:
 // sequences of 60 tokens of 72 234 and 194, of 40 175 and 133, of 88 276 and 222; of 128 tokens of 72 134 and 126) and changes
-// nothing elsewhere.  128 bytes for all would cost the backward of 80 and 96 3 %, of 56 2 %; 64, 96 and 128 forward do not care.
+// nothing elsewhere; likewise sequences of 60 and of 128 tokens of 8 (146 and 116, 87 and 86), of 24 (181 and 149, 110 and 90) and
+// of 104 (320 and 277, 193 and 197).  128 bytes for all would cost the backward of 80 and 96 3 %, of 56 2 %; 64, 96 and 128
+// forward do not care.
 CUtensorMapL2promotion l2_promotion(int32_t head_dim) {
     return head_dim % 16 != 0 && head_dim % 64 <= 40 ? CU_TENSOR_MAP_L2_PROMOTION_L2_128B : CU_TENSOR_MAP_L2_PROMOTION_L2_256B;
 }

@@ -359,8 +359,9 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             // Up to three barriers, each polled by a lane of its own (the others poll the first) and the loop left by a vote:
             // the time to see a barrier is spent once and not one barrier after the other, while the tensor pipe idles.
             // 65536 tokens, 16 heads of 64, one barrier after the other -> together: 300 tokens 494 -> 487 us, causal 404 ->
-            // 391; 1200 causal 690 -> 667; 4096 3176 -> 3154, causal 1718 -> 1679.  Waits for a single barrier stay with
-            // mbar_wait_warp (by the vote 0 to 2 % slower).
+            // 391; 1200 causal 690 -> 667; 4096 3176 -> 3154, causal 1718 -> 1679.  Waits that are always for a single barrier
+            // stay with mbar_wait_warp (by the vote 0 to 2 % slower); that for P^T's first half, with dkv_free in an item's first
+            // tile, is by the vote in every tile (a branch to mbar_wait_warp in the others: 0 to 1 % slower).
             auto wait = [&](int n, uint64_t* b0, uint32_t p0, uint64_t* b1, uint32_t p1, uint64_t* b2, uint32_t p2) {
                 uint64_t* b = n > 1 && lane == 1 ? b1 : n > 2 && lane == 2 ? b2 : b0;
                 const uint32_t par = n > 1 && lane == 1 ? p1 : n > 2 && lane == 2 ? p2 : p0;

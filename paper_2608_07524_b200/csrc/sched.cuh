@@ -20,7 +20,7 @@
 namespace dcp {
 
 constexpr int kTile = 128;            // rows of a Q tile / keys of a K,V tile
-constexpr int kFwdRowsPerItem = 256;  // a forward work item is two Q tiles of one (sequence, head)
+constexpr int kFwdRowsPerItem = 256;  // a forward work item is two Q tiles of one (sequence, head), or one where items are few
 constexpr int kMergeMaxLen = 64;      // sequences longer than this are never merged with their neighbours
 
 // Status codes a kernel may leave in the workspace's status word (0 = no error).
@@ -124,7 +124,7 @@ struct WorkItem {
     int32_t tok0;   // first token of the sequence in the packed batch
     int32_t len;    // sequence length
     int32_t head;
-    int32_t blk;    // row block inside the sequence (256 query rows forward, 128 keys backward)
+    int32_t blk;    // block inside the sequence: 256 or 128 query rows forward, 128 keys backward (256 on CTA pairs)
     int32_t tile0;  // index of the sequence's first 128-row tile among all tiles of the batch
 };
 

@@ -109,8 +109,8 @@ class StreamRunner:
     """Runs planned batches out of pre-allocated device buffers.
 
     `batch` holds one batch in input order (inputs and results); micro-batches of a plan that splits
-    the batch are gathered into `stage` (allocated on first need, sized like `batch`), run there and
-    scattered back.  The synthetic stream reuses the first rows of `batch` for every batch (the values
+    the batch run on their rows of it if these lie side by side, else they are gathered into `stage`
+    (allocated on first need, sized like `batch`), run there and scattered back.  The synthetic stream reuses the first rows of `batch` for every batch (the values
     are random either way).
     """
 
@@ -182,8 +182,9 @@ class StreamRunner:
                                     dv=buf.dv[:T], workspace=self.ws)
 
     def run_micro_batch(self, mb: MicroBatch, batch_tokens: Optional[int] = None) -> int:
-        """Enqueue one micro-batch: forward (+ recompute forward) + backward, in place on the batch
-        buffers if it has no copy list, else gathered into the staging buffers and scattered back.
+        """Enqueue one micro-batch: forward (+ recompute forward) + backward.  In place on the batch buffers if it has
+        no copy list; on their rows, with only lse copied, if its sequences are neighbours in the batch; else gathered
+        into the staging buffers and scattered back.
         batch_tokens = rows of the batch the micro-batch was cut from (needed for the lse planes)."""
         lens = np.asarray(mb.lengths, dtype=np.int32)
         cu_dev, seg_dev, n_seg, T = self._upload(lens, mb.seg)
