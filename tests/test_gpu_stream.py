@@ -12,7 +12,7 @@ import oracle
 from paper_2608_07524_b200 import binding as B
 from paper_2608_07524_b200 import inputs
 from paper_2608_07524_b200.profiler import intra_candidates, select_group_setting
-from paper_2608_07524_b200.stream import StreamRunner, plan_batch, plan_length_group
+from paper_2608_07524_b200.stream import BatchPlan, MicroBatch, StreamRunner, plan_batch, plan_length_group
 
 pytestmark = pytest.mark.gpu
 
@@ -183,8 +183,8 @@ def test_algorithm_1_candidates_over_batch_size_and_sequence_parallel_size():
     assert (idx, r, t) == oracle.intra_select(cands, tight, lam) and cands[idx][1] >= 2
 
 
-@pytest.mark.parametrize("batch_size,in_place", [(1, True), (2, True), (3, True), (5, None)])
-def test_neighbours_run_where_they_are(batch_size, in_place):
+@pytest.mark.parametrize("batch_size", [1, 2, 3])
+def test_neighbours_run_where_they_are(batch_size):
     """Micro-batches of sequences that lie side by side in the batch (a length group's) need no gather: same results as the
     batch in one piece, at the first, a middle and a last, shorter micro-batch, and no staging rows are ever allocated."""
     n, L, H, d = 5, 300, 3, 128
@@ -192,13 +192,36 @@ def test_neighbours_run_where_they_are(batch_size, in_place):
     r.run_batch(plan_length_group(n, L, n, 0), n * L)
     want = [x.clone() for x in (r.o, r.lse, r.dk, r.dv, r.dq)]
     for x in (r.o, r.lse, r.dk, r.dv, r.dq):
-        x.fill_(7.0)
+        x.fill_(float("nan"))
     plan = plan_length_group(n, L, batch_size, 1 if batch_size == 2 else 0)
+    assert len(plan.micro_batches) == -(-n // batch_size) > 1
     r.run_batch(plan, n * L)
     r.check()
     for a, b in zip((r.o, r.lse, r.dk, r.dv), want):
         assert torch.equal(a, b)
     assert float((r.dq.float() - want[4].float()).abs().max()) <= 2e-2       # fp32 atomics: order may differ
     assert r.stage is None
-    if in_place:
-        assert len(plan.micro_batches) == -(-n // batch_size) > 1
+
+
+@pytest.mark.parametrize("lengths", [[300, 411, 0, 129, 70, 512, 257], [300, 0, 411, 129, 70, 512, 257]], ids=["empty last", "empty first"])
+@pytest.mark.parametrize("order", [[0, 1, 2], [1, 2, 0], [2, 0, 1]], ids=str)
+def test_neighbours_and_gathered_sequences_in_one_plan(order, lengths):
+    """One runner, one plan, both forms, whichever comes first: neighbours of different lengths, an empty one among them, that do
+    not start the batch, the batch's end on its own, and sequences from either side of them, which alone need staging rows."""
+    mb_id, H, d, T = [1, 0, 0, 1, 1, 2, 2], 3, 128, sum(lengths)
+    r = StreamRunner(T, len(lengths), H, d, True, "cuda", value_seed=12)
+    whole = BatchPlan([0] * len(lengths), [0], 0, [MicroBatch(np.asarray(lengths, np.int32), 0)])
+    r.run_batch(whole, T)
+    want = [x.clone() for x in (r.o, r.lse, r.dk, r.dv, r.dq)]
+    for x in (r.o, r.lse, r.dk, r.dv, r.dq):
+        x.fill_(float("nan"))
+    offset, index, _, seg_offset, seg = B.dcp_plan_segments(lengths, mb_id, 3, 64)
+    for k in order:
+        idx = index[offset[k]: offset[k + 1]]
+        staged = r.stage is not None
+        r.run_micro_batch(MicroBatch(np.asarray(lengths, np.int32)[idx], k, idx, seg[seg_offset[k]: seg_offset[k + 1]]), T)
+        assert (r.stage is not None) == (staged or k == 1)
+    r.check()
+    for a, b in zip((r.o, r.lse, r.dk, r.dv), want):
+        assert torch.equal(a, b)
+    assert float((r.dq.float() - want[4].float()).abs().max()) <= 2e-2       # fp32 atomics: order may differ
