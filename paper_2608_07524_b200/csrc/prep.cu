@@ -430,7 +430,7 @@ struct BlockList {
 // copy fetches it.  Also zeroes the fp32 dQ accumulator blocks of sequences longer than direct_len, one key block of the main
 // kernel (shorter ones get their dQ written directly by it), the columns that hold data.  HBM-bound.  Zeroing behind a
 // pass's loads, head_dim's columns instead of D, and the loads in flight below (us before and after, 65536 tokens x 16 heads): 64
-// columns 109 -> 97, 72 columns 193 -> 139, 128 columns 212 -> 186 (5.9 TB/s); text batch 251 -> 227, 2-D model's spatial axis
+// columns 112 -> 101, 72 columns 195 -> 140, 128 columns 215 -> 190 (5.8 TB/s); text batch 251 -> 227, 2-D model's spatial axis
 // 386 -> 353, of 72 370 -> 267.
 constexpr int kPreCtas = 6;      // per SM: 40 registers a thread
 template <int D>
@@ -535,7 +535,7 @@ cudaError_t launch_bwd_pre(const __nv_bfloat16* o, const __nv_bfloat16* d_o, con
 // shared memory as bf16 and writes whole rows.  Rows past the sequence end are skipped, and so are
 // sequences of at most direct_len tokens, whose dQ the main kernel has already written.  A thread's eight loads of a pass lie
 // a constant distance apart, columns past head_dim are not read, and the grid is one wave of resident CTAs (us before and after,
-// 65536 tokens x 16 heads): 64 columns 75 -> 69, 72 columns 126 -> 92, 128 columns 147 -> 133; text batch 178 -> 160, 2-D
+// 65536 tokens x 16 heads): 64 columns 75 -> 68, 72 columns 127 -> 91, 128 columns 148 -> 130; text batch 178 -> 160, 2-D
 // model's spatial axis 253 -> 222.
 constexpr int kPostCtas = 4;     // per SM: 64 registers a thread, 35 KB of shared memory
 template <int D>
